@@ -62,7 +62,7 @@ AOParams Plan::ao_params() const {
   a.d0_d = d0_d; a.d0_hi = d0_hi; a.d0_lo = d0_lo; a.t0 = t0; a.kint = kint;
   for (int d = 0; d < 3; ++d) a.nb[d] = nb[d];
   a.nblk = nblk; a.lmax = lmax; a.nsa = nsa; a.blist = blist; a.bpre = bpre;
-  a.cs = cs;
+  a.cs = nullptr;
   return a;
 }
 
@@ -643,8 +643,7 @@ void free_plan(Plan* p) {
   void* bufs[] = {p->shells, p->atom_shell0, p->img_d, p->img_hi, p->img_lo, p->img_phase,
                   p->d0_d, p->d0_hi, p->d0_lo, p->t0, p->kint, p->psi, p->Y, p->scratch,
                   p->kc, p->xi, p->mmat, p->ek, p->dacc, p->status, p->h_c, p->h_kc, p->h_k,
-                  p->h_ex, p->ao_norm, p->cs, p->blist, p->bpre, p->shell_list_l[0], p->shell_list_l[1], p->shell_list_l[2],
-                  p->shell_list_l[3]};
+                  p->h_ex, p->ao_norm, p->cs, p->blist, p->bpre};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (p->scratch2) cudaFree(p->scratch2);
@@ -661,6 +660,7 @@ void free_plan(Plan* p) {
   if (p->aux) cudaStreamDestroy(p->aux);
   if (p->aux2) cudaStreamDestroy(p->aux2);
   if (p->tc) tc_plan_free(p->tc);
+  chi_free(p->chi);
   for (cudaEvent_t e : p->ev_used) cudaEventDestroy(e);
   for (cudaEvent_t e : p->ev_free) cudaEventDestroy(e);
   delete p;
@@ -733,14 +733,14 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
     return OCCRI_ECUDA;
   {
     StageTimer t(p, timed);
-    if (launch_scale_c<T>(*p, C, s) != cudaSuccess) return OCCRI_ECUDA;
-    if (launch_orbitals<T>(*p, s) != cudaSuccess) return OCCRI_ECUDA;
+    if (launch_slot_c<T>(*p, C, p->cs, 1.0, s) != cudaSuccess) return OCCRI_ECUDA;
+    if (launch_orbitals<T>(*p, 1, &p->cs, &p->psi, s) != cudaSuccess) return OCCRI_ECUDA;
     // the pair passes work on the periodic parts u = e^{-ik.r} psi: the pair density
     // conj(u_jk') u_ik is then periodic as it stands, and the accumulated periodic part
     // e^{-ik.r} Y_ik needs no phase either (Y is restored below)
     if (launch_phase_fields<T>(*p, p->psi, -1, s) != cudaSuccess) return OCCRI_ECUDA;
     t.done(OCCRI_STAGE_ORBITALS, p->nk);
-    launches += 2 + (p->nocc + kOrbChunk - 1) / kOrbChunk;
+    launches += 2 + chi_launches(*p, false);
   }
   {
     // Waves go round-robin over the plan's stream and one or two auxiliary ones, each with
@@ -834,10 +834,11 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
       if (launch_contract_tc(*p, s, &spans) != cudaSuccess) return OCCRI_ECUDA;
       launches += tc_plan_launches(p->tc);
     } else {
-      if (launch_contract<T>(*p, s) != cudaSuccess) return OCCRI_ECUDA;
-      for (int l = 0; l < 4; ++l)
-        if (!p->shells_by_l[l].empty())
-          launches += (p->nocc + contract_chunk<T>() - 1) / contract_chunk<T>();
+      // Y carries N_g/(4 pi) (see PairParams), hence -Omega 4 pi / (N_k N_g^2)
+      const double scale = -p->omega_cell * 4.0 * kPiD /
+                           ((double)p->nk * (double)p->ng * (double)p->ng);
+      if (launch_contract_field<T>(*p, p->Y, p->kc, scale, s) != cudaSuccess) return OCCRI_ECUDA;
+      launches += chi_launches(*p, true);
     }
     t.done(OCCRI_STAGE_CONTRACT, p->nk);
   }
@@ -875,8 +876,8 @@ int vjp_impl(Plan* p, const double2* C, double gEx, void* gC, double* gomega) {
     if (p->kernel.kind == OCCRI_ERFC || p->kernel.kind == OCCRI_ERF) {
       // periodic parts of the orbitals of C (the plan's copy may have been replaced by
       // an occri_orbitals call since the build)
-      if (launch_scale_c<T>(*p, C, s) != cudaSuccess) return OCCRI_ECUDA;
-      if (launch_orbitals<T>(*p, s) != cudaSuccess) return OCCRI_ECUDA;
+      if (launch_slot_c<T>(*p, C, p->cs, 1.0, s) != cudaSuccess) return OCCRI_ECUDA;
+      if (launch_orbitals<T>(*p, 1, &p->cs, &p->psi, s) != cudaSuccess) return OCCRI_ECUDA;
       if (launch_phase_fields<T>(*p, p->psi, -1, s) != cudaSuccess) return OCCRI_ECUDA;
       for (int k = 0; k < p->nk; ++k)
         for (int kp0 = k; kp0 < p->nk;) {
@@ -901,7 +902,7 @@ int vjp_full_impl(Plan* p, const double2* C, double gEx, const double2* gKC, con
   cudaStream_t s = p->stream;
   const size_t nkc = (size_t)p->nk * p->nao * p->nocc;
   const size_t orb = (size_t)p->nk * p->nocc * p->fs * sizeof(cplx_t<T>);
-  const size_t csb = (p->precision == OCCRI_FP64 ? sizeof(double2) : sizeof(float4)) * nkc;
+  const size_t csb = 16 * (size_t)p->nk * chi_slots(*p) * p->nocc;   // double2 or float4
   if (!p->gam) {   // first call: the adjoint workspaces
     bool ok = device_malloc(&p->gam, orb) == cudaSuccess &&
               device_malloc(&p->gpsi, orb) == cudaSuccess &&
@@ -926,11 +927,12 @@ int vjp_full_impl(Plan* p, const double2* C, double gEx, const double2* gKC, con
                                             p->gcf, p->nao, p->nocc, tol, p->status);
   // the adjoint orbital field g = -sum_mu chi_mu dL/dKC_mu (in units that leave out the
   // contraction's Omega/(N_k N_g)) and the orbitals of C, both as periodic parts
-  if (launch_scale_to<T>(*p, p->gkc, p->cs_g, -1.0, s) != cudaSuccess) return OCCRI_ECUDA;
-  if (launch_orbitals_to<T>(*p, p->cs_g, p->gam, s) != cudaSuccess) return OCCRI_ECUDA;
+  if (launch_slot_c<T>(*p, p->gkc, p->cs_g, -1.0, s) != cudaSuccess) return OCCRI_ECUDA;
+  if (launch_slot_c<T>(*p, C, p->cs, 1.0, s) != cudaSuccess) return OCCRI_ECUDA;
+  const void* coefs[2] = {p->cs_g, p->cs};
+  void* fields[2] = {p->gam, p->psi};
+  if (launch_orbitals<T>(*p, 2, coefs, fields, s) != cudaSuccess) return OCCRI_ECUDA;
   if (launch_phase_fields<T>(*p, p->gam, -1, s) != cudaSuccess) return OCCRI_ECUDA;
-  if (launch_scale_c<T>(*p, C, s) != cudaSuccess) return OCCRI_ECUDA;
-  if (launch_orbitals<T>(*p, s) != cudaSuccess) return OCCRI_ECUDA;
   if (launch_phase_fields<T>(*p, p->psi, -1, s) != cudaSuccess) return OCCRI_ECUDA;
   // (c)+(d): two round trips per unordered pair, dL/dpsi accumulated (and the omega
   // term of the kernel's derivative, for the erfc and erf kernels)
@@ -1386,7 +1388,6 @@ int occri_plan_create(occri_plan** out, const occri_cell* cell, const occri_kmes
     x.rcut2_f = (float)x.rcut2;
     rcut_max = std::max(rcut_max, rcut[s]);
     ao += 2 * x.l + 1;
-    p->shells_by_l[x.l].push_back(s);
   }
   std::vector<double> ao_norm(nao);
   for (int s = 0; s < p->nshell; ++s)
@@ -1570,16 +1571,8 @@ int occri_plan_create(occri_plan** out, const occri_cell* cell, const occri_kmes
   auto chk = [&](cudaError_t x) { if (e == cudaSuccess && x != cudaSuccess) e = x; };
   chk(upload(&p->shells, sh, &tot));
   chk(upload(&p->atom_shell0, atom_shell0, &tot));
-  for (int l = 0; l < 4; ++l) chk(upload(&p->shell_list_l[l], p->shells_by_l[l], &tot));
   chk(upload(&p->kint, p->kint_h, &tot));
   chk(upload(&p->ao_norm, ao_norm, &tot));
-  {
-    unsigned char* b = nullptr;
-    const size_t csb = (precision == OCCRI_FP64 ? sizeof(double2) : sizeof(float4)) *
-                       (size_t)p->nk * nao * nocc;
-    chk(dalloc(&b, csb, &tot));
-    p->cs = b;
-  }
   chk(upload(&p->t0, t0, &tot));
   chk(upload(&p->blist, blist, &tot));
   chk(upload(&p->bpre, bpre, &tot));
@@ -1602,6 +1595,16 @@ int occri_plan_create(occri_plan** out, const occri_cell* cell, const occri_kmes
     float2* ph = nullptr;
     chk(upload(&ph, ph_f, &tot));
     p->img_phase = ph;
+  }
+  if (e == cudaSuccess) {
+    std::vector<int> img_n;
+    for (const Img& m : imgs) img_n.insert(img_n.end(), m.n, m.n + 3);
+    chk(chi_create(p, sh, rcut, lists, bpre, img_n, t0, atom_shell0, &tot));
+  }
+  if (e == cudaSuccess) {
+    unsigned char* b = nullptr;
+    chk(dalloc(&b, 16 * (size_t)p->nk * chi_slots(*p) * nocc, &tot));   // double2 or float4
+    p->cs = b;
   }
   const size_t csz = (precision == OCCRI_FP64) ? sizeof(double2) : sizeof(float2);
   p->fs = (ng + 63) / 64 * 64;
@@ -1984,12 +1987,12 @@ int occri_orbitals(occri_plan* plan, const void* C_dev, void* psi_dev) {
   Plan* p = plan->p;
   cudaError_t e;
   if (p->precision == OCCRI_FP64) {
-    e = occri::launch_scale_c<double>(*p, (const double2*)C_dev, p->stream);
-    if (e == cudaSuccess) e = occri::launch_orbitals<double>(*p, p->stream);
+    e = occri::launch_slot_c<double>(*p, (const double2*)C_dev, p->cs, 1.0, p->stream);
+    if (e == cudaSuccess) e = occri::launch_orbitals<double>(*p, 1, &p->cs, &p->psi, p->stream);
     if (e == cudaSuccess) e = occri::launch_widen<double>(*p, psi_dev, p->stream);
   } else {
-    e = occri::launch_scale_c<float>(*p, (const double2*)C_dev, p->stream);
-    if (e == cudaSuccess) e = occri::launch_orbitals<float>(*p, p->stream);
+    e = occri::launch_slot_c<float>(*p, (const double2*)C_dev, p->cs, 1.0, p->stream);
+    if (e == cudaSuccess) e = occri::launch_orbitals<float>(*p, 1, &p->cs, &p->psi, p->stream);
     if (e == cudaSuccess) e = occri::launch_widen<float>(*p, psi_dev, p->stream);
   }
   return e == cudaSuccess ? OCCRI_OK : OCCRI_ECUDA;

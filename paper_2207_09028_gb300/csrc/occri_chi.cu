@@ -1,0 +1,978 @@
+// occri_chi.cu -- Bloch AOs on the grid in tiles, and the two products with them:
+//   (a) chi_{mu k}(r) = sum_T e^{i k.T} phi_mu(r - A - T)                     (Sec. II.A)
+//   (b) psi_{ik}(r) = sum_mu C^k_{mu i} chi_{mu k}(r)                          (Eq. occmo)
+//   (e) K_{mu i}(k) = -(Omega/(N_k N_g)) sum_r conj(chi_{mu k}(r)) Y_{ik}(r)   (Eq. occrik)
+//
+// chi_kernel forms chi for a run of point blocks (2 x 4 x 4 points each) and every k at once:
+// the Gaussian of an image is evaluated once, summed with the other images of its residue
+// class (lattice vectors equal modulo the k-mesh's supercell share e^{i k.T}), and only the
+// class sums meet the phases. orb_kernel and con_kernel are the products, one block per warp
+// with a point per lane. Blocks keep only the AOs that reach them: an atom's shells are
+// ordered by screening radius, so the AOs that reach a block are a prefix of the atom's slots.
+//
+// Before this, each step evaluated the Gaussians itself, once per four k-points in (b) and
+// once per k-point in (e), with every image's phases applied on the spot.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <mutex>
+#include <new>
+#include <numeric>
+#include <vector>
+
+#include "occri_ao.cuh"
+#include "occri_device.cuh"
+#include "occri_internal.h"
+
+namespace occri {
+
+// One shell in slot order.
+struct ChiShell {
+  double alpha_d, rcut2_d;
+  float alpha, alpha_lo, rcut2;
+  int l, slot, orig, exact;   // first slot within the atom; index in the basis; FP32 exponents
+};
+
+// Blocks [b0, b1): one filling of the chi buffer, with the contraction's work items and the
+// first of its rows_of entries.
+struct ChiChunk {
+  int b0, b1, item0, nitems, row_of0;
+};
+
+struct ChiTables {
+  std::vector<ChiChunk> chunks;
+  int nslots = 0;                 // slots of all atoms, each atom's padded to kChiPad
+  int ncls = 0, nkp = 0;          // residue classes in use; k-points padded to 8
+  int lsm = 0;                    // image records kept in shared memory (0: read from global)
+  int parts = 1;                  // CTAs per (block, atom) of chi_kernel
+  size_t chi_bytes = 0;
+  // device
+  ChiShell* shells = nullptr;     // [nshell] per atom, falling screening radius
+  int* slot0 = nullptr;           // [natm + 1] first slot of each atom
+  int* slot_ao = nullptr;         // [nslots] AO of a slot, or -1 (padding)
+  unsigned short* nsh = nullptr;  // [natm][nblk] shells that reach the block
+  int* aoff = nullptr;            // [nblk][natm + 1] slots of the block before atom a
+  long long* boff = nullptr;      // [nblk] slots of all blocks before this one in its chunk
+  unsigned short* t0i = nullptr;  // [natm][nblk] row of the class table (one per distinct T0)
+  int* cls = nullptr;             // [T0][nimg] class of T0 + T'
+  unsigned short* order = nullptr;   // [natm][nblk][lmax] list positions sorted by class
+  void* phase = nullptr;          // [ncls][nkp] e^{i k.T} of each class
+  int4* items = nullptr;          // contraction: (atom, first slot, first block, blocks)
+  int* border = nullptr;          // blocks per (chunk, atom) by falling number of slots
+  int2* rows = nullptr;           // runs of blocks: (first item in the chunk, slot groups)
+  int2* rows_of = nullptr;        // [chunk][natm] (first run, runs)
+  double* part = nullptr;         // [k][item][values] sums of the items
+  size_t part_bytes = 0;
+  void* chi = nullptr;            // [block][k][slot][32 points]
+  void* arena = nullptr;          // the one allocation behind all of these
+};
+
+namespace chi {
+
+using ao::Disp;
+
+constexpr int kPad = 4;         // slots per group: chi_kernel pads with zeros, the products
+                                // take kPad AOs at a time
+constexpr int kWarps = 4;       // warps of a chi_kernel CTA
+template <typename T> constexpr int rows() { return sizeof(T) == 4 ? 96 : 64; }
+
+template <typename T> struct Rec;
+template <> struct alignas(16) Rec<float> { float xh, yh, zh; int cls; float xl, yl, zl; int pad; };
+template <> struct alignas(16) Rec<double> { double x, y, z; int cls, pad; };
+
+template <typename T> struct CsT;
+template <> struct CsT<double> { using type = double2; };
+template <> struct CsT<float> { using type = float4; };
+
+struct Params {
+  AOParams a;
+  const ChiShell* shells;
+  const int* slot0;
+  const int* slot_ao;
+  const unsigned short* nsh;
+  const int* aoff;
+  const long long* boff;
+  const unsigned short* t0i;
+  const int* cls;
+  const unsigned short* order;
+  const void* phase;
+  const int4* items;
+  const int* border;
+  const int2* rows;
+  const int2* rows_of;
+  double* part;
+  const double* ao_norm;
+  int nslots, ncls, nkp, lsm, parts;
+};
+
+template <typename T>
+__device__ __forceinline__ Rec<T> load_rec(const Params& p, size_t list0, const int* cls, int j) {
+  const int id = p.a.blist[list0 + j];
+  Rec<T> r;
+  if constexpr (sizeof(T) == 4) {
+    r.xh = p.a.img_hi[id];
+    r.yh = p.a.img_hi[p.a.nimg + id];
+    r.zh = p.a.img_hi[2 * p.a.nimg + id];
+    r.xl = p.a.img_lo[id];
+    r.yl = p.a.img_lo[p.a.nimg + id];
+    r.zl = p.a.img_lo[2 * p.a.nimg + id];
+  } else {
+    r.x = p.a.img_d[id];
+    r.y = p.a.img_d[p.a.nimg + id];
+    r.z = p.a.img_d[2 * p.a.nimg + id];
+  }
+  r.cls = cls[id];
+  r.pad = 0;
+  return r;
+}
+
+// The 2L + 1 functions of a shell (without their norms) at displacement d - T, 0 past the
+// screening radius.
+template <int L>
+__device__ __forceinline__ void eval(const ChiShell& sh, const Disp<float>& d,
+                                     const Rec<float>& r, float (&v)[2 * L + 1]) {
+  float x, y, z, r2, e;
+  if (sh.exact) {
+    e = ao::exact_gauss(d, r.xh, r.yh, r.zh, r.xl, r.yl, r.zl, sh.alpha, sh.alpha_lo, &r2, &x, &y,
+                        &z);
+  } else {
+    x = (d.xh - r.xh) + (d.xl - r.xl);
+    y = (d.yh - r.yh) + (d.yl - r.yl);
+    z = (d.zh - r.zh) + (d.zl - r.zl);
+    r2 = x * x + y * y + z * z;
+    e = expf(-(sh.alpha * r2 + sh.alpha_lo * r2));
+  }
+  if (!(r2 <= sh.rcut2)) e = 0.f;
+  ao::solid<float, L>(x, y, z, v);
+#pragma unroll
+  for (int m = 0; m < 2 * L + 1; ++m) v[m] *= e;
+}
+template <int L>
+__device__ __forceinline__ void eval(const ChiShell& sh, const Disp<double>& d,
+                                     const Rec<double>& r, double (&v)[2 * L + 1]) {
+  const double x = d.x - r.x, y = d.y - r.y, z = d.z - r.z;
+  const double r2 = x * x + y * y + z * z;
+  double e = exp(-(sh.alpha_d * r2));
+  if (!(r2 <= sh.rcut2_d)) e = 0.0;
+  ao::solid<double, L>(x, y, z, v);
+#pragma unroll
+  for (int m = 0; m < 2 * L + 1; ++m) v[m] *= e;
+}
+
+// acc[b][m] += phases of KT k-points times the entries' values
+template <typename T, int KT, int NM>
+__device__ __forceinline__ void phase_sums(const cplx_t<T>* ph, int nkp, const T* ent,
+                                           const int* ecls, int ne, int k0, int lane,
+                                           T (&xr)[KT][NM], T (&xi)[KT][NM]) {
+  for (int e = 0; e < ne; ++e) {
+    const cplx_t<T>* row = ph + (size_t)ecls[e] * nkp + k0;
+    cplx_t<T> w[KT];
+    if constexpr (sizeof(T) == 4 && KT % 2 == 0) {
+#pragma unroll
+      for (int b = 0; b < KT; b += 2) {
+        const float4 q = __ldg(reinterpret_cast<const float4*>(row + b));
+        w[b] = cplx_t<T>{q.x, q.y};
+        w[b + 1] = cplx_t<T>{q.z, q.w};
+      }
+    } else {
+#pragma unroll
+      for (int b = 0; b < KT; ++b) w[b] = __ldg(row + b);
+    }
+    T v[NM];
+#pragma unroll
+    for (int m = 0; m < NM; ++m) v[m] = ent[(e * NM + m) * 32 + lane];
+#pragma unroll
+    for (int b = 0; b < KT; ++b)
+#pragma unroll
+      for (int m = 0; m < NM; ++m) {
+        xr[b][m] += w[b].x * v[m];
+        xi[b][m] += w[b].y * v[m];
+      }
+  }
+}
+
+// One shell at the warp's block: class sums into the warp's entries (a lane reads back only
+// what it wrote), then chi of every k. Where the entries run out, the sums so far go to chi
+// and the rest is added.
+template <typename T, int L, int KT, typename GetRec, typename GetOrder>
+__device__ __forceinline__ void shell_chi(const Params& p, const ChiShell& sh, const Disp<T>& d,
+                                          int np, int n_all, const GetRec& rec,
+                                          const GetOrder& order, T* ent, int* ecls,
+                                          cplx_t<T>* out, int kstride, int lane) {
+  constexpr int NM = 2 * L + 1;
+  constexpr int CAP = rows<T>() / NM;
+  const cplx_t<T>* ph = reinterpret_cast<const cplx_t<T>*>(p.phase);
+  const int nk = p.a.nk;
+  // Images in order of distance, each its own entry, or (where it saves more phase products
+  // than the scan costs) in order of class, with the images past the shell's reach skipped.
+  const bool fold = p.ncls == 1;
+  const bool by_class = !fold && p.order != nullptr &&
+                        (long long)(np - p.ncls) * (2 * nk * NM + 8) > 3 * n_all;
+  const int nt = by_class ? n_all : np;
+  bool first = true;
+  int ne = 0, cur = -1;
+  T acc[NM];
+#pragma unroll
+  for (int m = 0; m < NM; ++m) acc[m] = T(0);
+  auto close = [&]() {   // the class sum becomes an entry
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+      ent[(ne * NM + m) * 32 + lane] = acc[m];
+      acc[m] = T(0);
+    }
+    if (lane == 0) ecls[ne] = cur;
+    ++ne;
+  };
+  auto spill = [&]() {   // the entries' share of chi
+    __syncwarp();
+    for (int k0 = 0; k0 < nk; k0 += KT) {
+      T xr[KT][NM], xi[KT][NM];
+#pragma unroll
+      for (int b = 0; b < KT; ++b)
+#pragma unroll
+        for (int m = 0; m < NM; ++m) xr[b][m] = xi[b][m] = T(0);
+      phase_sums<T, KT, NM>(ph, p.nkp, ent, ecls, ne, k0, lane, xr, xi);
+#pragma unroll
+      for (int b = 0; b < KT; ++b) {
+        if (k0 + b >= nk) break;
+        cplx_t<T>* o = out + (size_t)(k0 + b) * kstride + lane;
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+          cplx_t<T> v{xr[b][m], xi[b][m]};
+          if (!first) {
+            const cplx_t<T> u = o[32 * m];
+            v.x += u.x;
+            v.y += u.y;
+          }
+          o[32 * m] = v;
+        }
+      }
+    }
+    __syncwarp();
+    ne = 0;
+    first = false;
+  };
+  for (int t = 0; t < nt; ++t) {
+    const int j = by_class ? order(t) : t;
+    if (j >= np) continue;   // uniform
+    const Rec<T> r = rec(j);
+    if (cur >= 0 && !fold && (!by_class || r.cls != cur)) {
+      close();
+      if (ne == CAP) spill();
+    }
+    cur = r.cls;
+    T v[NM];
+    eval<L>(sh, d, r, v);
+#pragma unroll
+    for (int m = 0; m < NM; ++m) acc[m] += v[m];
+  }
+  close();
+  spill();
+}
+
+// chi of the blocks [blk0, blk0 + gridDim.x) for one atom: warps take the atom's shells in
+// turn, a lane is a grid point. Each Gaussian is evaluated once for all k, so the kernel is
+// bound by its stores where there are many k-points and by the evaluation where there are few.
+template <typename T, int KS, int KL>
+__global__ void __launch_bounds__(32 * kWarps, 4)
+chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* ents = reinterpret_cast<T*>(smem_raw);
+  int* eclss = reinterpret_cast<int*>(ents + kWarps * rows<T>() * 32);
+  Rec<T>* recs = reinterpret_cast<Rec<T>*>(eclss + kWarps * rows<T>());
+  unsigned short* ord = reinterpret_cast<unsigned short*>(recs + p.lsm);
+  const int blk = blk0 + blockIdx.x, a = blockIdx.y;
+  const size_t ab = (size_t)a * p.a.nblk + blk;
+  const int nact = p.nsh[ab];
+  if (nact == 0) return;
+  const int s0 = p.a.atom_shell0[a];
+  const unsigned short* pre = p.a.bpre + ab * p.a.nsa;
+  const size_t list0 = ab * p.a.lmax;
+  const int n_all = pre[p.shells[s0].orig - s0];   // the widest shell's images
+  const int* cls = p.cls + (size_t)p.t0i[ab] * p.a.nimg;
+  const bool in_smem = p.lsm > 0;
+  if (in_smem) {
+    for (int j = threadIdx.x; j < n_all; j += blockDim.x) {
+      recs[j] = load_rec<T>(p, list0, cls, j);
+      if (p.order) ord[j] = p.order[list0 + j];
+    }
+    __syncthreads();
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  bool valid;
+  long long q;
+  const long long n = ao::block_point(p.a, blk, lane, &valid, &q);
+  Disp<T> d;
+  ao::load_disp(p.a, a, n, &d);
+  const int* aoff = p.aoff + (size_t)blk * (p.a.natm + 1);
+  const int kstride = 32 * aoff[p.a.natm];
+  cplx_t<T>* base = chi + (size_t)(p.boff[blk] * p.a.nk + aoff[a]) * 32;
+  T* ent = ents + warp * rows<T>() * 32;
+  int* ecls = eclss + warp * rows<T>();
+  auto rec = [&](int j) -> Rec<T> { return in_smem ? recs[j] : load_rec<T>(p, list0, cls, j); };
+  auto order = [&](int t) -> int { return in_smem ? ord[t] : p.order[list0 + t]; };
+  for (int s = warp + kWarps * blockIdx.z; s < nact; s += kWarps * gridDim.z) {
+    const ChiShell sh = p.shells[s0 + s];
+    const int np = pre[sh.orig - s0];
+    cplx_t<T>* out = base + 32 * (size_t)sh.slot;
+    switch (sh.l) {
+      case 0: shell_chi<T, 0, KS>(p, sh, d, np, n_all, rec, order, ent, ecls, out, kstride, lane); break;
+      case 1: shell_chi<T, 1, KS>(p, sh, d, np, n_all, rec, order, ent, ecls, out, kstride, lane); break;
+      case 2: shell_chi<T, 2, KL>(p, sh, d, np, n_all, rec, order, ent, ecls, out, kstride, lane); break;
+      default: shell_chi<T, 3, KL>(p, sh, d, np, n_all, rec, order, ent, ecls, out, kstride, lane); break;
+    }
+  }
+  if (blockIdx.z == 0 && warp == kWarps - 1) {   // padding slots of the atom's last group
+    const ChiShell& last = p.shells[s0 + nact - 1];
+    for (int s = last.slot + 2 * last.l + 1; s < aoff[a + 1] - aoff[a]; ++s)
+      for (int k = 0; k < p.a.nk; ++k)
+        base[(size_t)k * kstride + 32 * s + lane] = cplx_t<T>{T(0), T(0)};
+  }
+}
+
+// List positions of every (atom, block) in order of class, once at plan creation: a warp per
+// list, which appends the images of one class after another.
+__global__ void __launch_bounds__(256)
+order_kernel(Params p, unsigned short* __restrict__ order) {
+  const int ab = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int a = ab / p.a.nblk, s0 = p.a.atom_shell0[min(a, p.a.natm - 1)];
+  if (a >= p.a.natm || p.nsh[ab] == 0) return;
+  const size_t list0 = (size_t)ab * p.a.lmax;
+  const int n = p.a.bpre[(size_t)ab * p.a.nsa + p.shells[s0].orig - s0];
+  const int* cls = p.cls + (size_t)p.t0i[ab] * p.a.nimg;
+  int at = 0;
+  for (int c = 0; c < p.ncls && at < n; ++c)
+    for (int j0 = 0; j0 < n; j0 += 32) {
+      const int j = j0 + lane;
+      const bool in = j < n && cls[p.a.blist[list0 + j]] == c;
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (in) order[list0 + at + __popc(m & ((1u << lane) - 1u))] = (unsigned short)j;
+      at += __popc(m);
+    }
+}
+
+// t += c x; in FP32 the coefficient is a hi/lo pair
+__device__ __forceinline__ void cmac(const double2& c, const double2& x, double2& t) {
+  t.x += c.x * x.x - c.y * x.y;
+  t.y += c.x * x.y + c.y * x.x;
+}
+__device__ __forceinline__ void cmac(const float4& c, const float2& x, float2& t) {
+  t.x = fmaf(c.x, x.x, fmaf(-c.y, x.y, fmaf(c.z, x.x, fmaf(-c.w, x.y, t.x))));
+  t.y = fmaf(c.x, x.y, fmaf(c.y, x.x, fmaf(c.z, x.y, fmaf(c.w, x.x, t.y))));
+}
+
+// psi_ik at one block per warp: kPad AOs are summed on their own before they join the
+// orbital's sum, so that few roundings happen at its full size.
+template <typename T, int NI>
+__global__ void __launch_bounds__(128)
+orb_kernel(Params p, const cplx_t<T>* __restrict__ chi, const typename CsT<T>::type* __restrict__ cs,
+           cplx_t<T>* __restrict__ psi, int blk0, int nb, int i0) {
+  const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (w >= nb) return;
+  const int blk = blk0 + w, k = blockIdx.y, lane = threadIdx.x & 31;
+  const int nocc = p.a.nocc;
+  const int* aoff = p.aoff + (size_t)blk * (p.a.natm + 1);
+  const cplx_t<T>* x0 = chi + ((size_t)p.boff[blk] * p.a.nk + (size_t)k * aoff[p.a.natm]) * 32 + lane;
+  cplx_t<T> acc[NI];
+#pragma unroll
+  for (int i = 0; i < NI; ++i) acc[i] = cplx_t<T>{T(0), T(0)};
+  for (int a = 0; a < p.a.natm; ++a) {
+    const int n = aoff[a + 1] - aoff[a];
+    const cplx_t<T>* xa = x0 + (size_t)aoff[a] * 32;
+    const typename CsT<T>::type* ca = cs + ((size_t)k * p.nslots + p.slot0[a]) * nocc + i0;
+#pragma unroll 2
+    for (int s = 0; s < n; s += kPad) {
+      cplx_t<T> x[kPad];
+#pragma unroll
+      for (int u = 0; u < kPad; ++u) x[u] = __ldg(xa + (size_t)(s + u) * 32);
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        if (i0 + i >= nocc) break;
+        cplx_t<T> t{T(0), T(0)};
+#pragma unroll
+        for (int u = 0; u < kPad; ++u) cmac(__ldg(ca + (size_t)(s + u) * nocc + i), x[u], t);
+        acc[i].x += t.x;
+        acc[i].y += t.y;
+      }
+    }
+  }
+  bool valid;
+  long long q;
+  ao::block_point(p.a, blk, lane, &valid, &q);
+  if (!valid) return;
+#pragma unroll
+  for (int i = 0; i < NI; ++i)
+    if (i0 + i < nocc) psi[((size_t)k * nocc + i0 + i) * p.a.fs + q] = acc[i];
+}
+
+// Sum over the lanes of a warp of NV values per lane, by halving: after the exchange over lane
+// bit b each lane keeps half of its values. Lane l ends with the sums of the values j with
+// j mod (NV / 32) free and the rest its bit-reversed position (index returned through idx).
+// FP32 values travel as hi + lo pairs (error-free sums), so nothing is lost across lanes.
+__device__ __forceinline__ void pair_add(float& ah, float& al, float bh, float bl) {
+  float s, e;
+  ao::two_sum(ah, bh, s, e);
+  ah = s;
+  al = al + bl + e;
+}
+template <typename T, int NV>
+__device__ __forceinline__ void halve_lanes(T (&v)[NV], double (&out)[NV / 32], int lane) {
+  static_assert(NV % 32 == 0, "a whole number of values per lane");
+  if constexpr (sizeof(T) == 8) {
+#pragma unroll
+    for (int step = 0; step < 5; ++step) {
+      const int half = NV >> (step + 1);
+      const bool up = (lane >> (4 - step)) & 1;
+#pragma unroll
+      for (int j = 0; j < half; ++j) {
+        const T mine = up ? v[j + half] : v[j], other = up ? v[j] : v[j + half];
+        v[j] = mine + __shfl_xor_sync(0xffffffffu, other, 16 >> step);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < NV / 32; ++j) out[j] = v[j];
+  } else {
+    T lo[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) lo[j] = T(0);
+#pragma unroll
+    for (int step = 0; step < 5; ++step) {
+      const int half = NV >> (step + 1);
+      const bool up = (lane >> (4 - step)) & 1;
+#pragma unroll
+      for (int j = 0; j < half; ++j) {
+        T mh = up ? v[j + half] : v[j], ml = up ? lo[j + half] : lo[j];
+        const T oh = up ? v[j] : v[j + half], ol = up ? lo[j] : lo[j + half];
+        const T rh = __shfl_xor_sync(0xffffffffu, oh, 16 >> step);
+        const T rl = step ? __shfl_xor_sync(0xffffffffu, ol, 16 >> step) : T(0);
+        pair_add(mh, ml, rh, rl);
+        v[j] = mh;
+        lo[j] = ml;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < NV / 32; ++j) out[j] = (double)v[j] + (double)lo[j];
+  }
+}
+
+// Partial sums over r of conj(chi) F: a warp takes kPad AOs of an atom over a run of the blocks
+// they reach (work items, made with the plan), sums per lane in the working precision, then
+// over the lanes in 64 bits. sum_kernel adds the items in a fixed order, so that the result
+// does not depend on the order in which they ran.
+template <typename T, int NI>
+__global__ void __launch_bounds__(256, 2)
+con_kernel(Params p, const cplx_t<T>* __restrict__ chi, const cplx_t<T>* __restrict__ F,
+           int item0, int nitems, int i0) {
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (w >= nitems) return;
+  const int k = blockIdx.y, lane = threadIdx.x & 31;
+  const int4 it = p.items[item0 + w];
+  const int nocc = p.a.nocc;
+  const cplx_t<T>* f0 = F + ((size_t)k * nocc + i0) * p.a.fs;
+  constexpr int NV = 2 * kPad * NI;
+  T acc[NV];   // [slot][i][re, im]
+#pragma unroll
+  for (int j = 0; j < NV; ++j) acc[j] = T(0);
+#pragma unroll 1
+  for (int b = 0; b < it.w; ++b) {
+    const int blk = p.border[it.z + b];
+    const int* aoff = p.aoff + (size_t)blk * (p.a.natm + 1);
+    const cplx_t<T>* x0 = chi + ((size_t)p.boff[blk] * p.a.nk + (size_t)k * aoff[p.a.natm] +
+                                 aoff[it.x] + it.y) * 32 + lane;
+    cplx_t<T> x[kPad];
+#pragma unroll
+    for (int u = 0; u < kPad; ++u) x[u] = __ldg(x0 + 32 * u);
+    bool valid;
+    long long q;
+    ao::block_point(p.a, blk, lane, &valid, &q);
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      cplx_t<T> y{T(0), T(0)};
+      if (valid && i0 + i < nocc) y = __ldg(f0 + (size_t)i * p.a.fs + q);
+#pragma unroll
+      for (int u = 0; u < kPad; ++u) {   // conj(x) y
+        T& re = acc[2 * (u * NI + i)];
+        T& im = acc[2 * (u * NI + i) + 1];
+        re += x[u].x * y.x + x[u].y * y.y;
+        im += x[u].x * y.y - x[u].y * y.x;
+      }
+    }
+  }
+  double sum[NV / 32];
+  halve_lanes<T, NV>(acc, sum, lane);
+  // lane l holds the values l (NV / 32) + j
+  double* o = p.part + ((size_t)k * nitems + w) * NV + lane * (NV / 32);
+#pragma unroll
+  for (int j = 0; j < NV / 32; ++j) o[j] = sum[j];
+}
+
+// out[k][mu][i] += scale N_mu (sum of the items): one CTA per (slot group, k), a thread per
+// value and every kSumSplit-th run, the shares added in order.
+constexpr int kSumSplit = 8;
+template <int NI>
+__global__ void __launch_bounds__(2 * kPad * NI * kSumSplit)
+sum_kernel(Params p, double2* __restrict__ out, int row_of0, int nitems, int i0, double scale) {
+  constexpr int NV = 2 * kPad * NI;
+  __shared__ double share[kSumSplit][NV];
+  const int v = threadIdx.x % NV, z = threadIdx.x / NV, k = blockIdx.y;
+  int a = 0;
+  while ((int)blockIdx.x * kPad >= p.slot0[a + 1]) ++a;
+  const int g = (int)blockIdx.x - p.slot0[a] / kPad;
+  const int2 ro = p.rows_of[row_of0 + a];
+  const double* src = p.part + (size_t)k * nitems * NV + v;
+  double t = 0.0;
+#pragma unroll 4
+  for (int r = z; r < ro.y; r += kSumSplit) {
+    const int2 row = p.rows[ro.x + r];
+    if (g < row.y) t += src[(size_t)(row.x + g) * NV];
+  }
+  share[z][v] = t;
+  __syncthreads();
+  if (z != 0) return;
+  const int u = v / (2 * NI), i = (v / 2) % NI;
+  const int mu = p.slot_ao[blockIdx.x * kPad + u];
+  if (mu < 0 || i0 + i >= p.a.nocc) return;
+#pragma unroll
+  for (int y = 1; y < kSumSplit; ++y) t += share[y][v];
+  double* dst = reinterpret_cast<double*>(out + ((size_t)k * p.a.nao + mu) * p.a.nocc + i0 + i);
+  dst[v & 1] += scale * p.ao_norm[mu] * t;
+}
+
+// Coefficients factor N_mu X^k_{mu i} in slot order, formed in FP64 (hi/lo floats in FP32), 0
+// in padding slots.
+template <typename T>
+__global__ void slot_c_kernel(const double2* __restrict__ X, const double* __restrict__ nrm,
+                              const int* __restrict__ slot_ao, typename CsT<T>::type* __restrict__ out,
+                              int nao, int nocc, int nslots, long long n, double factor) {
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
+       e += (long long)gridDim.x * blockDim.x) {
+    const int i = (int)(e % nocc);
+    const long long ks = e / nocc;
+    const int mu = slot_ao[ks % nslots];
+    double x = 0.0, y = 0.0;
+    if (mu >= 0) {
+      const double2 c = X[((ks / nslots) * nao + mu) * nocc + i];
+      const double s = factor * nrm[mu];
+      x = s * c.x;
+      y = s * c.y;
+    }
+    if constexpr (sizeof(T) == 4) {
+      const float xh = (float)x, yh = (float)y;
+      out[e] = make_float4(xh, yh, (float)(x - (double)xh), (float)(y - (double)yh));
+    } else {
+      out[e] = make_double2(x, y);
+    }
+  }
+}
+
+Params params(const Plan& p) {
+  const ChiTables& t = *p.chi;
+  Params q;
+  q.a = p.ao_params();
+  q.shells = t.shells;
+  q.slot0 = t.slot0;
+  q.slot_ao = t.slot_ao;
+  q.nsh = t.nsh;
+  q.aoff = t.aoff;
+  q.boff = t.boff;
+  q.t0i = t.t0i;
+  q.cls = t.cls;
+  q.order = t.order;
+  q.phase = t.phase;
+  q.items = t.items;
+  q.border = t.border;
+  q.rows = t.rows;
+  q.rows_of = t.rows_of;
+  q.part = t.part;
+  q.ao_norm = p.ao_norm;
+  q.nslots = t.nslots;
+  q.ncls = t.ncls;
+  q.nkp = t.nkp;
+  q.lsm = t.lsm;
+  q.parts = t.parts;
+  return q;
+}
+
+template <typename T> size_t chi_smem(int lsm) {
+  return (size_t)kWarps * rows<T>() * (32 * sizeof(T) + sizeof(int)) +
+         (size_t)lsm * (sizeof(Rec<T>) + sizeof(unsigned short));
+}
+
+template <typename T, int KS, int KL>
+cudaError_t run_chi(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t s) {
+  const size_t sm = chi_smem<T>(q.lsm);
+  static std::mutex mu;
+  static size_t have[kMaxDevices] = {};
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    size_t& h = have[(p.device >= 0 && p.device < kMaxDevices) ? p.device : 0];
+    if (sm > h) {
+      const cudaError_t e = cudaFuncSetAttribute(
+          chi_kernel<T, KS, KL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (e != cudaSuccess) return e;
+      h = sm;
+    }
+  }
+  chi_kernel<T, KS, KL><<<dim3(c.b1 - c.b0, p.natm, q.parts), 32 * kWarps, sm, s>>>(
+      q, (cplx_t<T>*)p.chi->chi, c.b0);
+  return cudaGetLastError();
+}
+
+// k-points per pass over a shell's entries: as many as the registers hold, fewer for meshes
+// that would leave them idle
+template <typename T>
+cudaError_t fill(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t s) {
+  if (p.nk == 1) return run_chi<T, 1, 1>(p, q, c, s);
+  if constexpr (sizeof(T) == 4) {
+    if (p.nk <= 4) return run_chi<T, 4, 4>(p, q, c, s);
+    return run_chi<T, 8, 4>(p, q, c, s);
+  } else {
+    return run_chi<T, 4, 2>(p, q, c, s);
+  }
+}
+
+template <typename T, int NI>
+void run_orb(const Params& q, const cplx_t<T>* chi, const void* cs, void* out, const ChiChunk& c,
+             int i0, cudaStream_t s) {
+  orb_kernel<T, NI><<<dim3((c.b1 - c.b0 + 3) / 4, q.a.nk), 128, 0, s>>>(
+      q, chi, (const typename CsT<T>::type*)cs, (cplx_t<T>*)out, c.b0, c.b1 - c.b0, i0);
+}
+
+template <typename T>
+cudaError_t product_b(const Plan& p, const Params& q, const ChiChunk& c, const void* cs,
+                      void* out, cudaStream_t s) {
+  const cplx_t<T>* x = (const cplx_t<T>*)p.chi->chi;
+  for (int i0 = 0; i0 < p.nocc;) {
+    const int left = p.nocc - i0;
+    if (left <= 4) run_orb<T, 4>(q, x, cs, out, c, i0, s);
+    else if (left <= 8) run_orb<T, 8>(q, x, cs, out, c, i0, s);
+    else run_orb<T, 16>(q, x, cs, out, c, i0, s);
+    i0 += left <= 4 ? 4 : (left <= 8 ? 8 : 16);
+  }
+  return cudaGetLastError();
+}
+
+template <typename T, int NI>
+void run_con(const Plan& p, const Params& q, const ChiChunk& c, const void* F, double2* out,
+             int i0, double scale, cudaStream_t s) {
+  con_kernel<T, NI><<<dim3((c.nitems + 7) / 8, p.nk), 256, 0, s>>>(
+      q, (const cplx_t<T>*)p.chi->chi, (const cplx_t<T>*)F, c.item0, c.nitems, i0);
+  sum_kernel<NI><<<dim3(q.nslots / kPad, p.nk), 2 * kPad * NI * kSumSplit, 0, s>>>(
+      q, out, c.row_of0, c.nitems, i0, scale);
+}
+
+// orbitals per pass of con_kernel
+inline int con_width(int left, bool fp64) { return (fp64 || left <= 4) ? 4 : 8; }
+
+template <typename T>
+cudaError_t product_e(const Plan& p, const Params& q, const ChiChunk& c, const void* F,
+                      double2* out, double scale, cudaStream_t s) {
+  if (c.nitems == 0) return cudaSuccess;
+  for (int i0 = 0; i0 < p.nocc;) {
+    const int ni = con_width(p.nocc - i0, sizeof(T) == 8);
+    if (ni == 4) {
+      run_con<T, 4>(p, q, c, F, out, i0, scale, s);
+    } else if constexpr (sizeof(T) == 4) {
+      run_con<T, 8>(p, q, c, F, out, i0, scale, s);
+    }
+    i0 += ni;
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace chi
+
+template <typename T>
+cudaError_t launch_slot_c(const Plan& p, const double2* X, void* out, double factor,
+                          cudaStream_t s) {
+  const long long n = (long long)p.nk * p.chi->nslots * p.nocc;
+  chi::slot_c_kernel<T><<<2 * 152, 256, 0, s>>>(X, p.ao_norm, p.chi->slot_ao,
+                                                (typename chi::CsT<T>::type*)out, p.nao, p.nocc,
+                                                p.chi->nslots, n, factor);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_orbitals(const Plan& p, int nsets, const void* const* cs, void* const* out,
+                            cudaStream_t s) {
+  const chi::Params q = chi::params(p);
+  for (const ChiChunk& c : p.chi->chunks) {
+    cudaError_t e = chi::fill<T>(p, q, c, s);
+    for (int i = 0; i < nsets && e == cudaSuccess; ++i)
+      e = chi::product_b<T>(p, q, c, cs[i], out[i], s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+template <typename T>
+cudaError_t launch_contract_field(const Plan& p, const void* F, double2* out, double scale,
+                                  cudaStream_t s) {
+  const chi::Params q = chi::params(p);
+  for (const ChiChunk& c : p.chi->chunks) {
+    // one chunk: the buffer still holds chi from the orbitals of this call
+    cudaError_t e = p.chi->chunks.size() > 1 ? chi::fill<T>(p, q, c, s) : cudaSuccess;
+    if (e == cudaSuccess) e = chi::product_e<T>(p, q, c, F, out, scale, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+int chi_launches(const Plan& p, bool contract) {
+  const int nc = (int)p.chi->chunks.size();
+  const int per = contract ? (p.precision == OCCRI_FP64 ? 4 : 8) : 16;
+  const int products = (contract ? 2 : 1) * ((p.nocc + per - 1) / per);
+  return nc * (products + (contract && nc == 1 ? 0 : 1));
+}
+
+int chi_slots(const Plan& p) { return p.chi->nslots; }
+
+void chi_free(ChiTables* t) {
+  if (!t) return;
+  if (t->arena) cudaFree(t->arena);
+  delete t;
+}
+
+namespace {
+
+// Tables laid out one after another (256-byte steps) for one allocation and one copy.
+struct Arena {
+  std::vector<unsigned char> bytes;
+  template <typename X>
+  size_t put(const std::vector<X>& v) {
+    const size_t at = (bytes.size() + 255) / 256 * 256;
+    bytes.resize(at + v.size() * sizeof(X));
+    if (!v.empty()) std::memcpy(bytes.data() + at, v.data(), v.size() * sizeof(X));
+    return at;
+  }
+};
+
+}  // namespace
+
+cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vector<double>& rcut,
+                       const std::vector<std::vector<unsigned short>>& lists,
+                       const std::vector<unsigned short>& bpre, const std::vector<int>& img_n,
+                       const std::vector<int>& t0, const std::vector<int>& atom_shell0,
+                       size_t* total) {
+  ChiTables* t = new (std::nothrow) ChiTables();
+  if (!t) return cudaErrorMemoryAllocation;
+  p->chi = t;
+  const int natm = p->natm, nblk = p->nblk, nsa = p->nsa, lmax = p->lmax;
+  const bool fp64 = p->precision == OCCRI_FP64;
+  // slots: per atom, shells by falling screening radius
+  std::vector<ChiShell> shells(p->nshell);
+  std::vector<int> slot0(natm + 1, 0), slot_ao;
+  for (int a = 0; a < natm; ++a) {
+    slot0[a] = (int)slot_ao.size();
+    std::vector<int> idx(atom_shell0[a + 1] - atom_shell0[a]);
+    std::iota(idx.begin(), idx.end(), atom_shell0[a]);
+    std::stable_sort(idx.begin(), idx.end(), [&](int x, int y) { return rcut[x] > rcut[y]; });
+    for (size_t i = 0; i < idx.size(); ++i) {
+      const ShellDev& s = sh[idx[i]];
+      ChiShell& c = shells[atom_shell0[a] + i];
+      std::memset(&c, 0, sizeof(c));
+      c.alpha_d = s.alpha;
+      c.rcut2_d = s.rcut2;
+      c.alpha = s.alpha_f;
+      c.alpha_lo = s.alpha_lo;
+      c.rcut2 = s.rcut2_f;
+      c.l = s.l;
+      c.slot = (int)slot_ao.size() - slot0[a];
+      c.orig = idx[i];
+      c.exact = s.exact_arg;
+      for (int m = 0; m < 2 * s.l + 1; ++m) slot_ao.push_back(s.ao + m);
+    }
+    while ((slot_ao.size() - slot0[a]) % chi::kPad) slot_ao.push_back(-1);
+  }
+  slot0[natm] = (int)slot_ao.size();
+  t->nslots = slot0[natm];
+  // active shells and slots per (atom, block)
+  std::vector<unsigned short> nsh((size_t)natm * nblk, 0);
+  std::vector<int> aoff((size_t)nblk * (natm + 1), 0);
+  for (int b = 0; b < nblk; ++b)
+    for (int a = 0; a < natm; ++a) {
+      const size_t ab = (size_t)a * nblk + b;
+      int n = 0, slots = 0;
+      const int ns = atom_shell0[a + 1] - atom_shell0[a];
+      while (n < ns && bpre[ab * nsa + (shells[atom_shell0[a] + n].orig - atom_shell0[a])] > 0) {
+        const ChiShell& c = shells[atom_shell0[a] + n];
+        slots = c.slot + 2 * c.l + 1;
+        ++n;
+      }
+      nsh[ab] = (unsigned short)n;
+      slots = (slots + chi::kPad - 1) / chi::kPad * chi::kPad;
+      aoff[(size_t)b * (natm + 1) + a + 1] = aoff[(size_t)b * (natm + 1) + a] + slots;
+    }
+  // residue classes of T0 + T' modulo the k-mesh's supercell, a table row per distinct T0
+  const int Dc = p->D[0] * p->D[1] * p->D[2], nimg = p->nimg;
+  std::vector<int> id(Dc, -1), residue, cls, seen;
+  std::vector<unsigned short> t0i((size_t)natm * nblk);
+  for (size_t ab = 0; ab < t0i.size(); ++ab) {
+    size_t row = 0;
+    while (row < seen.size() && seen[row] != t0[ab]) ++row;
+    t0i[ab] = (unsigned short)row;
+    if (row < seen.size()) continue;
+    seen.push_back(t0[ab]);
+    int s0[3];
+    dev::unpack_t0(t0[ab], &s0[0], &s0[1], &s0[2]);
+    for (int j = 0; j < nimg; ++j) {
+      int r = 0;
+      for (int d = 0; d < 3; ++d) {
+        const int D = p->D[d];
+        r = r * D + ((s0[d] + img_n[3 * (size_t)j + d]) % D + D) % D;
+      }
+      if (id[r] < 0) {
+        id[r] = (int)residue.size();
+        residue.push_back(r);
+      }
+      cls.push_back(id[r]);
+    }
+  }
+  t->ncls = std::max(1, (int)residue.size());
+  t->nkp = (p->nk + 7) / 8 * 8;
+  std::vector<double2> phase((size_t)t->ncls * t->nkp, make_double2(0.0, 0.0));
+  for (size_t c = 0; c < residue.size(); ++c) {
+    const int n[3] = {residue[c] / (p->D[1] * p->D[2]), residue[c] / p->D[2] % p->D[1],
+                      residue[c] % p->D[2]};
+    for (int k = 0; k < p->nk; ++k) {
+      long long num = 0;
+      for (int d = 0; d < 3; ++d) num += (long long)p->kint_h[k * 3 + d] * n[d] * (Dc / p->D[d]);
+      num %= Dc;
+      const double ang = 2.0 * 3.14159265358979323846 * (double)num / (double)Dc;
+      phase[c * t->nkp + k] = make_double2(std::cos(ang), std::sin(ang));
+    }
+  }
+  // chunks of blocks, offsets, and the contraction's items
+  const size_t csz = fp64 ? sizeof(double2) : sizeof(float2);
+  const size_t slot_bytes = csz * 32 * (size_t)p->nk;
+  size_t all = 0, widest = 0;
+  for (int b = 0; b < nblk; ++b) {
+    const size_t n = slot_bytes * aoff[(size_t)b * (natm + 1) + natm];
+    all += n;
+    widest = std::max(widest, n);
+  }
+  size_t free_b = 0, dev_b = 0;
+  if (cudaMemGetInfo(&free_b, &dev_b) != cudaSuccess) return cudaGetLastError();
+  const size_t budget = all <= std::min(kChiKeepBytes, free_b / 4)
+                            ? std::max<size_t>(all, 1)
+                            : std::max(widest, std::min(kChiChunkBytes, free_b / 8));
+  std::vector<long long> boff(nblk, 0);
+  {
+    ChiChunk c{0, 0, 0, 0, 0};
+    long long slots = 0;
+    for (int b = 0; b < nblk; ++b) {
+      const int n = aoff[(size_t)b * (natm + 1) + natm];
+      if (b > c.b0 && slot_bytes * (slots + n) > budget) {
+        c.b1 = b;
+        t->chunks.push_back(c);
+        c.b0 = b;
+        slots = 0;
+      }
+      boff[b] = slots;
+      slots += n;
+      t->chi_bytes = std::max(t->chi_bytes, slot_bytes * (size_t)slots);
+    }
+    c.b1 = nblk;
+    t->chunks.push_back(c);
+  }
+  // Items: kPad slots of an atom over up to `run` of the blocks that reach them, enough items
+  // to fill the GPU (about 16 warps per scheduler) while a lane's FP32 sum stays short.
+  long long groups = 0;
+  for (int b = 0; b < nblk; ++b) groups += aoff[(size_t)b * (natm + 1) + natm] / chi::kPad;
+  const int run = (int)std::max<long long>(4, std::min<long long>(64, groups * p->nk / (152 * 64)));
+  std::vector<int4> items;
+  std::vector<int> border;
+  std::vector<int2> rows, rows_of;
+  for (ChiChunk& c : t->chunks) {
+    c.item0 = (int)items.size();
+    c.row_of0 = (int)rows_of.size();
+    for (int a = 0; a < natm; ++a) {
+      const int o0 = (int)border.size(), row0 = (int)rows.size();
+      auto slots = [&](int b) {
+        return aoff[(size_t)b * (natm + 1) + a + 1] - aoff[(size_t)b * (natm + 1) + a];
+      };
+      std::vector<int> bl(c.b1 - c.b0);
+      std::iota(bl.begin(), bl.end(), c.b0);
+      std::stable_sort(bl.begin(), bl.end(), [&](int x, int y) { return slots(x) > slots(y); });
+      border.insert(border.end(), bl.begin(), bl.end());
+      for (int r0 = 0; r0 < (int)bl.size() && slots(bl[r0]) > 0; r0 += run) {
+        rows.push_back(make_int2((int)items.size() - c.item0, slots(bl[r0]) / chi::kPad));
+        for (int s = 0; s < slots(bl[r0]); s += chi::kPad) {
+          int n = 0;
+          while (n < run && r0 + n < (int)bl.size() && slots(bl[r0 + n]) > s) ++n;
+          items.push_back(make_int4(a, s, o0 + r0, n));
+        }
+      }
+      rows_of.push_back(make_int2(row0, (int)rows.size() - row0));
+    }
+    c.nitems = (int)items.size() - c.item0;
+    t->part_bytes = std::max(t->part_bytes, sizeof(double) * 2 * chi::kPad *
+                                                (size_t)chi::con_width(p->nocc, fp64) *
+                                                (size_t)c.nitems * p->nk);
+  }
+  const int smem_lim = 160 * 1024;
+  const size_t need = fp64 ? chi::chi_smem<double>(lmax) : chi::chi_smem<float>(lmax);
+  t->lsm = need <= (size_t)smem_lim ? lmax : 0;
+  // several CTAs per (block, atom) where there are few of them (a Gamma cell)
+  t->parts = std::max(1, std::min(4, (int)(152LL * 12 / ((long long)nblk * natm))));
+
+  std::vector<float2> phase_f;
+  if (!fp64)
+    for (const double2& z : phase) phase_f.push_back(make_float2((float)z.x, (float)z.y));
+  Arena tab;
+  const size_t o_sh = tab.put(shells), o_s0 = tab.put(slot0), o_ao = tab.put(slot_ao),
+               o_nsh = tab.put(nsh), o_aoff = tab.put(aoff), o_boff = tab.put(boff),
+               o_t0i = tab.put(t0i), o_cls = tab.put(cls),
+               o_ph = fp64 ? tab.put(phase) : tab.put(phase_f), o_it = tab.put(items),
+               o_bd = tab.put(border), o_rows = tab.put(rows), o_ro = tab.put(rows_of);
+  // then the lists in order of class (where they hold several images of one), the items' sums
+  // and chi
+  const bool sorted = t->ncls > 1 && lmax > t->ncls;
+  auto align = [](size_t x) { return (x + 255) / 256 * 256; };
+  const size_t o_ord = align(tab.bytes.size());
+  const size_t o_part = align(o_ord + (sorted ? sizeof(short) * (size_t)natm * nblk * lmax : 0));
+  const size_t o_chi = align(o_part + t->part_bytes);
+  const size_t bytes = o_chi + std::max<size_t>(t->chi_bytes, 16);
+  *total += bytes;
+  cudaError_t e = device_malloc(&t->arena, bytes);
+  if (e != cudaSuccess) return e;
+  e = cudaMemcpy(t->arena, tab.bytes.data(), tab.bytes.size(), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return e;
+  unsigned char* d = (unsigned char*)t->arena;
+  t->shells = (ChiShell*)(d + o_sh);
+  t->slot0 = (int*)(d + o_s0);
+  t->slot_ao = (int*)(d + o_ao);
+  t->nsh = (unsigned short*)(d + o_nsh);
+  t->aoff = (int*)(d + o_aoff);
+  t->boff = (long long*)(d + o_boff);
+  t->t0i = (unsigned short*)(d + o_t0i);
+  t->cls = (int*)(d + o_cls);
+  t->phase = d + o_ph;
+  t->items = (int4*)(d + o_it);
+  t->border = (int*)(d + o_bd);
+  t->rows = (int2*)(d + o_rows);
+  t->rows_of = (int2*)(d + o_ro);
+  t->part = (double*)(d + o_part);
+  t->chi = d + o_chi;
+  if (sorted) {
+    t->order = (unsigned short*)(d + o_ord);   // after the copies, on their stream
+    chi::order_kernel<<<(natm * nblk + 7) / 8, 256>>>(chi::params(*p), t->order);
+    e = cudaGetLastError();
+  }
+  return e;
+}
+
+template cudaError_t launch_slot_c<float>(const Plan&, const double2*, void*, double, cudaStream_t);
+template cudaError_t launch_slot_c<double>(const Plan&, const double2*, void*, double, cudaStream_t);
+template cudaError_t launch_orbitals<float>(const Plan&, int, const void* const*, void* const*,
+                                            cudaStream_t);
+template cudaError_t launch_orbitals<double>(const Plan&, int, const void* const*, void* const*,
+                                             cudaStream_t);
+template cudaError_t launch_contract_field<float>(const Plan&, const void*, double2*, double,
+                                                  cudaStream_t);
+template cudaError_t launch_contract_field<double>(const Plan&, const void*, double2*, double,
+                                                   cudaStream_t);
+
+}  // namespace occri

@@ -52,7 +52,7 @@ __device__ __forceinline__ cplx_t<T> cis_frac_i(int num, int den, int sgn) {
 __host__ __device__ __forceinline__ int pack_t0(int a, int b, int c) {
   return (a & 1023) | ((b & 1023) << 10) | ((c & 1023) << 20);
 }
-__device__ __forceinline__ void unpack_t0(int v, int* a, int* b, int* c) {
+__host__ __device__ __forceinline__ void unpack_t0(int v, int* a, int* b, int* c) {
   const unsigned u = (unsigned)v;
   *a = (int)(u << 22) >> 22;
   *b = (int)(u << 12) >> 22;

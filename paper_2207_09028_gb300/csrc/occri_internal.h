@@ -68,6 +68,7 @@ struct AOParams {
 
 // Atoms a plan may have for the tensor-core contraction.
 constexpr int kMaxTcAtoms = 8;
+struct ChiTables;   // tables and buffer of the Bloch AOs (occri_chi.cu)
 struct TcPlan;   // tables and buffers of the tensor-core contraction (occri_contract_tc.cu)
 
 // Parameters of one wave of pair fields (steps c, d): output k, a block of k'.
@@ -138,12 +139,10 @@ struct Plan {
   int split_cd = 0;          // 1: passes C and D instead of the fused pass CD
   int wave_tables = 0;       // 1: each wave forms its kernel tables even where vq is held
   int tuned = 0;             // 1: the configuration came from the autotuner (or its cache)
-  std::vector<int> shells_by_l[4];
 
   // device tables
   ShellDev* shells = nullptr;
   int* atom_shell0 = nullptr;
-  int* shell_list_l[4] = {nullptr, nullptr, nullptr, nullptr};
   double* img_d = nullptr;
   float* img_hi = nullptr;
   float* img_lo = nullptr;
@@ -203,11 +202,12 @@ struct Plan {
   double* dacc = nullptr;    // [2] scratch accumulators (d E/d omega)
   int* status = nullptr;     // [2]: first device error code, k index
   bool have_kc = false;
+  ChiTables* chi = nullptr;  // Bloch AOs of the plan
   TcPlan* tc = nullptr;      // OCCRI_MIXED_TC: the tensor-core contraction's tables
   void* asm_scratch = nullptr;   // paper-form assembly: M, T, D (grown on demand)
   size_t asm_bytes = 0;
   double* ao_norm = nullptr; // [nao] N_lm per AO
-  void* cs = nullptr;        // scaled coefficients (see AOParams::cs)
+  void* cs = nullptr;        // [nk][slot][nocc] N_mu C: double2 (FP64) or float4 hi/lo (FP32)
 
   // host-call staging (allocated on first occri_k_build_host)
   double2* h_c = nullptr;
@@ -232,39 +232,49 @@ struct Plan {
   PairParams pair_params() const;
 };
 
-// orbitals per launch of the orbital kernel, and per launch of the contraction kernel
+// occri_orbitals_noalloc's kernel: orbitals per launch, and k-points per thread (the image
+// geometry is shared by them); its phase table e^{i k.T'} has its k rows padded with zeros to
+// a multiple of 4.
 constexpr int kOrbChunk = 8;
-// k-points per thread in the orbital kernel (the image geometry is shared by them);
-// the phase table e^{i k.T'} has its k rows padded with zeros to a multiple of 4.
 template <typename T> constexpr int orbital_kbatch() { return sizeof(T) == 4 ? 4 : 2; }
 constexpr int kPhasePadK = 4;
-template <typename T> constexpr int contract_chunk() { return sizeof(T) == 4 ? 8 : 4; }
+
+// The Bloch AOs of a run of point blocks stay in the plan's chi buffer from the orbitals to the
+// contraction of one call where all blocks take at most kChiKeepBytes; otherwise they are
+// formed again for the contraction, kChiChunkBytes at a time. (Writing and reading the buffer
+// costs about what forming chi does, so more memory than this buys little.)
+constexpr size_t kChiKeepBytes = (size_t)8 << 30;
+constexpr size_t kChiChunkBytes = (size_t)1 << 30;
+// Tables and buffer of the plan's AOs (occri_chi.cu), from the shells, their screening radii,
+// the image lists of every (atom, block) with their prefixes, the lattice coordinates of the
+// images and the blocks' T0. What it allocated is freed by chi_free, also after a failure.
+cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vector<double>& rcut,
+                       const std::vector<std::vector<unsigned short>>& lists,
+                       const std::vector<unsigned short>& bpre, const std::vector<int>& img_n,
+                       const std::vector<int>& t0, const std::vector<int>& atom_shell0,
+                       size_t* total);
+void chi_free(ChiTables* t);
+int chi_slots(const Plan& p);      // rows of a coefficient table (AOs in slot order, padded)
+int chi_launches(const Plan& p, bool contract);   // kernels of the orbitals or the contraction
 
 // ---- launchers (return cudaError_t of the launch) ----
+// Coefficients factor N_mu X of a [nk][nao][nocc] c128 array X, in slot order, into out.
 template <typename T>
-cudaError_t launch_scale_c(const Plan& p, const double2* C, cudaStream_t s);
+cudaError_t launch_slot_c(const Plan& p, const double2* X, void* out, double factor,
+                          cudaStream_t s);
+// Orbital fields out[i] of nsets coefficient tables cs[i].
 template <typename T>
-cudaError_t launch_orbitals(const Plan& p, cudaStream_t s);
-// k-points [k0, k0 + nkk) (nkk < 0: all from k0)
-template <typename T>
-cudaError_t launch_contract(const Plan& p, cudaStream_t s, int k0 = 0, int nkk = -1);
-// The same stages on other buffers (the adjoint): orbitals of the scaled coefficients cs
-// into out; scaled coefficients factor N_mu X of X into out; scale N_mu sum_r conj(chi) F
-// added into out.
-template <typename T>
-cudaError_t launch_orbitals_to(const Plan& p, const void* cs, void* out, cudaStream_t s,
-                               int k0 = 0, int nkk = -1);
-template <typename T>
-cudaError_t launch_scale_to(const Plan& p, const double2* X, void* out, double factor,
+cudaError_t launch_orbitals(const Plan& p, int nsets, const void* const* cs, void* const* out,
                             cudaStream_t s);
+// out[k][mu][i] += scale N_mu sum_r conj(chi) F_ik for an orbital-shaped field F; follows
+// launch_orbitals in the same call (the chi buffer may still hold the AOs).
 template <typename T>
 cudaError_t launch_contract_field(const Plan& p, const void* F, double2* out, double scale,
-                                  cudaStream_t s, int k0 = 0, int nkk = -1);
+                                  cudaStream_t s);
 // F[k][i][.] *= e^{sign i k.r} over the orbital-shaped field F (psi -> periodic parts
 // with sign -1 before the pair passes, accumulated periodic parts -> Y with +1 after).
 template <typename T>
-cudaError_t launch_phase_fields(const Plan& p, void* F, int sign, cudaStream_t s, int k0 = 0,
-                                int nkk = -1);
+cudaError_t launch_phase_fields(const Plan& p, void* F, int sign, cudaStream_t s);
 // Pair-wave launches over unordered pairs: diag = 1 is the wave (k, k) with fields
 // i <= j; diag = 0 covers k' in [kp0, kp0 + nkp), all kp0 > k, with every (i, j).
 // S is the wave's scratch and Y the accumulator the wave adds into (the plan's Y, or the

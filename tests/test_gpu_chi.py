@@ -1,0 +1,76 @@
+"""Bloch AOs in tiles (csrc/occri_chi.cu) where they change form: one class or many, entries that
+run out, lists in order of class, lists too long for shared memory, ragged point blocks, every
+width of the products, and k-points off a full mesh. Orbitals and K_{mu i} against the oracle."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import oracle as O
+from workloads import small_workload
+from workloads.synthetic import (analytic_overlap, lowdin_orthonormalize, random_coefficients)
+
+pytestmark = pytest.mark.gpu
+
+CASES = {
+    # Gamma: one class, several CTAs per block
+    "gamma": dict(mesh=(1, 1, 1), grid=(9, 9, 9), counts=(3, 2), lo=0.1, nocc=1),
+    # 2 and 8 classes, lists sorted by class, nk below and at the phase block
+    "class2": dict(mesh=(1, 1, 2), grid=(10, 10, 10), counts=(2, 2, 1), lo=0.1, nocc=5),
+    "class8": dict(mesh=(2, 2, 2), grid=(9, 9, 9), counts=(2, 1, 1), lo=0.1, nocc=4),
+    # 27 classes: d and f shells with more entries than fit, 9 and 17 orbitals
+    "spill": dict(mesh=(3, 3, 3), grid=(8, 8, 8), counts=(2, 1, 1, 1), lo=0.12, nocc=9),
+    "wide": dict(mesh=(1, 3, 1), grid=(8, 8, 8), counts=(3, 2, 1), lo=0.2, nocc=17),
+    # over 4,000 images in reach: the records stay in global memory
+    "long_list": dict(mesh=(1, 1, 2), grid=(8, 8, 8), counts=(1, 1), a_ang=2.0, lo=0.05, hi=0.05,
+                      nocc=1),
+}
+
+
+def _with_kfrac(w, kfrac):
+    """The same cell at other k-points, with orthonormal orbitals there."""
+    kfrac = np.asarray(kfrac, float)
+    s = analytic_overlap(w.lattice, w.xyz, w.shell_atom, w.shell_l, w.shell_alpha, kfrac)
+    x = random_coefficients(np.random.default_rng(3), len(kfrac), w.nao, w.nocc, True)
+    return dataclasses.replace(w, kfrac=kfrac, C=lowdin_orthonormalize(x, s))
+
+
+def _workload(name):
+    if name == "off_mesh":   # two points of a 1/8 mesh: as many classes as images
+        w = small_workload(mesh=(1, 1, 1), grid=(8, 8, 8), counts=(2, 1, 1), lo=0.15, nocc=2,
+                           seed=31, complex_c=True)
+        return _with_kfrac(w, [[0.125, 0.0, 0.375], [0.625, 0.25, 0.0]])
+    w = small_workload(seed=31, **CASES[name])
+    if name == "long_list":   # the AOs nearly cancel at k = 1/2: plain, not orthonormal, orbitals
+        w = dataclasses.replace(w, C=np.full_like(w.C, 0.3 + 0.1j))
+    return w
+
+
+@pytest.mark.parametrize("name", list(CASES) + ["off_mesh"])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_orbitals_and_contraction_match_oracle(name, precision):
+    import torch
+    import paper_2207_09028_gb300 as occri
+    w = _workload(name)
+    chi = O.bloch_aos(w.lattice, w.xyz, w.shell_atom, w.shell_l, w.shell_alpha, w.kfrac,
+                      grid=w.grid)
+    psi = O.orbitals_on_grid(chi, w.C)
+    g0 = O.g0_value(w.kernel, w.omega, w.g0_mode, w.lattice, w.kfrac)
+    kc = O.occri_kc(w.lattice, w.grid, w.kfrac, psi, chi, w.kernel, w.omega, g0)
+    plan = occri.Plan.from_workload(w, precision=precision)
+    C = torch.from_numpy(w.C).cuda()
+    got = plan.orbitals(C).cpu().numpy().reshape(psi.shape)
+    # The rounding of a sequential sum of n images of one sign is at most n u of it, u = 1.1e-16
+    # (FP64) or 6e-8 (FP32); the long list has n = 5,200 (FP64) or 4,000 (FP32) over two classes,
+    # the other cells about 100. FP32 bars: n u = 2.4e-4 and 6e-6 at most; the random-walk sizes
+    # sqrt(n) u = 4e-6 and 6e-7, with a margin of about 3, are asked for.
+    bar = 1e-12 if precision == "fp64" else (1.2e-5 if name == "long_list" else 2e-6)
+    assert np.abs(got - psi).max() <= bar * np.abs(psi).max()
+    KC = plan.build(C)[0]
+    # (The long list's orbital at Gamma is constant to 1e-4, so without its G = 0 term its density
+    # is what the sums above round off: K is compared in FP64 there.)
+    if name != "long_list" or precision == "fp64":
+        tol = 1e-10 if precision == "fp64" else 1e-5   # four orbitals in each term
+        assert np.abs(KC.cpu().numpy() - kc).max() <= tol * np.abs(kc).max()
+    # the contraction adds its partial sums in a fixed order
+    assert torch.equal(KC, plan.build(C)[0])
