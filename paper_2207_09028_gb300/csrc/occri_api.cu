@@ -659,7 +659,7 @@ void free_plan(Plan* p) {
     if (e) cudaEventDestroy(e);
   if (p->aux) cudaStreamDestroy(p->aux);
   if (p->aux2) cudaStreamDestroy(p->aux2);
-  if (p->tc) tc_plan_free(p->tc);
+  if (p->colmax) cudaFree(p->colmax);
   chi_free(p->chi);
   for (cudaEvent_t e : p->ev_used) cudaEventDestroy(e);
   for (cudaEvent_t e : p->ev_free) cudaEventDestroy(e);
@@ -814,7 +814,7 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
     StageTimer t(p, timed);
     if (launch_phase_fields<T>(*p, p->Y, +1, s) != cudaSuccess) return OCCRI_ECUDA;
     ++launches;
-    if (p->tc) {
+    if (p->precision == OCCRI_MIXED_TC) {
       // the GEMM kernels alone, one span per slab (stage OCCRI_STAGE_CONTRACT_GEMM)
       struct GemmSpans : LaunchHook {
         Plan* p;
@@ -832,7 +832,7 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
         }
       } spans(p, s, timed);
       if (launch_contract_tc(*p, s, &spans) != cudaSuccess) return OCCRI_ECUDA;
-      launches += tc_plan_launches(p->tc);
+      launches += tc_plan_launches(*p);
     } else {
       // Y carries N_g/(4 pi) (see PairParams), hence -Omega 4 pi / (N_k N_g^2)
       const double scale = -p->omega_cell * 4.0 * kPiD /
@@ -1653,6 +1653,7 @@ int occri_plan_create(occri_plan** out, const occri_cell* cell, const occri_kmes
   chk(dalloc(&p->mmat, (size_t)p->nk * nocc * nocc, &tot));
   chk(dalloc(&p->ek, (size_t)p->nk, &tot));
   chk(dalloc(&p->dacc, 2, &tot));
+  if (precision == OCCRI_MIXED_TC) chk(dalloc(&p->colmax, (size_t)p->nk * nocc, &tot));
   chk(dalloc(&p->status, 2, &tot));
   if (e == cudaSuccess) e = cudaMemset(p->status, 0, 2 * sizeof(int));
   if (e == cudaSuccess && p->vq)
@@ -1664,13 +1665,6 @@ int occri_plan_create(occri_plan** out, const occri_cell* cell, const occri_kmes
     cudaGetLastError();
     free_plan(p);
     return code;
-  }
-  if (precision == OCCRI_MIXED_TC) {
-    const int st = tc_plan_create(p, sh, cell->xyz, rcut, &tot);
-    if (st != OCCRI_OK) {
-      free_plan(p);
-      return st;
-    }
   }
   p->workspace_bytes = tot;
   {
@@ -1705,9 +1699,10 @@ int occri_plan_info(const occri_plan* plan, occri_plan_info_t* info) {
   info->workspace_bytes = p->workspace_bytes;
   info->fields_per_wave = p->nkp_wave * p->nocc * p->nocc;
   info->launches_per_build = p->launches_per_build;
-  info->contraction_tc = p->tc ? 1 : 0;
-  info->tc_stages = tc_plan_stages(p->tc);
-  info->tc_flops_per_stage = p->tc ? occri::tc_flops_per_stage() : 0.0;
+  const bool tc = p->precision == OCCRI_MIXED_TC;
+  info->contraction_tc = tc ? 1 : 0;
+  info->tc_stages = tc ? occri::tc_plan_stages(*p) : 0;
+  info->tc_flops_per_stage = tc ? occri::tc_flops_per_stage(p->nocc) : 0.0;
   return OCCRI_OK;
 }
 

@@ -23,58 +23,15 @@
 #include <vector>
 
 #include "occri_ao.cuh"
+#include "occri_chi.cuh"
 #include "occri_device.cuh"
 #include "occri_internal.h"
 
 namespace occri {
-
-// One shell in slot order.
-struct ChiShell {
-  double alpha_d, rcut2_d;
-  float alpha, alpha_lo, rcut2;
-  int l, slot, orig, exact;   // first slot within the atom; index in the basis; FP32 exponents
-};
-
-// Blocks [b0, b1): one filling of the chi buffer, with the contraction's work items and the
-// first of its rows_of entries.
-struct ChiChunk {
-  int b0, b1, item0, nitems, row_of0;
-};
-
-struct ChiTables {
-  std::vector<ChiChunk> chunks;
-  int nslots = 0;                 // slots of all atoms, each atom's padded to kChiPad
-  int ncls = 0, nkp = 0;          // residue classes in use; k-points padded to 8
-  int lsm = 0;                    // image records kept in shared memory (0: read from global)
-  int parts = 1;                  // CTAs per (block, atom) of chi_kernel
-  size_t chi_bytes = 0;
-  // device
-  ChiShell* shells = nullptr;     // [nshell] per atom, falling screening radius
-  int* slot0 = nullptr;           // [natm + 1] first slot of each atom
-  int* slot_ao = nullptr;         // [nslots] AO of a slot, or -1 (padding)
-  unsigned short* nsh = nullptr;  // [natm][nblk] shells that reach the block
-  int* aoff = nullptr;            // [nblk][natm + 1] slots of the block before atom a
-  long long* boff = nullptr;      // [nblk] slots of all blocks before this one in its chunk
-  unsigned short* t0i = nullptr;  // [natm][nblk] row of the class table (one per distinct T0)
-  int* cls = nullptr;             // [T0][nimg] class of T0 + T'
-  unsigned short* order = nullptr;   // [natm][nblk][lmax] list positions sorted by class
-  void* phase = nullptr;          // [ncls][nkp] e^{i k.T} of each class
-  int4* items = nullptr;          // contraction: (atom, first slot, first block, blocks)
-  int* border = nullptr;          // blocks per (chunk, atom) by falling number of slots
-  int2* rows = nullptr;           // runs of blocks: (first item in the chunk, slot groups)
-  int2* rows_of = nullptr;        // [chunk][natm] (first run, runs)
-  double* part = nullptr;         // [k][item][values] sums of the items
-  size_t part_bytes = 0;
-  void* chi = nullptr;            // [block][k][slot][32 points]
-  void* arena = nullptr;          // the one allocation behind all of these
-};
-
 namespace chi {
 
 using ao::Disp;
 
-constexpr int kPad = 4;         // slots per group: chi_kernel pads with zeros, the products
-                                // take kPad AOs at a time
 constexpr int kWarps = 4;       // warps of a chi_kernel CTA
 template <typename T> constexpr int rows() { return sizeof(T) == 4 ? 96 : 64; }
 
@@ -85,27 +42,6 @@ template <> struct alignas(16) Rec<double> { double x, y, z; int cls, pad; };
 template <typename T> struct CsT;
 template <> struct CsT<double> { using type = double2; };
 template <> struct CsT<float> { using type = float4; };
-
-struct Params {
-  AOParams a;
-  const ChiShell* shells;
-  const int* slot0;
-  const int* slot_ao;
-  const unsigned short* nsh;
-  const int* aoff;
-  const long long* boff;
-  const unsigned short* t0i;
-  const int* cls;
-  const unsigned short* order;
-  const void* phase;
-  const int4* items;
-  const int* border;
-  const int2* rows;
-  const int2* rows_of;
-  double* part;
-  const double* ao_norm;
-  int nslots, ncls, nkp, lsm, parts;
-};
 
 template <typename T>
 __device__ __forceinline__ Rec<T> load_rec(const Params& p, size_t list0, const int* cls, int j) {
@@ -586,6 +522,7 @@ Params params(const Plan& p) {
   q.rows = t.rows;
   q.rows_of = t.rows_of;
   q.part = t.part;
+  q.row_scale = t.row_scale;
   q.ao_norm = p.ao_norm;
   q.nslots = t.nslots;
   q.ncls = t.ncls;
@@ -682,6 +619,9 @@ cudaError_t product_e(const Plan& p, const Params& q, const ChiChunk& c, const v
   return cudaGetLastError();
 }
 
+template cudaError_t fill<float>(const Plan&, const Params&, const ChiChunk&, cudaStream_t);
+template cudaError_t fill<double>(const Plan&, const Params&, const ChiChunk&, cudaStream_t);
+
 }  // namespace chi
 
 template <typename T>
@@ -751,6 +691,13 @@ struct Arena {
 
 }  // namespace
 
+// Upper bound of |P_lm(d)| e^{-alpha d^2} over d: c_l (l / (2 alpha e))^{l/2}.
+static double shell_peak(int l, double alpha) {
+  static const double cl[4] = {1.0, 1.0, 2.0, 4.0};
+  if (l == 0) return 1.0;
+  return cl[l] * std::pow(l / (2.0 * alpha * std::exp(1.0)), 0.5 * l);
+}
+
 cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vector<double>& rcut,
                        const std::vector<std::vector<unsigned short>>& lists,
                        const std::vector<unsigned short>& bpre, const std::vector<int>& img_n,
@@ -759,6 +706,7 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   ChiTables* t = new (std::nothrow) ChiTables();
   if (!t) return cudaErrorMemoryAllocation;
   p->chi = t;
+  t->tile = p->precision == OCCRI_MIXED_TC ? kTcTile : 0;
   const int natm = p->natm, nblk = p->nblk, nsa = p->nsa, lmax = p->lmax;
   const bool fp64 = p->precision == OCCRI_FP64;
   // slots: per atom, shells by falling screening radius
@@ -788,6 +736,21 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   }
   slot0[natm] = (int)slot_ao.size();
   t->nslots = slot0[natm];
+  // FP16 scale of each slot: 2^13 over a bound of |chi| (the shell's largest value times the
+  // images that reach a block)
+  std::vector<float> row_scale(slot_ao.size(), 1.f);
+  if (t->tile > 0)
+    for (int a = 0; a < natm; ++a)
+      for (int i = atom_shell0[a]; i < atom_shell0[a + 1]; ++i) {
+        const ChiShell& c = shells[i];
+        int np = 1;
+        for (int b = 0; b < nblk; ++b)
+          np = std::max<int>(np, bpre[((size_t)a * nblk + b) * nsa + (c.orig - atom_shell0[a])]);
+        int e2 = 0;
+        std::frexp(shell_peak(c.l, c.alpha_d) * np, &e2);
+        for (int m = 0; m < 2 * c.l + 1; ++m)
+          row_scale[slot0[a] + c.slot + m] = (float)std::ldexp(1.0, 13 - e2);
+      }
   // active shells and slots per (atom, block)
   std::vector<unsigned short> nsh((size_t)natm * nblk, 0);
   std::vector<int> aoff((size_t)nblk * (natm + 1), 0);
@@ -877,11 +840,19 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
     c.b1 = nblk;
     t->chunks.push_back(c);
   }
-  // Items: kPad slots of an atom over up to `run` of the blocks that reach them, enough items
-  // to fill the GPU (about 16 warps per scheduler) while a lane's FP32 sum stays short.
+  // The contraction's items: a group of slots of an atom (kPad of them, or a tensor-core tile)
+  // over up to `run` of the blocks that reach the group. `run` gives enough items to fill the
+  // GPU (about 16 warps per scheduler, or three rounds of CTAs) while the FP32 sums stay short.
+  const int width = t->tile > 0 ? t->tile : chi::kPad;
   long long groups = 0;
-  for (int b = 0; b < nblk; ++b) groups += aoff[(size_t)b * (natm + 1) + natm] / chi::kPad;
-  const int run = (int)std::max<long long>(4, std::min<long long>(64, groups * p->nk / (152 * 64)));
+  for (int b = 0; b < nblk; ++b)
+    for (int a = 0; a < natm; ++a) {
+      const int* o = &aoff[(size_t)b * (natm + 1) + a];
+      groups += (o[1] - o[0] + width - 1) / width;
+    }
+  const long long want = t->tile > 0 ? 152 * 9 : 152 * 64;
+  int run = (int)std::max<long long>(4, std::min<long long>(64, groups * p->nk / want));
+  run = (run + 1) / 2 * 2;
   std::vector<int4> items;
   std::vector<int> border;
   std::vector<int2> rows, rows_of;
@@ -898,19 +869,21 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
       std::stable_sort(bl.begin(), bl.end(), [&](int x, int y) { return slots(x) > slots(y); });
       border.insert(border.end(), bl.begin(), bl.end());
       for (int r0 = 0; r0 < (int)bl.size() && slots(bl[r0]) > 0; r0 += run) {
-        rows.push_back(make_int2((int)items.size() - c.item0, slots(bl[r0]) / chi::kPad));
-        for (int s = 0; s < slots(bl[r0]); s += chi::kPad) {
+        rows.push_back(make_int2((int)items.size() - c.item0, (slots(bl[r0]) + width - 1) / width));
+        for (int s = 0; s < slots(bl[r0]); s += width) {
           int n = 0;
           while (n < run && r0 + n < (int)bl.size() && slots(bl[r0 + n]) > s) ++n;
           items.push_back(make_int4(a, s, o0 + r0, n));
+          t->item_pairs += (n + 1) / 2;
         }
       }
       rows_of.push_back(make_int2(row0, (int)rows.size() - row0));
     }
     c.nitems = (int)items.size() - c.item0;
-    t->part_bytes = std::max(t->part_bytes, sizeof(double) * 2 * chi::kPad *
-                                                (size_t)chi::con_width(p->nocc, fp64) *
-                                                (size_t)c.nitems * p->nk);
+    const size_t values = t->tile > 0
+                              ? tc_item_values(p->nocc)
+                              : 2 * (size_t)chi::kPad * chi::con_width(p->nocc, fp64);
+    t->part_bytes = std::max(t->part_bytes, sizeof(double) * values * (size_t)c.nitems * p->nk);
   }
   const int smem_lim = 160 * 1024;
   const size_t need = fp64 ? chi::chi_smem<double>(lmax) : chi::chi_smem<float>(lmax);
@@ -926,7 +899,8 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
                o_nsh = tab.put(nsh), o_aoff = tab.put(aoff), o_boff = tab.put(boff),
                o_t0i = tab.put(t0i), o_cls = tab.put(cls),
                o_ph = fp64 ? tab.put(phase) : tab.put(phase_f), o_it = tab.put(items),
-               o_bd = tab.put(border), o_rows = tab.put(rows), o_ro = tab.put(rows_of);
+               o_bd = tab.put(border), o_rows = tab.put(rows), o_ro = tab.put(rows_of),
+               o_rs = tab.put(row_scale);
   // then the lists in order of class (where they hold several images of one), the items' sums
   // and chi
   const bool sorted = t->ncls > 1 && lmax > t->ncls;
@@ -954,6 +928,7 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   t->border = (int*)(d + o_bd);
   t->rows = (int2*)(d + o_rows);
   t->rows_of = (int2*)(d + o_ro);
+  t->row_scale = (float*)(d + o_rs);
   t->part = (double*)(d + o_part);
   t->chi = d + o_chi;
   if (sorted) {

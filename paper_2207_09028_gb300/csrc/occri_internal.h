@@ -66,10 +66,7 @@ struct AOParams {
   const void* cs;            // [nk][nao][nocc] N_mu C^k_{mu i}: double2 (FP64) or float4 hi/lo (FP32)
 };
 
-// Atoms a plan may have for the tensor-core contraction.
-constexpr int kMaxTcAtoms = 8;
-struct ChiTables;   // tables and buffer of the Bloch AOs (occri_chi.cu)
-struct TcPlan;   // tables and buffers of the tensor-core contraction (occri_contract_tc.cu)
+struct ChiTables;   // tables and buffer of the Bloch AOs (occri_chi.cuh)
 
 // Parameters of one wave of pair fields (steps c, d): output k, a block of k'.
 constexpr int kFadN = 40;   // terms of the Faddeeva approximation (OCCRI_ERF_TRUNC)
@@ -203,7 +200,7 @@ struct Plan {
   int* status = nullptr;     // [2]: first device error code, k index
   bool have_kc = false;
   ChiTables* chi = nullptr;  // Bloch AOs of the plan
-  TcPlan* tc = nullptr;      // OCCRI_MIXED_TC: the tensor-core contraction's tables
+  unsigned* colmax = nullptr;   // OCCRI_MIXED_TC: [nk][nocc] largest |Re Y| + |Im Y|, float bits
   void* asm_scratch = nullptr;   // paper-form assembly: M, T, D (grown on demand)
   size_t asm_bytes = 0;
   double* ao_norm = nullptr; // [nao] N_lm per AO
@@ -318,22 +315,20 @@ inline int wave_targets(int nocc, int nkp, int diag) { return diag ? nocc : nocc
 template <typename T>
 cudaError_t launch_widen(const Plan& p, void* out, cudaStream_t s);
 
-// The tensor-core contraction (OCCRI_MIXED_TC): tables built at plan creation from the shells
-// (with their screening radii) and atom positions, freed with the plan; the launch turns the
-// Bloch-phased Y into FP16 hi/lo blocks and adds K_{mu i} into p.kc.
-int tc_plan_create(Plan* p, const std::vector<ShellDev>& shells, const double* xyz,
-                   const std::vector<double>& rcut, size_t* total);
-void tc_plan_free(TcPlan* t);
-long long tc_plan_stages(const TcPlan* t);
-int tc_plan_launches(const TcPlan* t);      // kernels one tensor-core contraction launches
-double tc_flops_per_stage();
+// The tensor-core contraction (OCCRI_MIXED_TC, occri_contract_tc.cu): adds K_{mu i} of the
+// accumulated Y into p.kc, from the chi buffer.
+constexpr int kTcTile = 64;                 // AO slots per tile (128 rows: Re and Im)
+size_t tc_item_values(int nocc);            // sums one work item leaves
+long long tc_plan_stages(const Plan& p);    // stages (pairs of point blocks) per contraction
+int tc_plan_launches(const Plan& p);        // kernels one tensor-core contraction launches
+double tc_flops_per_stage(int nocc);
 // Paper-form assembly and conduction-band helpers (occri_assemble.cu), on the plan's stream.
 cudaError_t launch_assemble_paper(Plan& p, int ncol, const double2* S, const double2* C,
                                   const double2* KC, double2* K);
 cudaError_t launch_gather_cols(const double2* all, double2* cr, long long rows, int nocc, int nr,
                                cudaStream_t s);
 cudaError_t launch_band_diff(const double2* all, const double2* rr, double2* out, long long rows,
-                             int nocc, int nr, cudaStream_t s);   // MMA flops of one stage of the tensor-core contraction   // stages of one contraction (0 without a plan)
+                             int nocc, int nr, cudaStream_t s);
 // Called around every GEMM launch of the tensor-core contraction (stage timing).
 struct LaunchHook {
   virtual void before() = 0;
