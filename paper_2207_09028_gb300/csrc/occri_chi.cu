@@ -20,8 +20,10 @@
 #include <mutex>
 #include <new>
 #include <numeric>
+#include <type_traits>
 #include <vector>
 
+#include "fft_reg.cuh"
 #include "occri_ao.cuh"
 #include "occri_chi.cuh"
 #include "occri_device.cuh"
@@ -32,8 +34,10 @@ namespace chi {
 
 using ao::Disp;
 
-constexpr int kWarps = 4;       // warps of a chi_kernel CTA
-template <typename T> constexpr int rows() { return sizeof(T) == 4 ? 96 : 64; }
+constexpr int kWarps = 8;       // most warps of a chi_kernel CTA
+constexpr int kRows = 48;       // entry rows of a warp (a value per lane each)
+constexpr int kCols = 8;        // AOs that the CTA takes together (wide shells)
+constexpr int kWide = 12;       // images from which a shell counts as wide
 
 template <typename T> struct Rec;
 template <> struct alignas(16) Rec<float> { float xh, yh, zh; int cls; float xl, yl, zl; int pad; };
@@ -129,39 +133,27 @@ __device__ __forceinline__ void phase_sums(const cplx_t<T>* ph, int nkp, const T
   }
 }
 
-// One shell at the warp's block: class sums into the warp's entries (a lane reads back only
-// what it wrote), then chi of every k. Where the entries run out, the sums so far go to chi
-// and the rest is added.
-template <typename T, int L, int KT, typename GetRec, typename GetOrder>
-__device__ __forceinline__ void shell_chi(const Params& p, const ChiShell& sh, const Disp<T>& d,
-                                          int np, int n_all, const GetRec& rec,
-                                          const GetOrder& order, T* ent, int* ecls,
-                                          cplx_t<T>* out, int kstride, int lane) {
+// A narrow shell, one warp: every image its own entry (a lane reads back only what it wrote),
+// then chi of every k. Where the entries run out, the sums so far go to chi and the rest is
+// added.
+template <typename T, int L, int KT, typename GetRec>
+__device__ __forceinline__ void narrow_shell(const Params& p, const ChiShell& sh,
+                                             const Disp<T>& d, int np, const GetRec& rec, T* ent,
+                                             int* ecls, cplx_t<T>* out, int kstride, int lane) {
   constexpr int NM = 2 * L + 1;
-  constexpr int CAP = rows<T>() / NM;
+  constexpr int CAP = kRows / NM;
   const cplx_t<T>* ph = reinterpret_cast<const cplx_t<T>*>(p.phase);
   const int nk = p.a.nk;
-  // Images in order of distance, each its own entry, or (where it saves more phase products
-  // than the scan costs) in order of class, with the images past the shell's reach skipped.
-  const bool fold = p.ncls == 1;
-  const bool by_class = !fold && p.order != nullptr &&
-                        (long long)(np - p.ncls) * (2 * nk * NM + 8) > 3 * n_all;
-  const int nt = by_class ? n_all : np;
-  bool first = true;
-  int ne = 0, cur = -1;
-  T acc[NM];
+  for (int j0 = 0; j0 < np; j0 += CAP) {
+    const int ne = min(CAP, np - j0);
+    for (int e = 0; e < ne; ++e) {
+      const Rec<T> r = rec(j0 + e);
+      T v[NM];
+      eval<L>(sh, d, r, v);
 #pragma unroll
-  for (int m = 0; m < NM; ++m) acc[m] = T(0);
-  auto close = [&]() {   // the class sum becomes an entry
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      ent[(ne * NM + m) * 32 + lane] = acc[m];
-      acc[m] = T(0);
+      for (int m = 0; m < NM; ++m) ent[(e * NM + m) * 32 + lane] = v[m];
+      if (lane == 0) ecls[e] = r.cls;
     }
-    if (lane == 0) ecls[ne] = cur;
-    ++ne;
-  };
-  auto spill = [&]() {   // the entries' share of chi
     __syncwarp();
     for (int k0 = 0; k0 < nk; k0 += KT) {
       T xr[KT][NM], xi[KT][NM];
@@ -177,7 +169,7 @@ __device__ __forceinline__ void shell_chi(const Params& p, const ChiShell& sh, c
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
           cplx_t<T> v{xr[b][m], xi[b][m]};
-          if (!first) {
+          if (j0 > 0) {
             const cplx_t<T> u = o[32 * m];
             v.x += u.x;
             v.y += u.y;
@@ -187,37 +179,157 @@ __device__ __forceinline__ void shell_chi(const Params& p, const ChiShell& sh, c
       }
     }
     __syncwarp();
-    ne = 0;
-    first = false;
-  };
-  for (int t = 0; t < nt; ++t) {
-    const int j = by_class ? order(t) : t;
-    if (j >= np) continue;   // uniform
-    const Rec<T> r = rec(j);
-    if (cur >= 0 && !fold && (!by_class || r.cls != cur)) {
-      close();
-      if (ne == CAP) spill();
+  }
+}
+
+// ---- wide shells: the class sums of up to kCols AOs in shared memory, then a discrete Fourier
+// transform over the classes, axis by axis (chi_k = sum_l e^{2 pi i k.l/D} Phi_l, Phi real: only
+// the non-negative half of the first axis is kept, the rest are conjugates). A column holds
+// one AO: rows ((l_0 D_1 + l_1) D_2 + l_2), a value per lane; after the first axis, row pairs
+// 2 k_0 (re) and 2 k_0 + 1 (im) in the place of l_0.
+template <typename F>
+__device__ __forceinline__ void by_length(int D, F&& f) {
+  switch (D) {
+    case 1: f(std::integral_constant<int, 1>{}); break;
+    case 2: f(std::integral_constant<int, 2>{}); break;
+    case 3: f(std::integral_constant<int, 3>{}); break;
+    case 4: f(std::integral_constant<int, 4>{}); break;
+    case 5: f(std::integral_constant<int, 5>{}); break;
+    case 6: f(std::integral_constant<int, 6>{}); break;
+    default: f(std::integral_constant<int, 8>{}); break;
+  }
+}
+
+// One column's transform; chi of every k of the mesh goes to out.
+template <typename T>
+__device__ __forceinline__ void mesh_dft(const Params& p, T* col, cplx_t<T>* out, int kstride,
+                                         int lane) {
+  const int D0 = p.a.D[0], D1 = p.a.D[1], D2 = p.a.D[2], H = D0 / 2 + 1, P = D1 * D2;
+  T* c = col + lane;
+  by_length(D0, [&](auto ND) {
+    constexpr int N = decltype(ND)::value;
+    for (int j = 0; j < P; ++j) {
+      T re[N], im[N];
+      fft::static_for<N>([&](auto I) {
+        constexpr int n = decltype(I)::value;
+        re[n] = c[(n * P + j) * 32];
+        im[n] = T(0);
+      });
+      fft::fft_dif<N, 1>(re, im);
+      fft::static_for<N>([&](auto I) {
+        constexpr int q = decltype(I)::value, k = fft::dif_rev(N, q);
+        if constexpr (k < N / 2 + 1) {
+          c[(2 * k * P + j) * 32] = re[q];
+          c[((2 * k + 1) * P + j) * 32] = im[q];
+        }
+      });
     }
-    cur = r.cls;
+  });
+  if (D1 > 1)
+    by_length(D1, [&](auto ND) {
+      constexpr int N = decltype(ND)::value;
+      for (int j = 0; j < H * D2; ++j) {
+        T* r = c + ((size_t)(j / D2) * 2 * P + j % D2) * 32;
+        T re[N], im[N];
+        fft::static_for<N>([&](auto I) {
+          constexpr int n = decltype(I)::value;
+          re[n] = r[n * D2 * 32];
+          im[n] = r[(P + n * D2) * 32];
+        });
+        fft::fft_dif<N, 1>(re, im);
+        fft::static_for<N>([&](auto I) {
+          constexpr int q = decltype(I)::value, k = fft::dif_rev(N, q);
+          r[k * D2 * 32] = re[q];
+          r[(P + k * D2) * 32] = im[q];
+        });
+      }
+    });
+  by_length(D2, [&](auto ND) {
+    constexpr int N = decltype(ND)::value;
+    for (int j = 0; j < H * D1; ++j) {
+      const int k0 = j / D1, k1 = j % D1;
+      const T* r = c + ((size_t)k0 * 2 * P + k1 * D2) * 32;
+      T re[N], im[N];
+      fft::static_for<N>([&](auto I) {
+        constexpr int n = decltype(I)::value;
+        re[n] = r[n * 32];
+        im[n] = r[(P + n) * 32];
+      });
+      fft::fft_dif<N, 1>(re, im);
+      const int g0 = (D0 - k0) % D0, g1 = (D1 - k1) % D1;   // -k on the first two axes
+      const int* at = p.kidx + (k0 * D1 + k1) * D2;
+      const int* neg = p.kidx + (g0 * D1 + g1) * D2;
+      fft::static_for<N>([&](auto I) {
+        constexpr int q = decltype(I)::value, k = fft::dif_rev(N, q);
+        const int i = at[k];
+        if (i >= 0) out[(size_t)i * kstride + lane] = cplx_t<T>{re[q], im[q]};
+        if (g0 != k0) {
+          const int n = neg[k == 0 ? 0 : N - k];
+          if (n >= 0) out[(size_t)n * kstride + lane] = cplx_t<T>{re[q], -im[q]};
+        }
+      });
+    }
+  });
+}
+
+// Class sums of the functions [m0, m0 + ncol) of one shell over a stretch [t0, t1) of the list
+// in order of class. A class that may continue from the stretch before (the first one of a
+// stretch) goes to `edge`, its number to *edge_cls; the others are this warp's alone.
+template <typename T, int L, typename GetRec, typename GetOrder>
+__device__ __forceinline__ void class_sums(const ChiShell& sh, const Disp<T>& d, int np, int t0,
+                                           int t1, int m0, int ncol, const GetRec& rec,
+                                           const GetOrder& order, T* cols, int col_rows, T* edge,
+                                           int* edge_cls, int lane) {
+  constexpr int NM = 2 * L + 1;
+  T acc[NM];
+#pragma unroll
+  for (int m = 0; m < NM; ++m) acc[m] = T(0);
+  int cur = -1, first = -1;
+  auto close = [&]() {
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+      const int c = m - m0;
+      if (c >= 0 && c < ncol) {
+        T* o = cur == first ? edge + c * 32 : cols + ((size_t)c * col_rows + cur) * 32;
+        o[lane] = acc[m];
+      }
+      acc[m] = T(0);
+    }
+  };
+  for (int t = t0; t < t1; ++t) {
+    const int j = order(t);
+    if (j >= np) continue;   // past the shell's reach (uniform)
+    const Rec<T> r = rec(j);
+    if (r.cls != cur) {
+      if (cur >= 0) close();
+      cur = r.cls;
+      if (first < 0) first = cur;
+    }
     T v[NM];
     eval<L>(sh, d, r, v);
 #pragma unroll
     for (int m = 0; m < NM; ++m) acc[m] += v[m];
   }
-  close();
-  spill();
+  if (cur >= 0) close();
+  if (lane == 0) *edge_cls = first;
 }
 
-// chi of the blocks [blk0, blk0 + gridDim.x) for one atom: warps take the atom's shells in
-// turn, a lane is a grid point. Each Gaussian is evaluated once for all k, so the kernel is
-// bound by its stores where there are many k-points and by the evaluation where there are few.
+// chi of the blocks [blk0, blk0 + gridDim.x) for one atom; a lane is a grid point. Every Gaussian
+// is evaluated once for all k. The atom's wide shells come first (they are a prefix of its
+// shells): the CTA takes as many as make kCols AOs, each warp a stretch of the images, then a
+// warp per AO transforms. The phases of a narrow shell's few images are applied one by one.
+// What bounds it: the stores at many k-points, the Gaussians at few. Phases times class sums
+// (a dense product over classes) instead of the transform took 43 ms per pass at 64 k, 350
+// AOs, 60^3: each broadcast phase costs the load path as much as a full vector.
 template <typename T, int KS, int KL>
-__global__ void __launch_bounds__(32 * kWarps, 4)
+__global__ void __launch_bounds__(32 * kWarps, 2)
 chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* ents = reinterpret_cast<T*>(smem_raw);
-  int* eclss = reinterpret_cast<int*>(ents + kWarps * rows<T>() * 32);
-  Rec<T>* recs = reinterpret_cast<Rec<T>*>(eclss + kWarps * rows<T>());
+  __shared__ T edge[kWarps][kCols][32];
+  __shared__ int edge_cls[kWarps][kCols];
+  T* buf = reinterpret_cast<T*>(smem_raw);   // entry rows of the warps, or columns
+  int* eclss = reinterpret_cast<int*>(buf + p.buf_rows * 32);
+  Rec<T>* recs = reinterpret_cast<Rec<T>*>(eclss + kWarps * kRows);
   unsigned short* ord = reinterpret_cast<unsigned short*>(recs + p.lsm);
   const int blk = blk0 + blockIdx.x, a = blockIdx.y;
   const size_t ab = (size_t)a * p.a.nblk + blk;
@@ -236,7 +348,7 @@ chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
     }
     __syncthreads();
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   bool valid;
   long long q;
   const long long n = ao::block_point(p.a, blk, lane, &valid, &q);
@@ -245,26 +357,85 @@ chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
   const int* aoff = p.aoff + (size_t)blk * (p.a.natm + 1);
   const int kstride = 32 * aoff[p.a.natm];
   cplx_t<T>* base = chi + (size_t)(p.boff[blk] * p.a.nk + aoff[a]) * 32;
-  T* ent = ents + warp * rows<T>() * 32;
-  int* ecls = eclss + warp * rows<T>();
   auto rec = [&](int j) -> Rec<T> { return in_smem ? recs[j] : load_rec<T>(p, list0, cls, j); };
   auto order = [&](int t) -> int { return in_smem ? ord[t] : p.order[list0 + t]; };
-  for (int s = warp + kWarps * blockIdx.z; s < nact; s += kWarps * gridDim.z) {
+  int s = 0;
+  if (p.ncol > 0) {
+    // groups of wide shells; the groups go round the CTAs of the (block, atom)
+    int m0 = 0, group = 0;
+    const int t0 = n_all * warp / nw, t1 = n_all * (warp + 1) / nw;
+    while (s < nact) {
+      // the group: functions m0.. of shell s, then whole shells while they fit
+      int e = s, cols = 0, next_m = 0;
+      if (pre[p.shells[s0 + s].orig - s0] < kWide) break;
+      while (e < nact) {
+        const ChiShell& sh = p.shells[s0 + e];
+        if (pre[sh.orig - s0] < kWide) break;
+        const int left = 2 * sh.l + 1 - (e == s ? m0 : 0);
+        if (cols + left > p.ncol) {
+          if (e == s) { next_m = m0 + p.ncol; cols = p.ncol; }   // a part of one shell
+          break;
+        }
+        cols += left;
+        ++e;
+      }
+      if (group % gridDim.z == blockIdx.z) {
+        for (int x = threadIdx.x; x < cols * p.col_rows * 32; x += blockDim.x) buf[x] = T(0);
+        for (int x = threadIdx.x; x < kWarps * kCols; x += blockDim.x)
+          (&edge_cls[0][0])[x] = -1;
+        __syncthreads();
+        for (int i = s, c = 0; i < e || (i == s && next_m > 0); ++i) {
+          const ChiShell sh = p.shells[s0 + i];
+          const int np = pre[sh.orig - s0], f = i == s ? m0 : 0;
+          const int nc = min(2 * sh.l + 1 - f, cols - c);
+          T* cb = buf + (size_t)c * p.col_rows * 32;
+          T* eb = &edge[warp][c][0];
+          switch (sh.l) {
+            case 0: class_sums<T, 0>(sh, d, np, t0, t1, f, nc, rec, order, cb, p.col_rows, eb, &edge_cls[warp][c], lane); break;
+            case 1: class_sums<T, 1>(sh, d, np, t0, t1, f, nc, rec, order, cb, p.col_rows, eb, &edge_cls[warp][c], lane); break;
+            case 2: class_sums<T, 2>(sh, d, np, t0, t1, f, nc, rec, order, cb, p.col_rows, eb, &edge_cls[warp][c], lane); break;
+            default: class_sums<T, 3>(sh, d, np, t0, t1, f, nc, rec, order, cb, p.col_rows, eb, &edge_cls[warp][c], lane); break;
+          }
+          // the shell's other columns share its stretch
+          __syncwarp();
+          if (lane > 0 && lane < nc) edge_cls[warp][c + lane] = edge_cls[warp][c];
+          c += nc;
+        }
+        __syncthreads();
+        for (int x = warp; x < cols; x += nw) {   // a warp per AO: the stretches' edges in
+          T* col = buf + (size_t)x * p.col_rows * 32;   // order, then the transform
+          for (int w = 0; w < nw; ++w) {
+            const int c = edge_cls[w][x];
+            if (c >= 0) col[c * 32 + lane] += edge[w][x][lane];
+          }
+          const int slot = p.shells[s0 + s].slot + m0 + x;
+          mesh_dft<T>(p, col, base + 32 * (size_t)slot, kstride, lane);
+        }
+        __syncthreads();
+      }
+      ++group;
+      s = next_m > 0 ? s : e;
+      m0 = next_m;
+    }
+  }
+  T* ent = buf + warp * kRows * 32;
+  int* ecls = eclss + warp * kRows;
+  for (s += warp + nw * blockIdx.z; s < nact; s += nw * gridDim.z) {
     const ChiShell sh = p.shells[s0 + s];
     const int np = pre[sh.orig - s0];
     cplx_t<T>* out = base + 32 * (size_t)sh.slot;
     switch (sh.l) {
-      case 0: shell_chi<T, 0, KS>(p, sh, d, np, n_all, rec, order, ent, ecls, out, kstride, lane); break;
-      case 1: shell_chi<T, 1, KS>(p, sh, d, np, n_all, rec, order, ent, ecls, out, kstride, lane); break;
-      case 2: shell_chi<T, 2, KL>(p, sh, d, np, n_all, rec, order, ent, ecls, out, kstride, lane); break;
-      default: shell_chi<T, 3, KL>(p, sh, d, np, n_all, rec, order, ent, ecls, out, kstride, lane); break;
+      case 0: narrow_shell<T, 0, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+      case 1: narrow_shell<T, 1, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+      case 2: narrow_shell<T, 2, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+      default: narrow_shell<T, 3, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
     }
   }
-  if (blockIdx.z == 0 && warp == kWarps - 1) {   // padding slots of the atom's last group
+  if (blockIdx.z == 0 && warp == nw - 1) {   // padding slots of the atom's last group
     const ChiShell& last = p.shells[s0 + nact - 1];
-    for (int s = last.slot + 2 * last.l + 1; s < aoff[a + 1] - aoff[a]; ++s)
+    for (int x = last.slot + 2 * last.l + 1; x < aoff[a + 1] - aoff[a]; ++x)
       for (int k = 0; k < p.a.nk; ++k)
-        base[(size_t)k * kstride + 32 * s + lane] = cplx_t<T>{T(0), T(0)};
+        base[(size_t)k * kstride + 32 * x + lane] = cplx_t<T>{T(0), T(0)};
   }
 }
 
@@ -529,17 +700,22 @@ Params params(const Plan& p) {
   q.nkp = t.nkp;
   q.lsm = t.lsm;
   q.parts = t.parts;
+  q.kidx = t.kidx;
+  q.ncol = t.ncol;
+  q.col_rows = t.col_rows;
+  q.buf_rows = t.buf_rows;
+  q.warps = t.warps;
   return q;
 }
 
-template <typename T> size_t chi_smem(int lsm) {
-  return (size_t)kWarps * rows<T>() * (32 * sizeof(T) + sizeof(int)) +
+template <typename T> size_t chi_smem(int buf_rows, int lsm) {
+  return (size_t)buf_rows * 32 * sizeof(T) + (size_t)kWarps * kRows * sizeof(int) +
          (size_t)lsm * (sizeof(Rec<T>) + sizeof(unsigned short));
 }
 
 template <typename T, int KS, int KL>
 cudaError_t run_chi(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t s) {
-  const size_t sm = chi_smem<T>(q.lsm);
+  const size_t sm = chi_smem<T>(q.buf_rows, q.lsm);
   static std::mutex mu;
   static size_t have[kMaxDevices] = {};
   {
@@ -552,7 +728,7 @@ cudaError_t run_chi(const Plan& p, const Params& q, const ChiChunk& c, cudaStrea
       h = sm;
     }
   }
-  chi_kernel<T, KS, KL><<<dim3(c.b1 - c.b0, p.natm, q.parts), 32 * kWarps, sm, s>>>(
+  chi_kernel<T, KS, KL><<<dim3(c.b1 - c.b0, p.natm, q.parts), 32 * q.warps, sm, s>>>(
       q, (cplx_t<T>*)p.chi->chi, c.b0);
   return cudaGetLastError();
 }
@@ -770,7 +946,13 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
     }
   // residue classes of T0 + T' modulo the k-mesh's supercell, a table row per distinct T0
   const int Dc = p->D[0] * p->D[1] * p->D[2], nimg = p->nimg;
+  const bool identity = Dc <= 4096;   // class = residue; beyond, the residues in use
   std::vector<int> id(Dc, -1), residue, cls, seen;
+  if (identity) {
+    residue.resize(Dc);
+    std::iota(residue.begin(), residue.end(), 0);
+    id = residue;
+  }
   std::vector<unsigned short> t0i((size_t)natm * nblk);
   for (size_t ab = 0; ab < t0i.size(); ++ab) {
     size_t row = 0;
@@ -885,9 +1067,28 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
                               : 2 * (size_t)chi::kPad * chi::con_width(p->nocc, fp64);
     t->part_bytes = std::max(t->part_bytes, sizeof(double) * values * (size_t)c.nitems * p->nk);
   }
-  const int smem_lim = 160 * 1024;
-  const size_t need = fp64 ? chi::chi_smem<double>(lmax) : chi::chi_smem<float>(lmax);
-  t->lsm = need <= (size_t)smem_lim ? lmax : 0;
+  // Wide shells go through the transform over classes where the mesh is (nearly) full, its
+  // k-points are distinct and its lengths are compiled; columns as the shared memory allows.
+  std::vector<int> kidx(identity ? Dc : 1, -1);
+  bool dft = identity && Dc <= 4 * p->nk;
+  for (int d = 0; d < 3; ++d) dft = dft && (p->D[d] <= 6 || p->D[d] == 8);
+  for (int k = 0; k < p->nk && dft; ++k) {
+    const int r = (p->kint_h[3 * k] * p->D[1] + p->kint_h[3 * k + 1]) * p->D[2] + p->kint_h[3 * k + 2];
+    if (kidx[r] >= 0) dft = false;
+    kidx[r] = k;
+  }
+  const int row_bytes = 32 * (fp64 ? 8 : 4);
+  t->col_rows = 2 * (p->D[0] / 2 + 1) * p->D[1] * p->D[2];
+  // 88 KB of columns leave room for two CTAs per SM; where that is under four AOs, one CTA
+  const long long col_bytes = (long long)t->col_rows * row_bytes;
+  const long long cols = (88 * 1024 / col_bytes >= 4 ? 88 : 176) * 1024 / col_bytes;
+  t->ncol = dft ? (int)std::min<long long>(chi::kCols, cols) : 0;
+  // small transforms: half the warps per CTA, so that fewer wait at its barriers
+  t->warps = t->ncol * t->col_rows <= 256 ? 4 : chi::kWarps;
+  t->buf_rows = std::max(t->ncol * t->col_rows, t->warps * chi::kRows);
+  const size_t need = fp64 ? chi::chi_smem<double>(t->buf_rows, lmax)
+                           : chi::chi_smem<float>(t->buf_rows, lmax);
+  t->lsm = need <= 200 * 1024 ? lmax : 0;
   // several CTAs per (block, atom) where there are few of them (a Gamma cell)
   t->parts = std::max(1, std::min(4, (int)(152LL * 12 / ((long long)nblk * natm))));
 
@@ -900,10 +1101,10 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
                o_t0i = tab.put(t0i), o_cls = tab.put(cls),
                o_ph = fp64 ? tab.put(phase) : tab.put(phase_f), o_it = tab.put(items),
                o_bd = tab.put(border), o_rows = tab.put(rows), o_ro = tab.put(rows_of),
-               o_rs = tab.put(row_scale);
-  // then the lists in order of class (where they hold several images of one), the items' sums
+               o_rs = tab.put(row_scale), o_ki = tab.put(kidx);
+  // then the lists in order of class (for the wide shells), the items' sums
   // and chi
-  const bool sorted = t->ncls > 1 && lmax > t->ncls;
+  const bool sorted = t->ncol > 0;
   auto align = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t o_ord = align(tab.bytes.size());
   const size_t o_part = align(o_ord + (sorted ? sizeof(short) * (size_t)natm * nblk * lmax : 0));
@@ -929,6 +1130,7 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   t->rows = (int2*)(d + o_rows);
   t->rows_of = (int2*)(d + o_ro);
   t->row_scale = (float*)(d + o_rs);
+  t->kidx = (int*)(d + o_ki);
   t->part = (double*)(d + o_part);
   t->chi = d + o_chi;
   if (sorted) {

@@ -26,6 +26,8 @@ struct ChiTables {
   int nslots = 0;                 // slots of all atoms, each atom's padded to kChiPad
   int ncls = 0, nkp = 0;          // residue classes in use; k-points padded to 8
   int lsm = 0;                    // image records kept in shared memory (0: read from global)
+  int ncol = 0, col_rows = 0;     // AOs per transform over classes (0: none), rows of one
+  int buf_rows = 0, warps = 0;    // rows of chi_kernel's buffer, warps of its CTAs
   int parts = 1;                  // CTAs per (block, atom) of chi_kernel
   int tile = 0;                   // slots per item of the tensor-core contraction, 0 without it
   long long item_pairs = 0;       // pairs of blocks over all items
@@ -39,6 +41,7 @@ struct ChiTables {
   long long* boff = nullptr;      // [nblk] slots of all blocks before this one in its chunk
   unsigned short* t0i = nullptr;  // [natm][nblk] row of the class table (one per distinct T0)
   int* cls = nullptr;             // [T0][nimg] class of T0 + T'
+  int* kidx = nullptr;            // [D_1 D_2 D_3] k-point at each mesh position, or -1
   unsigned short* order = nullptr;   // [natm][nblk][lmax] list positions sorted by class
   void* phase = nullptr;          // [ncls][nkp] e^{i k.T} of each class
   int4* items = nullptr;          // contraction: (atom, first slot, first block, blocks)
@@ -76,7 +79,8 @@ struct Params {
   double* part;
   const float* row_scale;
   const double* ao_norm;
-  int nslots, ncls, nkp, lsm, parts;
+  const int* kidx;
+  int nslots, ncls, nkp, lsm, parts, ncol, col_rows, buf_rows, warps;
 };
 
 Params params(const Plan& p);

@@ -1,6 +1,7 @@
-"""Bloch AOs in tiles (csrc/occri_chi.cu) where they change form: one class or many, entries that
-run out, lists in order of class, lists too long for shared memory, ragged point blocks, every
-width of the products, and k-points off a full mesh. Orbitals and K_{mu i} against the oracle."""
+"""Bloch AOs in tiles (csrc/occri_chi.cu) where they change form: the transform over classes at
+one class, full and partly filled axes and columns that take a part of a shell; meshes it does
+not take, with entries that run out; lists too long for shared memory, ragged point blocks,
+every width of the products. Orbitals and K_{mu i} against the oracle."""
 import dataclasses
 
 import numpy as np
@@ -15,12 +16,15 @@ pytestmark = pytest.mark.gpu
 CASES = {
     # Gamma: one class, several CTAs per block
     "gamma": dict(mesh=(1, 1, 1), grid=(9, 9, 9), counts=(3, 2), lo=0.1, nocc=1),
-    # 2 and 8 classes, lists sorted by class, nk below and at the phase block
-    "class2": dict(mesh=(1, 1, 2), grid=(10, 10, 10), counts=(2, 2, 1), lo=0.1, nocc=5),
+    # even and odd axes of the transform, wide and narrow shells side by side
+    "even": dict(mesh=(1, 4, 2), grid=(10, 10, 10), counts=(2, 2, 1), lo=0.1, nocc=5),
     "class8": dict(mesh=(2, 2, 2), grid=(9, 9, 9), counts=(2, 1, 1), lo=0.1, nocc=4),
-    # 27 classes: d and f shells with more entries than fit, 9 and 17 orbitals
-    "spill": dict(mesh=(3, 3, 3), grid=(8, 8, 8), counts=(2, 1, 1, 1), lo=0.12, nocc=9),
-    "wide": dict(mesh=(1, 3, 1), grid=(8, 8, 8), counts=(3, 2, 1), lo=0.2, nocc=17),
+    "odd": dict(mesh=(3, 3, 3), grid=(8, 8, 8), counts=(2, 1, 1, 1), lo=0.12, nocc=9),
+    "wide": dict(mesh=(5, 1, 1), grid=(8, 8, 8), counts=(3, 2, 1), lo=0.2, nocc=17),
+    # a length the transform does not take: an entry per image, more than fit
+    "seven": dict(mesh=(1, 1, 7), grid=(8, 8, 8), counts=(2, 1, 1, 1), lo=0.12, nocc=3),
+    # 100 classes: in FP64 an f shell does not fit the columns whole (orbitals only)
+    "columns": dict(mesh=(5, 4, 5), grid=(8, 8, 8), counts=(2, 0, 0, 1), lo=0.12, nocc=2),
     # over 4,000 images in reach: the records stay in global memory
     "long_list": dict(mesh=(1, 1, 2), grid=(8, 8, 8), counts=(1, 1), a_ang=2.0, lo=0.05, hi=0.05,
                       nocc=1),
@@ -55,8 +59,6 @@ def test_orbitals_and_contraction_match_oracle(name, precision):
     chi = O.bloch_aos(w.lattice, w.xyz, w.shell_atom, w.shell_l, w.shell_alpha, w.kfrac,
                       grid=w.grid)
     psi = O.orbitals_on_grid(chi, w.C)
-    g0 = O.g0_value(w.kernel, w.omega, w.g0_mode, w.lattice, w.kfrac)
-    kc = O.occri_kc(w.lattice, w.grid, w.kfrac, psi, chi, w.kernel, w.omega, g0)
     plan = occri.Plan.from_workload(w, precision=precision)
     C = torch.from_numpy(w.C).cuda()
     got = plan.orbitals(C).cpu().numpy().reshape(psi.shape)
@@ -66,6 +68,10 @@ def test_orbitals_and_contraction_match_oracle(name, precision):
     # sqrt(n) u = 4e-6 and 6e-7, with a margin of about 3, are asked for.
     bar = 1e-12 if precision == "fp64" else (1.2e-5 if name == "long_list" else 2e-6)
     assert np.abs(got - psi).max() <= bar * np.abs(psi).max()
+    if name == "columns":
+        return
+    g0 = O.g0_value(w.kernel, w.omega, w.g0_mode, w.lattice, w.kfrac)
+    kc = O.occri_kc(w.lattice, w.grid, w.kfrac, psi, chi, w.kernel, w.omega, g0)
     KC = plan.build(C)[0]
     # (The long list's orbital at Gamma is constant to 1e-4, so without its G = 0 term its density
     # is what the sums above round off: K is compared in FP64 there.)
