@@ -1,11 +1,13 @@
-// fft_reg.cuh -- one-thread, register-resident mixed-radix FFT of compile-time length.
+// fft_reg.cuh -- one-thread, register-resident FFT of compile-time length.
 //
-// A length-N transform lives in two register arrays re[], im[]. The decimation-
-// in-frequency recursion N = R*M (R in {4,3,5,2}) is unrolled completely at
-// compile time, so every index, every twiddle and the final digit permutation
-// are constants: twiddles become FMA immediates and the output permutation is a
-// register renaming. X[k] = sum_n x[n] e^{SIGN 2 pi i n k / N} with SIGN = -1
-// (forward) or +1 (inverse, unnormalised).
+// A length-N transform lives in registers. N = q_1 q_2 q_3 (its powers of 2, 3 and 5, which are
+// coprime) is split by the prime-factor algorithm (Good 1958): with n = sum n_i N/q_i and
+// k = the residues k_i (Chinese remainder theorem), e^{2 pi i n k/N} is the product of the
+// factors' own exponentials, so no twiddles stand between the factors. A prime power q runs the
+// decimation-in-frequency recursion q = R*M (R in {4,2,3,5}). Everything is unrolled at
+// compile time: every index, every twiddle and the output permutation are constants.
+// X[k] = sum_n x[n] e^{SIGN 2 pi i n k / N} with SIGN = -1 (forward) or +1 (inverse,
+// unnormalised).
 //
 // Twiddle values come from a constexpr sine/cosine (Taylor series after exact
 // integer octant reduction), evaluated by the compiler in double precision.
@@ -103,69 +105,101 @@ constexpr int dif_rev(int n, int p) {
   return r * dif_rev(m, p % m) + p / m;
 }
 
-// Inverse permutation: output index k is held at register position dif_pos(N, k).
-constexpr int dif_pos(int n, int k) {
-  for (int p = 0; p < n; ++p)
-    if (dif_rev(n, p) == k) return p;
-  return -1;
+// Coprime factors of a {2,3,5}-smooth N: its powers of 2, 3 and 5 (those above 1), in order.
+constexpr int prime_part(int n, int p) {
+  int q = 1;
+  while (n % p == 0) { q *= p; n /= p; }
+  return q;
+}
+constexpr int pf_count(int n) {
+  return (prime_part(n, 2) > 1) + (prime_part(n, 3) > 1) + (prime_part(n, 5) > 1);
+}
+constexpr int pf(int n, int i) {
+  for (int p : {2, 3, 5})
+    if (prime_part(n, p) > 1 && i-- == 0) return prime_part(n, p);
+  return 1;
+}
+constexpr int inv_mod(int a, int m) {
+  for (int x = 0; x < m; ++x)
+    if ((a * x) % m == 1 % m) return x;
+  return 0;
+}
+// The k modulo n with k = 1 modulo its factor q and 0 modulo the others.
+constexpr int crt_unit(int n, int q) { return (n / q) * inv_mod((n / q) % q, q) % n; }
+
+// Register p = sum n_i N/q_i (mod N) holds output X[pfa_out(N, p)] after pfa<N>.
+constexpr int pfa_out(int n, int p) {
+  int k = 0;
+  for (int i = 0; i < pf_count(n); ++i) {
+    const int q = pf(n, i);
+    const int ni = (p % q) * inv_mod((n / q) % q, q) % q;
+    k = (k + dif_rev(q, ni) * crt_unit(n, q)) % n;
+  }
+  return k;
 }
 
 // ---------------------------------------------------------------- butterflies
 
+// Elements A, A + S, ... of the TOT registers, indices modulo TOT.
 template <int SIGN, int A, int S, typename T, int TOT>
 OCCRI_HDI void dft2(T (&re)[TOT], T (&im)[TOT]) {
-  T ar = re[A], ai = im[A], br = re[A + S], bi = im[A + S];
-  re[A] = ar + br; im[A] = ai + bi;
-  re[A + S] = ar - br; im[A + S] = ai - bi;
+  constexpr int a = A % TOT, b = (A + S) % TOT;
+  const T ar = re[a], ai = im[a], br = re[b], bi = im[b];
+  re[a] = ar + br; im[a] = ai + bi;
+  re[b] = ar - br; im[b] = ai - bi;
 }
 
 template <int SIGN, int A, int S, typename T, int TOT>
 OCCRI_HDI void dft3(T (&re)[TOT], T (&im)[TOT]) {
-  constexpr double h = 0.86602540378443864676372317075293618;  // sqrt(3)/2
-  const T ar = re[A], ai = im[A];
-  const T t1r = re[A + S] + re[A + 2 * S], t1i = im[A + S] + im[A + 2 * S];
-  const T dr = re[A + S] - re[A + 2 * S], di = im[A + S] - im[A + 2 * S];
-  const T t2r = ar - T(0.5) * t1r, t2i = ai - T(0.5) * t1i;
-  // i * SIGN * h * d = (-SIGN h di, SIGN h dr)
-  const T ur = T(-SIGN * h) * di, ui = T(SIGN * h) * dr;
-  re[A] = ar + t1r; im[A] = ai + t1i;
-  re[A + S] = t2r + ur; im[A + S] = t2i + ui;
-  re[A + 2 * S] = t2r - ur; im[A + 2 * S] = t2i - ui;
+  constexpr int a = A % TOT, b = (A + S) % TOT, c = (A + 2 * S) % TOT;
+  constexpr T h = T(SIGN * 0.86602540378443864676372317075293618);  // sqrt(3)/2
+  const T t1r = re[b] + re[c], t1i = im[b] + im[c];
+  const T dr = re[b] - re[c], di = im[b] - im[c];
+  const T t2r = fma(T(-0.5), t1r, re[a]), t2i = fma(T(-0.5), t1i, im[a]);
+  re[a] = re[a] + t1r; im[a] = im[a] + t1i;
+  // t2 +- i SIGN h d
+  re[b] = fma(-h, di, t2r); im[b] = fma(h, dr, t2i);
+  re[c] = fma(h, di, t2r); im[c] = fma(-h, dr, t2i);
 }
 
 template <int SIGN, int A, int S, typename T, int TOT>
 OCCRI_HDI void dft4(T (&re)[TOT], T (&im)[TOT]) {
-  const T s0r = re[A] + re[A + 2 * S], s0i = im[A] + im[A + 2 * S];
-  const T d0r = re[A] - re[A + 2 * S], d0i = im[A] - im[A + 2 * S];
-  const T s1r = re[A + S] + re[A + 3 * S], s1i = im[A + S] + im[A + 3 * S];
-  const T d1r = re[A + S] - re[A + 3 * S], d1i = im[A + S] - im[A + 3 * S];
+  constexpr int a = A % TOT, b = (A + S) % TOT, c = (A + 2 * S) % TOT, d = (A + 3 * S) % TOT;
+  const T s0r = re[a] + re[c], s0i = im[a] + im[c];
+  const T d0r = re[a] - re[c], d0i = im[a] - im[c];
+  const T s1r = re[b] + re[d], s1i = im[b] + im[d];
+  const T d1r = re[b] - re[d], d1i = im[b] - im[d];
   // SIGN * i * d1 = (-SIGN d1i, SIGN d1r)
   const T jr = (SIGN > 0) ? -d1i : d1i;
   const T ji = (SIGN > 0) ? d1r : -d1r;
-  re[A] = s0r + s1r; im[A] = s0i + s1i;
-  re[A + 2 * S] = s0r - s1r; im[A + 2 * S] = s0i - s1i;
-  re[A + S] = d0r + jr; im[A + S] = d0i + ji;
-  re[A + 3 * S] = d0r - jr; im[A + 3 * S] = d0i - ji;
+  re[a] = s0r + s1r; im[a] = s0i + s1i;
+  re[c] = s0r - s1r; im[c] = s0i - s1i;
+  re[b] = d0r + jr; im[b] = d0i + ji;
+  re[d] = d0r - jr; im[d] = d0i - ji;
 }
 
+// Five points: the sines enter as s_1 (t3 + (s_2/s_1) t4) and s_1 ((s_2/s_1) t3 - t4), the
+// outer factor in the last multiply-adds: 32 operations.
 template <int SIGN, int A, int S, typename T, int TOT>
 OCCRI_HDI void dft5(T (&re)[TOT], T (&im)[TOT]) {
   constexpr CS w1 = cs2pi(1, 5), w2 = cs2pi(2, 5);
-  const T ar = re[A], ai = im[A];
-  const T t1r = re[A + S] + re[A + 4 * S], t1i = im[A + S] + im[A + 4 * S];
-  const T t2r = re[A + 2 * S] + re[A + 3 * S], t2i = im[A + 2 * S] + im[A + 3 * S];
-  const T t3r = re[A + S] - re[A + 4 * S], t3i = im[A + S] - im[A + 4 * S];
-  const T t4r = re[A + 2 * S] - re[A + 3 * S], t4i = im[A + 2 * S] - im[A + 3 * S];
-  const T c1 = T(w1.c), c2 = T(w2.c), s1 = T(SIGN * w1.s), s2 = T(SIGN * w2.s);
-  const T p1r = ar + c1 * t1r + c2 * t2r, p1i = ai + c1 * t1i + c2 * t2i;
-  const T p2r = ar + c2 * t1r + c1 * t2r, p2i = ai + c2 * t1i + c1 * t2i;
-  const T q1r = s1 * t3r + s2 * t4r, q1i = s1 * t3i + s2 * t4i;   // times i below
-  const T q2r = s2 * t3r - s1 * t4r, q2i = s2 * t3i - s1 * t4i;
-  re[A] = ar + t1r + t2r; im[A] = ai + t1i + t2i;
-  re[A + S] = p1r - q1i; im[A + S] = p1i + q1r;
-  re[A + 4 * S] = p1r + q1i; im[A + 4 * S] = p1i - q1r;
-  re[A + 2 * S] = p2r - q2i; im[A + 2 * S] = p2i + q2r;
-  re[A + 3 * S] = p2r + q2i; im[A + 3 * S] = p2i - q2r;
+  constexpr int e0 = A % TOT, e1 = (A + S) % TOT, e2 = (A + 2 * S) % TOT, e3 = (A + 3 * S) % TOT,
+                e4 = (A + 4 * S) % TOT;
+  const T ar = re[e0], ai = im[e0];
+  const T t1r = re[e1] + re[e4], t1i = im[e1] + im[e4];
+  const T t2r = re[e2] + re[e3], t2i = im[e2] + im[e3];
+  const T t3r = re[e1] - re[e4], t3i = im[e1] - im[e4];
+  const T t4r = re[e2] - re[e3], t4i = im[e2] - im[e3];
+  constexpr T c1 = T(w1.c), c2 = T(w2.c), s1 = T(SIGN * w1.s), r = T(w2.s / w1.s);
+  const T p1r = fma(c2, t2r, fma(c1, t1r, ar)), p1i = fma(c2, t2i, fma(c1, t1i, ai));
+  const T p2r = fma(c1, t2r, fma(c2, t1r, ar)), p2i = fma(c1, t2i, fma(c2, t1i, ai));
+  const T q1r = fma(r, t4r, t3r), q1i = fma(r, t4i, t3i);    // times i s_1 below
+  const T q2r = fma(r, t3r, -t4r), q2i = fma(r, t3i, -t4i);
+  re[e0] = ar + (t1r + t2r); im[e0] = ai + (t1i + t2i);
+  re[e1] = fma(-s1, q1i, p1r); im[e1] = fma(s1, q1r, p1i);
+  re[e4] = fma(s1, q1i, p1r); im[e4] = fma(-s1, q1r, p1i);
+  re[e2] = fma(-s1, q2i, p2r); im[e2] = fma(s1, q2r, p2i);
+  re[e3] = fma(s1, q2i, p2r); im[e3] = fma(-s1, q2r, p2i);
 }
 
 template <int R, int SIGN, int A, int S, typename T, int TOT>
@@ -177,9 +211,9 @@ OCCRI_HDI void small_dft(T (&re)[TOT], T (&im)[TOT]) {
 }
 
 // x[P] *= e^{SIGN 2 pi i E / N}
-template <int N, int SIGN, int E, int P, typename T, int TOT>
+template <int N, int SIGN, int E, int PP, typename T, int TOT>
 OCCRI_HDI void twiddle(T (&re)[TOT], T (&im)[TOT]) {
-  constexpr int e = E % N;
+  constexpr int e = E % N, P = PP % TOT;
   if constexpr (e == 0) {
   } else if constexpr (2 * e == N) {
     re[P] = -re[P]; im[P] = -im[P];
@@ -197,7 +231,7 @@ OCCRI_HDI void twiddle(T (&re)[TOT], T (&im)[TOT]) {
   }
 }
 
-// In-place DIF of the N elements at positions A + S*idx.
+// In-place DIF of the N elements at positions A + S*idx (modulo TOT).
 template <int N, int SIGN, int A, int S, typename T, int TOT>
 OCCRI_HDI void dif(T (&re)[TOT], T (&im)[TOT]) {
   if constexpr (N == 1) {
@@ -220,26 +254,15 @@ OCCRI_HDI void dif(T (&re)[TOT], T (&im)[TOT]) {
   }
 }
 
-// Full transform: after the call, register p holds X[dif_rev(N, p)].
+// Full transform: after the call, register p holds X[pfa_out(N, p)].
 template <int N, int SIGN, typename T>
-OCCRI_HDI void fft_dif(T (&re)[N], T (&im)[N]) {
+OCCRI_HDI void pfa(T (&re)[N], T (&im)[N]) {
   static_assert(smooth235(N), "FFT length must be {2,3,5}-smooth");
-  dif<N, SIGN, 0, 1>(re, im);
-}
-
-// Reorder registers from DIF order to natural order (compile-time renaming).
-template <int N, typename T>
-OCCRI_HDI void dif_to_natural(T (&re)[N], T (&im)[N]) {
-  T r2[N], i2[N];
-  static_for<N>([&](auto K) {
-    constexpr int k = decltype(K)::value;
-    r2[k] = re[dif_pos(N, k)];
-    i2[k] = im[dif_pos(N, k)];
-  });
-  static_for<N>([&](auto K) {
-    constexpr int k = decltype(K)::value;
-    re[k] = r2[k];
-    im[k] = i2[k];
+  static_for<pf_count(N)>([&](auto F) {
+    constexpr int q = pf(N, decltype(F)::value), S = N / q;
+    // the transforms of length q: one per value of the other factors' indices, i.e. per
+    // multiple of q modulo N
+    static_for<S>([&](auto J) { dif<q, SIGN, (decltype(J)::value * q) % N, S>(re, im); });
   });
 }
 
@@ -289,6 +312,13 @@ __device__ __forceinline__ u64 mul_i(u64 x) {
   unpack(x, r, i);
   return SGN > 0 ? pack(-i, r) : pack(i, -r);
 }
+// (a - b) with its halves exchanged, for a later multiply-add by (-s, s) = i s
+__device__ __forceinline__ u64 sub_swap(u64 a, u64 b) {
+  float ar, ai, br, bi;
+  unpack(a, ar, ai);
+  unpack(b, br, bi);
+  return pack(ai - bi, ar - br);
+}
 // x * (c + i s), scalar on the halves so that c and s stay instruction immediates
 __device__ __forceinline__ u64 cmul_const(u64 x, float c, float s) {
   float r, i;
@@ -299,60 +329,62 @@ __device__ __forceinline__ u64 cmul_const(u64 x, float c, float s) {
 
 template <int SIGN, int A, int S, int TOT>
 __device__ __forceinline__ void pdft2(pk::u64 (&x)[TOT]) {
-  const pk::u64 a = x[A], b = x[A + S];
-  x[A] = pk::add(a, b);
-  x[A + S] = pk::sub(a, b);
+  constexpr int e0 = A % TOT, e1 = (A + S) % TOT;
+  const pk::u64 a = x[e0], b = x[e1];
+  x[e0] = pk::add(a, b);
+  x[e1] = pk::sub(a, b);
 }
 
 template <int SIGN, int A, int S, int TOT>
 __device__ __forceinline__ void pdft3(pk::u64 (&x)[TOT]) {
-  constexpr double h = 0.86602540378443864676372317075293618;  // sqrt(3)/2
-  const pk::u64 a = x[A];
-  const pk::u64 t1 = pk::add(x[A + S], x[A + 2 * S]);
-  const pk::u64 d = pk::sub(x[A + S], x[A + 2 * S]);
+  constexpr int e0 = A % TOT, e1 = (A + S) % TOT, e2 = (A + 2 * S) % TOT;
+  constexpr float h = float(SIGN * 0.86602540378443864676372317075293618);  // sqrt(3)/2
+  const pk::u64 a = x[e0];
+  const pk::u64 t1 = pk::add(x[e1], x[e2]);
+  const pk::u64 d = pk::sub_swap(x[e1], x[e2]);
   const pk::u64 t2 = pk::fma(t1, pk::splat(-0.5f), a);
-  float dr, di;
-  pk::unpack(d, dr, di);
-  // i * SIGN * h * d = (-SIGN h di, SIGN h dr)
-  const pk::u64 u = pk::pack(float(-SIGN * h) * di, float(SIGN * h) * dr);
-  x[A] = pk::add(a, t1);
-  x[A + S] = pk::add(t2, u);
-  x[A + 2 * S] = pk::sub(t2, u);
+  x[e0] = pk::add(a, t1);
+  x[e1] = pk::fma(d, pk::pack(-h, h), t2);   // t2 + i h (x1 - x2)
+  x[e2] = pk::fma(d, pk::pack(h, -h), t2);
 }
 
 template <int SIGN, int A, int S, int TOT>
 __device__ __forceinline__ void pdft4(pk::u64 (&x)[TOT]) {
-  const pk::u64 s0 = pk::add(x[A], x[A + 2 * S]);
-  const pk::u64 d0 = pk::sub(x[A], x[A + 2 * S]);
-  const pk::u64 s1 = pk::add(x[A + S], x[A + 3 * S]);
-  const pk::u64 d1 = pk::sub(x[A + S], x[A + 3 * S]);
-  const pk::u64 j = pk::mul_i<SIGN>(d1);   // SIGN * i * d1
-  x[A] = pk::add(s0, s1);
-  x[A + 2 * S] = pk::sub(s0, s1);
-  x[A + S] = pk::add(d0, j);
-  x[A + 3 * S] = pk::sub(d0, j);
+  constexpr int e0 = A % TOT, e1 = (A + S) % TOT, e2 = (A + 2 * S) % TOT, e3 = (A + 3 * S) % TOT;
+  constexpr float h = float(SIGN);
+  const pk::u64 s0 = pk::add(x[e0], x[e2]);
+  const pk::u64 d0 = pk::sub(x[e0], x[e2]);
+  const pk::u64 s1 = pk::add(x[e1], x[e3]);
+  const pk::u64 d1 = pk::sub_swap(x[e1], x[e3]);
+  x[e0] = pk::add(s0, s1);
+  x[e2] = pk::sub(s0, s1);
+  x[e1] = pk::fma(d1, pk::pack(-h, h), d0);   // d0 + i SIGN (x1 - x3)
+  x[e3] = pk::fma(d1, pk::pack(h, -h), d0);
 }
 
+// As dft5, the terms that multiply i with their halves exchanged.
 template <int SIGN, int A, int S, int TOT>
 __device__ __forceinline__ void pdft5(pk::u64 (&x)[TOT]) {
   constexpr CS w1 = cs2pi(1, 5), w2 = cs2pi(2, 5);
-  const pk::u64 a = x[A];
-  const pk::u64 t1 = pk::add(x[A + S], x[A + 4 * S]);
-  const pk::u64 t2 = pk::add(x[A + 2 * S], x[A + 3 * S]);
-  const pk::u64 t3 = pk::sub(x[A + S], x[A + 4 * S]);
-  const pk::u64 t4 = pk::sub(x[A + 2 * S], x[A + 3 * S]);
+  constexpr int e0 = A % TOT, e1 = (A + S) % TOT, e2 = (A + 2 * S) % TOT, e3 = (A + 3 * S) % TOT,
+                e4 = (A + 4 * S) % TOT;
+  const pk::u64 a = x[e0];
+  const pk::u64 t1 = pk::add(x[e1], x[e4]);
+  const pk::u64 t2 = pk::add(x[e2], x[e3]);
+  const pk::u64 t3 = pk::sub_swap(x[e1], x[e4]);
+  const pk::u64 t4 = pk::sub_swap(x[e2], x[e3]);
   const pk::u64 c1 = pk::splat(float(w1.c)), c2 = pk::splat(float(w2.c));
-  const pk::u64 s1 = pk::splat(float(SIGN * w1.s)), s2 = pk::splat(float(SIGN * w2.s));
+  constexpr float s1 = float(SIGN * w1.s), r = float(w2.s / w1.s);
   const pk::u64 p1 = pk::fma(t2, c2, pk::fma(t1, c1, a));
   const pk::u64 p2 = pk::fma(t2, c1, pk::fma(t1, c2, a));
-  const pk::u64 q1 = pk::fma(t4, s2, pk::mul(t3, s1));                       // times i below
-  const pk::u64 q2 = pk::fma(t4, pk::splat(float(-SIGN * w1.s)), pk::mul(t3, s2));
-  const pk::u64 iq1 = pk::mul_i<1>(q1), iq2 = pk::mul_i<1>(q2);
-  x[A] = pk::add(pk::add(a, t1), t2);
-  x[A + S] = pk::add(p1, iq1);
-  x[A + 4 * S] = pk::sub(p1, iq1);
-  x[A + 2 * S] = pk::add(p2, iq2);
-  x[A + 3 * S] = pk::sub(p2, iq2);
+  const pk::u64 q1 = pk::fma(t4, pk::splat(r), t3);              // t3 + r t4
+  const pk::u64 q2 = pk::fma(t3, pk::splat(-r), t4);             // -(r t3 - t4)
+  const pk::u64 up = pk::pack(-s1, s1), dn = pk::pack(s1, -s1);  // times i s_1, -i s_1
+  x[e0] = pk::add(pk::add(t1, t2), a);
+  x[e1] = pk::fma(q1, up, p1);
+  x[e4] = pk::fma(q1, dn, p1);
+  x[e2] = pk::fma(q2, dn, p2);
+  x[e3] = pk::fma(q2, up, p2);
 }
 
 template <int R, int SIGN, int A, int S, int TOT>
@@ -364,9 +396,9 @@ __device__ __forceinline__ void psmall_dft(pk::u64 (&x)[TOT]) {
 }
 
 // x[P] *= e^{SIGN 2 pi i E / N}
-template <int N, int SIGN, int E, int P, int TOT>
+template <int N, int SIGN, int E, int PP, int TOT>
 __device__ __forceinline__ void ptwiddle(pk::u64 (&x)[TOT]) {
-  constexpr int e = E % N;
+  constexpr int e = E % N, P = PP % TOT;
   if constexpr (e == 0) {
   } else if constexpr (2 * e == N) {
     x[P] = pk::sub(pk::splat(0.0f), x[P]);
@@ -401,11 +433,14 @@ __device__ __forceinline__ void pdif(pk::u64 (&x)[TOT]) {
   }
 }
 
-// Packed FP32 transform: after the call, x[p] holds X[dif_rev(N, p)].
+// Packed FP32 transform: after the call, x[p] holds X[pfa_out(N, p)].
 template <int N, int SIGN>
-__device__ __forceinline__ void pfft_dif(pk::u64 (&x)[N]) {
+__device__ __forceinline__ void ppfa(pk::u64 (&x)[N]) {
   static_assert(smooth235(N), "FFT length must be {2,3,5}-smooth");
-  pdif<N, SIGN, 0, 1>(x);
+  static_for<pf_count(N)>([&](auto F) {
+    constexpr int q = pf(N, decltype(F)::value), S = N / q;
+    static_for<S>([&](auto J) { pdif<q, SIGN, (decltype(J)::value * q) % N, S>(x); });
+  });
 }
 #endif
 

@@ -215,9 +215,9 @@ __device__ __forceinline__ void mesh_dft(const Params& p, T* col, cplx_t<T>* out
         re[n] = c[(n * P + j) * 32];
         im[n] = T(0);
       });
-      fft::fft_dif<N, 1>(re, im);
+      fft::pfa<N, 1>(re, im);
       fft::static_for<N>([&](auto I) {
-        constexpr int q = decltype(I)::value, k = fft::dif_rev(N, q);
+        constexpr int q = decltype(I)::value, k = fft::pfa_out(N, q);
         if constexpr (k < N / 2 + 1) {
           c[(2 * k * P + j) * 32] = re[q];
           c[((2 * k + 1) * P + j) * 32] = im[q];
@@ -236,9 +236,9 @@ __device__ __forceinline__ void mesh_dft(const Params& p, T* col, cplx_t<T>* out
           re[n] = r[n * D2 * 32];
           im[n] = r[(P + n * D2) * 32];
         });
-        fft::fft_dif<N, 1>(re, im);
+        fft::pfa<N, 1>(re, im);
         fft::static_for<N>([&](auto I) {
-          constexpr int q = decltype(I)::value, k = fft::dif_rev(N, q);
+          constexpr int q = decltype(I)::value, k = fft::pfa_out(N, q);
           r[k * D2 * 32] = re[q];
           r[(P + k * D2) * 32] = im[q];
         });
@@ -255,12 +255,12 @@ __device__ __forceinline__ void mesh_dft(const Params& p, T* col, cplx_t<T>* out
         re[n] = r[n * 32];
         im[n] = r[(P + n) * 32];
       });
-      fft::fft_dif<N, 1>(re, im);
+      fft::pfa<N, 1>(re, im);
       const int g0 = (D0 - k0) % D0, g1 = (D1 - k1) % D1;   // -k on the first two axes
       const int* at = p.kidx + (k0 * D1 + k1) * D2;
       const int* neg = p.kidx + (g0 * D1 + g1) * D2;
       fft::static_for<N>([&](auto I) {
-        constexpr int q = decltype(I)::value, k = fft::dif_rev(N, q);
+        constexpr int q = decltype(I)::value, k = fft::pfa_out(N, q);
         const int i = at[k];
         if (i >= 0) out[(size_t)i * kstride + lane] = cplx_t<T>{re[q], im[q]};
         if (g0 != k0) {

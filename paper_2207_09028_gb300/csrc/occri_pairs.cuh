@@ -46,26 +46,27 @@ using dev::exp_t;
 using dev::expm1_t;
 
 constexpr int pitch(int n) { return (n % 2 == 0) ? n + 1 : n; }
-// Even edges use two threads per line (radix-2 split, see line_fft2), odd edges one.
+// Even edges use two threads per line (see line_fft2), odd edges one.
 constexpr int line_split(int n) { return (n % 2 == 0) ? 2 : 1; }
 constexpr int round32(int n) { return (n + 31) / 32 * 32; }
-// Where the two halves of a split line live. true: adjacent lanes of one warp, so that
-// both halves' loads of the same element are one shared-memory broadcast (the
-// half-dependent twiddle is then computed by both and selected). false: the halves of
-// lines 32w..32w+31 in warps 2w (h = 0) and 2w + 1 (h = 1), half-dependent code uniform
-// over each warp, every load its own shared-memory access.
-constexpr bool kPairLanes = false;
-constexpr int threads_for(int n) {
-  return line_split(n) == 1 ? round32(n) : (kPairLanes ? round32(2 * n) : 2 * round32(n));
+// Where the two halves of a split line live. FP32: neighbouring lanes of one warp, which read
+// the line's elements together (one broadcast for both, half the shared-memory wavefronts of
+// two warps; the transform passes are bound by those) and need no barrier wider than the warp.
+// FP64: lines 32 v .. 32 v + 31 in warps 2 v (half 0) and 2 v + 1 (half 1), so that half 0 skips
+// the twiddles (FP64 arithmetic is what bounds those passes).
+template <typename T> constexpr bool pair_lanes() { return sizeof(T) == 4; }
+template <typename T> constexpr int threads_for(int n) {
+  return line_split(n) == 1 ? round32(n) : (pair_lanes<T>() ? round32(2 * n) : 2 * round32(n));
 }
-// resident CTAs per SM requested from the register allocator
-constexpr int min_blocks(int n, int elem_bytes) {
-  return elem_bytes > 8 ? (n <= 32 ? 4 : 2) : (n <= 32 ? 8 : 4);
+// resident CTAs per SM requested from the register allocator: 512 threads per SM in FP32 (768 in
+// pass A, 80 registers), but for odd edges, whose threads hold a whole line
+template <typename T> constexpr int min_blocks(int n) {
+  return sizeof(T) > 4 ? (n <= 32 ? 4 : 2)
+                       : (line_split(n) == 2 ? 512 / threads_for<T>(n) : (n <= 32 ? 8 : 4));
 }
-// pass A (29 KB of shared memory at 60^3, FP32) runs six CTAs per SM (80 registers, no
-// spills): 4 % faster than five at 60^3; a seventh (72 registers) was 7 % slower
-constexpr int min_blocks_a(int n, int elem_bytes) {
-  return elem_bytes > 8 ? min_blocks(n, elem_bytes) : (n <= 32 ? 8 : 6);
+template <typename T> constexpr int min_blocks_a(int n) {
+  return sizeof(T) > 4 ? min_blocks<T>(n)
+                       : (line_split(n) == 2 ? 768 / threads_for<T>(n) : (n <= 32 ? 8 : 6));
 }
 // f(|G+q|)/(4 pi) of Eq. recipcoul for |G+q|^2 = g2 = g2h + g2l > 0 (a hi + lo pair).
 // The truncated Coulomb kernel (1 - cos(x R_c))/x^2 = 2 sin^2(x R_c/2)/x^2 is evaluated in
@@ -168,13 +169,13 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(PENDING));
 }
 
-// body(r, c) for every element of an N x N block, in a CTA of threads_for(N) threads:
+// body(r, c) for every element of an N x N block, in a CTA of threads_for<T>(N) threads:
 // thread t < RT N takes column c = t mod N and rows t / N, t / N + RT, ... (RT = the
-// threads_for(N) / N rows in flight), so the row is an induction variable and the
+// threads_for<T>(N) / N rows in flight), so the row is an induction variable and the
 // addresses advance by constant steps instead of being re-derived from a flat index.
-template <int N, typename F>
+template <typename T, int N, typename F>
 __device__ __forceinline__ void plane_loop(F&& body) {
-  constexpr int RT = threads_for(N) / N;
+  constexpr int RT = threads_for<T>(N) / N;
   static_assert(RT >= 1, "a thread per column");
   const int t = threadIdx.x;
   if (t < RT * N) {
@@ -187,19 +188,54 @@ __device__ __forceinline__ void plane_loop(F&& body) {
 // Copy a contiguous N x N plane into shared memory with row pitch P.
 template <typename T, int N, int P>
 __device__ __forceinline__ void stage_plane(cplx_t<T>* dst, const cplx_t<T>* src) {
-  plane_loop<N>([&](int r, int c) { cp_async<sizeof(cplx_t<T>)>(dst + r * P + c, src + r * N + c); });
+  plane_loop<T, N>([&](int r, int c) { cp_async<sizeof(cplx_t<T>)>(dst + r * P + c, src + r * N + c); });
 }
 
 // ------------------------------------------------------------------ one line transform
-// DFT (e^{-2 pi i m n / N}) of the N elements at base[m * stride], in place, with the
-// whole line in registers. The unnormalised inverse (e^{+2 pi i m n / N}) is the same
-// transform with output k stored at index (N - k) mod N. post(k, re, im) sees output
-// index k (after that reversal) before the store (store is skipped when !store). Every
-// call site has its own unrolled copy with a compile-time stride, so no address is
-// computed at run time from a stride.
-template <typename T, int N, typename Post>
-__device__ __forceinline__ void line_fft(cplx_t<T>* base, int stride, bool inverse, bool store,
-                                         Post&& post) {
+// DFT (e^{-2 pi i m n / N}; INV: e^{+2 pi i m n / N}, unnormalised) of the N elements at
+// base[m * stride], in place, with the whole line in registers. post(K, W, re, im) sees output
+// index K (+ the half's shift, below) before the store (no store with STORE = false). Every
+// call site has its own unrolled copy with a compile-time stride, so no address is computed
+// at run time from a stride.
+//
+// Two threads per line (even N = q m, q its power of 2, m odd): with k = (k_q, k_m) by residues,
+// half h forms the outputs with k_q = 2 t + h from
+//   y_h[n'] = (x[n'] + (-1)^h x[n' + q/2]) e^{-+2 pi i h n' / q},   n' < q/2 along the factor q,
+// which is a register transform of length N/2 (prime factors q/2 and those of m). Only n'
+// has a twiddle, so q = 2 needs none and q = 4 a product with i; the radix-2 split of the
+// natural order that this replaced needed N/2 - 1.
+// Output K of half 0 and of half 1 differ by E = crt_unit(N, q) modulo N: half 1's index is
+// K + E (W = 0) or K + E - N (W = 1), K known at compile time.
+template <int N> struct Split {
+  static constexpr int q = fft::prime_part(N, 2), M = N / 2, E = fft::crt_unit(N, q);
+  // index along the factor f of register p's element
+  static constexpr int along(int p, int f, int len) {
+    return (p % f) * fft::inv_mod((len / f) % f, f) % f;
+  }
+  static constexpr int n_half(int p) { return q / 2 > 1 ? along(p, q / 2, M) : 0; }
+  static constexpr int in(int p) {   // memory index of register p's first element
+    int n = n_half(p) * (N / q);
+    for (int f : {fft::prime_part(N, 3), fft::prime_part(N, 5)})
+      if (f > 1) n += along(p, f, M) * (N / f);
+    return n % N;
+  }
+  static constexpr int out(int p) {  // half 0's output index of register p
+    int k = 2 * (q / 2 > 1 ? fft::dif_rev(q / 2, n_half(p)) : 0) * E;
+    for (int f : {fft::prime_part(N, 3), fft::prime_part(N, 5)})
+      if (f > 1) k += fft::dif_rev(f, along(p, f, M)) * fft::crt_unit(N, f);
+    return k % N;
+  }
+};
+// Index shift of half h for outputs of class W.
+template <int N> __device__ __forceinline__ int half_shift(int h, int w) {
+  if constexpr (line_split(N) == 1) return 0;
+  else return h * (Split<N>::E - w * N);
+}
+template <int V> using IntC = std::integral_constant<int, V>;
+
+template <typename T, int N, bool INV, bool STORE, typename Post>
+__device__ __forceinline__ void line_fft(cplx_t<T>* base, int stride, Post&& post) {
+  constexpr int SG = INV ? 1 : -1;
   if constexpr (std::is_same<T, float>::value) {   // packed FP32 core
     fft::pk::u64 x[N];
     fft::static_for<N>([&](auto I) {
@@ -207,16 +243,13 @@ __device__ __forceinline__ void line_fft(cplx_t<T>* base, int stride, bool inver
       const float2 v = base[m * stride];
       x[m] = fft::pk::pack(v.x, v.y);
     });
-    fft::pfft_dif<N, -1>(x);
+    fft::ppfa<N, SG>(x);
     fft::static_for<N>([&](auto I) {
-      constexpr int q = decltype(I)::value;
-      constexpr int k = fft::dif_rev(N, q);
-      constexpr int kr = (N - k) % N;
-      const int ks = inverse ? kr : k;
+      constexpr int p = decltype(I)::value, k = fft::pfa_out(N, p);
       float re, im;
-      fft::pk::unpack(x[q], re, im);
-      post(ks, re, im);
-      if (store) base[ks * stride] = mk<T>(re, im);
+      fft::pk::unpack(x[p], re, im);
+      post(IntC<k>{}, IntC<0>{}, re, im);
+      if (STORE) base[k * stride] = mk<T>(re, im);
     });
   } else {
     T re[N], im[N];
@@ -226,170 +259,152 @@ __device__ __forceinline__ void line_fft(cplx_t<T>* base, int stride, bool inver
       re[m] = v.x;
       im[m] = v.y;
     });
-    fft::fft_dif<N, -1>(re, im);
+    fft::pfa<N, SG>(re, im);
     fft::static_for<N>([&](auto I) {
-      constexpr int q = decltype(I)::value;
-      constexpr int k = fft::dif_rev(N, q);
-      constexpr int kr = (N - k) % N;
-      const int ks = inverse ? kr : k;
-      post(ks, re[q], im[q]);
-      if (store) base[ks * stride] = mk<T>(re[q], im[q]);
+      constexpr int p = decltype(I)::value, k = fft::pfa_out(N, p);
+      post(IntC<k>{}, IntC<0>{}, re[p], im[p]);
+      if (STORE) base[k * stride] = mk<T>(re[p], im[p]);
     });
   }
 }
 
-// Two threads per line (even N), adjacent lanes or two warps (kPairLanes). Half h forms
-//   y_h[n] = (x[n] + (-1)^h x[n + N/2]) e^{-2 pi i h n / N},   n < N/2,
-// from the whole line in shared memory and transforms it with an N/2-point register
-// FFT, which gives the outputs X[2k + h] (radix-2 decimation in frequency). inverse,
-// store and post as in line_fft; `valid` is false for padding threads, which compute
-// on a duplicate line but neither store nor call post. The pair synchronises between
-// its loads and its stores: __syncwarp for adjacent lanes, else named barrier `bar`
-// (1 or 2: at most two pairs of warps per CTA, N <= 64), or with bar = 0 the whole CTA
-// (every thread of the CTA then calls it).
+// The two-thread form; `valid` is false for padding threads, which compute on a duplicate line
+// but neither store nor call post. Between its loads and its stores a pair synchronises:
+// lanes of one warp by __syncwarp, two warps by named barrier `bar` (1 or 2: at most two pairs
+// of warps per CTA, N <= 64); with bar = 0 the whole CTA does (every thread then calls it).
 struct NoMid {
   __device__ __forceinline__ void operator()() const {}
 };
 
-template <typename T, int N, typename Post, typename Mid = NoMid>
-__device__ __forceinline__ void line_fft2(cplx_t<T>* base, int stride, bool inverse, bool store,
-                                          int h, bool valid, int bar, Post&& post,
-                                          Mid&& mid = Mid()) {
-  constexpr int M = N / 2;
+template <typename T, int N, bool INV, bool STORE, typename Post, typename Mid = NoMid>
+__device__ __forceinline__ void line_fft2(cplx_t<T>* base, int stride, int h, bool valid, int bar,
+                                          Post&& post, Mid&& mid = Mid()) {
+  using SP = Split<N>;
+  constexpr int M = N / 2, SG = INV ? 1 : -1;
   auto pair_barrier = [&]() {
-    if constexpr (kPairLanes) {
-      __syncwarp();
-    } else if (bar == 0) {   // warp-uniform; immediate barrier ids
+    if (bar == 0) {   // warp-uniform; immediate barrier ids
       __syncthreads();
+    } else if constexpr (pair_lanes<T>()) {
+      __syncwarp();
     } else if (bar == 1) {
       asm volatile("bar.sync 1, 64;\n" ::: "memory");
     } else {
       asm volatile("bar.sync 2, 64;\n" ::: "memory");
     }
   };
-  if constexpr (std::is_same<T, float>::value) {   // packed FP32 core
+  cplx_t<T>* st[2] = {base + half_shift<N>(h, 0) * stride, base + half_shift<N>(h, 1) * stride};
+  auto wrap = [](int k) constexpr { return k + SP::E >= N ? 1 : 0; };
+  if constexpr (std::is_same<T, float>::value) {   // packed FP32 core, no branch on h
     using fft::pk::u64;
     u64 x[M];
-    if constexpr (kPairLanes) {   // both halves in one warp: no branch on h
-      fft::static_for<M>([&](auto I) {
-        constexpr int n = decltype(I)::value;
-        constexpr fft::CS w = fft::cs2pi(n, N);     // e^{-2 pi i n / N} = c - i s
-        const float2 a = base[n * stride], b = base[(n + M) * stride];
-        const u64 pa = fft::pk::pack(a.x, a.y), pb = fft::pk::pack(b.x, b.y);
-        if constexpr (n == 0) {
-          x[n] = h ? fft::pk::sub(pa, pb) : fft::pk::add(pa, pb);
-        } else {
-          const u64 t = fft::pk::cmul_const(fft::pk::sub(pa, pb), float(w.c), float(-w.s));
-          x[n] = h ? t : fft::pk::add(pa, pb);
-        }
-      });
-    } else if (h == 0) {
-      fft::static_for<M>([&](auto I) {
-        constexpr int n = decltype(I)::value;
-        const float2 a = base[n * stride], b = base[(n + M) * stride];
-        x[n] = fft::pk::add(fft::pk::pack(a.x, a.y), fft::pk::pack(b.x, b.y));
-      });
-    } else {
-      fft::static_for<M>([&](auto I) {
-        constexpr int n = decltype(I)::value;
-        constexpr fft::CS w = fft::cs2pi(n, N);     // e^{-2 pi i n / N} = c - i s
-        const float2 a = base[n * stride], b = base[(n + M) * stride];
-        const u64 d = fft::pk::sub(fft::pk::pack(a.x, a.y), fft::pk::pack(b.x, b.y));
-        if constexpr (n == 0)
-          x[n] = d;
-        else
-          x[n] = fft::pk::cmul_const(d, float(w.c), float(-w.s));
-      });
-    }
-    pair_barrier();
-    mid();   // every line of the CTA is in registers when bar == 0
-    fft::pfft_dif<M, -1>(x);
+    const float sg = h ? -1.f : 1.f;
+    const u64 sg2 = fft::pk::pack(sg, sg);
     fft::static_for<M>([&](auto I) {
-      constexpr int q = decltype(I)::value;
-      const int k = 2 * fft::dif_rev(M, q) + h;
-      const int ks = inverse ? (k == 0 ? 0 : N - k) : k;
-      if (valid) {
-        float re, im;
-        fft::pk::unpack(x[q], re, im);
-        post(ks, re, im);
-        if (store) base[ks * stride] = mk<T>(re, im);
+      constexpr int p = decltype(I)::value, n = SP::in(p), e = SP::n_half(p);
+      const float2 a = base[n * stride], b = base[((n + M) % N) * stride];
+      x[p] = fft::pk::fma(fft::pk::pack(b.x, b.y), sg2, fft::pk::pack(a.x, a.y));
+      if constexpr (4 * e == SP::q) {          // half 1: times -+i
+        float r, i;
+        fft::pk::unpack(x[p], r, i);
+        x[p] = fft::pk::pack(h ? -SG * i : r, h ? SG * r : i);
+      } else if constexpr (e != 0) {
+        constexpr fft::CS w = fft::cs2pi(e, SP::q);
+        const float c = h ? float(w.c) : 1.f, s = h ? float(SG * w.s) : 0.f;
+        float r, i;
+        fft::pk::unpack(x[p], r, i);
+        x[p] = fft::pk::pack(r * c - i * s, r * s + i * c);
       }
     });
+    pair_barrier();
+    mid();   // every line of the CTA is in registers when bar == 0
+    fft::ppfa<M, SG>(x);
+    if (valid) {
+      fft::static_for<M>([&](auto I) {
+        constexpr int p = decltype(I)::value, k = SP::out(p), w = wrap(k);
+        float re, im;
+        fft::pk::unpack(x[p], re, im);
+        post(IntC<k>{}, IntC<w>{}, re, im);
+        if (STORE) st[w][k * stride] = mk<T>(re, im);
+      });
+    }
   } else {
     T re[M], im[M];
     if (h == 0) {
       fft::static_for<M>([&](auto I) {
-        constexpr int n = decltype(I)::value;
-        const cplx_t<T> a = base[n * stride], b = base[(n + M) * stride];
-        re[n] = a.x + b.x;
-        im[n] = a.y + b.y;
+        constexpr int p = decltype(I)::value, n = SP::in(p);
+        const cplx_t<T> a = base[n * stride], b = base[((n + M) % N) * stride];
+        re[p] = a.x + b.x;
+        im[p] = a.y + b.y;
       });
     } else {
       fft::static_for<M>([&](auto I) {
-        constexpr int n = decltype(I)::value;
-        constexpr fft::CS w = fft::cs2pi(n, N);     // e^{-2 pi i n / N} = c - i s
-        const cplx_t<T> a = base[n * stride], b = base[(n + M) * stride];
-        const T yr = a.x - b.x, yi = a.y - b.y;
-        if constexpr (n == 0) {
-          re[n] = yr;
-          im[n] = yi;
-        } else {
-          re[n] = yr * T(w.c) + yi * T(w.s);
-          im[n] = yi * T(w.c) - yr * T(w.s);
-        }
+        constexpr int p = decltype(I)::value, n = SP::in(p), e = SP::n_half(p);
+        const cplx_t<T> a = base[n * stride], b = base[((n + M) % N) * stride];
+        re[p] = a.x - b.x;
+        im[p] = a.y - b.y;
+        fft::twiddle<SP::q, SG, e, p>(re, im);
       });
     }
     pair_barrier();
     mid();   // every line of the CTA is in registers when bar == 0
-    fft::fft_dif<M, -1>(re, im);
-    fft::static_for<M>([&](auto I) {
-      constexpr int q = decltype(I)::value;
-      const int k = 2 * fft::dif_rev(M, q) + h;
-      const int ks = inverse ? (k == 0 ? 0 : N - k) : k;
-      if (valid) {
-        post(ks, re[q], im[q]);
-        if (store) base[ks * stride] = mk<T>(re[q], im[q]);
-      }
-    });
-  }
-}
-
-// One transform job over the N lines of a plane (rows: along the contiguous index;
-// columns: along the pitched index); every thread of the CTA must call it.
-// As run_lines for even N, with the pair barrier made CTA-wide and mid() called after it by
-// every thread: the plane in shared memory is free from then on (every line is in registers).
-template <typename T, int N, typename Post, typename Mid>
-__device__ __forceinline__ void run_lines_then(cplx_t<T>* plane, int P, bool rows, bool inverse,
-                                               Post&& post, Mid&& mid) {
-  static_assert(line_split(N) == 2, "even edges");
-  const int w = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
-  const int line0 = kPairLanes ? (int)threadIdx.x >> 1 : (w >> 1) * 32 + lane;
-  const int h = kPairLanes ? (int)threadIdx.x & 1 : w & 1;
-  const bool valid = line0 < N;
-  const int line = valid ? line0 : N - 1;
-  line_fft2<T, N>(rows ? plane + line * P : plane + line, rows ? 1 : P, inverse, false, h, valid,
-                  0, [&](int k, T& re, T& im) { post(line, k, re, im); }, mid);
-}
-
-template <typename T, int N, typename Post>
-__device__ __forceinline__ void run_lines(cplx_t<T>* plane, int P, bool rows, bool inverse,
-                                          bool store, Post&& post) {
-  if constexpr (line_split(N) == 2) {
-    const int w = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
-    const int line0 = kPairLanes ? (int)threadIdx.x >> 1 : (w >> 1) * 32 + lane;
-    const int h = kPairLanes ? (int)threadIdx.x & 1 : w & 1;
-    const bool valid = line0 < N;
-    const int line = valid ? line0 : N - 1;
-    line_fft2<T, N>(rows ? plane + line * P : plane + line, rows ? 1 : P, inverse, store, h,
-                    valid, 1 + (w >> 1), [&](int k, T& re, T& im) { post(line, k, re, im); });
-  } else {
-    if (threadIdx.x < N) {
-      const int line = threadIdx.x;
-      line_fft<T, N>(rows ? plane + line * P : plane + line, rows ? 1 : P, inverse, store,
-                     [&](int k, T& re, T& im) { post(line, k, re, im); });
+    fft::pfa<M, SG>(re, im);
+    if (valid) {
+      fft::static_for<M>([&](auto I) {
+        constexpr int p = decltype(I)::value, k = SP::out(p), w = wrap(k);
+        post(IntC<k>{}, IntC<w>{}, re[p], im[p]);
+        if (STORE) st[w][k * stride] = mk<T>(re[p], im[p]);
+      });
     }
   }
 }
+
+// The plane line of this thread and its half. In FP32 the half warps hold the even and the odd
+// lines of a warp's sixteen: half 1's stores are an odd distance from half 0's, so the two
+// never share a bank.
+struct LineId { int line, h; bool valid; };
+template <typename T, int N> __device__ __forceinline__ LineId line_id() {
+  const int w = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+  LineId r;
+  if constexpr (line_split(N) == 1) {
+    r.line = threadIdx.x;
+    r.h = 0;
+  } else if constexpr (pair_lanes<T>()) {
+    r.line = 16 * w + 2 * ((lane >> 1) & 7) + (lane >> 4);
+    r.h = lane & 1;
+  } else {
+    r.line = (w >> 1) * 32 + lane;
+    r.h = w & 1;
+  }
+  r.valid = r.line < N;
+  if (!r.valid) r.line = N - 1;
+  return r;
+}
+
+// One transform job over the N lines of a plane (ROWS: along the contiguous index; else
+// along the pitched index); every thread of the CTA must call it.
+template <typename T, int N, bool ROWS, bool INV, bool STORE, typename Post>
+__device__ __forceinline__ void run_lines(cplx_t<T>* plane, int P, const LineId& id, Post&& post) {
+  cplx_t<T>* base = ROWS ? plane + id.line * P : plane + id.line;
+  if constexpr (line_split(N) == 2) {
+    line_fft2<T, N, INV, STORE>(base, ROWS ? 1 : P, id.h, id.valid, 1 + ((int)threadIdx.x >> 6),
+                                post);
+  } else {
+    if (id.valid) line_fft<T, N, INV, STORE>(base, ROWS ? 1 : P, post);
+  }
+}
+// As run_lines for even N without a store, with the pair barrier made CTA-wide and mid() called
+// after it by every thread: the plane in shared memory is free from then on (every line is in
+// registers).
+template <typename T, int N, bool ROWS, bool INV, typename Post, typename Mid>
+__device__ __forceinline__ void run_lines_then(cplx_t<T>* plane, int P, const LineId& id,
+                                               Post&& post, Mid&& mid) {
+  static_assert(line_split(N) == 2, "even edges");
+  line_fft2<T, N, INV, false>(ROWS ? plane + id.line * P : plane + id.line, ROWS ? 1 : P, id.h,
+                              id.valid, 0, post, mid);
+}
+struct NoPost {
+  template <typename... A> __device__ __forceinline__ void operator()(A&&...) const {}
+};
 
 // ------------------------------------------------------------------ kernel values per bin
 // Per-CTA table for axis 1 and per-column constants for axes 2, 3 give, for the first
@@ -587,7 +602,7 @@ __device__ __forceinline__ long long qtab_index(const PairParams& p, int kpl) {
 // (m3, kpl, z) fills rows m1 = z (mod kVtabSplit) of plane m3.
 constexpr int kVtabSplit = 4;
 template <typename T, int N>
-__global__ void __launch_bounds__(threads_for(N))
+__global__ void __launch_bounds__(threads_for<T>(N))
 vtab_kernel(T* __restrict__ vt, PairParams p) {
   __shared__ Axis1<T> ax1[N];
   const int m3 = blockIdx.x, kpl = blockIdx.y;
@@ -599,7 +614,7 @@ vtab_kernel(T* __restrict__ vt, PairParams p) {
 // The plan's kernel tables (qtab_index order), once at plan creation: CTA (t, m3, z) fills
 // rows m1 = z (mod kVtabSplit) of plane m3 of table t.
 template <typename T, int N>
-__global__ void __launch_bounds__(threads_for(N))
+__global__ void __launch_bounds__(threads_for<T>(N))
 qtab_kernel(T* __restrict__ vq, PairParams p) {
   __shared__ Axis1<T> ax1[N];
   const int m3 = blockIdx.y;
@@ -622,7 +637,7 @@ qtab_kernel(T* __restrict__ vq, PairParams p) {
 // With ADJ (the adjoint build): the field is sigma = conj(u_jk') g_ik + conj(g_jk') u_ik,
 // g being the adjoint orbital field, i.e. the change of rho when u moves along g.
 template <typename T, int N, bool ADJ = false>
-__global__ void __launch_bounds__(threads_for(N), min_blocks_a(N, sizeof(cplx_t<T>)))
+__global__ void __launch_bounds__(threads_for<T>(N), min_blocks_a<T>(N))
 pass_a(const cplx_t<T>* __restrict__ psi, cplx_t<T>* __restrict__ S, PairParams p,
        const cplx_t<T>* __restrict__ gam = nullptr, T* __restrict__ vt = nullptr) {
   using C2 = cplx_t<T>;
@@ -652,7 +667,7 @@ pass_a(const cplx_t<T>* __restrict__ psi, cplx_t<T>* __restrict__ S, PairParams 
   if constexpr (ADJ) {
     const C2* gi = gam + (size_t)(p.k * p.nocc + fi.i) * p.fs + (size_t)n1 * N;
     const C2* gj = gam + (size_t)(kp * p.nocc + fi.j) * p.fs + (size_t)n1 * N;
-    plane_loop<N>([&](int n3, int n2) {
+    plane_loop<T, N>([&](int n3, int n2) {
       const size_t off = (size_t)n3 * N * N + n2;
       const C2 a = cmulc<T>(__ldg(pj + off), __ldg(gi + off));
       const C2 b = cmulc<T>(__ldg(gj + off), __ldg(pi + off));
@@ -662,7 +677,7 @@ pass_a(const cplx_t<T>* __restrict__ psi, cplx_t<T>* __restrict__ S, PairParams 
     // two points per 16-byte load: N/2 threads per row, more bytes in flight per thread
     // (every plane row starts 16-byte aligned: fs, N and the column are even)
     constexpr int H = N / 2;
-    constexpr int RT2 = threads_for(N) / H;
+    constexpr int RT2 = threads_for<T>(N) / H;
     const int t = threadIdx.x;
     if (t < RT2 * H) {
       const int c = 2 * (t % H);
@@ -677,19 +692,21 @@ pass_a(const cplx_t<T>* __restrict__ psi, cplx_t<T>* __restrict__ S, PairParams 
       }
     }
   } else {
-    plane_loop<N>([&](int n3, int n2) {
+    plane_loop<T, N>([&](int n3, int n2) {
       const size_t off = (size_t)n3 * N * N + n2;
       pl[n2 * P + n3] = cmulc<T>(__ldg(pj + off), __ldg(pi + off));
     });
   }
   __syncthreads();
   // columns (line n3, along n2), then rows (line m2, along n3); the rows' outputs go
-  // straight to S[f][m3][n1][m2], a warp's lanes on consecutive m2
-  run_lines<T, N>(pl, P, false, false, true, [](int, int, T&, T&) {});
+  // straight to S[f][m3][n1][m2], a half warp's lanes on consecutive m2
+  const LineId id = line_id<T, N>();
+  run_lines<T, N, false, false, true>(pl, P, id, NoPost());
   __syncthreads();
-  C2* out = S + (size_t)f * p.fs;
-  run_lines<T, N>(pl, P, true, false, false, [&](int line, int k, T& re, T& im) {
-    out[((size_t)k * N + n1) * N + line] = mk<T>(re, im);
+  C2* o0 = S + (size_t)f * p.fs + n1 * N + id.line;
+  C2* out[2] = {o0 + half_shift<N>(id.h, 0) * N * N, o0 + half_shift<N>(id.h, 1) * N * N};
+  run_lines<T, N, true, false, false>(pl, P, id, [&](auto K, auto W, T& re, T& im) {
+    out[decltype(W)::value][decltype(K)::value * N * N] = mk<T>(re, im);
   });
 }
 
@@ -748,6 +765,8 @@ __device__ __forceinline__ void pass_b_body(cplx_t<T>* __restrict__ S, const Pai
   if (i0 < i1) stage(i0);
   cp_async_commit();
   T dsum = T(0);
+  const LineId id = line_id<T, N>();
+  const int sh[2] = {half_shift<N>(id.h, 0) * N + id.line, half_shift<N>(id.h, 1) * N + id.line};
 #pragma unroll 1
   for (int it = i0; it < i1; ++it) {
     const int m3 = it / nf, f = it - (it / nf) * nf;
@@ -763,10 +782,9 @@ __device__ __forceinline__ void pass_b_body(cplx_t<T>* __restrict__ S, const Pai
     __syncthreads();
     // an unordered pair stands for itself and its reverse, except (k, k, i, i)
     const T wgt = (p.diag && fi.i == fi.j) ? T(1) : T(2);
-    // columns (m2 = line): forward along n1, times v (the only forward transform, so its
-    // output indices are constants)
-    run_lines<T, N>(plane, P, false, false, !DOMEGA, [&](int line, int k, T& re, T& im) {
-      const T v = vtab[k * N + line];
+    // columns (m2 = line): forward along n1, times v
+    run_lines<T, N, false, false, !DOMEGA>(plane, P, id, [&](auto K, auto W, T& re, T& im) {
+      const T v = vtab[sh[decltype(W)::value] + decltype(K)::value * N];
       if constexpr (DOMEGA) {
         dsum += wgt * v * (re * re + im * im);
       } else {
@@ -777,20 +795,23 @@ __device__ __forceinline__ void pass_b_body(cplx_t<T>* __restrict__ S, const Pai
     __syncthreads();
     if constexpr (!DOMEGA) {
       // inverse along m2 (rows), then along m1 (columns); the columns' outputs go straight
-      // to S[f][m3][n1][n2], a warp's lanes on consecutive n2
-      run_lines<T, N>(plane, P, true, true, true, [](int, int, T&, T&) {});
+      // to S[f][m3][n1][n2], a half warp's lanes on consecutive n2
+      run_lines<T, N, true, true, true>(plane, P, id, NoPost());
       __syncthreads();
       C2* buf = S + (size_t)f * p.fs + (size_t)m3 * N * N;
-      auto out = [&](int line, int k, T& re, T& im) { buf[(size_t)k * N + line] = mk<T>(re, im); };
+      C2* bo[2] = {buf + sh[0], buf + sh[1]};
+      auto out = [&](auto K, auto W, T& re, T& im) {
+        bo[decltype(W)::value][decltype(K)::value * N] = mk<T>(re, im);
+      };
       if constexpr (line_split(N) == 2) {
         // the next item's copies start as soon as every line of this last transform is in
         // registers, and overlap its arithmetic and stores
-        run_lines_then<T, N>(plane, P, false, true, out, [&]() {
+        run_lines_then<T, N, false, true>(plane, P, id, out, [&]() {
           if (it + 1 < i1) stage(it + 1);
           cp_async_commit();
         });
       } else {
-        run_lines<T, N>(plane, P, false, true, false, out);
+        run_lines<T, N, false, true, false>(plane, P, id, out);
         __syncthreads();   // releases the buffers for the next item's copies
         if (it + 1 < i1) stage(it + 1);
         cp_async_commit();
@@ -814,13 +835,13 @@ __device__ __forceinline__ void pass_b_body(cplx_t<T>* __restrict__ S, const Pai
 }
 
 template <typename T, int N>
-__global__ void __launch_bounds__(threads_for(N), min_blocks(N, sizeof(cplx_t<T>)))
+__global__ void __launch_bounds__(threads_for<T>(N), min_blocks<T>(N))
 pass_b(cplx_t<T>* __restrict__ S, PairParams p, const T* __restrict__ vt) {
   pass_b_body<T, N, false>(S, p, vt, nullptr);
 }
 
 template <typename T, int N>
-__global__ void __launch_bounds__(threads_for(N), min_blocks(N, sizeof(cplx_t<T>)))
+__global__ void __launch_bounds__(threads_for<T>(N), min_blocks<T>(N))
 pass_b_domega(cplx_t<T>* __restrict__ S, PairParams p, double* dacc) {
   pass_b_body<T, N, true>(S, p, nullptr, dacc);
 }
@@ -840,7 +861,7 @@ int resident_slots(K kernel, int threads, size_t smem) {
 // S[f][n3][n1][n2]. This is the periodic part e^{-iq.r} W of the potential, which is
 // what the accumulation of periodic parts needs.
 template <typename T, int N>
-__global__ void __launch_bounds__(threads_for(N), min_blocks(N, sizeof(cplx_t<T>)))
+__global__ void __launch_bounds__(threads_for<T>(N), min_blocks<T>(N))
 pass_c(cplx_t<T>* __restrict__ S, PairParams p) {
   using C2 = cplx_t<T>;
   constexpr int P = pitch(N);
@@ -849,16 +870,16 @@ pass_c(cplx_t<T>* __restrict__ S, PairParams p) {
   const int n1 = blockIdx.x;
   const int f = blockIdx.y;
   C2* rows = S + (size_t)f * p.fs + (size_t)n1 * N;   // row m3 at rows + m3 N^2
-  plane_loop<N>([&](int m3, int n2) {
+  plane_loop<T, N>([&](int m3, int n2) {
     cp_async<sizeof(C2)>(cur + m3 * P + n2, rows + (size_t)m3 * N * N + n2);
   });
   cp_async_commit();
   cp_async_wait<0>();
   __syncthreads();
   // columns (n2 = line): inverse along m3
-  run_lines<T, N>(cur, P, false, true, true, [](int, int, T&, T&) {});
+  run_lines<T, N, false, true, true>(cur, P, line_id<T, N>(), NoPost());
   __syncthreads();
-  plane_loop<N>([&](int n3, int n2) { rows[(size_t)n3 * N * N + n2] = cur[n3 * P + n2]; });
+  plane_loop<T, N>([&](int n3, int n2) { rows[(size_t)n3 * N * N + n2] = cur[n3 * P + n2]; });
 }
 
 // ------------------------------------------------------------------ pass D
@@ -1339,17 +1360,20 @@ pass_cd(const float2* __restrict__ S, const float2* __restrict__ psi, float2* __
 #pragma unroll 1
       for (int l0 = 0; l0 < lines; l0 += per_round) {
         if constexpr (SP == 2) {
-          const int w = t >> 5;
-          const int line0 = l0 + (w >> 1) * 32 + (t & 31);
+          // a warp's sixteen lines are four fields of four columns: even and odd fields in
+          // different half warps, whose stores then hit different banks (pitch 4 mod 16)
+          static_assert(CW == 4, "lane order");
+          const int lane = t & 31;
+          const int line0 = l0 + 16 * (t >> 5) + ((lane >> 1) & 3) + 4 * (lane >> 4) +
+                            8 * ((lane >> 3) & 1);
           const bool valid = line0 < lines;
           const int line = valid ? line0 : lines - 1;
-          line_fft2<float, N>(Wb + (line / CW) * PP + line % CW, CW, true, true, w & 1, valid, 0,
-                              [](int, float&, float&) {});
+          line_fft2<float, N, true, true>(Wb + (line / CW) * PP + line % CW, CW, lane & 1, valid,
+                                          1, NoPost());
         } else {
           const int line = l0 + t;
           if (line < lines)
-            line_fft<float, N>(Wb + (line / CW) * PP + line % CW, CW, true, true,
-                               [](int, float&, float&) {});
+            line_fft<float, N, true, true>(Wb + (line / CW) * PP + line % CW, CW, NoPost());
         }
       }
     }
@@ -1442,7 +1466,7 @@ pass_cd(const float2* __restrict__ S, const float2* __restrict__ psi, float2* __
 // and sum_m (dv/d omega)/(4 pi) Re(conj(sigma^) rho^) is added to *dacc, weight 1/2 for
 // a field (k, k, i, i) of a diagonal wave (the only pair that is its own reverse).
 template <typename T, int N>
-__global__ void __launch_bounds__(threads_for(N), min_blocks(N, sizeof(cplx_t<T>)))
+__global__ void __launch_bounds__(threads_for<T>(N), min_blocks<T>(N))
 pass_b_domega2(const cplx_t<T>* __restrict__ S0, const cplx_t<T>* __restrict__ S1,
                PairParams p, double* __restrict__ dacc) {
   using C2 = cplx_t<T>;
@@ -1464,17 +1488,17 @@ pass_b_domega2(const cplx_t<T>* __restrict__ S0, const cplx_t<T>* __restrict__ S
   cp_async_wait<0>();
   __syncthreads();
   T dsum = T(0);
-#pragma unroll 1
-  for (int job = 0; job < 2; ++job) {   // rho^ (stored), then sigma^ (paired with rho^)
-    run_lines<T, N>(job == 0 ? rho : sig, P, false, false, job == 0,
-                    [&](int line, int k, T& re, T& im) {
-                      if (job == 1) {
-                        const C2 r = rho[k * P + line];
-                        dsum += vtab[k * N + line] * (re * r.x + im * r.y);
-                      }
-                    });
-    __syncthreads();
-  }
+  const LineId id = line_id<T, N>();
+  const int s0 = half_shift<N>(id.h, 0), s1 = half_shift<N>(id.h, 1);
+  run_lines<T, N, false, false, true>(rho, P, id, NoPost());   // rho^ (stored)
+  __syncthreads();
+  const C2* rr[2] = {rho + s0 * P + id.line, rho + s1 * P + id.line};
+  const T* vv[2] = {vtab + s0 * N + id.line, vtab + s1 * N + id.line};
+  run_lines<T, N, false, false, false>(sig, P, id, [&](auto K, auto W, T& re, T& im) {
+    constexpr int k = decltype(K)::value, w = decltype(W)::value;
+    const C2 r = rr[w][k * P];
+    dsum += vv[w][k * N] * (re * r.x + im * r.y);
+  });
   double part = double(dsum);
   for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
@@ -1609,7 +1633,7 @@ template <typename T, int N>
 cudaError_t run_wave(const PairParams& p, const cplx_t<T>* psi, cplx_t<T>* S, cplx_t<T>* Y,
                      cudaStream_t st, cudaEvent_t* ev, cudaEvent_t ev_y) {
   using C2 = cplx_t<T>;
-  const int nt = threads_for(N);
+  const int nt = threads_for<T>(N);
   const int nf = wave_fields(p.nocc, p.nkp, p.diag);
   const size_t sa = smem_a<N>(sizeof(C2));
   const size_t sb = smem_b<N>(sizeof(C2), sizeof(Axis1<T>));
@@ -1659,7 +1683,7 @@ template <typename T, int N>
 cudaError_t run_domega_wave(const PairParams& p, const cplx_t<T>* psi, cplx_t<T>* S,
                             double* dacc, cudaStream_t st) {
   using C2 = cplx_t<T>;
-  const int nt = threads_for(N);
+  const int nt = threads_for<T>(N);
   const int nf = wave_fields(p.nocc, p.nkp, p.diag);
   const size_t sa = smem_a<N>(sizeof(C2));
   const size_t sb = smem_b<N>(sizeof(C2), sizeof(Axis1<T>));
@@ -1682,7 +1706,7 @@ cudaError_t run_vjp_wave(const PairParams& p, const cplx_t<T>* psi, const cplx_t
                          cplx_t<T>* S0, cplx_t<T>* S1, cplx_t<T>* G, double* dacc,
                          cudaStream_t st) {
   using C2 = cplx_t<T>;
-  const int nt = threads_for(N);
+  const int nt = threads_for<T>(N);
   const int nf = wave_fields(p.nocc, p.nkp, p.diag);
   const size_t sa = smem_a<N>(sizeof(C2));
   const size_t sb = smem_b<N>(sizeof(C2), sizeof(Axis1<T>));
@@ -1718,7 +1742,7 @@ cudaError_t run_vjp_wave(const PairParams& p, const cplx_t<T>* psi, const cplx_t
 template <typename T, int N>
 cudaError_t run_qtables(const PairParams& p, T* vq, cudaStream_t st) {
   const unsigned nq = (unsigned)((2 * p.D[0] - 1) * (2 * p.D[1] - 1) * (2 * p.D[2] - 1));
-  qtab_kernel<T, N><<<dim3(nq, N, kVtabSplit), threads_for(N), 0, st>>>(vq, p);
+  qtab_kernel<T, N><<<dim3(nq, N, kVtabSplit), threads_for<T>(N), 0, st>>>(vq, p);
   return cudaGetLastError();
 }
 
