@@ -344,102 +344,200 @@ __device__ void record_status(int* status, int code, int k) {
   if (atomicCAS(status, 0, code) == 0) status[1] = k;
 }
 
-// One CTA per k: M = C^H KC (Hermitised), -M = L L^H, xi = KC L^{-H},
-// K = -xi xi^H, ek[k] = Re Tr M.
+// Step (f), first half: M = C^H KC (Hermitised), -M = L L^H per k, ek[k] = Re Tr M and E_x.
+// gridDim.x CTAs per k sum a share of the rows each; the last one to finish adds the shares in
+// order and factorises (a warp, a lane per row of the column), the last k's also sums E_x. One
+// CTA and one thread for all of it took 31 us at Gamma and, with the K product that
+// ace_k_kernel now spreads over the GPU, 1.9 ms at 64 k, 350 AOs, nocc 8: an SM adds two FP64
+// products per cycle. `ticket` holds nk + 1 counters, zero between builds.
 __global__ void __launch_bounds__(256)
-ace_kernel(const double2* __restrict__ C, const double2* __restrict__ kc, double2* __restrict__ xi,
-           double2* __restrict__ mout, double* __restrict__ ek, double2* __restrict__ K, int nao,
-           int nocc, double pivot_tol, int* status) {
+ace_factor_kernel(const double2* __restrict__ C, const double2* __restrict__ kc,
+                  double2* __restrict__ share, double2* __restrict__ mout,
+                  double2* __restrict__ lout, int* __restrict__ okout, double* __restrict__ ek,
+                  double* __restrict__ ex, int nk, int nao, int nocc, double pivot_tol,
+                  int* __restrict__ ticket, int* status) {
   extern __shared__ double2 sm[];
-  double2* M = sm;                   // nocc*nocc
-  double2* L = sm + nocc * nocc;     // nocc*nocc
-  __shared__ int ok;
-  const int k = blockIdx.x;
+  const int nn = nocc * nocc;
+  double2* A = sm;        // the share, then all of C^H KC, then L
+  double2* M = sm + nn;
+  __shared__ int last, ok;
+  const int k = blockIdx.y, S = gridDim.x;
+  const int mu0 = (int)((long long)nao * blockIdx.x / S), mu1 = (int)((long long)nao * (blockIdx.x + 1) / S);
   const double2* Ck = C + (size_t)k * nao * nocc;
   const double2* KCk = kc + (size_t)k * nao * nocc;
-  for (int e = threadIdx.x; e < nocc * nocc; e += blockDim.x) {
-    const int i = e / nocc, j = e - (e / nocc) * nocc;
-    double sr = 0.0, si = 0.0;
-    for (int mu = 0; mu < nao; ++mu) {
-      const double2 c = Ck[(size_t)mu * nocc + i], x = KCk[(size_t)mu * nocc + j];
-      sr += c.x * x.x + c.y * x.y;   // conj(c) * x
-      si += c.x * x.y - c.y * x.x;
+  // rows split over the threads that share an element, their sums added in order
+  const int per = max(1, min(16, 256 / nn));   // threads per element
+  __shared__ double2 red[256];
+  for (int e0 = 0; e0 < nn; e0 += 256 / per) {
+    const int e = e0 + (int)threadIdx.x / per, z = (int)threadIdx.x % per;
+    double2 t = make_double2(0.0, 0.0);
+    const bool in = e < nn && (int)threadIdx.x < 256 / per * per;
+    if (in) {
+      const int i = e / nocc, j = e - i * nocc;
+#pragma unroll 4
+      for (int mu = mu0 + z; mu < mu1; mu += per) {
+        const double2 c = Ck[(size_t)mu * nocc + i], x = KCk[(size_t)mu * nocc + j];
+        t.x += c.x * x.x + c.y * x.y;   // conj(c) * x
+        t.y += c.x * x.y - c.y * x.x;
+      }
     }
-    L[e] = make_double2(sr, si);
+    __syncthreads();
+    red[threadIdx.x] = t;
+    __syncthreads();
+    if (in && z == 0) {
+      for (int y = 1; y < per; ++y) {
+        t.x += red[threadIdx.x + y].x;
+        t.y += red[threadIdx.x + y].y;
+      }
+      A[e] = t;
+    }
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < nocc * nocc; e += blockDim.x) {
+  if (S > 1) {
+    double2* mine = share + ((size_t)k * S + blockIdx.x) * nn;
+    for (int e = threadIdx.x; e < nn; e += blockDim.x) mine[e] = A[e];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&ticket[k], 1) == S - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int e = threadIdx.x; e < nn; e += blockDim.x) {
+      double2 t = make_double2(0.0, 0.0);
+      for (int x = 0; x < S; ++x) {
+        const double2 v = __ldcg(share + ((size_t)k * S + x) * nn + e);
+        t.x += v.x;
+        t.y += v.y;
+      }
+      A[e] = t;
+    }
+    if (threadIdx.x == 0) ticket[k] = 0;
+    __syncthreads();
+  }
+  for (int e = threadIdx.x; e < nn; e += blockDim.x) {
     const int i = e / nocc, j = e - (e / nocc) * nocc;
-    const double2 a = L[i * nocc + j], b = L[j * nocc + i];
+    const double2 a = A[i * nocc + j], b = A[j * nocc + i];
     M[e] = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    ok = 1;
-    double tr = 0.0;
-    for (int i = 0; i < nocc; ++i) tr += M[i * nocc + i].x;
-    ek[k] = tr;
-    for (int e = 0; e < nocc * nocc; ++e) mout[(size_t)k * nocc * nocc + e] = M[e];
-    // Cholesky of A = -M (lower, complex Hermitian); a pivot at or below
-    // pivot_tol * max_j A_jj counts as not positive definite.
-    double amax = 0.0;
-    for (int j = 0; j < nocc; ++j) amax = fmax(amax, -M[j * nocc + j].x);
-    for (int j = 0; j < nocc && ok; ++j) {
-      double d = -M[j * nocc + j].x;
-      for (int l = 0; l < j; ++l) d -= L[j * nocc + l].x * L[j * nocc + l].x + L[j * nocc + l].y * L[j * nocc + l].y;
-      if (!(d > pivot_tol * amax) || !isfinite(d)) { ok = 0; break; }
-      const double ljj = sqrt(d);
-      L[j * nocc + j] = make_double2(ljj, 0.0);
-      for (int i = j + 1; i < nocc; ++i) {
-        double ar = -M[i * nocc + j].x, ai = -M[i * nocc + j].y;
-        for (int l = 0; l < j; ++l) {  // - L_il conj(L_jl)
-          const double2 x = L[i * nocc + l], y = L[j * nocc + l];
-          ar -= x.x * y.x + x.y * y.y;
-          ai -= x.y * y.x - x.x * y.y;
-        }
-        L[i * nocc + j] = make_double2(ar / ljj, ai / ljj);
-      }
-      for (int i = 0; i < j; ++i) L[i * nocc + j] = make_double2(0.0, 0.0);
-    }
-    if (!ok) record_status(status, OCCRI_ENOTPD, k);
-  }
-  __syncthreads();
-  if (!ok) return;
-  // xi L^H = KC  ->  xi_j = (KC_j - sum_{l<j} xi_l conj(L_jl)) / L_jj
-  double2* xik = xi + (size_t)k * nao * nocc;
-  for (int mu = threadIdx.x; mu < nao; mu += blockDim.x) {
+  for (int e = threadIdx.x; e < nn; e += blockDim.x) mout[(size_t)k * nn + e] = M[e];
+  if (threadIdx.x < 32) {
+    // Cholesky of -M (lower, complex Hermitian), column by column with lane i on row i (nocc
+    // <= 32); a pivot at or below pivot_tol * max_j (-M_jj) counts as not positive definite.
+    const int i = threadIdx.x;
+    double tr = 0.0, amax = 0.0;
     for (int j = 0; j < nocc; ++j) {
-      double2 v = KCk[(size_t)mu * nocc + j];
-      for (int l = 0; l < j; ++l) {
-        const double2 x = xik[(size_t)mu * nocc + l], y = L[j * nocc + l];
-        v.x -= x.x * y.x + x.y * y.y;
-        v.y -= x.y * y.x - x.x * y.y;
+      tr += M[j * nocc + j].x;
+      amax = fmax(amax, -M[j * nocc + j].x);
+    }
+    int good = 1;
+    for (int j = 0; j < nocc; ++j) {
+      double2 v = make_double2(0.0, 0.0);
+      if (i >= j && i < nocc) {
+        v = make_double2(-M[i * nocc + j].x, -M[i * nocc + j].y);
+        for (int l = 0; l < j; ++l) {  // - L_il conj(L_jl)
+          const double2 x = A[i * nocc + l], y = A[j * nocc + l];
+          v.x -= x.x * y.x + x.y * y.y;
+          v.y -= x.y * y.x - x.x * y.y;
+        }
       }
-      const double ljj = L[j * nocc + j].x;
-      xik[(size_t)mu * nocc + j] = make_double2(v.x / ljj, v.y / ljj);
+      const double d = __shfl_sync(0xffffffffu, v.x, j);
+      if (!(d > pivot_tol * amax) || !isfinite(d)) { good = 0; break; }
+      const double ljj = sqrt(d);
+      __syncwarp();
+      if (i < nocc)
+        A[i * nocc + j] = i < j ? make_double2(0.0, 0.0)
+                                : (i == j ? make_double2(ljj, 0.0) : make_double2(v.x / ljj, v.y / ljj));
+      __syncwarp();
+    }
+    if (i == 0) {
+      ok = good;
+      okout[k] = good;
+      ek[k] = tr;
+      if (!good) record_status(status, OCCRI_ENOTPD, k);
     }
   }
   __syncthreads();
-  if (K == nullptr) return;
-  double2* Kk = K + (size_t)k * nao * nao;
-  for (size_t e = threadIdx.x; e < (size_t)nao * nao; e += blockDim.x) {
-    const int mu = (int)(e / nao), nu = (int)(e - (e / nao) * nao);
-    double sr = 0.0, si = 0.0;
-    for (int j = 0; j < nocc; ++j) {  // xi_mu conj(xi_nu)
-      const double2 a = xik[(size_t)mu * nocc + j], b = xik[(size_t)nu * nocc + j];
-      sr += a.x * b.x + a.y * b.y;
-      si += a.y * b.x - a.x * b.y;
+  if (ok)
+    for (int e = threadIdx.x; e < nn; e += blockDim.x) lout[(size_t)k * nn + e] = A[e];
+  if (ex == nullptr) return;
+  if (threadIdx.x < 32) {   // the last k adds the energies in order
+    int all = 0;
+    if (threadIdx.x == 0) {
+      __threadfence();
+      all = atomicAdd(&ticket[nk], 1) == nk - 1;
+      __threadfence();
     }
-    Kk[e] = make_double2(-sr, -si);
+    if (!__shfl_sync(0xffffffffu, all, 0)) return;
+    double s = 0.0;
+    for (int q = threadIdx.x; q < nk; q += 32) s += __ldcg(ek + q);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) {
+      *ex = s / nk;
+      ticket[nk] = 0;
+    }
   }
 }
 
-__global__ void ex_kernel(const double* __restrict__ ek, int nk, double* __restrict__ ex) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int k = 0; k < nk; ++k) s += ek[k];
-    *ex = s / nk;
+// Step (f), second half: xi L^H = KC and K = -xi xi^H, a CTA per (tile pair bi <= bj of TILE AOs,
+// k). Each CTA solves its own rows of xi; the tile below the diagonal is the conjugate of the
+// one above it.
+template <int TILE>
+__global__ void __launch_bounds__(256)
+ace_k_kernel(const double2* __restrict__ kc, const double2* __restrict__ lmat,
+             const int* __restrict__ okin, double2* __restrict__ K, int nao, int nocc, int T) {
+  extern __shared__ double2 sm[];
+  double2* L = sm;                    // nocc x nocc
+  double2* X = sm + nocc * nocc;      // [2 TILE][nocc + 1]
+  const int k = blockIdx.y, pitch = nocc + 1;
+  if (!okin[k]) return;
+  int bi = 0, bj = blockIdx.x;
+  while (bj >= T - bi) { bj -= T - bi; ++bi; }
+  bj += bi;
+  for (int e = threadIdx.x; e < nocc * nocc; e += blockDim.x) L[e] = lmat[(size_t)k * nocc * nocc + e];
+  for (int e = threadIdx.x; e < 2 * TILE * nocc; e += blockDim.x) {
+    const int r = e / nocc, j = e - r * nocc;
+    const int mu = (r < TILE ? bi * TILE + r : bj * TILE + r - TILE);
+    X[r * pitch + j] = mu < nao ? kc[((size_t)k * nao + mu) * nocc + j] : make_double2(0.0, 0.0);
   }
+  __syncthreads();
+  for (int r = threadIdx.x; r < 2 * TILE; r += blockDim.x) {
+    // xi_j = (KC_j - sum_{l<j} xi_l conj(L_jl)) / L_jj
+    double2* x = X + r * pitch;
+    for (int j = 0; j < nocc; ++j) {
+      double2 v = x[j];
+      for (int l = 0; l < j; ++l) {
+        const double2 u = x[l], y = L[j * nocc + l];
+        v.x -= u.x * y.x + u.y * y.y;
+        v.y -= u.y * y.x - u.x * y.y;
+      }
+      const double ljj = L[j * nocc + j].x;
+      x[j] = make_double2(v.x / ljj, v.y / ljj);
+    }
+  }
+  __syncthreads();
+  double2* Kk = K + (size_t)k * nao * nao;
+  for (int e = threadIdx.x; e < TILE * TILE; e += blockDim.x) {
+    const int r = e / TILE, c = e - r * TILE;
+    const int mu = bi * TILE + r, nu = bj * TILE + c;
+    if (mu >= nao || nu >= nao || (bi == bj && nu < mu)) continue;
+    const double2* a = X + r * pitch;
+    const double2* b = X + (TILE + c) * pitch;
+    double sr = 0.0, si = 0.0;
+    for (int j = 0; j < nocc; ++j) {  // xi_mu conj(xi_nu)
+      sr += a[j].x * b[j].x + a[j].y * b[j].y;
+      si += a[j].y * b[j].x - a[j].x * b[j].y;
+    }
+    if (mu == nu) si = 0.0;   // |xi|^2, up to what its products' rounding leaves
+    Kk[(size_t)mu * nao + nu] = make_double2(-sr, -si);
+    if (mu != nu) Kk[(size_t)nu * nao + mu] = make_double2(-sr, si);
+  }
+}
+
+// CTAs per k of ace_factor_kernel: about 4,000 FP64 products of the Gram matrix each
+int ace_shares(const Plan& p) {
+  const long long work = 4LL * p.nao * p.nocc * p.nocc;
+  return (int)std::max(1LL, std::min(16LL, work / 16000));
 }
 
 __global__ void scale_copy_kernel(const double2* __restrict__ in, double2* __restrict__ out,
@@ -617,16 +715,21 @@ ace_adjoint_kernel(const double2* __restrict__ C, const double2* __restrict__ kc
   }
 }
 
-// y += a + b over n complex values (the streams' private accumulators into Y)
+// y += a + b (b may be null) over n complex values (the streams' accumulators into Y)
 template <typename C2>
 __global__ void add3_kernel(C2* __restrict__ y, const C2* __restrict__ a, const C2* __restrict__ b,
                             long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     C2 v = y[i];
-    const C2 u = a[i], w = b[i];
-    v.x += u.x + w.x;
-    v.y += u.y + w.y;
+    C2 u = a[i];
+    if (b) {
+      const C2 w = b[i];
+      u.x += w.x;
+      u.y += w.y;
+    }
+    v.x += u.x;
+    v.y += u.y;
     y[i] = v;
   }
 }
@@ -642,7 +745,7 @@ void free_plan(Plan* p) {
   if (!p) return;
   void* bufs[] = {p->shells, p->atom_shell0, p->img_d, p->img_hi, p->img_lo, p->img_phase,
                   p->d0_d, p->d0_hi, p->d0_lo, p->t0, p->kint, p->psi, p->Y, p->scratch,
-                  p->kc, p->xi, p->mmat, p->ek, p->dacc, p->status, p->h_c, p->h_kc, p->h_k,
+                  p->kc, p->lmat, p->ace_share, p->ace_ok, p->mmat, p->ek, p->dacc, p->status, p->h_c, p->h_kc, p->h_k,
                   p->h_ex, p->ao_norm, p->cs, p->blist, p->bpre};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -725,12 +828,16 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
   const bool timed = p->timing_every != 0;   // > 0: sampled waves too; -1: stage spans only
   long long launches = 0;
   const size_t orb = (size_t)p->nk * p->nocc * p->fs;
+  // streams that get a wave (a Gamma build has one wave)
+  long long nwaves = 0;
+  for (int k = 0; k < p->nk; ++k)
+    nwaves += 1 + (p->nk - k - 1 + p->nkp_wave - 1) / p->nkp_wave;
+  const int ns = (int)std::min<long long>(p->nstreams, nwaves);
+  const bool split_y = ns > 1 && p->Yx[0] && p->Yx[1];
   if (cudaMemsetAsync(p->Y, 0, orb * sizeof(cplx_t<T>), s) != cudaSuccess) return OCCRI_ECUDA;
-  for (void* yx : p->Yx)
-    if (yx && cudaMemsetAsync(yx, 0, orb * sizeof(cplx_t<T>), s) != cudaSuccess)
+  for (int o = 1; o < ns && split_y; ++o)
+    if (cudaMemsetAsync(p->Yx[o - 1], 0, orb * sizeof(cplx_t<T>), s) != cudaSuccess)
       return OCCRI_ECUDA;
-  if (cudaMemsetAsync(p->kc, 0, sizeof(double2) * (size_t)p->nk * p->nao * p->nocc, s) != cudaSuccess)
-    return OCCRI_ECUDA;
   {
     StageTimer t(p, timed);
     if (launch_slot_c<T>(*p, C, p->cs, 1.0, s) != cudaSuccess) return OCCRI_ECUDA;
@@ -748,21 +855,19 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
     // streams by ev_y. A sampled wave runs alone (the streams wait for each other around
     // it) so that its pass times are not mixed with another stream's work.
     StageTimer all(p, timed);
-    const int ns = p->nstreams;
     cudaStream_t st[3] = {s, p->aux, p->aux2};
     void* sc[3] = {p->scratch, p->scratch2, p->scratch3};
     // with private accumulators per stream, no wave waits for another stream's Y updates
-    const bool split_y = p->Yx[0] && p->Yx[1];
     void* yacc[3] = {p->Y, split_y ? p->Yx[0] : p->Y, split_y ? p->Yx[1] : p->Y};
-    cudaEvent_t ev_y = split_y ? nullptr : p->ev_y;
+    cudaEvent_t ev_y = split_y || ns == 1 ? nullptr : p->ev_y;
     cudaEvent_t join[3] = {nullptr, p->ev_join, p->ev_join2};
     cudaEvent_t iso[3] = {p->ev_iso, p->ev_iso2, p->ev_iso3};
-    if (cudaEventRecord(p->ev_fork, s) != cudaSuccess) return OCCRI_ECUDA;
+    if (ns > 1 && cudaEventRecord(p->ev_fork, s) != cudaSuccess) return OCCRI_ECUDA;
     for (int o = 1; o < ns; ++o)
       if (cudaStreamWaitEvent(st[o], p->ev_fork, 0) != cudaSuccess) return OCCRI_ECUDA;
     // the first wave's accumulation waits on this record (within the same build, which
     // keeps the chain inside a captured graph when the build is captured)
-    if (cudaEventRecord(p->ev_y, s) != cudaSuccess) return OCCRI_ECUDA;
+    if (ev_y && cudaEventRecord(ev_y, s) != cudaSuccess) return OCCRI_ECUDA;
     // every other stream's work so far precedes the next work of stream w
     auto isolate = [&](int w) {
       for (int o = 0; o < ns; ++o)
@@ -805,7 +910,8 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
         return OCCRI_ECUDA;
     if (split_y) {
       add3_kernel<<<8 * 152, 256, 0, s>>>((cplx_t<T>*)p->Y, (const cplx_t<T>*)p->Yx[0],
-                                          (const cplx_t<T>*)p->Yx[1], (long long)orb);
+                                          ns > 2 ? (const cplx_t<T>*)p->Yx[1] : nullptr,
+                                          (long long)orb);
       ++launches;
     }
     all.done(OCCRI_STAGE_PAIRS, fields);
@@ -844,13 +950,25 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
   }
   {
     StageTimer t(p, timed);
-    const size_t sm = 2 * sizeof(double2) * (size_t)p->nocc * p->nocc;
+    const size_t nn = (size_t)p->nocc * p->nocc;
     const double tol = (p->precision == OCCRI_FP64) ? 1e-10 : 1e-5;
-    ace_kernel<<<p->nk, 256, sm, s>>>(C, p->kc, p->xi, p->mmat, p->ek, (double2*)K, p->nao,
-                                      p->nocc, tol, p->status);
+    ace_factor_kernel<<<dim3(ace_shares(*p), p->nk), 256, 2 * sizeof(double2) * nn, s>>>(
+        C, p->kc, p->ace_share, p->mmat, p->lmat, p->ace_ok, p->ek, Ex, p->nk, p->nao, p->nocc,
+        tol, p->ace_ticket, p->status);
     ++launches;
-    if (Ex) {
-      ex_kernel<<<1, 32, 0, s>>>(p->ek, p->nk, Ex);
+    if (K) {
+      // tiles of 32 AOs, or 16 where those are fewer than the SMs (or too large at nocc 32)
+      auto rows = [&](int tile) { return (p->nao + tile - 1) / tile; };
+      auto pairs = [&](int tile) { return rows(tile) * (rows(tile) + 1) / 2; };
+      const int tile = (long long)pairs(32) * p->nk >= 152 && p->nocc < 32 ? 32 : 16;
+      const size_t sm = sizeof(double2) * (nn + 2 * (size_t)tile * (p->nocc + 1));
+      const dim3 grid(pairs(tile), p->nk);
+      if (tile == 32)
+        ace_k_kernel<32><<<grid, 256, sm, s>>>(p->kc, p->lmat, p->ace_ok, (double2*)K, p->nao,
+                                               p->nocc, rows(tile));
+      else
+        ace_k_kernel<16><<<grid, 256, sm, s>>>(p->kc, p->lmat, p->ace_ok, (double2*)K, p->nao,
+                                               p->nocc, rows(tile));
       ++launches;
     }
     t.done(OCCRI_STAGE_ASSEMBLE, p->nk);
@@ -951,7 +1069,6 @@ int vjp_full_impl(Plan* p, const double2* C, double gEx, const double2* gKC, con
   // (b): dL/dC_{mu i} = sum_r conj(chi_mu) dL/dpsi_i; the transforms carry N_g/(4 pi)
   // and g carried N_k N_g/Omega, hence the factor 4 pi Omega/(N_k N_g^2)
   if (launch_phase_fields<T>(*p, p->gpsi, +1, s) != cudaSuccess) return OCCRI_ECUDA;
-  if (cudaMemsetAsync(p->gacc, 0, nkc * sizeof(double2), s) != cudaSuccess) return OCCRI_ECUDA;
   const double ngd = (double)p->ng;
   const double scale = 4.0 * kPiD * p->omega_cell / ((double)p->nk * ngd * ngd);
   if (launch_contract_field<T>(*p, p->gpsi, p->gacc, scale, s) != cudaSuccess) return OCCRI_ECUDA;
@@ -1649,13 +1766,17 @@ int occri_plan_create(occri_plan** out, const occri_cell* cell, const occri_kmes
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   p->nstreams = 3;
   chk(dalloc(&p->kc, (size_t)p->nk * nao * nocc, &tot));
-  chk(dalloc(&p->xi, (size_t)p->nk * nao * nocc, &tot));
+  chk(dalloc(&p->lmat, (size_t)p->nk * nocc * nocc, &tot));
+  chk(dalloc(&p->ace_share, (size_t)p->nk * ace_shares(*p) * nocc * nocc, &tot));
+  chk(dalloc(&p->ace_ok, 2 * (size_t)p->nk + 1, &tot));   // flags, then the tickets
+  p->ace_ticket = p->ace_ok ? p->ace_ok + p->nk : nullptr;
   chk(dalloc(&p->mmat, (size_t)p->nk * nocc * nocc, &tot));
   chk(dalloc(&p->ek, (size_t)p->nk, &tot));
   chk(dalloc(&p->dacc, 2, &tot));
   if (precision == OCCRI_MIXED_TC) chk(dalloc(&p->colmax, (size_t)p->nk * nocc, &tot));
   chk(dalloc(&p->status, 2, &tot));
   if (e == cudaSuccess) e = cudaMemset(p->status, 0, 2 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(p->ace_ok, 0, sizeof(int) * (2 * (size_t)p->nk + 1));
   if (e == cudaSuccess && p->vq)
     e = precision == OCCRI_FP64 ? launch_qtables<double>(*p, p->stream)
                                 : launch_qtables<float>(*p, p->stream);

@@ -615,12 +615,12 @@ con_kernel(Params p, const cplx_t<T>* __restrict__ chi, const cplx_t<T>* __restr
   for (int j = 0; j < NV / 32; ++j) o[j] = sum[j];
 }
 
-// out[k][mu][i] += scale N_mu (sum of the items): one CTA per (slot group, k), a thread per
-// value and every kSumSplit-th run, the shares added in order.
+// out[k][mu][i] = scale N_mu (sum of the items), or += after the first chunk: one CTA per (slot
+// group, k), a thread per value and every kSumSplit-th run, the shares added in order.
 constexpr int kSumSplit = 8;
 template <int NI>
 __global__ void __launch_bounds__(2 * kPad * NI * kSumSplit)
-sum_kernel(Params p, double2* __restrict__ out, int row_of0, int nitems, int i0, double scale) {
+sum_kernel(Params p, double2* __restrict__ out, int row_of0, int nitems, int i0, double scale, int add) {
   constexpr int NV = 2 * kPad * NI;
   __shared__ double share[kSumSplit][NV];
   const int v = threadIdx.x % NV, z = threadIdx.x / NV, k = blockIdx.y;
@@ -644,7 +644,8 @@ sum_kernel(Params p, double2* __restrict__ out, int row_of0, int nitems, int i0,
 #pragma unroll
   for (int y = 1; y < kSumSplit; ++y) t += share[y][v];
   double* dst = reinterpret_cast<double*>(out + ((size_t)k * p.a.nao + mu) * p.a.nocc + i0 + i);
-  dst[v & 1] += scale * p.ao_norm[mu] * t;
+  t *= scale * p.ao_norm[mu];
+  dst[v & 1] = add ? dst[v & 1] + t : t;
 }
 
 // Coefficients factor N_mu X^k_{mu i} in slot order, formed in FP64 (hi/lo floats in FP32), 0
@@ -770,10 +771,11 @@ cudaError_t product_b(const Plan& p, const Params& q, const ChiChunk& c, const v
 template <typename T, int NI>
 void run_con(const Plan& p, const Params& q, const ChiChunk& c, const void* F, double2* out,
              int i0, double scale, cudaStream_t s) {
-  con_kernel<T, NI><<<dim3((c.nitems + 7) / 8, p.nk), 256, 0, s>>>(
+  if (c.nitems > 0)
+    con_kernel<T, NI><<<dim3((c.nitems + 7) / 8, p.nk), 256, 0, s>>>(
       q, (const cplx_t<T>*)p.chi->chi, (const cplx_t<T>*)F, c.item0, c.nitems, i0);
   sum_kernel<NI><<<dim3(q.nslots / kPad, p.nk), 2 * kPad * NI * kSumSplit, 0, s>>>(
-      q, out, c.row_of0, c.nitems, i0, scale);
+      q, out, c.row_of0, c.nitems, i0, scale, c.b0 > 0 ? 1 : 0);
 }
 
 // orbitals per pass of con_kernel
@@ -782,7 +784,6 @@ inline int con_width(int left, bool fp64) { return (fp64 || left <= 4) ? 4 : 8; 
 template <typename T>
 cudaError_t product_e(const Plan& p, const Params& q, const ChiChunk& c, const void* F,
                       double2* out, double scale, cudaStream_t s) {
-  if (c.nitems == 0) return cudaSuccess;
   for (int i0 = 0; i0 < p.nocc;) {
     const int ni = con_width(p.nocc - i0, sizeof(T) == 8);
     if (ni == 4) {
@@ -1084,7 +1085,9 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   const long long cols = (88 * 1024 / col_bytes >= 4 ? 88 : 176) * 1024 / col_bytes;
   t->ncol = dft ? (int)std::min<long long>(chi::kCols, cols) : 0;
   // small transforms: half the warps per CTA, so that fewer wait at its barriers
-  t->warps = t->ncol * t->col_rows <= 256 ? 4 : chi::kWarps;
+  // (but not where the CTAs are few: a Gamma cell)
+  const bool few = (long long)nblk * natm < 152 * 8;
+  t->warps = t->ncol * t->col_rows <= 256 && !few ? 4 : chi::kWarps;
   t->buf_rows = std::max(t->ncol * t->col_rows, t->warps * chi::kRows);
   const size_t need = fp64 ? chi::chi_smem<double>(t->buf_rows, lmax)
                            : chi::chi_smem<float>(t->buf_rows, lmax);

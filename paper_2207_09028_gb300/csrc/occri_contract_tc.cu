@@ -287,12 +287,12 @@ con_tc_kernel(chi::Params p, const float2* __restrict__ chi, const float2* __res
   if (warp == 0) tc::tmem_dealloc(tmem, COLS);
 }
 
-// kc[k][mu][i] += scale N_mu (sum of the items): a CTA per (eight slots, k), 32 threads per slot
+// kc[k][mu][i] = scale N_mu (sum of the items), or += after the first chunk: a CTA per (eight slots, k), 32 threads per slot
 // over the orbitals and parts, the items of a slot in order.
 template <int N>
 __global__ void __launch_bounds__(256)
 sum_tc_kernel(chi::Params p, const unsigned* __restrict__ colmax, double2* __restrict__ kc,
-              int row_of0, int nitems, double scale) {
+              int row_of0, int nitems, double scale, int add) {
   constexpr int NI = N / 2;
   const int slot = blockIdx.x * 8 + (threadIdx.x >> 5), k = blockIdx.y, nocc = p.a.nocc;
   if (slot >= p.nslots) return;
@@ -316,7 +316,7 @@ sum_tc_kernel(chi::Params p, const unsigned* __restrict__ colmax, double2* __res
     const double f = scale * p.ao_norm[mu] / (double)p.row_scale[slot] *
                      ldexp(1.0, col_exp(colmax[(size_t)k * nocc + i]) - 13);
     double* dst = reinterpret_cast<double*>(kc + ((size_t)k * p.a.nao + mu) * nocc + i);
-    dst[im] += f * t;
+    dst[im] = add ? dst[im] + f * t : f * t;
   }
 }
 
@@ -332,14 +332,15 @@ cudaError_t run(const Plan& p, const chi::Params& q, const ChiChunk& c, double s
     cudaFuncSetAttribute(con_tc_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     return 1;
   });
-  if (c.nitems == 0) return cudaSuccess;
   if (hook) hook->before();
-  con_tc_kernel<N><<<dim3(c.nitems, p.nk), kThreads, smem, s>>>(
-      q, (const float2*)p.chi->chi, (const float2*)p.Y, p.colmax, c.item0, c.nitems, p.status,
-      p.wait_ns);
+  if (c.nitems > 0)
+    con_tc_kernel<N><<<dim3(c.nitems, p.nk), kThreads, smem, s>>>(
+        q, (const float2*)p.chi->chi, (const float2*)p.Y, p.colmax, c.item0, c.nitems, p.status,
+        p.wait_ns);
   if (hook) hook->after();
   sum_tc_kernel<N><<<dim3((q.nslots + 7) / 8, p.nk), 256, 0, s>>>(q, p.colmax, p.kc, c.row_of0,
-                                                                  c.nitems, scale);
+                                                                  c.nitems, scale,
+                                                                  c.b0 > 0 ? 1 : 0);
   return cudaGetLastError();
 }
 

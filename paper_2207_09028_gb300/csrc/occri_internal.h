@@ -193,7 +193,10 @@ struct Plan {
   double2* gcf = nullptr;    // [nk][nao][nocc] dL/dC through the assembly alone
   double2* gacc = nullptr;   // [nk][nao][nocc] dL/dC through the orbitals
   double2* kc = nullptr;     // [nk][nao][nocc]
-  double2* xi = nullptr;     // [nk][nao][nocc]
+  double2* lmat = nullptr;   // [nk][nocc][nocc] Cholesky factor of -M
+  double2* ace_share = nullptr;   // [nk][shares][nocc][nocc] shares of C^H KC
+  int* ace_ok = nullptr;     // [nk] factorised; then the counters (zero between builds)
+  int* ace_ticket = nullptr;
   double2* mmat = nullptr;   // [nk][nocc][nocc]
   double* ek = nullptr;      // [nk]
   double* dacc = nullptr;    // [2] scratch accumulators (d E/d omega)
@@ -263,7 +266,7 @@ cudaError_t launch_slot_c(const Plan& p, const double2* X, void* out, double fac
 template <typename T>
 cudaError_t launch_orbitals(const Plan& p, int nsets, const void* const* cs, void* const* out,
                             cudaStream_t s);
-// out[k][mu][i] += scale N_mu sum_r conj(chi) F_ik for an orbital-shaped field F; follows
+// out[k][mu][i] = scale N_mu sum_r conj(chi) F_ik for an orbital-shaped field F; follows
 // launch_orbitals in the same call (the chi buffer may still hold the AOs).
 template <typename T>
 cudaError_t launch_contract_field(const Plan& p, const void* F, double2* out, double scale,
@@ -315,7 +318,7 @@ inline int wave_targets(int nocc, int nkp, int diag) { return diag ? nocc : nocc
 template <typename T>
 cudaError_t launch_widen(const Plan& p, void* out, cudaStream_t s);
 
-// The tensor-core contraction (OCCRI_MIXED_TC, occri_contract_tc.cu): adds K_{mu i} of the
+// The tensor-core contraction (OCCRI_MIXED_TC, occri_contract_tc.cu): K_{mu i} of the
 // accumulated Y into p.kc, from the chi buffer.
 constexpr int kTcTile = 64;                 // AO slots per tile (128 rows: Re and Im)
 size_t tc_item_values(int nocc);            // sums one work item leaves
