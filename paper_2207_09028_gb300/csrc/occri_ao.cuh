@@ -63,10 +63,10 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   const float bb = s - a;
   e = (a - (s - bb)) + (b - bb);
 }
-__device__ __forceinline__ float exact_gauss(const Disp<float>& d, float txh, float tyh,
-                                             float tzh, float txl, float tyl, float tzl,
-                                             float ah_, float al_, float* r2h, float* x,
-                                             float* y, float* z) {
+// d - T rounded to FP32 in *x, *y, *z, and r^2 as *r2h + *r2l.
+__device__ __forceinline__ void exact_r2(const Disp<float>& d, float txh, float tyh, float tzh,
+                                         float txl, float tyl, float tzl, float* r2h, float* r2l,
+                                         float* x, float* y, float* z) {
   float c[3], cl[3];
   const float dh[3] = {d.xh, d.yh, d.zh}, dl[3] = {d.xl, d.yl, d.zl};
   const float th[3] = {txh, tyh, tzh}, tl[3] = {txl, tyl, tzl};
@@ -86,13 +86,20 @@ __device__ __forceinline__ float exact_gauss(const Disp<float>& d, float txh, fl
   float s1, e1, s2, e2;
   two_sum(ph[0], ph[1], s1, e1);
   two_sum(s1, ph[2], s2, e2);
-  const float rl = (e1 + e2) + (pl[0] + pl[1] + pl[2]);
+  *r2l = (e1 + e2) + (pl[0] + pl[1] + pl[2]);
   *r2h = s2;
-  const float ah = ah_ * s2;
-  const float al = fmaf(ah_, s2, -ah) + ah_ * rl + al_ * s2;
   *x = c[0] + cl[0];
   *y = c[1] + cl[1];
   *z = c[2] + cl[2];
+}
+__device__ __forceinline__ float exact_gauss(const Disp<float>& d, float txh, float tyh,
+                                             float tzh, float txl, float tyl, float tzl,
+                                             float ah_, float al_, float* r2h, float* x,
+                                             float* y, float* z) {
+  float r2l;
+  exact_r2(d, txh, tyh, tzh, txl, tyl, tzl, r2h, &r2l, x, y, z);
+  const float ah = ah_ * *r2h;
+  const float al = fmaf(ah_, *r2h, -ah) + ah_ * r2l + al_ * *r2h;
   return expf(-ah) * (1.0f - al);
 }
 

@@ -35,8 +35,9 @@ namespace chi {
 using ao::Disp;
 
 constexpr int kWarps = 8;       // most warps of a chi_kernel CTA
-constexpr int kRows = 48;       // entry rows of a warp (a value per lane each)
-constexpr int kCols = 8;        // AOs that the CTA takes together (wide shells)
+constexpr int kFold = 8;        // most classes of a mesh whose shells take a warp each
+constexpr int kRows = 7 * kFold;   // entry rows of a warp (a value per lane each)
+constexpr int kCols = 10;       // AOs that the CTA takes together (wide shells)
 constexpr int kWide = 12;       // images from which a shell counts as wide
 
 template <typename T> struct Rec;
@@ -182,6 +183,79 @@ __device__ __forceinline__ void narrow_shell(const Params& p, const ChiShell& sh
   }
 }
 
+// A shell on a mesh of at most kFold classes, one warp: class sums in the warp's rows (row
+// class NM + m; a lane reads back only what it wrote), then chi of every k. Where every axis
+// has one or two points the phases are signs and chi is real: sums and differences over the axes
+// (a Walsh-Hadamard transform); else the classes' phases as in narrow_shell.
+template <typename T, int L, int KT, typename GetRec>
+__device__ __forceinline__ void fold_shell(const Params& p, const ChiShell& sh, const Disp<T>& d,
+                                           int np, const GetRec& rec, T* ent, int* ecls,
+                                           cplx_t<T>* out, int kstride, int lane) {
+  constexpr int NM = 2 * L + 1;
+  const int nc = p.ncls, nk = p.a.nk;
+  T* e0 = ent + lane;
+  for (int x = 0; x < nc * NM; ++x) e0[x * 32] = T(0);
+  Rec<T> next = rec(0);
+  for (int j = 0; j < np; ++j) {
+    const Rec<T> r = next;
+    if (j + 1 < np) next = rec(j + 1);
+    T v[NM];
+    eval<L>(sh, d, r, v);
+    T* o = e0 + r.cls * (NM * 32);
+#pragma unroll
+    for (int m = 0; m < NM; ++m) o[m * 32] += v[m];
+  }
+  if (p.signs) {
+    int off[kFold];   // where each class index's k goes, or -1
+#pragma unroll
+    for (int c = 0; c < kFold; ++c) {
+      const int k = c < nc ? p.kidx[c] : -1;
+      off[c] = k >= 0 ? k * kstride + lane : -1;
+    }
+    // rolled: the straight-line form missed the instruction cache
+#pragma unroll 1
+    for (int m = 0; m < NM; ++m) {
+      T f[kFold];
+#pragma unroll
+      for (int c = 0; c < kFold; ++c) f[c] = c < nc ? e0[(c * NM + m) * 32] : T(0);
+#pragma unroll
+      for (int st = 1; st < kFold; st *= 2) {
+        if (st >= nc) break;
+#pragma unroll
+        for (int c = 0; c < kFold; ++c)
+          if (!(c & st)) {
+            const T u = f[c], w = f[c + st];
+            f[c] = u + w;
+            f[c + st] = u - w;
+          }
+      }
+#pragma unroll
+      for (int c = 0; c < kFold; ++c)
+        if (off[c] >= 0) out[off[c] + 32 * m] = cplx_t<T>{f[c], T(0)};
+    }
+    return;
+  }
+  __syncwarp();
+  if (lane < nc) ecls[lane] = lane;
+  __syncwarp();
+  for (int k0 = 0; k0 < nk; k0 += KT) {
+    T xr[KT][NM], xi[KT][NM];
+#pragma unroll
+    for (int b = 0; b < KT; ++b)
+#pragma unroll
+      for (int m = 0; m < NM; ++m) xr[b][m] = xi[b][m] = T(0);
+    phase_sums<T, KT, NM>(reinterpret_cast<const cplx_t<T>*>(p.phase), p.nkp, ent, ecls, nc, k0,
+                          lane, xr, xi);
+#pragma unroll
+    for (int b = 0; b < KT; ++b) {
+      if (k0 + b >= nk) break;
+#pragma unroll
+      for (int m = 0; m < NM; ++m)
+        out[(size_t)(k0 + b) * kstride + 32 * m + lane] = cplx_t<T>{xr[b][m], xi[b][m]};
+    }
+  }
+}
+
 // ---- wide shells: the class sums of up to kCols AOs in shared memory, then a discrete Fourier
 // transform over the classes, axis by axis (chi_k = sum_l e^{2 pi i k.l/D} Phi_l, Phi real: only
 // the non-negative half of the first axis is kept, the rest are conjugates). A column holds
@@ -272,43 +346,120 @@ __device__ __forceinline__ void mesh_dft(const Params& p, T* col, cplx_t<T>* out
   });
 }
 
-// Class sums of the functions [m0, m0 + ncol) of one shell over a stretch [t0, t1) of the list
+// Displacement, r^2 and what the shells need of them for one image. In FP32 shells with an exact
+// exponent want r^2 as a hi + lo pair (see ao::exact_gauss); the others take lo = 0 and alpha
+// r^2 in one rounding less.
+template <typename T> struct Geo;
+template <> struct Geo<float> {
+  float x, y, z, rh, rl;
+  __device__ __forceinline__ Geo(const Disp<float>& d, const Rec<float>& r, bool exact) {
+    if (exact) {
+      ao::exact_r2(d, r.xh, r.yh, r.zh, r.xl, r.yl, r.zl, &rh, &rl, &x, &y, &z);
+    } else {
+      x = (d.xh - r.xh) + (d.xl - r.xl);
+      y = (d.yh - r.yh) + (d.yl - r.yl);
+      z = (d.zh - r.zh) + (d.zl - r.zl);
+      rh = x * x + y * y + z * z;
+      rl = 0.f;
+    }
+  }
+  __device__ __forceinline__ float gauss(float alpha, float alpha_lo, float rcut2,
+                                         bool exact) const {
+    float e;
+    if (exact) {
+      const float ah = alpha * rh;
+      const float al = fmaf(alpha, rh, -ah) + alpha * rl + alpha_lo * rh;
+      e = expf(-ah) * (1.0f - al);
+    } else {
+      e = expf(-(alpha * rh + alpha_lo * rh));
+    }
+    return rh <= rcut2 ? e : 0.f;
+  }
+};
+template <> struct Geo<double> {
+  double x, y, z, r2;
+  __device__ __forceinline__ Geo(const Disp<double>& d, const Rec<double>& r, bool)
+      : x(d.x - r.x), y(d.y - r.y), z(d.z - r.z) {
+    r2 = x * x + y * y + z * z;
+  }
+  __device__ __forceinline__ double gauss(double alpha, double, double rcut2, bool) const {
+    const double e = exp(-(alpha * r2));
+    return r2 <= rcut2 ? e : 0.0;
+  }
+};
+
+// Shells of one angular momentum that share their images' displacements: as many as fit the
+// columns and the registers.
+template <int L> constexpr int group_shells() { return L == 0 ? 8 : (L == 1 ? 3 : (L == 2 ? 2 : 1)); }
+
+// Class sums of ns shells (functions [m0, m0 + nm) of each) over a stretch [t0, t1) of the list
 // in order of class. A class that may continue from the stretch before (the first one of a
-// stretch) goes to `edge`, its number to *edge_cls; the others are this warp's alone.
+// stretch) goes to `edge`, its number to *edge_cls; the others are this warp's alone. The
+// shells come by falling reach, np[s] images each.
 template <typename T, int L, typename GetRec, typename GetOrder>
-__device__ __forceinline__ void class_sums(const ChiShell& sh, const Disp<T>& d, int np, int t0,
-                                           int t1, int m0, int ncol, const GetRec& rec,
-                                           const GetOrder& order, T* cols, int col_rows, T* edge,
-                                           int* edge_cls, int lane) {
-  constexpr int NM = 2 * L + 1;
-  T acc[NM];
+__device__ __forceinline__ void class_sums(const ChiShell* shells, const int* np, int ns,
+                                           const Disp<T>& d, int t0, int t1, int m0, int nm,
+                                           const GetRec& rec, const GetOrder& order, T* cols,
+                                           int col_rows, T* edge, int* edge_cls, int lane) {
+  constexpr int NM = 2 * L + 1, NS = group_shells<L>();
+  T acc[NS][NM], alpha[NS], alpha_lo[NS], rcut2[NS];
+  int n[NS];
+  bool exact = false;   // one exact exponent: all of the group's
 #pragma unroll
-  for (int m = 0; m < NM; ++m) acc[m] = T(0);
+  for (int s = 0; s < NS; ++s) {
+    const int q = min(s, ns - 1);
+    exact = exact || shells[q].exact;
+    n[s] = s < ns ? np[s] : 0;
+    if constexpr (sizeof(T) == 4) {
+      alpha[s] = shells[q].alpha;
+      alpha_lo[s] = shells[q].alpha_lo;
+      rcut2[s] = shells[q].rcut2;
+    } else {
+      alpha[s] = shells[q].alpha_d;
+      alpha_lo[s] = T(0);
+      rcut2[s] = shells[q].rcut2_d;
+    }
+#pragma unroll
+    for (int m = 0; m < NM; ++m) acc[s][m] = T(0);
+  }
   int cur = -1, first = -1;
   auto close = [&]() {
 #pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      const int c = m - m0;
-      if (c >= 0 && c < ncol) {
-        T* o = cur == first ? edge + c * 32 : cols + ((size_t)c * col_rows + cur) * 32;
-        o[lane] = acc[m];
+    for (int s = 0; s < NS; ++s) {
+      if (s >= ns) break;
+#pragma unroll
+      for (int m = 0; m < NM; ++m) {
+        const int c = s * nm + m - m0;
+        if (m >= m0 && m < m0 + nm) {
+          T* o = cur == first ? edge + c * 32 : cols + ((size_t)c * col_rows + cur) * 32;
+          o[lane] = acc[s][m];
+        }
+        acc[s][m] = T(0);
       }
-      acc[m] = T(0);
     }
   };
+  int next = t0 < t1 ? order(t0) : 0;
   for (int t = t0; t < t1; ++t) {
-    const int j = order(t);
-    if (j >= np) continue;   // past the shell's reach (uniform)
+    const int j = next;
+    if (t + 1 < t1) next = order(t + 1);
+    if (j >= n[0]) continue;   // past every shell's reach (uniform)
     const Rec<T> r = rec(j);
     if (r.cls != cur) {
       if (cur >= 0) close();
       cur = r.cls;
       if (first < 0) first = cur;
     }
-    T v[NM];
-    eval<L>(sh, d, r, v);
+    const Geo<T> g(d, r, exact);
+    T P[NM];
+    ao::solid<T, L>(g.x, g.y, g.z, P);
 #pragma unroll
-    for (int m = 0; m < NM; ++m) acc[m] += v[m];
+    for (int s = 0; s < NS; ++s) {
+      if (j < n[s]) {
+        const T e = g.gauss(alpha[s], alpha_lo[s], rcut2[s], exact);
+#pragma unroll
+        for (int m = 0; m < NM; ++m) acc[s][m] += P[m] * e;
+      }
+    }
   }
   if (cur >= 0) close();
   if (lane == 0) *edge_cls = first;
@@ -316,8 +467,8 @@ __device__ __forceinline__ void class_sums(const ChiShell& sh, const Disp<T>& d,
 
 // chi of the blocks [blk0, blk0 + gridDim.x) for one atom; a lane is a grid point. Every Gaussian
 // is evaluated once for all k. The atom's wide shells come first (they are a prefix of its
-// shells): the CTA takes as many as make kCols AOs, each warp a stretch of the images, then a
-// warp per AO transforms. The phases of a narrow shell's few images are applied one by one.
+// shells): the CTA takes a few of one angular momentum, which share their images' distances,
+// each warp a stretch of the images, then a warp per AO transforms. The phases of a narrow shell's few images are applied one by one.
 // What bounds it: the stores at many k-points, the Gaussians at few. Phases times class sums
 // (a dense product over classes) instead of the transform took 43 ms per pass at 64 k, 350
 // AOs, 60^3: each broadcast phase costs the load path as much as a full vector.
@@ -326,11 +477,12 @@ __global__ void __launch_bounds__(32 * kWarps, 2)
 chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ T edge[kWarps][kCols][32];
-  __shared__ int edge_cls[kWarps][kCols];
+  __shared__ int edge_cls[kWarps];
   T* buf = reinterpret_cast<T*>(smem_raw);   // entry rows of the warps, or columns
   int* eclss = reinterpret_cast<int*>(buf + p.buf_rows * 32);
   Rec<T>* recs = reinterpret_cast<Rec<T>*>(eclss + kWarps * kRows);
-  unsigned short* ord = reinterpret_cast<unsigned short*>(recs + p.lsm);
+  int* lnp = reinterpret_cast<int*>(recs + p.lsm);   // images << 2 | l of the atom's shells
+  unsigned short* ord = reinterpret_cast<unsigned short*>(lnp + p.a.nsa);
   const int blk = blk0 + blockIdx.x, a = blockIdx.y;
   const size_t ab = (size_t)a * p.a.nblk + blk;
   const int nact = p.nsh[ab];
@@ -341,13 +493,17 @@ chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
   const int n_all = pre[p.shells[s0].orig - s0];   // the widest shell's images
   const int* cls = p.cls + (size_t)p.t0i[ab] * p.a.nimg;
   const bool in_smem = p.lsm > 0;
+  for (int x = threadIdx.x; x < nact; x += blockDim.x) {
+    const ChiShell& sh = p.shells[s0 + x];
+    lnp[x] = pre[sh.orig - s0] << 2 | sh.l;
+  }
   if (in_smem) {
     for (int j = threadIdx.x; j < n_all; j += blockDim.x) {
       recs[j] = load_rec<T>(p, list0, cls, j);
       if (p.order) ord[j] = p.order[list0 + j];
     }
-    __syncthreads();
   }
+  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   bool valid;
   long long q;
@@ -359,71 +515,95 @@ chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
   cplx_t<T>* base = chi + (size_t)(p.boff[blk] * p.a.nk + aoff[a]) * 32;
   auto rec = [&](int j) -> Rec<T> { return in_smem ? recs[j] : load_rec<T>(p, list0, cls, j); };
   auto order = [&](int t) -> int { return in_smem ? ord[t] : p.order[list0 + t]; };
-  int s = 0;
+  __shared__ ChiShell gsh[8];
+  __shared__ int gnp[8], gidx[8], gslot[kCols], gns, gm0, gnm, gnext, gl;
+  int wide = 0;   // wide shells (a prefix)
   if (p.ncol > 0) {
-    // groups of wide shells; the groups go round the CTAs of the (block, atom)
-    int m0 = 0, group = 0;
+    while (wide < nact && lnp[wide] >> 2 >= kWide) ++wide;
+    // Groups of one angular momentum, in turn over the CTAs of the (block, atom)
     const int t0 = n_all * warp / nw, t1 = n_all * (warp + 1) / nw;
-    while (s < nact) {
-      // the group: functions m0.. of shell s, then whole shells while they fit
-      int e = s, cols = 0, next_m = 0;
-      if (pre[p.shells[s0 + s].orig - s0] < kWide) break;
-      while (e < nact) {
-        const ChiShell& sh = p.shells[s0 + e];
-        if (pre[sh.orig - s0] < kWide) break;
-        const int left = 2 * sh.l + 1 - (e == s ? m0 : 0);
-        if (cols + left > p.ncol) {
-          if (e == s) { next_m = m0 + p.ncol; cols = p.ncol; }   // a part of one shell
-          break;
+    int at = 0, m0 = 0, l = 0;   // next shell to look at, its first function
+    for (int group = 0; l < 4; ++group) {
+      __syncthreads();   // the group before is done with the columns and the list
+      if (threadIdx.x == 0) {
+        int ns = 0, x = at;
+        const int full = 2 * l + 1, nm = min(full - m0, p.ncol);   // functions of each shell
+        const int most = max(1, min(l == 0 ? group_shells<0>() : (l == 1 ? group_shells<1>() :
+                                    (l == 2 ? group_shells<2>() : 1)), p.ncol / full));
+        for (; x < wide && ns < most; ++x) {
+          if ((lnp[x] & 3) != l) continue;
+          gnp[ns] = lnp[x] >> 2;
+          gidx[ns++] = s0 + x;
+          if (m0 + nm < full) break;   // a part of one shell: the rest of it next
         }
-        cols += left;
-        ++e;
+        gns = ns;
+        gm0 = m0;
+        gnm = nm;
+        gl = l;
+        gnext = ns > 0 && m0 + nm < full ? x : -1 - x;
       }
-      if (group % gridDim.z == blockIdx.z) {
-        for (int x = threadIdx.x; x < cols * p.col_rows * 32; x += blockDim.x) buf[x] = T(0);
-        for (int x = threadIdx.x; x < kWarps * kCols; x += blockDim.x)
-          (&edge_cls[0][0])[x] = -1;
-        __syncthreads();
-        for (int i = s, c = 0; i < e || (i == s && next_m > 0); ++i) {
-          const ChiShell sh = p.shells[s0 + i];
-          const int np = pre[sh.orig - s0], f = i == s ? m0 : 0;
-          const int nc = min(2 * sh.l + 1 - f, cols - c);
-          T* cb = buf + (size_t)c * p.col_rows * 32;
-          T* eb = &edge[warp][c][0];
-          switch (sh.l) {
-            case 0: class_sums<T, 0>(sh, d, np, t0, t1, f, nc, rec, order, cb, p.col_rows, eb, &edge_cls[warp][c], lane); break;
-            case 1: class_sums<T, 1>(sh, d, np, t0, t1, f, nc, rec, order, cb, p.col_rows, eb, &edge_cls[warp][c], lane); break;
-            case 2: class_sums<T, 2>(sh, d, np, t0, t1, f, nc, rec, order, cb, p.col_rows, eb, &edge_cls[warp][c], lane); break;
-            default: class_sums<T, 3>(sh, d, np, t0, t1, f, nc, rec, order, cb, p.col_rows, eb, &edge_cls[warp][c], lane); break;
-          }
-          // the shell's other columns share its stretch
-          __syncwarp();
-          if (lane > 0 && lane < nc) edge_cls[warp][c + lane] = edge_cls[warp][c];
-          c += nc;
+      __syncthreads();
+      const int ns = gns, nm = gnm, gm = gm0;
+      if (gnext >= 0) {   // stay at this shell
+        at = gnext;
+        m0 = gm + nm;
+      } else {
+        at = -1 - gnext;
+        m0 = 0;
+        if (ns == 0) {    // no more of this angular momentum
+          ++l;
+          at = 0;
+          --group;
+          continue;
         }
-        __syncthreads();
-        for (int x = warp; x < cols; x += nw) {   // a warp per AO: the stretches' edges in
-          T* col = buf + (size_t)x * p.col_rows * 32;   // order, then the transform
-          for (int w = 0; w < nw; ++w) {
-            const int c = edge_cls[w][x];
-            if (c >= 0) col[c * 32 + lane] += edge[w][x][lane];
-          }
-          const int slot = p.shells[s0 + s].slot + m0 + x;
-          mesh_dft<T>(p, col, base + 32 * (size_t)slot, kstride, lane);
-        }
-        __syncthreads();
       }
-      ++group;
-      s = next_m > 0 ? s : e;
-      m0 = next_m;
+      if (group % gridDim.z != blockIdx.z) continue;
+      const int cols = ns * nm;
+      if ((int)threadIdx.x < ns) {
+        const ChiShell sh = p.shells[gidx[threadIdx.x]];
+        gsh[threadIdx.x] = sh;
+        for (int m = 0; m < nm; ++m) gslot[threadIdx.x * nm + m] = sh.slot + gm + m;
+      }
+      for (int c = 0; c < cols; ++c)   // the classes' rows (the transform fills the others)
+        for (int x = threadIdx.x; x < p.ncls * 32; x += blockDim.x)
+          buf[(size_t)c * p.col_rows * 32 + x] = T(0);
+      __syncthreads();
+      T* eb = &edge[warp][0][0];
+      int* ec = &edge_cls[warp];
+      switch (gl) {
+        case 0: class_sums<T, 0>(gsh, gnp, ns, d, t0, t1, gm, nm, rec, order, buf, p.col_rows, eb, ec, lane); break;
+        case 1: class_sums<T, 1>(gsh, gnp, ns, d, t0, t1, gm, nm, rec, order, buf, p.col_rows, eb, ec, lane); break;
+        case 2: class_sums<T, 2>(gsh, gnp, ns, d, t0, t1, gm, nm, rec, order, buf, p.col_rows, eb, ec, lane); break;
+        default: class_sums<T, 3>(gsh, gnp, ns, d, t0, t1, gm, nm, rec, order, buf, p.col_rows, eb, ec, lane); break;
+      }
+      __syncthreads();
+      for (int x = warp; x < cols; x += nw) {   // a warp per AO: the stretches' edges in
+        T* col = buf + (size_t)x * p.col_rows * 32;   // order, then the transform
+        for (int w = 0; w < nw; ++w) {
+          const int c = edge_cls[w];
+          if (c >= 0) col[c * 32 + lane] += edge[w][x][lane];
+        }
+        mesh_dft<T>(p, col, base + 32 * (size_t)gslot[x], kstride, lane);
+      }
     }
+    __syncthreads();
   }
+  int s = wide;
   T* ent = buf + warp * kRows * 32;
   int* ecls = eclss + warp * kRows;
   for (s += warp + nw * blockIdx.z; s < nact; s += nw * gridDim.z) {
     const ChiShell sh = p.shells[s0 + s];
     const int np = pre[sh.orig - s0];
     cplx_t<T>* out = base + 32 * (size_t)sh.slot;
+    if (p.ncls <= kFold) {
+      switch (sh.l) {
+        case 0: fold_shell<T, 0, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+        case 1: fold_shell<T, 1, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+        case 2: fold_shell<T, 2, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+        default: fold_shell<T, 3, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+      }
+      continue;
+    }
     switch (sh.l) {
       case 0: narrow_shell<T, 0, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
       case 1: narrow_shell<T, 1, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
@@ -460,6 +640,18 @@ order_kernel(Params p, unsigned short* __restrict__ order) {
     }
 }
 
+// chi is read once: past L1, which holds what is shared (coefficients, orbital fields).
+__device__ __forceinline__ float2 stream_ld(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 stream_ld(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+
 // t += c x; in FP32 the coefficient is a hi/lo pair
 __device__ __forceinline__ void cmac(const double2& c, const double2& x, double2& t) {
   t.x += c.x * x.x - c.y * x.y;
@@ -470,48 +662,92 @@ __device__ __forceinline__ void cmac(const float4& c, const float2& x, float2& t
   t.y = fmaf(c.x, x.y, fmaf(c.y, x.x, fmaf(c.z, x.y, fmaf(c.w, x.x, t.y))));
 }
 
-// psi_ik at one block per warp: kPad AOs are summed on their own before they join the
-// orbital's sum, so that few roundings happen at its full size.
-template <typename T, int NI>
+// psi_ik at NB consecutive blocks per warp: kPad AOs are summed on their own before they join
+// the orbital's sum, so that few roundings happen at its full size. In FP32 a coefficient,
+// the same for every lane, costs the load path as much as a value per lane: up to four
+// orbitals take two blocks (64 k, 200 AOs, 48^3, nocc 4: orbitals and AOs 5.5 -> 5.0 ms); with
+// eight the wider tile's registers cost what it saves (350 AOs, 8 k, 60^3: 1.52 against 1.50 ms).
+template <typename T, int NI> constexpr int orb_blocks() { return sizeof(T) == 4 && NI == 4 ? 2 : 1; }
+template <typename T, int NI, int NB>
 __global__ void __launch_bounds__(128)
 orb_kernel(Params p, const cplx_t<T>* __restrict__ chi, const typename CsT<T>::type* __restrict__ cs,
            cplx_t<T>* __restrict__ psi, int blk0, int nb, int i0) {
-  const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int w = NB * (blockIdx.x * 4 + (threadIdx.x >> 5));
   if (w >= nb) return;
-  const int blk = blk0 + w, k = blockIdx.y, lane = threadIdx.x & 31;
-  const int nocc = p.a.nocc;
-  const int* aoff = p.aoff + (size_t)blk * (p.a.natm + 1);
-  const cplx_t<T>* x0 = chi + ((size_t)p.boff[blk] * p.a.nk + (size_t)k * aoff[p.a.natm]) * 32 + lane;
-  cplx_t<T> acc[NI];
+  const int k = blockIdx.y, lane = threadIdx.x & 31;
+  const int nocc = p.a.nocc, blk = blk0 + w, nlast = min(NB, nb - w) - 1;
+  const int* aoff[NB];
+  const cplx_t<T>* x0[NB];
 #pragma unroll
-  for (int i = 0; i < NI; ++i) acc[i] = cplx_t<T>{T(0), T(0)};
-  for (int a = 0; a < p.a.natm; ++a) {
-    const int n = aoff[a + 1] - aoff[a];
-    const cplx_t<T>* xa = x0 + (size_t)aoff[a] * 32;
-    const typename CsT<T>::type* ca = cs + ((size_t)k * p.nslots + p.slot0[a]) * nocc + i0;
-#pragma unroll 2
-    for (int s = 0; s < n; s += kPad) {
-      cplx_t<T> x[kPad];
+  for (int b = 0; b < NB; ++b) {   // past the last block: the last one again, not stored
+    const int q = blk + min(b, nlast);
+    aoff[b] = p.aoff + (size_t)q * (p.a.natm + 1);
+    x0[b] = chi + ((size_t)p.boff[q] * p.a.nk + (size_t)k * aoff[b][p.a.natm]) * 32 + lane;
+  }
+  cplx_t<T> acc[NB][NI];
 #pragma unroll
-      for (int u = 0; u < kPad; ++u) x[u] = __ldg(xa + (size_t)(s + u) * 32);
+  for (int b = 0; b < NB; ++b)
 #pragma unroll
-      for (int i = 0; i < NI; ++i) {
-        if (i0 + i >= nocc) break;
-        cplx_t<T> t{T(0), T(0)};
+    for (int i = 0; i < NI; ++i) acc[b][i] = cplx_t<T>{T(0), T(0)};
+  // slots [s, s + kPad) of an atom for the blocks [b0, b1) of the warp
+  auto group = [&](const cplx_t<T>* (&xa)[NB], const typename CsT<T>::type* ca, int s, auto B0,
+                   auto B1) {
+    constexpr int b0 = decltype(B0)::value, b1 = decltype(B1)::value;
+    cplx_t<T> x[NB][kPad];
 #pragma unroll
-        for (int u = 0; u < kPad; ++u) cmac(__ldg(ca + (size_t)(s + u) * nocc + i), x[u], t);
-        acc[i].x += t.x;
-        acc[i].y += t.y;
+    for (int b = b0; b < b1; ++b)
+#pragma unroll
+      for (int u = 0; u < kPad; ++u) x[b][u] = stream_ld(xa[b] + (size_t)(s + u) * 32);
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      if (i0 + i >= nocc) break;
+      cplx_t<T> t[NB];
+#pragma unroll
+      for (int b = b0; b < b1; ++b) t[b] = cplx_t<T>{T(0), T(0)};
+#pragma unroll
+      for (int u = 0; u < kPad; ++u) {
+        const typename CsT<T>::type c = __ldg(ca + (size_t)(s + u) * nocc + i);
+#pragma unroll
+        for (int b = b0; b < b1; ++b) cmac(c, x[b][u], t[b]);
+      }
+#pragma unroll
+      for (int b = b0; b < b1; ++b) {
+        acc[b][i].x += t[b].x;
+        acc[b][i].y += t[b].y;
       }
     }
-  }
-  bool valid;
-  long long q;
-  ao::block_point(p.a, blk, lane, &valid, &q);
-  if (!valid) return;
+  };
+  using Zero = std::integral_constant<int, 0>;
+  using One = std::integral_constant<int, 1>;
+  using All = std::integral_constant<int, NB>;
+  for (int a = 0; a < p.a.natm; ++a) {
+    int n[NB], both = 1 << 30;
+    const cplx_t<T>* xa[NB];
 #pragma unroll
-  for (int i = 0; i < NI; ++i)
-    if (i0 + i < nocc) psi[((size_t)k * nocc + i0 + i) * p.a.fs + q] = acc[i];
+    for (int b = 0; b < NB; ++b) {
+      n[b] = aoff[b][a + 1] - aoff[b][a];
+      xa[b] = x0[b] + (size_t)aoff[b][a] * 32;
+      both = min(both, n[b]);
+    }
+    const typename CsT<T>::type* ca = cs + ((size_t)k * p.nslots + p.slot0[a]) * nocc + i0;
+#pragma unroll 2
+    for (int s = 0; s < both; s += kPad) group(xa, ca, s, Zero{}, All{});
+    if constexpr (NB == 2) {   // what only one of the blocks has
+      for (int s = both; s < n[0]; s += kPad) group(xa, ca, s, Zero{}, One{});
+      for (int s = both; s < n[1]; s += kPad) group(xa, ca, s, One{}, All{});
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    if (b > nlast) break;
+    bool valid;
+    long long q;
+    ao::block_point(p.a, blk + b, lane, &valid, &q);
+    if (!valid) continue;
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+      if (i0 + i < nocc) psi[((size_t)k * nocc + i0 + i) * p.a.fs + q] = acc[b][i];
+  }
 }
 
 // Sum over the lanes of a warp of NV values per lane, by halving: after the exchange over lane
@@ -590,7 +826,7 @@ con_kernel(Params p, const cplx_t<T>* __restrict__ chi, const cplx_t<T>* __restr
                                  aoff[it.x] + it.y) * 32 + lane;
     cplx_t<T> x[kPad];
 #pragma unroll
-    for (int u = 0; u < kPad; ++u) x[u] = __ldg(x0 + 32 * u);
+    for (int u = 0; u < kPad; ++u) x[u] = stream_ld(x0 + 32 * u);
     bool valid;
     long long q;
     ao::block_point(p.a, blk, lane, &valid, &q);
@@ -706,17 +942,18 @@ Params params(const Plan& p) {
   q.col_rows = t.col_rows;
   q.buf_rows = t.buf_rows;
   q.warps = t.warps;
+  q.signs = t.signs;
   return q;
 }
 
-template <typename T> size_t chi_smem(int buf_rows, int lsm) {
-  return (size_t)buf_rows * 32 * sizeof(T) + (size_t)kWarps * kRows * sizeof(int) +
+template <typename T> size_t chi_smem(int buf_rows, int lsm, int nsa) {
+  return (size_t)buf_rows * 32 * sizeof(T) + (size_t)(kWarps * kRows + nsa) * sizeof(int) +
          (size_t)lsm * (sizeof(Rec<T>) + sizeof(unsigned short));
 }
 
 template <typename T, int KS, int KL>
 cudaError_t run_chi(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t s) {
-  const size_t sm = chi_smem<T>(q.buf_rows, q.lsm);
+  const size_t sm = chi_smem<T>(q.buf_rows, q.lsm, q.a.nsa);
   static std::mutex mu;
   static size_t have[kMaxDevices] = {};
   {
@@ -750,8 +987,15 @@ cudaError_t fill(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t
 template <typename T, int NI>
 void run_orb(const Params& q, const cplx_t<T>* chi, const void* cs, void* out, const ChiChunk& c,
              int i0, cudaStream_t s) {
-  orb_kernel<T, NI><<<dim3((c.b1 - c.b0 + 3) / 4, q.a.nk), 128, 0, s>>>(
-      q, chi, (const typename CsT<T>::type*)cs, (cplx_t<T>*)out, c.b0, c.b1 - c.b0, i0);
+  // one block per warp where two would leave SMs without work
+  const int nb = c.b1 - c.b0;
+  constexpr int NB = orb_blocks<T, NI>();
+  if (NB == 1 || (long long)nb * q.a.nk < 152 * 64)
+    orb_kernel<T, NI, 1><<<dim3((nb + 3) / 4, q.a.nk), 128, 0, s>>>(
+        q, chi, (const typename CsT<T>::type*)cs, (cplx_t<T>*)out, c.b0, nb, i0);
+  else
+    orb_kernel<T, NI, NB><<<dim3((nb + 7) / 8, q.a.nk), 128, 0, s>>>(
+        q, chi, (const typename CsT<T>::type*)cs, (cplx_t<T>*)out, c.b0, nb, i0);
 }
 
 template <typename T>
@@ -1078,22 +1322,22 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
     if (kidx[r] >= 0) dft = false;
     kidx[r] = k;
   }
+  t->signs = dft && Dc <= chi::kFold && p->D[0] <= 2 && p->D[1] <= 2 && p->D[2] <= 2;
+  dft = dft && Dc > chi::kFold;   // up to kFold classes every shell takes one warp (fold_shell)
   const int row_bytes = 32 * (fp64 ? 8 : 4);
   t->col_rows = 2 * (p->D[0] / 2 + 1) * p->D[1] * p->D[2];
   // 88 KB of columns leave room for two CTAs per SM; where that is under four AOs, one CTA
   const long long col_bytes = (long long)t->col_rows * row_bytes;
   const long long cols = (88 * 1024 / col_bytes >= 4 ? 88 : 176) * 1024 / col_bytes;
   t->ncol = dft ? (int)std::min<long long>(chi::kCols, cols) : 0;
-  // small transforms: half the warps per CTA, so that fewer wait at its barriers
-  // (but not where the CTAs are few: a Gamma cell)
-  const bool few = (long long)nblk * natm < 152 * 8;
-  t->warps = t->ncol * t->col_rows <= 256 && !few ? 4 : chi::kWarps;
+  // without the transform nothing crosses warps: smaller CTAs
+  t->warps = t->ncol > 0 ? chi::kWarps : 4;
   t->buf_rows = std::max(t->ncol * t->col_rows, t->warps * chi::kRows);
-  const size_t need = fp64 ? chi::chi_smem<double>(t->buf_rows, lmax)
-                           : chi::chi_smem<float>(t->buf_rows, lmax);
+  const size_t need = fp64 ? chi::chi_smem<double>(t->buf_rows, lmax, nsa)
+                           : chi::chi_smem<float>(t->buf_rows, lmax, nsa);
   t->lsm = need <= 200 * 1024 ? lmax : 0;
   // several CTAs per (block, atom) where there are few of them (a Gamma cell)
-  t->parts = std::max(1, std::min(4, (int)(152LL * 12 / ((long long)nblk * natm))));
+  t->parts = std::max(1, std::min(4, (int)(152LL * 4 / ((long long)nblk * natm))));
 
   std::vector<float2> phase_f;
   if (!fp64)

@@ -28,6 +28,7 @@ struct ChiTables {
   int lsm = 0;                    // image records kept in shared memory (0: read from global)
   int ncol = 0, col_rows = 0;     // AOs per transform over classes (0: none), rows of one
   int buf_rows = 0, warps = 0;    // rows of chi_kernel's buffer, warps of its CTAs
+  int signs = 0;                  // every phase of the mesh is a sign (axes of one or two points)
   int parts = 1;                  // CTAs per (block, atom) of chi_kernel
   int tile = 0;                   // slots per item of the tensor-core contraction, 0 without it
   long long item_pairs = 0;       // pairs of blocks over all items
@@ -80,7 +81,7 @@ struct Params {
   const float* row_scale;
   const double* ao_norm;
   const int* kidx;
-  int nslots, ncls, nkp, lsm, parts, ncol, col_rows, buf_rows, warps;
+  int nslots, ncls, nkp, lsm, parts, ncol, col_rows, buf_rows, warps, signs;
 };
 
 Params params(const Plan& p);
