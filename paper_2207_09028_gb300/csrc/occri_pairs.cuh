@@ -601,13 +601,14 @@ __device__ __forceinline__ long long qtab_index(const PairParams& p, int kpl) {
 // copy plane by plane (instead of every pass-B CTA forming the planes it meets). CTA
 // (m3, kpl, z) fills rows m1 = z (mod kVtabSplit) of plane m3.
 constexpr int kVtabSplit = 4;
-template <typename T, int N>
+// DERIV: the tables of dv/domega, for the omega passes.
+template <typename T, int N, bool DERIV = false>
 __global__ void __launch_bounds__(threads_for<T>(N))
 vtab_kernel(T* __restrict__ vt, PairParams p) {
   __shared__ Axis1<T> ax1[N];
   const int m3 = blockIdx.x, kpl = blockIdx.y;
   const MetricHL<T> gm(p);
-  fill_vtab<T, N, false>(p, gm, m3, kpl, ax1, vt + ((size_t)kpl * N + m3) * N * N,
+  fill_vtab<T, N, DERIV>(p, gm, m3, kpl, ax1, vt + ((size_t)kpl * N + m3) * N * N,
                          (int)blockIdx.z, kVtabSplit);
 }
 
@@ -724,8 +725,8 @@ pass_a(const cplx_t<T>* __restrict__ psi, cplx_t<T>* __restrict__ S, PairParams 
 // plane of kernel values is copied in (from the wave's tables, vt) only when (m3, k')
 // changes, in the same cp.async group as the item's plane. One plane buffer per CTA: a
 // fourth CTA per SM hides the copies better than a second buffer did.
-// With DOMEGA: the forward part only, accumulating sum_m (dv/d omega)/(4 pi) |rho^(m)|^2,
-// with the derivative's kernel values formed in the CTA.
+// With DOMEGA: the forward part only, accumulating sum_m (dv/d omega)/(4 pi) |rho^(m)|^2, vt
+// holding the derivative's tables.
 template <typename T, int N>
 __device__ __forceinline__ void copy_table(T* dst, const T* src) {
   // even N: N^2 values are a whole number of 16-byte pieces, and every plane of the
@@ -744,28 +745,25 @@ __device__ __forceinline__ void pass_b_body(cplx_t<T>* __restrict__ S, const Pai
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* plane = reinterpret_cast<C2*>(smem_raw);                 // [n1][m2]
   T* vtab = reinterpret_cast<T*>(plane + N * P);               // [m1][m2] v or dv
-  Axis1<T>* ax1 = reinterpret_cast<Axis1<T>*>(vtab + N * N);   // [m1] (DOMEGA)
   __shared__ double red[4];
   const int nf = wave_fields(p.nocc, p.nkp, p.diag);
   const int items = N * nf;
   const int per = (items + (int)gridDim.x - 1) / (int)gridDim.x;
   const int i0 = min(items, (int)blockIdx.x * per);
   const int i1 = min(items, i0 + per);
-  const MetricHL<T> gm(p);
   int m3_tab = -1, kpl_tab = -1;
   // the item's plane and, where (m3, k') changes, its plane of kernel values
   auto stage = [&](int it) {
     const int m3 = it / nf, f = it - (it / nf) * nf;
     stage_plane<T, N, P>(plane, S + (size_t)f * p.fs + (size_t)m3 * N * N);
-    if constexpr (!DOMEGA) {
-      const int kpl = field_idx(f, p.nocc, p.diag).kpl;
-      if (m3 != m3_tab || kpl != kpl_tab) {   // uniform over the CTA
-        m3_tab = m3;
-        kpl_tab = kpl;
-        const T* tab = p.vq ? static_cast<const T*>(p.vq) + (size_t)qtab_index(p, kpl) * N * N * N
-                            : vt + (size_t)kpl * N * N * N;
-        copy_table<T, N>(vtab, tab + (size_t)m3 * N * N);
-      }
+    const int kpl = field_idx(f, p.nocc, p.diag).kpl;
+    if (m3 != m3_tab || kpl != kpl_tab) {   // uniform over the CTA
+      m3_tab = m3;
+      kpl_tab = kpl;
+      const T* tab = p.vq && !DOMEGA
+                         ? static_cast<const T*>(p.vq) + (size_t)qtab_index(p, kpl) * N * N * N
+                         : vt + (size_t)kpl * N * N * N;
+      copy_table<T, N>(vtab, tab + (size_t)m3 * N * N);
     }
   };
   if (i0 < i1) stage(i0);
@@ -777,13 +775,6 @@ __device__ __forceinline__ void pass_b_body(cplx_t<T>* __restrict__ S, const Pai
   for (int it = i0; it < i1; ++it) {
     const int m3 = it / nf, f = it - (it / nf) * nf;
     const FieldIdx fi = field_idx(f, p.nocc, p.diag);
-    if constexpr (DOMEGA) {
-      if (fi.kpl != kpl_tab || m3 != m3_tab) {   // uniform over the CTA
-        kpl_tab = fi.kpl;
-        m3_tab = m3;
-        fill_vtab<T, N, true>(p, gm, m3, fi.kpl, ax1, vtab, 0, 1);
-      }
-    }
     cp_async_wait<0>();   // this item's plane (and table) have landed
     __syncthreads();
     // an unordered pair stands for itself and its reverse, except (k, k, i, i)
@@ -823,6 +814,7 @@ __device__ __forceinline__ void pass_b_body(cplx_t<T>* __restrict__ S, const Pai
         cp_async_commit();
       }
     } else {
+      // the barrier above: every line has read the plane and its kernel values
       if (it + 1 < i1) stage(it + 1);
       cp_async_commit();
     }
@@ -848,8 +840,8 @@ pass_b(cplx_t<T>* __restrict__ S, PairParams p, const T* __restrict__ vt) {
 
 template <typename T, int N>
 __global__ void __launch_bounds__(threads_for<T>(N), min_blocks<T>(N))
-pass_b_domega(cplx_t<T>* __restrict__ S, PairParams p, double* dacc) {
-  pass_b_body<T, N, true>(S, p, nullptr, dacc);
+pass_b_domega(cplx_t<T>* __restrict__ S, PairParams p, const T* __restrict__ vt, double* dacc) {
+  pass_b_body<T, N, true>(S, p, vt, dacc);
 }
 
 // Resident CTA slots of a kernel on this device (SMs x CTAs per SM), at least 1.
@@ -1473,23 +1465,21 @@ pass_cd(const float2* __restrict__ S, const float2* __restrict__ psi, float2* __
 template <typename T, int N>
 __global__ void __launch_bounds__(threads_for<T>(N), min_blocks<T>(N))
 pass_b_domega2(const cplx_t<T>* __restrict__ S0, const cplx_t<T>* __restrict__ S1,
-               PairParams p, double* __restrict__ dacc) {
+               PairParams p, const T* __restrict__ vt, double* __restrict__ dacc) {
   using C2 = cplx_t<T>;
   constexpr int P = pitch(N);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* rho = reinterpret_cast<C2*>(smem_raw);                     // [n1][m2]
   C2* sig = rho + N * P;
-  Axis1<T>* ax1 = reinterpret_cast<Axis1<T>*>(sig + N * P);     // [m1]
-  T* vtab = reinterpret_cast<T*>(ax1 + N);                       // [m1][m2] dv/(4 pi)
+  T* vtab = reinterpret_cast<T*>(sig + N * P);                   // [m1][m2] dv/(4 pi)
   __shared__ double red[4];
   const int m3 = blockIdx.x;
   const int f = blockIdx.y;
   const FieldIdx fi = field_idx(f, p.nocc, p.diag);
   stage_plane<T, N, P>(rho, S0 + (size_t)f * p.fs + (size_t)m3 * N * N);
   stage_plane<T, N, P>(sig, S1 + (size_t)f * p.fs + (size_t)m3 * N * N);
+  copy_table<T, N>(vtab, vt + ((size_t)fi.kpl * N + m3) * N * N);
   cp_async_commit();
-  const MetricHL<T> gm(p);
-  fill_vtab<T, N, true>(p, gm, m3, fi.kpl, ax1, vtab, 0, 1);
   cp_async_wait<0>();
   __syncthreads();
   T dsum = T(0);
@@ -1522,14 +1512,23 @@ pass_b_domega2(const cplx_t<T>* __restrict__ S0, const cplx_t<T>* __restrict__ S
 // orbital field and u the orbitals, every unordered pair (k, k', i, j) adds
 //   G_ik  += u_jk' Z_ij + g_jk' W_ij,      G_jk' += u_ik conj(Z_ij) + g_ik conj(W_ij),
 // a field (k, k, i, i) of a diagonal wave only the first. NOC >= nocc.
+// A warp takes 32 points and every G-th k' of the wave (G = 1, 2, 4 or 8 warps share the points;
+// their sums for G_ik meet in shared memory, in order): a wave of few points and many k'
+// otherwise leaves most of the GPU without a thread (27 k' at 30^3: 70 us with a thread per
+// point over all k').
 template <typename T, int NOC>
 __global__ void __launch_bounds__(256)
 pass_e(const cplx_t<T>* __restrict__ SW, const cplx_t<T>* __restrict__ SZ,
        const cplx_t<T>* __restrict__ psi, const cplx_t<T>* __restrict__ gam,
-       cplx_t<T>* __restrict__ G, PairParams p) {
+       cplx_t<T>* __restrict__ G, PairParams p, int share) {
   using C2 = cplx_t<T>;
+  __shared__ C2 part[8][32];
   const long long ng = p.ng;
-  const int nocc = p.nocc;
+  const int nocc = p.nocc, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int first = warp % share, pw = warp / share, per = 8 / share;   // k' share, points
+  const long long r0 = ((long long)blockIdx.x * per + pw) * 32 + lane;
+  const bool valid = r0 < ng;
+  const long long r = valid ? r0 : ng - 1;
   auto mac = [](C2& acc, C2 a, C2 b) {   // acc += a * b
     acc.x += a.x * b.x - a.y * b.y;
     acc.y += a.x * b.y + a.y * b.x;
@@ -1538,60 +1537,59 @@ pass_e(const cplx_t<T>* __restrict__ SW, const cplx_t<T>* __restrict__ SZ,
     acc.x += a.x * b.x + a.y * b.y;
     acc.y += a.y * b.x - a.x * b.y;
   };
-  for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < ng;
-       r += (long long)gridDim.x * blockDim.x) {
-    C2 uk[NOC], gk[NOC], acc[NOC];
+  C2 uk[NOC], gk[NOC], acc[NOC];
 #pragma unroll
-    for (int i = 0; i < NOC; ++i) {
-      uk[i] = gk[i] = acc[i] = mk<T>(T(0), T(0));
-      if (i < nocc) {
-        uk[i] = __ldg(psi + (size_t)(p.k * nocc + i) * p.fs + r);
-        gk[i] = __ldg(gam + (size_t)(p.k * nocc + i) * p.fs + r);
+  for (int i = 0; i < NOC; ++i) {
+    uk[i] = gk[i] = acc[i] = mk<T>(T(0), T(0));
+    if (i < nocc) {
+      uk[i] = __ldg(psi + (size_t)(p.k * nocc + i) * p.fs + r);
+      gk[i] = __ldg(gam + (size_t)(p.k * nocc + i) * p.fs + r);
+    }
+  }
+  if (p.diag) {   // share = 1
+#pragma unroll
+    for (int j = 0; j < NOC; ++j) {
+      if (j >= nocc) break;
+#pragma unroll
+      for (int i = 0; i <= j; ++i) {
+        const size_t f = (size_t)diag_field(i, j, nocc) * p.fs + r;
+        const C2 w = __ldg(SW + f), z = __ldg(SZ + f);
+        mac(acc[i], uk[j], z);
+        mac(acc[i], gk[j], w);
+        if (i < j) {
+          macc(acc[j], uk[i], z);
+          macc(acc[j], gk[i], w);
+        }
       }
     }
-    if (p.diag) {
+  } else {
+#pragma unroll 1
+    for (int kpl = first; kpl < p.nkp; kpl += share) {
+      const int kp = p.kp0 + kpl;
+      C2 uq[NOC], gq[NOC], accq[NOC];
 #pragma unroll
       for (int j = 0; j < NOC; ++j) {
-        if (j >= nocc) break;
-#pragma unroll
-        for (int i = 0; i <= j; ++i) {
-          const size_t f = (size_t)diag_field(i, j, nocc) * p.fs + r;
-          const C2 w = __ldg(SW + f), z = __ldg(SZ + f);
-          mac(acc[i], uk[j], z);
-          mac(acc[i], gk[j], w);
-          if (i < j) {
-            macc(acc[j], uk[i], z);
-            macc(acc[j], gk[i], w);
-          }
+        uq[j] = gq[j] = accq[j] = mk<T>(T(0), T(0));
+        if (j < nocc) {
+          uq[j] = __ldg(psi + (size_t)(kp * nocc + j) * p.fs + r);
+          gq[j] = __ldg(gam + (size_t)(kp * nocc + j) * p.fs + r);
         }
       }
-    } else {
-#pragma unroll 1
-      for (int kpl = 0; kpl < p.nkp; ++kpl) {
-        const int kp = p.kp0 + kpl;
-        C2 uq[NOC], gq[NOC], accq[NOC];
+#pragma unroll
+      for (int i = 0; i < NOC; ++i) {
+        if (i >= nocc) break;
 #pragma unroll
         for (int j = 0; j < NOC; ++j) {
-          uq[j] = gq[j] = accq[j] = mk<T>(T(0), T(0));
-          if (j < nocc) {
-            uq[j] = __ldg(psi + (size_t)(kp * nocc + j) * p.fs + r);
-            gq[j] = __ldg(gam + (size_t)(kp * nocc + j) * p.fs + r);
-          }
+          if (j >= nocc) break;
+          const size_t f = (size_t)((kpl * nocc + i) * nocc + j) * p.fs + r;
+          const C2 w = __ldg(SW + f), z = __ldg(SZ + f);
+          mac(acc[i], uq[j], z);
+          mac(acc[i], gq[j], w);
+          macc(accq[j], uk[i], z);
+          macc(accq[j], gk[i], w);
         }
-#pragma unroll
-        for (int i = 0; i < NOC; ++i) {
-          if (i >= nocc) break;
-#pragma unroll
-          for (int j = 0; j < NOC; ++j) {
-            if (j >= nocc) break;
-            const size_t f = (size_t)((kpl * nocc + i) * nocc + j) * p.fs + r;
-            const C2 w = __ldg(SW + f), z = __ldg(SZ + f);
-            mac(acc[i], uq[j], z);
-            mac(acc[i], gq[j], w);
-            macc(accq[j], uk[i], z);
-            macc(accq[j], gk[i], w);
-          }
-        }
+      }
+      if (valid) {
 #pragma unroll
         for (int j = 0; j < NOC; ++j) {
           if (j >= nocc) break;
@@ -1603,9 +1601,21 @@ pass_e(const cplx_t<T>* __restrict__ SW, const cplx_t<T>* __restrict__ SZ,
         }
       }
     }
+  }
 #pragma unroll
-    for (int i = 0; i < NOC; ++i) {
-      if (i >= nocc) break;
+  for (int i = 0; i < NOC; ++i) {
+    if (i >= nocc) break;
+    if (share > 1) {
+      __syncthreads();
+      part[warp][lane] = acc[i];
+      __syncthreads();
+      for (int w = 1; w < share && first == 0; ++w) {
+        const C2 v = part[warp + w][lane];
+        acc[i].x += v.x;
+        acc[i].y += v.y;
+      }
+    }
+    if (valid && first == 0) {
       C2* g = G + (size_t)(p.k * nocc + i) * p.fs + r;
       C2 v = *g;
       v.x += acc[i].x;
@@ -1619,17 +1629,19 @@ template <typename T>
 cudaError_t launch_pass_e(const PairParams& p, const cplx_t<T>* SW, const cplx_t<T>* SZ,
                           const cplx_t<T>* psi, const cplx_t<T>* gam, cplx_t<T>* G,
                           cudaStream_t st) {
-  const unsigned nb = (unsigned)std::min<long long>((p.ng + 255) / 256, 152LL * 8);
-  if (p.nocc <= 4) pass_e<T, 4><<<nb, 256, 0, st>>>(SW, SZ, psi, gam, G, p);
-  else if (p.nocc <= 8) pass_e<T, 8><<<nb, 256, 0, st>>>(SW, SZ, psi, gam, G, p);
-  else if (p.nocc <= 16) pass_e<T, 16><<<nb, 256, 0, st>>>(SW, SZ, psi, gam, G, p);
-  else pass_e<T, 32><<<nb, 256, 0, st>>>(SW, SZ, psi, gam, G, p);
+  int share = 1;
+  while (!p.diag && 2 * share <= std::min(8, p.nkp)) share *= 2;
+  const unsigned nb = (unsigned)((p.ng * share + 255) / 256);
+  if (p.nocc <= 4) pass_e<T, 4><<<nb, 256, 0, st>>>(SW, SZ, psi, gam, G, p, share);
+  else if (p.nocc <= 8) pass_e<T, 8><<<nb, 256, 0, st>>>(SW, SZ, psi, gam, G, p, share);
+  else if (p.nocc <= 16) pass_e<T, 16><<<nb, 256, 0, st>>>(SW, SZ, psi, gam, G, p, share);
+  else pass_e<T, 32><<<nb, 256, 0, st>>>(SW, SZ, psi, gam, G, p, share);
   return cudaGetLastError();
 }
 
 template <int N> constexpr size_t smem_a(size_t csz) { return csz * N * pitch(N); }
-template <int N> constexpr size_t smem_b(size_t csz, size_t tab) {
-  return csz * N * pitch(N) + N * tab + csz / 2 * N * N;
+template <int N> constexpr size_t smem_b(size_t csz) {   // a plane and its kernel values
+  return csz * N * pitch(N) + csz / 2 * N * N;
 }
 
 template <int N> constexpr size_t smem_c(size_t csz) { return csz * N * pitch(N); }
@@ -1641,7 +1653,7 @@ cudaError_t run_wave(const PairParams& p, const cplx_t<T>* psi, cplx_t<T>* S, cp
   const int nt = threads_for<T>(N);
   const int nf = wave_fields(p.nocc, p.nkp, p.diag);
   const size_t sa = smem_a<N>(sizeof(C2));
-  const size_t sb = smem_b<N>(sizeof(C2), sizeof(Axis1<T>));
+  const size_t sb = smem_b<N>(sizeof(C2));
   const size_t sc = smem_c<N>(sizeof(C2));
   static DeviceCache cache;   // per device: attributes set, resident pass-B slots
   const int slots_b = cache.get(p.device, [&] {
@@ -1691,7 +1703,7 @@ cudaError_t run_domega_wave(const PairParams& p, const cplx_t<T>* psi, cplx_t<T>
   const int nt = threads_for<T>(N);
   const int nf = wave_fields(p.nocc, p.nkp, p.diag);
   const size_t sa = smem_a<N>(sizeof(C2));
-  const size_t sb = smem_b<N>(sizeof(C2), sizeof(Axis1<T>));
+  const size_t sb = smem_b<N>(sizeof(C2));
   static DeviceCache cache;   // per device: attributes set, resident pass-B slots
   const int slots_b = cache.get(p.device, [&] {
     cudaFuncSetAttribute(pass_a<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sa);
@@ -1700,21 +1712,24 @@ cudaError_t run_domega_wave(const PairParams& p, const cplx_t<T>* psi, cplx_t<T>
     return resident_slots(pass_b_domega<T, N>, nt, sb);
   });
   pass_a<T, N><<<dim3(N, nf), nt, sa, st>>>(psi, S, p);
-  pass_b_domega<T, N><<<std::min(N * nf, slots_b), nt, sb, st>>>(S, p, dacc);
+  T* vt = reinterpret_cast<T*>(reinterpret_cast<char*>(S) + p.vt_off);
+  vtab_kernel<T, N, true><<<dim3(N, p.diag ? 1 : p.nkp, kVtabSplit), nt, 0, st>>>(vt, p);
+  pass_b_domega<T, N><<<std::min(N * nf, slots_b), nt, sb, st>>>(S, p, vt, dacc);
   return cudaGetLastError();
 }
 
 // One wave of the adjoint: the forward potentials W into S0, the potentials Z of the
-// adjoint densities into S1 (the same three transform passes), then pass E.
+// adjoint densities into S1 (the same three transform passes), then pass E. The two chains run on
+// two streams between their common points (the omega term and pass E), ev0 and ev1 in between.
 template <typename T, int N>
 cudaError_t run_vjp_wave(const PairParams& p, const cplx_t<T>* psi, const cplx_t<T>* gam,
                          cplx_t<T>* S0, cplx_t<T>* S1, cplx_t<T>* G, double* dacc,
-                         cudaStream_t st) {
+                         cudaStream_t st, cudaStream_t st2, cudaEvent_t ev0, cudaEvent_t ev1) {
   using C2 = cplx_t<T>;
   const int nt = threads_for<T>(N);
   const int nf = wave_fields(p.nocc, p.nkp, p.diag);
   const size_t sa = smem_a<N>(sizeof(C2));
-  const size_t sb = smem_b<N>(sizeof(C2), sizeof(Axis1<T>));
+  const size_t sb = smem_b<N>(sizeof(C2));
   const size_t sc = smem_c<N>(sizeof(C2));
   static DeviceCache cache;   // per device: attributes set, resident pass-B slots
   const int slots_b = cache.get(p.device, [&] {
@@ -1728,18 +1743,31 @@ cudaError_t run_vjp_wave(const PairParams& p, const cplx_t<T>* psi, const cplx_t
                          (int)(sb + sizeof(C2) * N * pitch(N)));
     return resident_slots(pass_b<T, N>, nt, sb);
   });
-  pass_a<T, N, false><<<dim3(N, nf), nt, sa, st>>>(psi, S0, p, nullptr);
-  pass_a<T, N, true><<<dim3(N, nf), nt, sa, st>>>(psi, S1, p, gam);
-  if (dacc)
-    pass_b_domega2<T, N><<<dim3(N, nf), nt, sb + sizeof(C2) * N * pitch(N), st>>>(S0, S1, p,
-                                                                                dacc);
+  cudaError_t e = cudaSuccess;
+  auto chk = [&](cudaError_t y) { if (e == cudaSuccess) e = y; };
+  auto after = [&](cudaStream_t a, cudaStream_t b, cudaEvent_t ev) {   // b goes on after a
+    chk(cudaEventRecord(ev, a));
+    chk(cudaStreamWaitEvent(b, ev, 0));
+  };
   T* vt = reinterpret_cast<T*>(reinterpret_cast<char*>(S0) + p.vt_off);
-  if (!p.vq) vtab_kernel<T, N><<<dim3(N, p.diag ? 1 : p.nkp, kVtabSplit), nt, 0, st>>>(vt, p);
+  const dim3 tab(N, p.diag ? 1 : p.nkp, kVtabSplit);
+  after(st, st2, ev0);
+  pass_a<T, N, false><<<dim3(N, nf), nt, sa, st>>>(psi, S0, p, nullptr);
+  pass_a<T, N, true><<<dim3(N, nf), nt, sa, st2>>>(psi, S1, p, gam);
+  if (dacc) {
+    vtab_kernel<T, N, true><<<tab, nt, 0, st>>>(vt, p);
+    after(st2, st, ev1);
+    pass_b_domega2<T, N><<<dim3(N, nf), nt, sb + sizeof(C2) * N * pitch(N), st>>>(S0, S1, p, vt,
+                                                                                dacc);
+  }
+  if (!p.vq) vtab_kernel<T, N><<<tab, nt, 0, st>>>(vt, p);
+  if (dacc || !p.vq) after(st, st2, ev0);
   pass_b<T, N><<<std::min(N * nf, slots_b), nt, sb, st>>>(S0, p, vt);
   pass_c<T, N><<<dim3(N, nf), nt, sc, st>>>(S0, p);
-  pass_b<T, N><<<std::min(N * nf, slots_b), nt, sb, st>>>(S1, p, vt);
-  pass_c<T, N><<<dim3(N, nf), nt, sc, st>>>(S1, p);
-  const cudaError_t e = launch_pass_e<T>(p, S0, S1, psi, gam, G, st);
+  pass_b<T, N><<<std::min(N * nf, slots_b), nt, sb, st2>>>(S1, p, vt);
+  pass_c<T, N><<<dim3(N, nf), nt, sc, st2>>>(S1, p);
+  after(st2, st, ev1);
+  chk(launch_pass_e<T>(p, S0, S1, psi, gam, G, st));
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

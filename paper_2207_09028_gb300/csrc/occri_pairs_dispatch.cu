@@ -76,7 +76,8 @@ cudaError_t launch_vjp_wave(const Plan& p, int k, int kp0, int nkp, int diag, do
   switch (p.N[0]) {
 #define OCCRI_VJP_CASE(NN) \
   case NN:                 \
-    return pairs::run_vjp_wave<T, NN>(pp, psi, gam, S0, S1, G, dacc, s);
+    return pairs::run_vjp_wave<T, NN>(pp, psi, gam, S0, S1, G, dacc, s, p.aux, p.ev_iso,   \
+                                      p.ev_iso2);
     OCCRI_FOR_EACH_N(OCCRI_VJP_CASE)
 #undef OCCRI_VJP_CASE
     default:

@@ -13,8 +13,8 @@ template cudaError_t run_qtables<double, 32>(const PairParams&, double*, cudaStr
 template cudaError_t run_wave<double, 36>(const PairParams&, const cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, cudaStream_t, cudaEvent_t*, cudaEvent_t);
 template cudaError_t run_domega_wave<double, 36>(const PairParams&, const cplx_t<double>*, cplx_t<double>*, double*, cudaStream_t);
 template cudaError_t run_qtables<double, 36>(const PairParams&, double*, cudaStream_t);
-template cudaError_t run_vjp_wave<double, 30>(const PairParams&, const cplx_t<double>*, const cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, double*, cudaStream_t);
-template cudaError_t run_vjp_wave<double, 32>(const PairParams&, const cplx_t<double>*, const cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, double*, cudaStream_t);
-template cudaError_t run_vjp_wave<double, 36>(const PairParams&, const cplx_t<double>*, const cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, double*, cudaStream_t);
+template cudaError_t run_vjp_wave<double, 30>(const PairParams&, const cplx_t<double>*, const cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, double*, cudaStream_t, cudaStream_t, cudaEvent_t, cudaEvent_t);
+template cudaError_t run_vjp_wave<double, 32>(const PairParams&, const cplx_t<double>*, const cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, double*, cudaStream_t, cudaStream_t, cudaEvent_t, cudaEvent_t);
+template cudaError_t run_vjp_wave<double, 36>(const PairParams&, const cplx_t<double>*, const cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, cplx_t<double>*, double*, cudaStream_t, cudaStream_t, cudaEvent_t, cudaEvent_t);
 }  // namespace pairs
 }  // namespace occri
