@@ -355,7 +355,7 @@ def tensor_roofline(info: dict, contract_ms: float, peak_tflops: float, peak_kin
     if not info.get("contraction_tc") or st <= 0 or contract_ms <= 0 or fps <= 0:
         return None
     achieved = fps * st / (contract_ms / 1e3) / 1e12
-    return {"kernel": "contract_tc_kernel (tcgen05.mma kind::f16, FP16 hi/lo x3, FP32 accumulate)",
+    return {"kernel": "con_tc_kernel (tcgen05.mma kind::f16, FP16 hi/lo x3, FP32 accumulate)",
             "bound": "tensor", "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
             "frac": achieved / peak_tflops, "peak_kind": peak_kind, "stages": st,
             "flops_per_stage": fps, "gemm_ms": contract_ms, "stage_ms": stage_ms,

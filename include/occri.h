@@ -84,15 +84,11 @@ typedef enum {
  * OCCRI_MIXED: AO evaluation, orbitals, pair densities, FFTs, the kernel multiply
  *   and the Y accumulation in FP32; the contraction (e) accumulates per thread in
  *   FP32 and across threads in FP64; assembly (f) and E_x in FP64.
- * OCCRI_MIXED_TC: as OCCRI_MIXED, but the contraction (e) runs on the tensor cores as
- *   one GEMM over the grid points of the k-mesh's supercell: the AOs periodised over the
- *   supercell (generated on the fly) times Y, both split into FP16 hi + lo parts with
- *   power-of-two scalings, three FP16 products with FP32 accumulation per term; each
- *   32-point product leaves tensor memory at once, times the phase of its supercell offset,
- *   into FP32 running sums over at most 16 point tiles, and FP64 sums beyond.
- *   Where the supercell has more than 512 cells, the cell more than 8 atoms, or a tile of 32
- *   grid points more than 128 supercell images in reach (small supercells), the plan keeps
- *   the CUDA-core contraction of OCCRI_MIXED; occri_plan_info reports which one it uses. */
+ * OCCRI_MIXED_TC: as OCCRI_MIXED, but the contraction (e) runs on the tensor cores, per k as a
+ *   real GEMM over the grid points: rows Re and Im of the Bloch AOs, columns Re and Im of Y,
+ *   both split into FP16 hi + lo parts with power-of-two scalings, three FP16 products with
+ *   FP32 accumulation per term; each 16-point product leaves tensor memory after its stage
+ *   into FP32 running sums over at most 64 blocks of 32 points, and FP64 sums beyond. */
 typedef enum { OCCRI_FP64 = 0, OCCRI_MIXED = 1, OCCRI_MIXED_TC = 2 } occri_precision;
 
 typedef struct {
@@ -139,12 +135,13 @@ typedef struct {
   size_t workspace_bytes;  /* device bytes owned by the plan */
   int fields_per_wave;     /* pair fields transformed per launch group */
   long long launches_per_build;  /* kernels one occri_k_build launches */
-  int contraction_tc;      /* 1: step (e) runs on the tensor cores (OCCRI_MIXED_TC where the
-                              supercell admits it), 0: on the CUDA cores */
+  int contraction_tc;      /* 1: step (e) runs on the tensor cores (OCCRI_MIXED_TC), 0: on
+                              the CUDA cores */
   long long tc_stages;     /* tensor-core contraction: stages per build, else 0 */
   double tc_flops_per_stage;  /* MMA flops one stage issues: 3 products (FP16 hi/lo) of
-                                 M = 128 AO rows, N = 192 (Re, Im of 96 (k, i) columns),
-                                 K = 32 grid points, i.e. 3 x 2 M N K */
+                                 M = 128 rows (Re, Im of 64 AOs), N = 16, 32 or 64 columns
+                                 (Re, Im of up to 8, 16 or 32 orbitals), K = 64 grid points,
+                                 i.e. 3 x 2 M N K */
 } occri_plan_info_t;
 
 /* Stages reported by occri_plan_stage_times. */
@@ -160,8 +157,8 @@ enum {
   OCCRI_STAGE_ASSEMBLE = 5,  /* (f) */
   OCCRI_STAGE_PAIRS = 6,     /* (c)+(d): the whole loop over pair waves, wall time */
   OCCRI_STAGE_CONTRACT_GEMM = 7,  /* (e) on the tensor cores: the GEMM kernels alone (inside
-                                     OCCRI_STAGE_CONTRACT, which also holds the Y conversion
-                                     and the A-block generation) */
+                                     OCCRI_STAGE_CONTRACT, which also holds the Y scales, the
+                                     sums over work items and, on large problems, the AOs) */
   OCCRI_NSTAGES = 8
 };
 
@@ -176,7 +173,10 @@ typedef struct occri_plan occri_plan;
  * cudaStream_t or NULL (legacy default stream). The plan lives on the device current at
  * this call: every later call on it makes that device current for its duration and then
  * restores the caller's. Among its workspaces are the kernel tables v/(4 pi) of every integer
- * k - k' on the mesh, formed here where they take at most 4 GiB (occri_tune_t.wave_tables).
+ * k - k' on the mesh, formed here where they take at most 4 GiB (occri_tune_t.wave_tables),
+ * and a buffer for the Bloch AOs of the grid (all of them where they take at most 8 GiB and a
+ * quarter of the free memory, else 1 GiB or an eighth of it), filled by every call that needs
+ * them.
  * On success *out owns a plan to be destroyed with occri_plan_destroy; on failure *out is
  * NULL. */
 int occri_plan_create(occri_plan **out, const occri_cell *cell, const occri_kmesh *kmesh,
@@ -274,8 +274,9 @@ int occri_k_assemble_paper(occri_plan *plan, int ncol, const void *S_dev, const 
  * build (the bands' own terms), so it costs one build of each.
  * C_all_dev: device c128 [nk][nao][nocc + nr], occupied columns first.
  * KCr_dev  : device c128 [nk][nao][nr], written.
- * Both builds run on plan_all's stream; the call synchronises it, allocates and frees a
- * temporary of 16 nk nao (nocc + 3 nr) bytes (OCCRI_ENOMEM), and returns the first device
+ * Both builds run on plan_all's stream; the call synchronises it, keeps a buffer of
+ * 16 nk nao (nocc + 3 nr) bytes with plan_all (allocated by the first call that needs it:
+ * OCCRI_ENOMEM), and returns the first device
  * error of either build (as occri_plan_sync). OCCRI_EINVAL if the plans differ in anything
  * but nocc, or plan_r's nocc is not below plan_all's. */
 int occri_k_build_conduction(occri_plan *plan_all, occri_plan *plan_r, const void *C_all_dev,

@@ -239,32 +239,35 @@ __global__ void widen_kernel(const cplx_t<T>* __restrict__ in, double2* __restri
 }
 
 
-// F[k][i][q] *= e^{sign i k.r_q} for every orbital field of every k-point (fields'
-// point order q = (n3 N + n1) N + n2, cubic grid of edge N). With sign = -1 this turns
-// the Bloch orbitals psi_ik into their periodic parts u_ik = e^{-ik.r} psi_ik, with
-// sign = +1 it turns the accumulated periodic parts back into Y_ik. The phase is
-// 2 pi sum_d kint_d n_d / (D_d N), reduced exactly in integers.
+// F[k][i][q] = (F + a + b) e^{i k.r_q} for every orbital field of every k-point (fields' point order
+// q = (n3 N + n1) N + n2, cubic grid of edge N): the streams' sums of periodic parts become Y_ik.
 template <typename T>
-__global__ void phase_fields_kernel(cplx_t<T>* __restrict__ F, const int* __restrict__ kint,
-                                    int k0, int nk, int nocc, int N, long long fs, int D0, int D1,
-                                    int D2, int sign) {
+__global__ void phase_fields_kernel(cplx_t<T>* __restrict__ F, const cplx_t<T>* __restrict__ a,
+                                    const cplx_t<T>* __restrict__ b, const int* __restrict__ kint,
+                                    int nk, int nocc, int N, long long fs, int D0, int D1, int D2) {
   const long long ng = (long long)N * N * N;
-  const long long Dc = (long long)D0 * D1 * D2;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nk * ng;
        e += (long long)gridDim.x * blockDim.x) {
-    const int k = k0 + (int)(e / ng);
-    const long long q = e - (long long)(k - k0) * ng;
+    const int k = (int)(e / ng);
+    const long long q = e - (long long)k * ng;
     const int n3 = (int)(q / ((long long)N * N));
     const int rem = (int)(q - (long long)n3 * N * N);
-    const int n1 = rem / N, n2 = rem - (rem / N) * N;
-    const long long num = (long long)kint[3 * k] * n1 * (Dc / D0) +
-                          (long long)kint[3 * k + 1] * n2 * (Dc / D1) +
-                          (long long)kint[3 * k + 2] * n3 * (Dc / D2);
-    const cplx_t<T> ph = dev::cis_frac<T>(num, Dc * N, sign);
-    cplx_t<T>* f = F + (size_t)k * nocc * fs + q;
+    const cplx_t<T> ph = point_phase<T>(kint + 3 * k, D0, D1, D2, N, rem / N, rem % N, n3, +1);
+    const size_t at = (size_t)k * nocc * fs + q;
     for (int i = 0; i < nocc; ++i) {
-      const cplx_t<T> v = f[(size_t)i * fs];
-      f[(size_t)i * fs] = cplx_t<T>{v.x * ph.x - v.y * ph.y, v.x * ph.y + v.y * ph.x};
+      const size_t f = at + (size_t)i * fs;
+      cplx_t<T> v = F[f];
+      if (a) {
+        cplx_t<T> u = a[f];
+        if (b) {
+          const cplx_t<T> w = b[f];
+          u.x += w.x;
+          u.y += w.y;
+        }
+        v.x += u.x;
+        v.y += u.y;
+      }
+      F[f] = dev::cmul<T>(v, ph);
     }
   }
 }
@@ -272,13 +275,17 @@ __global__ void phase_fields_kernel(cplx_t<T>* __restrict__ F, const int* __rest
 }  // namespace ao
 
 template <typename T>
-cudaError_t launch_phase_fields(const Plan& p, void* F, int sign, cudaStream_t s) {
-  ao::phase_fields_kernel<T><<<8 * 152, 256, 0, s>>>((cplx_t<T>*)F, p.kint, 0, p.nk, p.nocc,
-                                                      p.N[0], p.fs, p.D[0], p.D[1], p.D[2], sign);
+cudaError_t launch_phase_fields(const Plan& p, void* F, const void* a, const void* b,
+                                cudaStream_t s) {
+  ao::phase_fields_kernel<T><<<8 * 152, 256, 0, s>>>((cplx_t<T>*)F, (const cplx_t<T>*)a,
+                                                      (const cplx_t<T>*)b, p.kint, p.nk, p.nocc,
+                                                      p.N[0], p.fs, p.D[0], p.D[1], p.D[2]);
   return cudaGetLastError();
 }
-template cudaError_t launch_phase_fields<float>(const Plan&, void*, int, cudaStream_t);
-template cudaError_t launch_phase_fields<double>(const Plan&, void*, int, cudaStream_t);
+template cudaError_t launch_phase_fields<float>(const Plan&, void*, const void*, const void*,
+                                                cudaStream_t);
+template cudaError_t launch_phase_fields<double>(const Plan&, void*, const void*, const void*,
+                                                 cudaStream_t);
 
 template <typename T>
 cudaError_t launch_widen(const Plan& p, void* out, cudaStream_t s) {

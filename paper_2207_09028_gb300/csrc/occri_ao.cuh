@@ -122,5 +122,16 @@ __device__ __forceinline__ long long block_point(const AOParams& p, int blk, int
   return ((long long)n1 * p.N[1] + n2) * p.N[2] + n3;
 }
 
+// e^{sign i k.r} at grid point (n1, n2, n3): the phase 2 pi sum_d kint_d n_d / (D_d N) of k = kint / D,
+// reduced exactly in integers.
+template <typename T>
+__device__ __forceinline__ cplx_t<T> point_phase(const int* kint, int D0, int D1, int D2, int N,
+                                                 int n1, int n2, int n3, int sign) {
+  const long long Dc = (long long)D0 * D1 * D2;
+  const long long num = (long long)kint[0] * n1 * (Dc / D0) + (long long)kint[1] * n2 * (Dc / D1) +
+                        (long long)kint[2] * n3 * (Dc / D2);
+  return cis_frac<T>(num, Dc * N, sign);
+}
+
 }  // namespace ao
 }  // namespace occri

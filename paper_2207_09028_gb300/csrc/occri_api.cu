@@ -715,25 +715,6 @@ ace_adjoint_kernel(const double2* __restrict__ C, const double2* __restrict__ kc
   }
 }
 
-// y += a + b (b may be null) over n complex values (the streams' accumulators into Y)
-template <typename C2>
-__global__ void add3_kernel(C2* __restrict__ y, const C2* __restrict__ a, const C2* __restrict__ b,
-                            long long n) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    C2 v = y[i];
-    C2 u = a[i];
-    if (b) {
-      const C2 w = b[i];
-      u.x += w.x;
-      u.y += w.y;
-    }
-    v.x += u.x;
-    v.y += u.y;
-    y[i] = v;
-  }
-}
-
 __global__ void add_kernel(const double2* __restrict__ a, const double2* __restrict__ b,
                            double2* __restrict__ out, long long n) {
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
@@ -745,7 +726,7 @@ void free_plan(Plan* p) {
   if (!p) return;
   void* bufs[] = {p->shells, p->atom_shell0, p->img_d, p->img_hi, p->img_lo, p->img_phase,
                   p->d0_d, p->d0_hi, p->d0_lo, p->t0, p->kint, p->psi, p->Y, p->scratch,
-                  p->kc, p->lmat, p->ace_share, p->ace_ok, p->mmat, p->ek, p->dacc, p->status, p->h_c, p->h_kc, p->h_k,
+                  p->kc, p->lmat, p->ace_share, p->ace_ok, p->mmat, p->ek, p->dacc, p->h_c, p->h_kc, p->h_k,
                   p->h_ex, p->ao_norm, p->cs, p->blist, p->bpre};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -763,6 +744,8 @@ void free_plan(Plan* p) {
   if (p->aux) cudaStreamDestroy(p->aux);
   if (p->aux2) cudaStreamDestroy(p->aux2);
   if (p->colmax) cudaFree(p->colmax);
+  if (p->status_h) cudaFreeHost(p->status_h);
+  if (p->bands) cudaFree(p->bands);
   chi_free(p->chi);
   for (cudaEvent_t e : p->ev_used) cudaEventDestroy(e);
   for (cudaEvent_t e : p->ev_free) cudaEventDestroy(e);
@@ -776,6 +759,17 @@ void free_plan(Plan* p) {
 using occri::Plan;
 
 namespace occri_impl {
+
+// The device status of the plan's finished work (its stream has been synchronised), cleared for
+// the next calls.
+int take_status(Plan* p, int* bad_k) {
+  volatile int* st = p->status_h;
+  const int code = st[0];
+  if (code == 0) return OCCRI_OK;
+  if (bad_k) *bad_k = st[1];
+  st[0] = 0;
+  return code;
+}
 
 cudaEvent_t take_event(Plan* p) {
   cudaEvent_t e = nullptr;
@@ -841,13 +835,12 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
   {
     StageTimer t(p, timed);
     if (launch_slot_c<T>(*p, C, p->cs, 1.0, s) != cudaSuccess) return OCCRI_ECUDA;
-    if (launch_orbitals<T>(*p, 1, &p->cs, &p->psi, s) != cudaSuccess) return OCCRI_ECUDA;
     // the pair passes work on the periodic parts u = e^{-ik.r} psi: the pair density
     // conj(u_jk') u_ik is then periodic as it stands, and the accumulated periodic part
     // e^{-ik.r} Y_ik needs no phase either (Y is restored below)
-    if (launch_phase_fields<T>(*p, p->psi, -1, s) != cudaSuccess) return OCCRI_ECUDA;
+    if (launch_orbitals<T>(*p, 1, &p->cs, &p->psi, true, s) != cudaSuccess) return OCCRI_ECUDA;
     t.done(OCCRI_STAGE_ORBITALS, p->nk);
-    launches += 2 + chi_launches(*p, false);
+    launches += 1 + chi_launches(*p, false);
   }
   {
     // Waves go round-robin over the plan's stream and one or two auxiliary ones, each with
@@ -908,17 +901,13 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
       if (cudaEventRecord(join[o], st[o]) != cudaSuccess ||
           cudaStreamWaitEvent(s, join[o], 0) != cudaSuccess)
         return OCCRI_ECUDA;
-    if (split_y) {
-      add3_kernel<<<8 * 152, 256, 0, s>>>((cplx_t<T>*)p->Y, (const cplx_t<T>*)p->Yx[0],
-                                          ns > 2 ? (const cplx_t<T>*)p->Yx[1] : nullptr,
-                                          (long long)orb);
-      ++launches;
-    }
     all.done(OCCRI_STAGE_PAIRS, fields);
   }
   {
     StageTimer t(p, timed);
-    if (launch_phase_fields<T>(*p, p->Y, +1, s) != cudaSuccess) return OCCRI_ECUDA;
+    if (launch_phase_fields<T>(*p, p->Y, split_y ? p->Yx[0] : nullptr,
+                               split_y && ns > 2 ? p->Yx[1] : nullptr, s) != cudaSuccess)
+      return OCCRI_ECUDA;
     ++launches;
     if (p->precision == OCCRI_MIXED_TC) {
       // the GEMM kernels alone, one span per slab (stage OCCRI_STAGE_CONTRACT_GEMM)
@@ -937,13 +926,13 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
           t = nullptr;
         }
       } spans(p, s, timed);
-      if (launch_contract_tc(*p, s, &spans) != cudaSuccess) return OCCRI_ECUDA;
+      if (launch_contract_tc(*p, (double2*)KC, s, &spans) != cudaSuccess) return OCCRI_ECUDA;
       launches += tc_plan_launches(*p);
     } else {
       // Y carries N_g/(4 pi) (see PairParams), hence -Omega 4 pi / (N_k N_g^2)
       const double scale = -p->omega_cell * 4.0 * kPiD /
                            ((double)p->nk * (double)p->ng * (double)p->ng);
-      if (launch_contract_field<T>(*p, p->Y, p->kc, scale, s) != cudaSuccess) return OCCRI_ECUDA;
+      if (launch_contract_field<T>(*p, p->Y, p->kc, (double2*)KC, scale, s) != cudaSuccess) return OCCRI_ECUDA;
       launches += chi_launches(*p, true);
     }
     t.done(OCCRI_STAGE_CONTRACT, p->nk);
@@ -973,10 +962,6 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
     }
     t.done(OCCRI_STAGE_ASSEMBLE, p->nk);
   }
-  if (KC &&
-      cudaMemcpyAsync(KC, p->kc, sizeof(double2) * (size_t)p->nk * p->nao * p->nocc,
-                      cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-    return OCCRI_ECUDA;
   if (cudaGetLastError() != cudaSuccess) return OCCRI_ECUDA;
   p->have_kc = true;
   p->launches_per_build = launches;
@@ -995,8 +980,7 @@ int vjp_impl(Plan* p, const double2* C, double gEx, void* gC, double* gomega) {
       // periodic parts of the orbitals of C (the plan's copy may have been replaced by
       // an occri_orbitals call since the build)
       if (launch_slot_c<T>(*p, C, p->cs, 1.0, s) != cudaSuccess) return OCCRI_ECUDA;
-      if (launch_orbitals<T>(*p, 1, &p->cs, &p->psi, s) != cudaSuccess) return OCCRI_ECUDA;
-      if (launch_phase_fields<T>(*p, p->psi, -1, s) != cudaSuccess) return OCCRI_ECUDA;
+      if (launch_orbitals<T>(*p, 1, &p->cs, &p->psi, true, s) != cudaSuccess) return OCCRI_ECUDA;
       for (int k = 0; k < p->nk; ++k)
         for (int kp0 = k; kp0 < p->nk;) {
           const int diag = (kp0 == k) ? 1 : 0;
@@ -1049,9 +1033,7 @@ int vjp_full_impl(Plan* p, const double2* C, double gEx, const double2* gKC, con
   if (launch_slot_c<T>(*p, C, p->cs, 1.0, s) != cudaSuccess) return OCCRI_ECUDA;
   const void* coefs[2] = {p->cs_g, p->cs};
   void* fields[2] = {p->gam, p->psi};
-  if (launch_orbitals<T>(*p, 2, coefs, fields, s) != cudaSuccess) return OCCRI_ECUDA;
-  if (launch_phase_fields<T>(*p, p->gam, -1, s) != cudaSuccess) return OCCRI_ECUDA;
-  if (launch_phase_fields<T>(*p, p->psi, -1, s) != cudaSuccess) return OCCRI_ECUDA;
+  if (launch_orbitals<T>(*p, 2, coefs, fields, true, s) != cudaSuccess) return OCCRI_ECUDA;
   // (c)+(d): two round trips per unordered pair, dL/dpsi accumulated (and the omega
   // term of the kernel's derivative, for the erfc and erf kernels)
   if (cudaMemsetAsync(p->gpsi, 0, orb, s) != cudaSuccess) return OCCRI_ECUDA;
@@ -1068,10 +1050,10 @@ int vjp_full_impl(Plan* p, const double2* C, double gEx, const double2* gKC, con
     }
   // (b): dL/dC_{mu i} = sum_r conj(chi_mu) dL/dpsi_i; the transforms carry N_g/(4 pi)
   // and g carried N_k N_g/Omega, hence the factor 4 pi Omega/(N_k N_g^2)
-  if (launch_phase_fields<T>(*p, p->gpsi, +1, s) != cudaSuccess) return OCCRI_ECUDA;
+  if (launch_phase_fields<T>(*p, p->gpsi, nullptr, nullptr, s) != cudaSuccess) return OCCRI_ECUDA;
   const double ngd = (double)p->ng;
   const double scale = 4.0 * kPiD * p->omega_cell / ((double)p->nk * ngd * ngd);
-  if (launch_contract_field<T>(*p, p->gpsi, p->gacc, scale, s) != cudaSuccess) return OCCRI_ECUDA;
+  if (launch_contract_field<T>(*p, p->gpsi, p->gacc, nullptr, scale, s) != cudaSuccess) return OCCRI_ECUDA;
   add_kernel<<<4 * 152, 256, 0, s>>>(p->gcf, p->gacc, gC, (long long)nkc);
   // dL/d omega = Re <dL/dKC, dKC/d omega>: the same units as the gradient of C
   if (gomega) domega_finish_kernel<<<1, 32, 0, s>>>(p->dacc, scale, gomega);
@@ -1774,8 +1756,13 @@ int occri_plan_create(occri_plan** out, const occri_cell* cell, const occri_kmes
   chk(dalloc(&p->ek, (size_t)p->nk, &tot));
   chk(dalloc(&p->dacc, 2, &tot));
   if (precision == OCCRI_MIXED_TC) chk(dalloc(&p->colmax, (size_t)p->nk * nocc, &tot));
-  chk(dalloc(&p->status, 2, &tot));
-  if (e == cudaSuccess) e = cudaMemset(p->status, 0, 2 * sizeof(int));
+  // mapped host memory: a kernel writes it only when something failed, and a sync reads it
+  // without a copy (cudaMemcpy of eight bytes took about 10 us of every synchronised call)
+  if (e == cudaSuccess) e = cudaHostAlloc((void**)&p->status_h, 2 * sizeof(int), cudaHostAllocMapped);
+  if (e == cudaSuccess) {
+    p->status_h[0] = p->status_h[1] = 0;
+    e = cudaHostGetDevicePointer((void**)&p->status, p->status_h, 0);
+  }
   if (e == cudaSuccess) e = cudaMemset(p->ace_ok, 0, sizeof(int) * (2 * (size_t)p->nk + 1));
   if (e == cudaSuccess && p->vq)
     e = precision == OCCRI_FP64 ? launch_qtables<double>(*p, p->stream)
@@ -1882,14 +1869,7 @@ int occri_plan_sync(occri_plan* plan, int* bad_k) {
   if (!guard.ok) return OCCRI_ECUDA;
   Plan* p = plan->p;
   if (cudaStreamSynchronize(p->stream) != cudaSuccess) return OCCRI_ECUDA;
-  int st[2] = {0, -1};
-  if (cudaMemcpy(st, p->status, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return OCCRI_ECUDA;
-  if (st[0] != 0) {
-    if (cudaMemset(p->status, 0, sizeof(st)) != cudaSuccess) return OCCRI_ECUDA;
-    if (bad_k) *bad_k = st[1];
-    return st[0];
-  }
-  return OCCRI_OK;
+  return occri_impl::take_status(p, bad_k);
 }
 
 
@@ -1990,13 +1970,20 @@ int occri_k_build_conduction(occri_plan* plan_all, occri_plan* plan_r, const voi
   if (!guard.ok) return OCCRI_ECUDA;
   const int nr = pr->nocc, nocc = pa->nocc - nr;
   const long long rows = (long long)pa->nk * pa->nao;
-  void* buf = nullptr;
   const size_t b_all = sizeof(double2) * (size_t)rows * pa->nocc;
   const size_t b_r = sizeof(double2) * (size_t)rows * nr;
-  if (occri::device_malloc(&buf, b_all + 2 * b_r) != cudaSuccess) {
-    cudaGetLastError();
-    return OCCRI_ENOMEM;
+  if (pa->bands_bytes < b_all + 2 * b_r) {   // kept with the plan
+    if (pa->bands) cudaFree(pa->bands);
+    pa->bands = nullptr;
+    pa->bands_bytes = 0;
+    if (occri::device_malloc(&pa->bands, b_all + 2 * b_r) != cudaSuccess) {
+      cudaGetLastError();
+      pa->bands = nullptr;
+      return OCCRI_ENOMEM;
+    }
+    pa->bands_bytes = b_all + 2 * b_r;
   }
+  void* buf = pa->bands;
   double2* kc_all = (double2*)buf;
   double2* c_r = (double2*)((unsigned char*)buf + b_all);
   double2* kc_r = (double2*)((unsigned char*)buf + b_all + b_r);
@@ -2015,7 +2002,6 @@ int occri_k_build_conduction(occri_plan* plan_all, occri_plan* plan_r, const voi
     st = OCCRI_ECUDA;
   if (cudaStreamSynchronize(pa->stream) != cudaSuccess && st == OCCRI_OK) st = OCCRI_ECUDA;
   pr->stream = keep;
-  cudaFree(buf);
   if (st != OCCRI_OK) {
     cudaGetLastError();
     return st;
@@ -2104,11 +2090,11 @@ int occri_orbitals(occri_plan* plan, const void* C_dev, void* psi_dev) {
   cudaError_t e;
   if (p->precision == OCCRI_FP64) {
     e = occri::launch_slot_c<double>(*p, (const double2*)C_dev, p->cs, 1.0, p->stream);
-    if (e == cudaSuccess) e = occri::launch_orbitals<double>(*p, 1, &p->cs, &p->psi, p->stream);
+    if (e == cudaSuccess) e = occri::launch_orbitals<double>(*p, 1, &p->cs, &p->psi, false, p->stream);
     if (e == cudaSuccess) e = occri::launch_widen<double>(*p, psi_dev, p->stream);
   } else {
     e = occri::launch_slot_c<float>(*p, (const double2*)C_dev, p->cs, 1.0, p->stream);
-    if (e == cudaSuccess) e = occri::launch_orbitals<float>(*p, 1, &p->cs, &p->psi, p->stream);
+    if (e == cudaSuccess) e = occri::launch_orbitals<float>(*p, 1, &p->cs, &p->psi, false, p->stream);
     if (e == cudaSuccess) e = occri::launch_widen<float>(*p, psi_dev, p->stream);
   }
   return e == cudaSuccess ? OCCRI_OK : OCCRI_ECUDA;
@@ -2218,16 +2204,12 @@ int occri_batch_sync(occri_batch* b, int* bad_cell, int* bad_k) {
   int first = OCCRI_OK;
   for (size_t i = 0; i < b->plans.size(); ++i) {
     Plan* p = b->plans[i]->p;
-    int st[2] = {0, -1};
-    if (cudaMemcpy(st, p->status, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess)
-      return OCCRI_ECUDA;
-    if (st[0] != 0) {
-      if (cudaMemset(p->status, 0, sizeof(st)) != cudaSuccess) return OCCRI_ECUDA;
-      if (first == OCCRI_OK) {
-        first = st[0];
-        if (bad_cell) *bad_cell = (int)i;
-        if (bad_k) *bad_k = st[1];
-      }
+    int k = -1;
+    const int st = occri_impl::take_status(p, &k);
+    if (st != OCCRI_OK && first == OCCRI_OK) {
+      first = st;
+      if (bad_cell) *bad_cell = (int)i;
+      if (bad_k) *bad_k = k;
     }
   }
   return first;

@@ -671,7 +671,7 @@ template <typename T, int NI> constexpr int orb_blocks() { return sizeof(T) == 4
 template <typename T, int NI, int NB>
 __global__ void __launch_bounds__(128)
 orb_kernel(Params p, const cplx_t<T>* __restrict__ chi, const typename CsT<T>::type* __restrict__ cs,
-           cplx_t<T>* __restrict__ psi, int blk0, int nb, int i0) {
+           cplx_t<T>* __restrict__ psi, int blk0, int nb, int i0, int periodic) {
   const int w = NB * (blockIdx.x * 4 + (threadIdx.x >> 5));
   if (w >= nb) return;
   const int k = blockIdx.y, lane = threadIdx.x & 31;
@@ -742,8 +742,16 @@ orb_kernel(Params p, const cplx_t<T>* __restrict__ chi, const typename CsT<T>::t
     if (b > nlast) break;
     bool valid;
     long long q;
-    ao::block_point(p.a, blk + b, lane, &valid, &q);
+    const long long n = ao::block_point(p.a, blk + b, lane, &valid, &q);
     if (!valid) continue;
+    if (periodic) {   // u = e^{-ik.r} psi
+      const int N = p.a.N[0];
+      const int n3 = (int)(n % N), n2 = (int)(n / N % N), n1 = (int)(n / ((long long)N * N));
+      const cplx_t<T> ph = ao::point_phase<T>(p.a.kint + 3 * k, p.a.D[0], p.a.D[1], p.a.D[2], N,
+                                              n1, n2, n3, -1);
+#pragma unroll
+      for (int i = 0; i < NI; ++i) acc[b][i] = dev::cmul<T>(acc[b][i], ph);
+    }
 #pragma unroll
     for (int i = 0; i < NI; ++i)
       if (i0 + i < nocc) psi[((size_t)k * nocc + i0 + i) * p.a.fs + q] = acc[b][i];
@@ -856,7 +864,7 @@ con_kernel(Params p, const cplx_t<T>* __restrict__ chi, const cplx_t<T>* __restr
 constexpr int kSumSplit = 8;
 template <int NI>
 __global__ void __launch_bounds__(2 * kPad * NI * kSumSplit)
-sum_kernel(Params p, double2* __restrict__ out, int row_of0, int nitems, int i0, double scale, int add) {
+sum_kernel(Params p, double2* __restrict__ out, double2* __restrict__ copy, int row_of0, int nitems, int i0, double scale, int add) {
   constexpr int NV = 2 * kPad * NI;
   __shared__ double share[kSumSplit][NV];
   const int v = threadIdx.x % NV, z = threadIdx.x / NV, k = blockIdx.y;
@@ -879,9 +887,12 @@ sum_kernel(Params p, double2* __restrict__ out, int row_of0, int nitems, int i0,
   if (mu < 0 || i0 + i >= p.a.nocc) return;
 #pragma unroll
   for (int y = 1; y < kSumSplit; ++y) t += share[y][v];
-  double* dst = reinterpret_cast<double*>(out + ((size_t)k * p.a.nao + mu) * p.a.nocc + i0 + i);
+  const size_t at = 2 * (((size_t)k * p.a.nao + mu) * p.a.nocc + i0 + i) + (v & 1);
+  double* dst = reinterpret_cast<double*>(out) + at;
   t *= scale * p.ao_norm[mu];
-  dst[v & 1] = add ? dst[v & 1] + t : t;
+  if (add) t += *dst;
+  *dst = t;
+  if (copy) reinterpret_cast<double*>(copy)[at] = t;
 }
 
 // Coefficients factor N_mu X^k_{mu i} in slot order, formed in FP64 (hi/lo floats in FP32), 0
@@ -986,27 +997,27 @@ cudaError_t fill(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t
 
 template <typename T, int NI>
 void run_orb(const Params& q, const cplx_t<T>* chi, const void* cs, void* out, const ChiChunk& c,
-             int i0, cudaStream_t s) {
+             int i0, int periodic, cudaStream_t s) {
   // one block per warp where two would leave SMs without work
   const int nb = c.b1 - c.b0;
   constexpr int NB = orb_blocks<T, NI>();
   if (NB == 1 || (long long)nb * q.a.nk < 152 * 64)
     orb_kernel<T, NI, 1><<<dim3((nb + 3) / 4, q.a.nk), 128, 0, s>>>(
-        q, chi, (const typename CsT<T>::type*)cs, (cplx_t<T>*)out, c.b0, nb, i0);
+        q, chi, (const typename CsT<T>::type*)cs, (cplx_t<T>*)out, c.b0, nb, i0, periodic);
   else
     orb_kernel<T, NI, NB><<<dim3((nb + 7) / 8, q.a.nk), 128, 0, s>>>(
-        q, chi, (const typename CsT<T>::type*)cs, (cplx_t<T>*)out, c.b0, nb, i0);
+        q, chi, (const typename CsT<T>::type*)cs, (cplx_t<T>*)out, c.b0, nb, i0, periodic);
 }
 
 template <typename T>
 cudaError_t product_b(const Plan& p, const Params& q, const ChiChunk& c, const void* cs,
-                      void* out, cudaStream_t s) {
+                      void* out, int periodic, cudaStream_t s) {
   const cplx_t<T>* x = (const cplx_t<T>*)p.chi->chi;
   for (int i0 = 0; i0 < p.nocc;) {
     const int left = p.nocc - i0;
-    if (left <= 4) run_orb<T, 4>(q, x, cs, out, c, i0, s);
-    else if (left <= 8) run_orb<T, 8>(q, x, cs, out, c, i0, s);
-    else run_orb<T, 16>(q, x, cs, out, c, i0, s);
+    if (left <= 4) run_orb<T, 4>(q, x, cs, out, c, i0, periodic, s);
+    else if (left <= 8) run_orb<T, 8>(q, x, cs, out, c, i0, periodic, s);
+    else run_orb<T, 16>(q, x, cs, out, c, i0, periodic, s);
     i0 += left <= 4 ? 4 : (left <= 8 ? 8 : 16);
   }
   return cudaGetLastError();
@@ -1014,12 +1025,12 @@ cudaError_t product_b(const Plan& p, const Params& q, const ChiChunk& c, const v
 
 template <typename T, int NI>
 void run_con(const Plan& p, const Params& q, const ChiChunk& c, const void* F, double2* out,
-             int i0, double scale, cudaStream_t s) {
+             double2* copy, int i0, double scale, cudaStream_t s) {
   if (c.nitems > 0)
     con_kernel<T, NI><<<dim3((c.nitems + 7) / 8, p.nk), 256, 0, s>>>(
       q, (const cplx_t<T>*)p.chi->chi, (const cplx_t<T>*)F, c.item0, c.nitems, i0);
   sum_kernel<NI><<<dim3(q.nslots / kPad, p.nk), 2 * kPad * NI * kSumSplit, 0, s>>>(
-      q, out, c.row_of0, c.nitems, i0, scale, c.b0 > 0 ? 1 : 0);
+      q, out, copy, c.row_of0, c.nitems, i0, scale, c.b0 > 0 ? 1 : 0);
 }
 
 // orbitals per pass of con_kernel
@@ -1027,13 +1038,13 @@ inline int con_width(int left, bool fp64) { return (fp64 || left <= 4) ? 4 : 8; 
 
 template <typename T>
 cudaError_t product_e(const Plan& p, const Params& q, const ChiChunk& c, const void* F,
-                      double2* out, double scale, cudaStream_t s) {
+                      double2* out, double2* copy, double scale, cudaStream_t s) {
   for (int i0 = 0; i0 < p.nocc;) {
     const int ni = con_width(p.nocc - i0, sizeof(T) == 8);
     if (ni == 4) {
-      run_con<T, 4>(p, q, c, F, out, i0, scale, s);
+      run_con<T, 4>(p, q, c, F, out, copy, i0, scale, s);
     } else if constexpr (sizeof(T) == 4) {
-      run_con<T, 8>(p, q, c, F, out, i0, scale, s);
+      run_con<T, 8>(p, q, c, F, out, copy, i0, scale, s);
     }
     i0 += ni;
   }
@@ -1057,25 +1068,25 @@ cudaError_t launch_slot_c(const Plan& p, const double2* X, void* out, double fac
 
 template <typename T>
 cudaError_t launch_orbitals(const Plan& p, int nsets, const void* const* cs, void* const* out,
-                            cudaStream_t s) {
+                            bool periodic, cudaStream_t s) {
   const chi::Params q = chi::params(p);
   for (const ChiChunk& c : p.chi->chunks) {
     cudaError_t e = chi::fill<T>(p, q, c, s);
     for (int i = 0; i < nsets && e == cudaSuccess; ++i)
-      e = chi::product_b<T>(p, q, c, cs[i], out[i], s);
+      e = chi::product_b<T>(p, q, c, cs[i], out[i], periodic, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
 template <typename T>
-cudaError_t launch_contract_field(const Plan& p, const void* F, double2* out, double scale,
-                                  cudaStream_t s) {
+cudaError_t launch_contract_field(const Plan& p, const void* F, double2* out, double2* copy,
+                                  double scale, cudaStream_t s) {
   const chi::Params q = chi::params(p);
   for (const ChiChunk& c : p.chi->chunks) {
     // one chunk: the buffer still holds chi from the orbitals of this call
     cudaError_t e = p.chi->chunks.size() > 1 ? chi::fill<T>(p, q, c, s) : cudaSuccess;
-    if (e == cudaSuccess) e = chi::product_e<T>(p, q, c, F, out, scale, s);
+    if (e == cudaSuccess) e = chi::product_e<T>(p, q, c, F, out, copy, scale, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1391,12 +1402,12 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
 template cudaError_t launch_slot_c<float>(const Plan&, const double2*, void*, double, cudaStream_t);
 template cudaError_t launch_slot_c<double>(const Plan&, const double2*, void*, double, cudaStream_t);
 template cudaError_t launch_orbitals<float>(const Plan&, int, const void* const*, void* const*,
-                                            cudaStream_t);
+                                            bool, cudaStream_t);
 template cudaError_t launch_orbitals<double>(const Plan&, int, const void* const*, void* const*,
-                                             cudaStream_t);
-template cudaError_t launch_contract_field<float>(const Plan&, const void*, double2*, double,
-                                                  cudaStream_t);
-template cudaError_t launch_contract_field<double>(const Plan&, const void*, double2*, double,
-                                                   cudaStream_t);
+                                             bool, cudaStream_t);
+template cudaError_t launch_contract_field<float>(const Plan&, const void*, double2*, double2*,
+                                                  double, cudaStream_t);
+template cudaError_t launch_contract_field<double>(const Plan&, const void*, double2*, double2*,
+                                                   double, cudaStream_t);
 
 }  // namespace occri

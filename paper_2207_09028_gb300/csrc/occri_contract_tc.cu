@@ -245,8 +245,9 @@ con_tc_kernel(chi::Params p, const float2* __restrict__ chi, const float2* __res
     if constexpr (NI == 8) load8(st);
   };
   fetch(0);
+  int st = 0;   // stages issued
 #pragma unroll 1
-  for (int st = 0; st < nst; ++st) {
+  for (; st < nst; ++st) {
     if (st > 0) {
       ok = tc::mbar_wait(tc::smem_u32(&bar.done), (unsigned)((st - 1) & 1), wait_ns);
       if (ok) take();
@@ -272,11 +273,10 @@ con_tc_kernel(chi::Params p, const float2* __restrict__ chi, const float2* __res
     }
     if (st + 1 < nst) fetch(st + 1);
   }
-  if (ok) {
-    ok = tc::mbar_wait(tc::smem_u32(&bar.done), (unsigned)((nst - 1) & 1), wait_ns);
-    if (ok) take();
-  }
-  if (!ok && lane == 0) fail(status);
+  // the last stage issued (after a timeout too: nothing is in flight when the CTA leaves)
+  const bool last = tc::mbar_wait(tc::smem_u32(&bar.done), (unsigned)((st - 1) & 1), wait_ns);
+  if (ok && last) take();
+  if (!ok || !last) fail(status);
   // part[k][item][row][column]
   double* o = p.part + ((size_t)k * nitems + w) * kM * N +
               (size_t)(32 * (warp & 3) + lane) * N + NI * (warp >> 2);
@@ -292,7 +292,7 @@ con_tc_kernel(chi::Params p, const float2* __restrict__ chi, const float2* __res
 template <int N>
 __global__ void __launch_bounds__(256)
 sum_tc_kernel(chi::Params p, const unsigned* __restrict__ colmax, double2* __restrict__ kc,
-              int row_of0, int nitems, double scale, int add) {
+              double2* __restrict__ copy, int row_of0, int nitems, double scale, int add) {
   constexpr int NI = N / 2;
   const int slot = blockIdx.x * 8 + (threadIdx.x >> 5), k = blockIdx.y, nocc = p.a.nocc;
   if (slot >= p.nslots) return;
@@ -315,16 +315,19 @@ sum_tc_kernel(chi::Params p, const unsigned* __restrict__ colmax, double2* __res
     }
     const double f = scale * p.ao_norm[mu] / (double)p.row_scale[slot] *
                      ldexp(1.0, col_exp(colmax[(size_t)k * nocc + i]) - 13);
-    double* dst = reinterpret_cast<double*>(kc + ((size_t)k * p.a.nao + mu) * nocc + i);
-    dst[im] = add ? dst[im] + f * t : f * t;
+    const size_t at = 2 * (((size_t)k * p.a.nao + mu) * nocc + i) + im;
+    double* dst = reinterpret_cast<double*>(kc) + at;
+    t = add ? *dst + f * t : f * t;
+    *dst = t;
+    if (copy) reinterpret_cast<double*>(copy)[at] = t;
   }
 }
 
 constexpr int width(int nocc) { return nocc <= 8 ? 16 : (nocc <= 16 ? 32 : 64); }
 
 template <int N>
-cudaError_t run(const Plan& p, const chi::Params& q, const ChiChunk& c, double scale,
-                cudaStream_t s, LaunchHook* hook) {
+cudaError_t run(const Plan& p, const chi::Params& q, const ChiChunk& c, double2* copy,
+                double scale, cudaStream_t s, LaunchHook* hook) {
   constexpr size_t smem = 2 * (size_t)(op_bytes(kM) + op_bytes(N)) + sizeof(Smem);
   static_assert(smem <= 75 * 1024, "three CTAs per SM");
   static DeviceCache attr;
@@ -338,7 +341,7 @@ cudaError_t run(const Plan& p, const chi::Params& q, const ChiChunk& c, double s
         q, (const float2*)p.chi->chi, (const float2*)p.Y, p.colmax, c.item0, c.nitems, p.status,
         p.wait_ns);
   if (hook) hook->after();
-  sum_tc_kernel<N><<<dim3((q.nslots + 7) / 8, p.nk), 256, 0, s>>>(q, p.colmax, p.kc, c.row_of0,
+  sum_tc_kernel<N><<<dim3((q.nslots + 7) / 8, p.nk), 256, 0, s>>>(q, p.colmax, p.kc, copy, c.row_of0,
                                                                   c.nitems, scale,
                                                                   c.b0 > 0 ? 1 : 0);
   return cudaGetLastError();
@@ -354,7 +357,7 @@ int tc_plan_launches(const Plan& p) {
   return 1 + 2 * nc + (nc > 1 ? nc : 0);
 }
 
-cudaError_t launch_contract_tc(const Plan& p, cudaStream_t s, LaunchHook* hook) {
+cudaError_t launch_contract_tc(const Plan& p, double2* copy, cudaStream_t s, LaunchHook* hook) {
   using namespace tcc;
   const chi::Params q = chi::params(p);
   // Y carries N_g/(4 pi) (see PairParams), hence -Omega 4 pi / (N_k N_g^2)
@@ -370,9 +373,9 @@ cudaError_t launch_contract_tc(const Plan& p, cudaStream_t s, LaunchHook* hook) 
     e = p.chi->chunks.size() > 1 ? chi::fill<float>(p, q, c, s) : cudaGetLastError();
     if (e != cudaSuccess) return e;
     switch (width(p.nocc)) {
-      case 16: e = run<16>(p, q, c, scale, s, hook); break;
-      case 32: e = run<32>(p, q, c, scale, s, hook); break;
-      default: e = run<64>(p, q, c, scale, s, hook); break;
+      case 16: e = run<16>(p, q, c, copy, scale, s, hook); break;
+      case 32: e = run<32>(p, q, c, copy, scale, s, hook); break;
+      default: e = run<64>(p, q, c, copy, scale, s, hook); break;
     }
     if (e != cudaSuccess) return e;
   }

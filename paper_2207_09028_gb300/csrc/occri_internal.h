@@ -200,7 +200,10 @@ struct Plan {
   double2* mmat = nullptr;   // [nk][nocc][nocc]
   double* ek = nullptr;      // [nk]
   double* dacc = nullptr;    // [2] scratch accumulators (d E/d omega)
-  int* status = nullptr;     // [2]: first device error code, k index
+  int* status = nullptr;     // [2]: first device error code, k index (device address of status_h)
+  int* status_h = nullptr;   // mapped host memory
+  void* bands = nullptr;     // conduction-band columns: both builds' K_{mu i} and the bands
+  size_t bands_bytes = 0;
   bool have_kc = false;
   ChiTables* chi = nullptr;  // Bloch AOs of the plan
   unsigned* colmax = nullptr;   // OCCRI_MIXED_TC: [nk][nocc] largest |Re Y| + |Im Y|, float bits
@@ -262,19 +265,21 @@ int chi_launches(const Plan& p, bool contract);   // kernels of the orbitals or 
 template <typename T>
 cudaError_t launch_slot_c(const Plan& p, const double2* X, void* out, double factor,
                           cudaStream_t s);
-// Orbital fields out[i] of nsets coefficient tables cs[i].
+// Orbital fields out[i] of nsets coefficient tables cs[i], or their periodic parts e^{-ik.r} psi.
 template <typename T>
 cudaError_t launch_orbitals(const Plan& p, int nsets, const void* const* cs, void* const* out,
-                            cudaStream_t s);
+                            bool periodic, cudaStream_t s);
 // out[k][mu][i] = scale N_mu sum_r conj(chi) F_ik for an orbital-shaped field F; follows
-// launch_orbitals in the same call (the chi buffer may still hold the AOs).
+// launch_orbitals in the same call (the chi buffer may still hold the AOs). copy (may be null)
+// receives the same values.
 template <typename T>
-cudaError_t launch_contract_field(const Plan& p, const void* F, double2* out, double scale,
-                                  cudaStream_t s);
-// F[k][i][.] *= e^{sign i k.r} over the orbital-shaped field F (psi -> periodic parts
-// with sign -1 before the pair passes, accumulated periodic parts -> Y with +1 after).
+cudaError_t launch_contract_field(const Plan& p, const void* F, double2* out, double2* copy,
+                                  double scale, cudaStream_t s);
+// F[k][i][.] = (F + a + b) e^{i k.r} over the orbital-shaped field F (accumulated periodic parts
+// -> Y; a and b, either may be null, are the other streams' accumulators).
 template <typename T>
-cudaError_t launch_phase_fields(const Plan& p, void* F, int sign, cudaStream_t s);
+cudaError_t launch_phase_fields(const Plan& p, void* F, const void* a, const void* b,
+                                cudaStream_t s);
 // Pair-wave launches over unordered pairs: diag = 1 is the wave (k, k) with fields
 // i <= j; diag = 0 covers k' in [kp0, kp0 + nkp), all kp0 > k, with every (i, j).
 // S is the wave's scratch and Y the accumulator the wave adds into (the plan's Y, or the
@@ -338,7 +343,8 @@ struct LaunchHook {
   virtual void after() = 0;
   virtual ~LaunchHook() = default;
 };
-cudaError_t launch_contract_tc(const Plan& p, cudaStream_t s, LaunchHook* hook = nullptr);
+cudaError_t launch_contract_tc(const Plan& p, double2* copy, cudaStream_t s,
+                               LaunchHook* hook = nullptr);
 
 // Launch settings derived once per kernel instantiation and device (function attributes,
 // resident-slot counts): each entry is filled under a lock the first time a plan on that

@@ -58,11 +58,17 @@ template <typename T> constexpr bool pair_lanes() { return sizeof(T) == 4; }
 template <typename T> constexpr int threads_for(int n) {
   return line_split(n) == 1 ? round32(n) : (pair_lanes<T>() ? round32(2 * n) : 2 * round32(n));
 }
-// resident CTAs per SM requested from the register allocator: 512 threads per SM in FP32 (768 in
-// pass A, 80 registers), but for odd edges, whose threads hold a whole line
+// Resident CTAs per SM requested from the register allocator. FP32: 640 threads per SM where
+// their planes and kernel values leave 58 KB and more of the SM's memory to the L1 cache
+// (pass B at 48^3 15.3 -> 14.1 ms per 32,896 fields), else 512 (at 60^3 five CTAs of 128
+// threads took 134 ms per 131,328 fields, four 114); 768 in pass A (80 registers). Odd edges,
+// whose threads hold a whole line, and FP64 run fewer.
+constexpr int plane_smem(int n, int elem) { return n * pitch(n) * elem + n * n * elem / 2; }
 template <typename T> constexpr int min_blocks(int n) {
-  return sizeof(T) > 4 ? (n <= 32 ? 4 : 2)
-                       : (line_split(n) == 2 ? 512 / threads_for<T>(n) : (n <= 32 ? 8 : 4));
+  if (sizeof(T) > 4) return n <= 32 ? 4 : 2;
+  if (line_split(n) == 1) return n <= 32 ? 8 : 4;
+  const int more = 640 / threads_for<T>(n);
+  return more * plane_smem(n, 8) <= 170 * 1024 ? more : 512 / threads_for<T>(n);
 }
 template <typename T> constexpr int min_blocks_a(int n) {
   return sizeof(T) > 4 ? min_blocks<T>(n)
