@@ -35,6 +35,7 @@ namespace chi {
 using ao::Disp;
 
 constexpr int kWarps = 8;       // most warps of a chi_kernel CTA
+constexpr int kFoldWarps = 4;   // warps of its CTAs where no class sums cross warps
 constexpr int kFold = 8;        // most classes of a mesh whose shells take a warp each
 constexpr int kRows = 7 * kFold;   // entry rows of a warp (a value per lane each)
 constexpr int kCols = 10;       // AOs that the CTA takes together (wide shells)
@@ -186,7 +187,8 @@ __device__ __forceinline__ void narrow_shell(const Params& p, const ChiShell& sh
 // A shell on a mesh of at most kFold classes, one warp: class sums in the warp's rows (row
 // class NM + m; a lane reads back only what it wrote), then chi of every k. Where every axis
 // has one or two points the phases are signs and chi is real: sums and differences over the axes
-// (a Walsh-Hadamard transform); else the classes' phases as in narrow_shell.
+// (a Walsh-Hadamard transform), and the buffer holds real values; else the classes' phases as in
+// narrow_shell.
 template <typename T, int L, int KT, typename GetRec>
 __device__ __forceinline__ void fold_shell(const Params& p, const ChiShell& sh, const Disp<T>& d,
                                            int np, const GetRec& rec, T* ent, int* ecls,
@@ -231,7 +233,7 @@ __device__ __forceinline__ void fold_shell(const Params& p, const ChiShell& sh, 
       }
 #pragma unroll
       for (int c = 0; c < kFold; ++c)
-        if (off[c] >= 0) out[off[c] + 32 * m] = cplx_t<T>{f[c], T(0)};
+        if (off[c] >= 0) reinterpret_cast<T*>(out)[off[c] + 32 * m] = f[c];
     }
     return;
   }
@@ -472,8 +474,11 @@ __device__ __forceinline__ void class_sums(const ChiShell* shells, const int* np
 // What bounds it: the stores at many k-points, the Gaussians at few. Phases times class sums
 // (a dense product over classes) instead of the transform took 43 ms per pass at 64 k, 350
 // AOs, 60^3: each broadcast phase costs the load path as much as a full vector.
-template <typename T, int KS, int KL>
-__global__ void __launch_bounds__(32 * kWarps, 2)
+// FOLD: meshes of up to kFold classes (fold_shell alone, CTAs of kFoldWarps: with fewer registers
+// more of them fit; at six CTAs the phases' kernel spills and is 3 % slower).
+template <typename T, int KS, int KL, bool FOLD>
+__global__ void __launch_bounds__(32 * (FOLD ? kFoldWarps : kWarps),
+                                  !FOLD ? 2 : (sizeof(T) == 8 ? 4 : (KS == 1 ? 6 : 5)))
 chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ T edge[kWarps][kCols][32];
@@ -512,13 +517,16 @@ chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
   ao::load_disp(p.a, a, n, &d);
   const int* aoff = p.aoff + (size_t)blk * (p.a.natm + 1);
   const int kstride = 32 * aoff[p.a.natm];
-  cplx_t<T>* base = chi + (size_t)(p.boff[blk] * p.a.nk + aoff[a]) * 32;
+  const size_t base0 = (size_t)(p.boff[blk] * p.a.nk + aoff[a]) * 32;
+  // (real values: the same offsets in T)
+  cplx_t<T>* base = p.signs ? reinterpret_cast<cplx_t<T>*>(reinterpret_cast<T*>(chi) + base0)
+                            : chi + base0;
   auto rec = [&](int j) -> Rec<T> { return in_smem ? recs[j] : load_rec<T>(p, list0, cls, j); };
   auto order = [&](int t) -> int { return in_smem ? ord[t] : p.order[list0 + t]; };
   __shared__ ChiShell gsh[8];
   __shared__ int gnp[8], gidx[8], gslot[kCols], gns, gm0, gnm, gnext, gl;
   int wide = 0;   // wide shells (a prefix)
-  if (p.ncol > 0) {
+  if constexpr (!FOLD) if (p.ncol > 0) {
     while (wide < nact && lnp[wide] >> 2 >= kWide) ++wide;
     // Groups of one angular momentum, in turn over the CTAs of the (block, atom)
     const int t0 = n_all * warp / nw, t1 = n_all * (warp + 1) / nw;
@@ -594,28 +602,32 @@ chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
   for (s += warp + nw * blockIdx.z; s < nact; s += nw * gridDim.z) {
     const ChiShell sh = p.shells[s0 + s];
     const int np = pre[sh.orig - s0];
-    cplx_t<T>* out = base + 32 * (size_t)sh.slot;
-    if (p.ncls <= kFold) {
+    cplx_t<T>* out = p.signs ? reinterpret_cast<cplx_t<T>*>(reinterpret_cast<T*>(base) + 32 * sh.slot)
+                             : base + 32 * (size_t)sh.slot;
+    if constexpr (FOLD) {
       switch (sh.l) {
         case 0: fold_shell<T, 0, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
         case 1: fold_shell<T, 1, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
         case 2: fold_shell<T, 2, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
         default: fold_shell<T, 3, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
       }
-      continue;
-    }
-    switch (sh.l) {
-      case 0: narrow_shell<T, 0, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
-      case 1: narrow_shell<T, 1, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
-      case 2: narrow_shell<T, 2, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
-      default: narrow_shell<T, 3, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+    } else {
+      switch (sh.l) {
+        case 0: narrow_shell<T, 0, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+        case 1: narrow_shell<T, 1, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+        case 2: narrow_shell<T, 2, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+        default: narrow_shell<T, 3, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+      }
     }
   }
   if (blockIdx.z == 0 && warp == nw - 1) {   // padding slots of the atom's last group
     const ChiShell& last = p.shells[s0 + nact - 1];
     for (int x = last.slot + 2 * last.l + 1; x < aoff[a + 1] - aoff[a]; ++x)
-      for (int k = 0; k < p.a.nk; ++k)
-        base[(size_t)k * kstride + 32 * x + lane] = cplx_t<T>{T(0), T(0)};
+      for (int k = 0; k < p.a.nk; ++k) {
+        const size_t o = (size_t)k * kstride + 32 * x + lane;
+        if (p.signs) reinterpret_cast<T*>(base)[o] = T(0);
+        else base[o] = cplx_t<T>{T(0), T(0)};
+      }
   }
 }
 
@@ -652,6 +664,21 @@ __device__ __forceinline__ double2 stream_ld(const double2* p) {
   return v;
 }
 
+__device__ __forceinline__ float stream_ld(const float* p) {
+  float v;
+  asm volatile("ld.global.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double stream_ld(const double* p) {
+  double v;
+  asm volatile("ld.global.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+
+// chi as the products read it: real on meshes whose phases are signs (half the bytes and half
+// the products)
+template <typename T, bool REAL> using chi_t = std::conditional_t<REAL, T, cplx_t<T>>;
+
 // t += c x; in FP32 the coefficient is a hi/lo pair
 __device__ __forceinline__ void cmac(const double2& c, const double2& x, double2& t) {
   t.x += c.x * x.x - c.y * x.y;
@@ -662,22 +689,32 @@ __device__ __forceinline__ void cmac(const float4& c, const float2& x, float2& t
   t.y = fmaf(c.x, x.y, fmaf(c.y, x.x, fmaf(c.z, x.y, fmaf(c.w, x.x, t.y))));
 }
 
+__device__ __forceinline__ void cmac(const double2& c, double x, double2& t) {
+  t.x += c.x * x;
+  t.y += c.y * x;
+}
+__device__ __forceinline__ void cmac(const float4& c, float x, float2& t) {
+  t.x = fmaf(c.x, x, fmaf(c.z, x, t.x));
+  t.y = fmaf(c.y, x, fmaf(c.w, x, t.y));
+}
+
 // psi_ik at NB consecutive blocks per warp: kPad AOs are summed on their own before they join
 // the orbital's sum, so that few roundings happen at its full size. In FP32 a coefficient,
 // the same for every lane, costs the load path as much as a value per lane: up to four
 // orbitals take two blocks (64 k, 200 AOs, 48^3, nocc 4: orbitals and AOs 5.5 -> 5.0 ms); with
 // eight the wider tile's registers cost what it saves (350 AOs, 8 k, 60^3: 1.52 against 1.50 ms).
 template <typename T, int NI> constexpr int orb_blocks() { return sizeof(T) == 4 && NI == 4 ? 2 : 1; }
-template <typename T, int NI, int NB>
+template <typename T, int NI, int NB, bool REAL>
 __global__ void __launch_bounds__(128)
-orb_kernel(Params p, const cplx_t<T>* __restrict__ chi, const typename CsT<T>::type* __restrict__ cs,
+orb_kernel(Params p, const chi_t<T, REAL>* __restrict__ chi, const typename CsT<T>::type* __restrict__ cs,
            cplx_t<T>* __restrict__ psi, int blk0, int nb, int i0, int periodic) {
   const int w = NB * (blockIdx.x * 4 + (threadIdx.x >> 5));
   if (w >= nb) return;
   const int k = blockIdx.y, lane = threadIdx.x & 31;
   const int nocc = p.a.nocc, blk = blk0 + w, nlast = min(NB, nb - w) - 1;
+  using X = chi_t<T, REAL>;
   const int* aoff[NB];
-  const cplx_t<T>* x0[NB];
+  const X* x0[NB];
 #pragma unroll
   for (int b = 0; b < NB; ++b) {   // past the last block: the last one again, not stored
     const int q = blk + min(b, nlast);
@@ -690,10 +727,10 @@ orb_kernel(Params p, const cplx_t<T>* __restrict__ chi, const typename CsT<T>::t
 #pragma unroll
     for (int i = 0; i < NI; ++i) acc[b][i] = cplx_t<T>{T(0), T(0)};
   // slots [s, s + kPad) of an atom for the blocks [b0, b1) of the warp
-  auto group = [&](const cplx_t<T>* (&xa)[NB], const typename CsT<T>::type* ca, int s, auto B0,
+  auto group = [&](const X* (&xa)[NB], const typename CsT<T>::type* ca, int s, auto B0,
                    auto B1) {
     constexpr int b0 = decltype(B0)::value, b1 = decltype(B1)::value;
-    cplx_t<T> x[NB][kPad];
+    X x[NB][kPad];
 #pragma unroll
     for (int b = b0; b < b1; ++b)
 #pragma unroll
@@ -722,7 +759,7 @@ orb_kernel(Params p, const cplx_t<T>* __restrict__ chi, const typename CsT<T>::t
   using All = std::integral_constant<int, NB>;
   for (int a = 0; a < p.a.natm; ++a) {
     int n[NB], both = 1 << 30;
-    const cplx_t<T>* xa[NB];
+    const X* xa[NB];
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       n[b] = aoff[b][a + 1] - aoff[b][a];
@@ -812,9 +849,9 @@ __device__ __forceinline__ void halve_lanes(T (&v)[NV], double (&out)[NV / 32], 
 // they reach (work items, made with the plan), sums per lane in the working precision, then
 // over the lanes in 64 bits. sum_kernel adds the items in a fixed order, so that the result
 // does not depend on the order in which they ran.
-template <typename T, int NI>
+template <typename T, int NI, bool REAL>
 __global__ void __launch_bounds__(256, 2)
-con_kernel(Params p, const cplx_t<T>* __restrict__ chi, const cplx_t<T>* __restrict__ F,
+con_kernel(Params p, const chi_t<T, REAL>* __restrict__ chi, const cplx_t<T>* __restrict__ F,
            int item0, int nitems, int i0) {
   const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (w >= nitems) return;
@@ -830,9 +867,9 @@ con_kernel(Params p, const cplx_t<T>* __restrict__ chi, const cplx_t<T>* __restr
   for (int b = 0; b < it.w; ++b) {
     const int blk = p.border[it.z + b];
     const int* aoff = p.aoff + (size_t)blk * (p.a.natm + 1);
-    const cplx_t<T>* x0 = chi + ((size_t)p.boff[blk] * p.a.nk + (size_t)k * aoff[p.a.natm] +
-                                 aoff[it.x] + it.y) * 32 + lane;
-    cplx_t<T> x[kPad];
+    const chi_t<T, REAL>* x0 = chi + ((size_t)p.boff[blk] * p.a.nk + (size_t)k * aoff[p.a.natm] +
+                                      aoff[it.x] + it.y) * 32 + lane;
+    chi_t<T, REAL> x[kPad];
 #pragma unroll
     for (int u = 0; u < kPad; ++u) x[u] = stream_ld(x0 + 32 * u);
     bool valid;
@@ -846,8 +883,13 @@ con_kernel(Params p, const cplx_t<T>* __restrict__ chi, const cplx_t<T>* __restr
       for (int u = 0; u < kPad; ++u) {   // conj(x) y
         T& re = acc[2 * (u * NI + i)];
         T& im = acc[2 * (u * NI + i) + 1];
-        re += x[u].x * y.x + x[u].y * y.y;
-        im += x[u].x * y.y - x[u].y * y.x;
+        if constexpr (REAL) {
+          re += x[u] * y.x;
+          im += x[u] * y.y;
+        } else {
+          re += x[u].x * y.x + x[u].y * y.y;
+          im += x[u].x * y.y - x[u].y * y.x;
+        }
       }
     }
   }
@@ -962,8 +1004,8 @@ template <typename T> size_t chi_smem(int buf_rows, int lsm, int nsa) {
          (size_t)lsm * (sizeof(Rec<T>) + sizeof(unsigned short));
 }
 
-template <typename T, int KS, int KL>
-cudaError_t run_chi(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t s) {
+template <typename T, int KS, int KL, bool FOLD>
+cudaError_t run_chi_as(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t s) {
   const size_t sm = chi_smem<T>(q.buf_rows, q.lsm, q.a.nsa);
   static std::mutex mu;
   static size_t have[kMaxDevices] = {};
@@ -972,14 +1014,19 @@ cudaError_t run_chi(const Plan& p, const Params& q, const ChiChunk& c, cudaStrea
     size_t& h = have[(p.device >= 0 && p.device < kMaxDevices) ? p.device : 0];
     if (sm > h) {
       const cudaError_t e = cudaFuncSetAttribute(
-          chi_kernel<T, KS, KL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+          chi_kernel<T, KS, KL, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
       h = sm;
     }
   }
-  chi_kernel<T, KS, KL><<<dim3(c.b1 - c.b0, p.natm, q.parts), 32 * q.warps, sm, s>>>(
+  chi_kernel<T, KS, KL, FOLD><<<dim3(c.b1 - c.b0, p.natm, q.parts), 32 * q.warps, sm, s>>>(
       q, (cplx_t<T>*)p.chi->chi, c.b0);
   return cudaGetLastError();
+}
+template <typename T, int KS, int KL>
+cudaError_t run_chi(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t s) {
+  return q.ncls <= kFold ? run_chi_as<T, KS, KL, true>(p, q, c, s)
+                         : run_chi_as<T, KS, KL, false>(p, q, c, s);
 }
 
 // k-points per pass over a shell's entries: as many as the registers hold, fewer for meshes
@@ -995,24 +1042,32 @@ cudaError_t fill(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t
   }
 }
 
-template <typename T, int NI>
-void run_orb(const Params& q, const cplx_t<T>* chi, const void* cs, void* out, const ChiChunk& c,
-             int i0, int periodic, cudaStream_t s) {
+template <typename T, int NI, bool REAL>
+void run_orb_as(const Params& q, const void* chi, const void* cs, void* out, const ChiChunk& c,
+                int i0, int periodic, cudaStream_t s) {
   // one block per warp where two would leave SMs without work
   const int nb = c.b1 - c.b0;
   constexpr int NB = orb_blocks<T, NI>();
+  const auto* x = (const chi_t<T, REAL>*)chi;
+  const auto* cf = (const typename CsT<T>::type*)cs;
   if (NB == 1 || (long long)nb * q.a.nk < 152 * 64)
-    orb_kernel<T, NI, 1><<<dim3((nb + 3) / 4, q.a.nk), 128, 0, s>>>(
-        q, chi, (const typename CsT<T>::type*)cs, (cplx_t<T>*)out, c.b0, nb, i0, periodic);
+    orb_kernel<T, NI, 1, REAL><<<dim3((nb + 3) / 4, q.a.nk), 128, 0, s>>>(
+        q, x, cf, (cplx_t<T>*)out, c.b0, nb, i0, periodic);
   else
-    orb_kernel<T, NI, NB><<<dim3((nb + 7) / 8, q.a.nk), 128, 0, s>>>(
-        q, chi, (const typename CsT<T>::type*)cs, (cplx_t<T>*)out, c.b0, nb, i0, periodic);
+    orb_kernel<T, NI, NB, REAL><<<dim3((nb + 7) / 8, q.a.nk), 128, 0, s>>>(
+        q, x, cf, (cplx_t<T>*)out, c.b0, nb, i0, periodic);
+}
+template <typename T, int NI>
+void run_orb(const Params& q, const void* chi, const void* cs, void* out, const ChiChunk& c,
+             int i0, int periodic, cudaStream_t s) {
+  if (q.signs) run_orb_as<T, NI, true>(q, chi, cs, out, c, i0, periodic, s);
+  else run_orb_as<T, NI, false>(q, chi, cs, out, c, i0, periodic, s);
 }
 
 template <typename T>
 cudaError_t product_b(const Plan& p, const Params& q, const ChiChunk& c, const void* cs,
                       void* out, int periodic, cudaStream_t s) {
-  const cplx_t<T>* x = (const cplx_t<T>*)p.chi->chi;
+  const void* x = p.chi->chi;
   for (int i0 = 0; i0 < p.nocc;) {
     const int left = p.nocc - i0;
     if (left <= 4) run_orb<T, 4>(q, x, cs, out, c, i0, periodic, s);
@@ -1026,9 +1081,13 @@ cudaError_t product_b(const Plan& p, const Params& q, const ChiChunk& c, const v
 template <typename T, int NI>
 void run_con(const Plan& p, const Params& q, const ChiChunk& c, const void* F, double2* out,
              double2* copy, int i0, double scale, cudaStream_t s) {
-  if (c.nitems > 0)
-    con_kernel<T, NI><<<dim3((c.nitems + 7) / 8, p.nk), 256, 0, s>>>(
-      q, (const cplx_t<T>*)p.chi->chi, (const cplx_t<T>*)F, c.item0, c.nitems, i0);
+  const dim3 grid((c.nitems + 7) / 8, p.nk);
+  if (c.nitems > 0 && q.signs)
+    con_kernel<T, NI, true><<<grid, 256, 0, s>>>(q, (const T*)p.chi->chi, (const cplx_t<T>*)F,
+                                                 c.item0, c.nitems, i0);
+  else if (c.nitems > 0)
+    con_kernel<T, NI, false><<<grid, 256, 0, s>>>(q, (const cplx_t<T>*)p.chi->chi,
+                                                  (const cplx_t<T>*)F, c.item0, c.nitems, i0);
   sum_kernel<NI><<<dim3(q.nslots / kPad, p.nk), 2 * kPad * NI * kSumSplit, 0, s>>>(
       q, out, copy, c.row_of0, c.nitems, i0, scale, c.b0 > 0 ? 1 : 0);
 }
@@ -1245,8 +1304,20 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
       phase[c * t->nkp + k] = make_double2(std::cos(ang), std::sin(ang));
     }
   }
+  // Wide shells go through the transform over classes where the mesh is (nearly) full, its
+  // k-points are distinct and its lengths are compiled; columns as the shared memory allows.
+  std::vector<int> kidx(identity ? Dc : 1, -1);
+  bool dft = identity && Dc <= 4 * p->nk;
+  for (int d = 0; d < 3; ++d) dft = dft && (p->D[d] <= 6 || p->D[d] == 8);
+  for (int k = 0; k < p->nk && dft; ++k) {
+    const int r = (p->kint_h[3 * k] * p->D[1] + p->kint_h[3 * k + 1]) * p->D[2] + p->kint_h[3 * k + 2];
+    if (kidx[r] >= 0) dft = false;
+    kidx[r] = k;
+  }
+  t->signs = dft && Dc <= chi::kFold && p->D[0] <= 2 && p->D[1] <= 2 && p->D[2] <= 2;
+  dft = dft && Dc > chi::kFold;   // up to kFold classes every shell takes one warp (fold_shell)
   // chunks of blocks, offsets, and the contraction's items
-  const size_t csz = fp64 ? sizeof(double2) : sizeof(float2);
+  const size_t csz = (fp64 ? sizeof(double) : sizeof(float)) * (t->signs ? 1 : 2);
   const size_t slot_bytes = csz * 32 * (size_t)p->nk;
   size_t all = 0, widest = 0;
   for (int b = 0; b < nblk; ++b) {
@@ -1323,18 +1394,6 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
                               : 2 * (size_t)chi::kPad * chi::con_width(p->nocc, fp64);
     t->part_bytes = std::max(t->part_bytes, sizeof(double) * values * (size_t)c.nitems * p->nk);
   }
-  // Wide shells go through the transform over classes where the mesh is (nearly) full, its
-  // k-points are distinct and its lengths are compiled; columns as the shared memory allows.
-  std::vector<int> kidx(identity ? Dc : 1, -1);
-  bool dft = identity && Dc <= 4 * p->nk;
-  for (int d = 0; d < 3; ++d) dft = dft && (p->D[d] <= 6 || p->D[d] == 8);
-  for (int k = 0; k < p->nk && dft; ++k) {
-    const int r = (p->kint_h[3 * k] * p->D[1] + p->kint_h[3 * k + 1]) * p->D[2] + p->kint_h[3 * k + 2];
-    if (kidx[r] >= 0) dft = false;
-    kidx[r] = k;
-  }
-  t->signs = dft && Dc <= chi::kFold && p->D[0] <= 2 && p->D[1] <= 2 && p->D[2] <= 2;
-  dft = dft && Dc > chi::kFold;   // up to kFold classes every shell takes one warp (fold_shell)
   const int row_bytes = 32 * (fp64 ? 8 : 4);
   t->col_rows = 2 * (p->D[0] / 2 + 1) * p->D[1] * p->D[2];
   // 88 KB of columns leave room for two CTAs per SM; where that is under four AOs, one CTA
@@ -1342,7 +1401,7 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   const long long cols = (88 * 1024 / col_bytes >= 4 ? 88 : 176) * 1024 / col_bytes;
   t->ncol = dft ? (int)std::min<long long>(chi::kCols, cols) : 0;
   // without the transform nothing crosses warps: smaller CTAs
-  t->warps = t->ncol > 0 ? chi::kWarps : 4;
+  t->warps = t->ncol > 0 ? chi::kWarps : chi::kFoldWarps;
   t->buf_rows = std::max(t->ncol * t->col_rows, t->warps * chi::kRows);
   const size_t need = fp64 ? chi::chi_smem<double>(t->buf_rows, lmax, nsa)
                            : chi::chi_smem<float>(t->buf_rows, lmax, nsa);

@@ -52,7 +52,7 @@ struct ChiTables {
   double* part = nullptr;         // [k][item][values] sums of the items
   float* row_scale = nullptr;     // [nslots] tensor-core contraction: FP16 scale of a slot
   size_t part_bytes = 0;
-  void* chi = nullptr;            // [block][k][slot][32 points]
+  void* chi = nullptr;            // [block][k][slot][32 points], complex, or real with signs
   void* arena = nullptr;          // the one allocation behind all of these
 };
 

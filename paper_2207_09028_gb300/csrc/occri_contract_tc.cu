@@ -89,9 +89,9 @@ struct Smem {
 };
 
 // One work item per CTA: kTcTile slots of an atom over a run of blocks, at one k.
-template <int N>
+template <int N, bool REAL>
 __global__ void __launch_bounds__(kThreads, N == 64 ? 2 : 3)
-con_tc_kernel(chi::Params p, const float2* __restrict__ chi, const float2* __restrict__ Y,
+con_tc_kernel(chi::Params p, const void* __restrict__ chi, const float2* __restrict__ Y,
               const unsigned* __restrict__ colmax, int item0, int nitems, int* status,
               long long wait_ns) {
   constexpr int NI = N / 2;                       // orbitals, padded
@@ -130,13 +130,20 @@ con_tc_kernel(chi::Params p, const float2* __restrict__ chi, const float2* __res
       const int blk = have ? p.border[it.z + 2 * st + h] : 0;
       const int* aoff = p.aoff + (size_t)blk * (p.a.natm + 1);
       const int n = have ? aoff[it.x + 1] - aoff[it.x] - it.y : 0;   // slots of the tile here
-      const float2* x = chi + ((size_t)p.boff[blk] * p.a.nk + (size_t)k * aoff[p.a.natm] +
-                               aoff[it.x] + it.y) * 32 + pt;
+      const size_t x = ((size_t)p.boff[blk] * p.a.nk + (size_t)k * aoff[p.a.natm] + aoff[it.x] +
+                        it.y) * 32 + pt;
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
         const int slot = 8 * warp + 2 * s + odd;
-        av[h][s] = slot < n ? __ldg(reinterpret_cast<const float4*>(x + 32 * slot))
-                            : make_float4(0.f, 0.f, 0.f, 0.f);
+        av[h][s] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (slot < n) {
+          if constexpr (REAL) {
+            const float2 v = __ldg(reinterpret_cast<const float2*>((const float*)chi + x + 32 * slot));
+            av[h][s] = make_float4(v.x, 0.f, v.y, 0.f);
+          } else {
+            av[h][s] = __ldg(reinterpret_cast<const float4*>((const float2*)chi + x + 32 * slot));
+          }
+        }
       }
       if constexpr (HB == 0) continue;
       bool v0, v1;
@@ -287,32 +294,43 @@ con_tc_kernel(chi::Params p, const float2* __restrict__ chi, const float2* __res
   if (warp == 0) tc::tmem_dealloc(tmem, COLS);
 }
 
-// kc[k][mu][i] = scale N_mu (sum of the items), or += after the first chunk: a CTA per (eight slots, k), 32 threads per slot
-// over the orbitals and parts, the items of a slot in order.
+// kc[k][mu][i] = scale N_mu (sum of the items), or += after the first chunk: a CTA per (slot, k),
+// a lane per orbital and part, every eighth run of items per warp, the warps' shares added in
+// order.
 template <int N>
 __global__ void __launch_bounds__(256)
 sum_tc_kernel(chi::Params p, const unsigned* __restrict__ colmax, double2* __restrict__ kc,
               double2* __restrict__ copy, int row_of0, int nitems, double scale, int add) {
-  constexpr int NI = N / 2;
-  const int slot = blockIdx.x * 8 + (threadIdx.x >> 5), k = blockIdx.y, nocc = p.a.nocc;
-  if (slot >= p.nslots) return;
+  constexpr int NI = N / 2, Z = 8;
+  __shared__ double share[Z][2 * NI];
+  const int slot = blockIdx.x, k = blockIdx.y, nocc = p.a.nocc;
   const int mu = p.slot_ao[slot];
   if (mu < 0) return;
   int a = 0;
   while (slot >= p.slot0[a + 1]) ++a;
   const int s = slot - p.slot0[a], g = s / kTcTile, r = s % kTcTile;
   const int2 ro = p.rows_of[row_of0 + a];
-  for (int v = threadIdx.x & 31; v < 2 * nocc; v += 32) {
+  const int z = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double* src = p.part + ((size_t)k * nitems * kM + r) * N;
+  for (int v = lane; v < 2 * nocc; v += 32) {
     const int i = v >> 1, im = v & 1;
-    const double* src = p.part + ((size_t)k * nitems * kM + r) * N;
     double t = 0.0;
 #pragma unroll 4
-    for (int y = 0; y < ro.y; ++y) {
+    for (int y = z; y < ro.y; y += Z) {
       const int2 row = p.rows[ro.x + y];
       if (g >= row.y) continue;
       const double* q = src + (size_t)(row.x + g) * kM * N;
       t += im ? q[NI + i] - q[kTcTile * N + i] : q[i] + q[kTcTile * N + NI + i];
     }
+    share[z][v] = t;
+  }
+  __syncthreads();
+  if (z != 0) return;
+  for (int v = lane; v < 2 * nocc; v += 32) {
+    const int i = v >> 1, im = v & 1;
+    double t = 0.0;
+#pragma unroll
+    for (int y = 0; y < Z; ++y) t += share[y][v];
     const double f = scale * p.ao_norm[mu] / (double)p.row_scale[slot] *
                      ldexp(1.0, col_exp(colmax[(size_t)k * nocc + i]) - 13);
     const size_t at = 2 * (((size_t)k * p.a.nao + mu) * nocc + i) + im;
@@ -332,16 +350,23 @@ cudaError_t run(const Plan& p, const chi::Params& q, const ChiChunk& c, double2*
   static_assert(smem <= 75 * 1024, "three CTAs per SM");
   static DeviceCache attr;
   attr.get(p.device, [&] {
-    cudaFuncSetAttribute(con_tc_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(con_tc_kernel<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+    cudaFuncSetAttribute(con_tc_kernel<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
     return 1;
   });
+  const dim3 grid(c.nitems, p.nk);
   if (hook) hook->before();
-  if (c.nitems > 0)
-    con_tc_kernel<N><<<dim3(c.nitems, p.nk), kThreads, smem, s>>>(
-        q, (const float2*)p.chi->chi, (const float2*)p.Y, p.colmax, c.item0, c.nitems, p.status,
-        p.wait_ns);
+  if (c.nitems > 0 && q.signs)
+    con_tc_kernel<N, true><<<grid, kThreads, smem, s>>>(q, p.chi->chi, (const float2*)p.Y, p.colmax,
+                                                        c.item0, c.nitems, p.status, p.wait_ns);
+  else if (c.nitems > 0)
+    con_tc_kernel<N, false><<<grid, kThreads, smem, s>>>(q, p.chi->chi, (const float2*)p.Y,
+                                                         p.colmax, c.item0, c.nitems, p.status,
+                                                         p.wait_ns);
   if (hook) hook->after();
-  sum_tc_kernel<N><<<dim3((q.nslots + 7) / 8, p.nk), 256, 0, s>>>(q, p.colmax, p.kc, copy, c.row_of0,
+  sum_tc_kernel<N><<<dim3(q.nslots, p.nk), 256, 0, s>>>(q, p.colmax, p.kc, copy, c.row_of0,
                                                                   c.nitems, scale,
                                                                   c.b0 > 0 ? 1 : 0);
   return cudaGetLastError();
