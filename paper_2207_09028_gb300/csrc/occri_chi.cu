@@ -703,7 +703,9 @@ __device__ __forceinline__ void cmac(const float4& c, float x, float2& t) {
 // the same for every lane, costs the load path as much as a value per lane: up to four
 // orbitals take two blocks (64 k, 200 AOs, 48^3, nocc 4: orbitals and AOs 5.5 -> 5.0 ms); with
 // eight the wider tile's registers cost what it saves (350 AOs, 8 k, 60^3: 1.52 against 1.50 ms).
-template <typename T, int NI> constexpr int orb_blocks() { return sizeof(T) == 4 && NI == 4 ? 2 : 1; }
+template <typename T, int NI, bool REAL> constexpr int orb_blocks() {
+  return sizeof(T) == 4 && (REAL || NI == 4) ? 2 : 1;
+}
 template <typename T, int NI, int NB, bool REAL>
 __global__ void __launch_bounds__(128)
 orb_kernel(Params p, const chi_t<T, REAL>* __restrict__ chi, const typename CsT<T>::type* __restrict__ cs,
@@ -1047,7 +1049,7 @@ void run_orb_as(const Params& q, const void* chi, const void* cs, void* out, con
                 int i0, int periodic, cudaStream_t s) {
   // one block per warp where two would leave SMs without work
   const int nb = c.b1 - c.b0;
-  constexpr int NB = orb_blocks<T, NI>();
+  constexpr int NB = orb_blocks<T, NI, REAL>();
   const auto* x = (const chi_t<T, REAL>*)chi;
   const auto* cf = (const typename CsT<T>::type*)cs;
   if (NB == 1 || (long long)nb * q.a.nk < 152 * 64)

@@ -80,3 +80,26 @@ def test_orbitals_and_contraction_match_oracle(name, precision):
         assert np.abs(KC.cpu().numpy() - kc).max() <= tol * np.abs(kc).max()
     # the contraction adds its partial sums in a fixed order
     assert torch.equal(KC, plan.build(C)[0])
+
+
+@pytest.fixture(scope="module")
+def ragged():
+    w = small_workload(mesh=(1, 2, 2), grid=(45, 45, 45), counts=(3, 1), lo=0.15, nocc=2, seed=37,
+                       complex_c=True)
+    return w, O.bloch_aos(w.lattice, w.xyz, w.shell_atom, w.shell_l, w.shell_alpha, w.kfrac,
+                          grid=w.grid)
+
+
+@pytest.mark.parametrize("nocc", [3, 7, 12])
+def test_orbitals_two_blocks_per_warp(ragged, nocc):
+    """Enough ragged blocks that a warp takes two (which differ in the AOs that reach them)."""
+    import torch
+    import paper_2207_09028_gb300 as occri
+    w, chi = ragged
+    c = np.random.default_rng(5).standard_normal((2, w.nk, w.nao, nocc))
+    w = dataclasses.replace(w, nocc=nocc, C=c[0] + 1j * c[1])
+    psi = O.orbitals_on_grid(chi, w.C)
+    plan = occri.Plan.from_workload(w, precision="mixed")
+    got = plan.orbitals(torch.from_numpy(w.C).cuda()).cpu().numpy().reshape(psi.shape)
+    # the bar above: sqrt(n) u for n of about 100 images and AOs, with a margin of about 3
+    assert np.abs(got - psi).max() <= 2e-6 * np.abs(psi).max()
