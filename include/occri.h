@@ -84,7 +84,8 @@ typedef enum {
  * OCCRI_MIXED: AO evaluation, orbitals, pair densities, FFTs, the kernel multiply
  *   and the Y accumulation in FP32; the contraction (e) accumulates per thread in
  *   FP32 and across threads in FP64; assembly (f) and E_x in FP64.
- * OCCRI_MIXED_TC: as OCCRI_MIXED, but the contraction (e) runs on the tensor cores, per k as a
+ * OCCRI_MIXED_TC: as OCCRI_MIXED, but at two and more k-points the contraction (e) runs on the
+ *   tensor cores, per k as a
  *   real GEMM over the grid points: rows Re and Im of the Bloch AOs, columns Re and Im of Y,
  *   both split into FP16 hi + lo parts with power-of-two scalings, three FP16 products with
  *   FP32 accumulation per term; each 16-point product leaves tensor memory after its stage

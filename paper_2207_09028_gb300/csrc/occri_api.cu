@@ -909,7 +909,7 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
                                split_y && ns > 2 ? p->Yx[1] : nullptr, s) != cudaSuccess)
       return OCCRI_ECUDA;
     ++launches;
-    if (p->precision == OCCRI_MIXED_TC) {
+    if (tc_contraction(*p)) {
       // the GEMM kernels alone, one span per slab (stage OCCRI_STAGE_CONTRACT_GEMM)
       struct GemmSpans : LaunchHook {
         Plan* p;
@@ -1755,7 +1755,7 @@ int occri_plan_create(occri_plan** out, const occri_cell* cell, const occri_kmes
   chk(dalloc(&p->mmat, (size_t)p->nk * nocc * nocc, &tot));
   chk(dalloc(&p->ek, (size_t)p->nk, &tot));
   chk(dalloc(&p->dacc, 2, &tot));
-  if (precision == OCCRI_MIXED_TC) chk(dalloc(&p->colmax, (size_t)p->nk * nocc, &tot));
+  if (tc_contraction(*p)) chk(dalloc(&p->colmax, (size_t)p->nk * nocc, &tot));
   // mapped host memory: a kernel writes it only when something failed, and a sync reads it
   // without a copy (cudaMemcpy of eight bytes took about 10 us of every synchronised call)
   if (e == cudaSuccess) e = cudaHostAlloc((void**)&p->status_h, 2 * sizeof(int), cudaHostAllocMapped);
@@ -1807,7 +1807,7 @@ int occri_plan_info(const occri_plan* plan, occri_plan_info_t* info) {
   info->workspace_bytes = p->workspace_bytes;
   info->fields_per_wave = p->nkp_wave * p->nocc * p->nocc;
   info->launches_per_build = p->launches_per_build;
-  const bool tc = p->precision == OCCRI_MIXED_TC;
+  const bool tc = occri::tc_contraction(*p);
   info->contraction_tc = tc ? 1 : 0;
   info->tc_stages = tc ? occri::tc_plan_stages(*p) : 0;
   info->tc_flops_per_stage = tc ? occri::tc_flops_per_stage(p->nocc) : 0.0;

@@ -1199,7 +1199,7 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   ChiTables* t = new (std::nothrow) ChiTables();
   if (!t) return cudaErrorMemoryAllocation;
   p->chi = t;
-  t->tile = p->precision == OCCRI_MIXED_TC ? kTcTile : 0;
+  t->tile = tc_contraction(*p) ? kTcTile : 0;
   const int natm = p->natm, nblk = p->nblk, nsa = p->nsa, lmax = p->lmax;
   const bool fp64 = p->precision == OCCRI_FP64;
   // slots: per atom, shells by falling screening radius
