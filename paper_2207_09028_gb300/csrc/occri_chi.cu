@@ -1083,15 +1083,15 @@ cudaError_t product_b(const Plan& p, const Params& q, const ChiChunk& c, const v
 template <typename T, int NI>
 void run_con(const Plan& p, const Params& q, const ChiChunk& c, const void* F, double2* out,
              double2* copy, int i0, double scale, cudaStream_t s) {
-  const dim3 grid((c.nitems + 7) / 8, p.nk);
-  if (c.nitems > 0 && q.signs)
+  const dim3 grid((c.con.nitems + 7) / 8, p.nk);
+  if (c.con.nitems > 0 && q.signs)
     con_kernel<T, NI, true><<<grid, 256, 0, s>>>(q, (const T*)p.chi->chi, (const cplx_t<T>*)F,
-                                                 c.item0, c.nitems, i0);
-  else if (c.nitems > 0)
+                                                 c.con.item0, c.con.nitems, i0);
+  else if (c.con.nitems > 0)
     con_kernel<T, NI, false><<<grid, 256, 0, s>>>(q, (const cplx_t<T>*)p.chi->chi,
-                                                  (const cplx_t<T>*)F, c.item0, c.nitems, i0);
+                                                  (const cplx_t<T>*)F, c.con.item0, c.con.nitems, i0);
   sum_kernel<NI><<<dim3(q.nslots / kPad, p.nk), 2 * kPad * NI * kSumSplit, 0, s>>>(
-      q, out, copy, c.row_of0, c.nitems, i0, scale, c.b0 > 0 ? 1 : 0);
+      q, out, copy, c.con.row_of0, c.con.nitems, i0, scale, c.b0 > 0 ? 1 : 0);
 }
 
 // orbitals per pass of con_kernel
@@ -1334,7 +1334,7 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
                             : std::max(widest, std::min(kChiChunkBytes, free_b / 8));
   std::vector<long long> boff(nblk, 0);
   {
-    ChiChunk c{0, 0, 0, 0, 0};
+    ChiChunk c;
     long long slots = 0;
     for (int b = 0; b < nblk; ++b) {
       const int n = aoff[(size_t)b * (natm + 1) + natm];
@@ -1354,47 +1354,58 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   // The contraction's items: a group of slots of an atom (kPad of them, or a tensor-core tile)
   // over up to `run` of the blocks that reach the group. `run` gives enough items to fill the
   // GPU (about 16 warps per scheduler, or three rounds of CTAs) while the FP32 sums stay short.
-  const int width = t->tile > 0 ? t->tile : chi::kPad;
-  long long groups = 0;
-  for (int b = 0; b < nblk; ++b)
-    for (int a = 0; a < natm; ++a) {
-      const int* o = &aoff[(size_t)b * (natm + 1) + a];
-      groups += (o[1] - o[0] + width - 1) / width;
-    }
-  const long long want = t->tile > 0 ? 152 * 9 : 152 * 64;
-  int run = (int)std::max<long long>(4, std::min<long long>(64, groups * p->nk / want));
-  run = (run + 1) / 2 * 2;
   std::vector<int4> items;
   std::vector<int> border;
   std::vector<int2> rows, rows_of;
-  for (ChiChunk& c : t->chunks) {
-    c.item0 = (int)items.size();
-    c.row_of0 = (int)rows_of.size();
+  auto slots = [&](int a, int b) {
+    return aoff[(size_t)b * (natm + 1) + a + 1] - aoff[(size_t)b * (natm + 1) + a];
+  };
+  auto run_length = [&](int width, long long want) {
+    long long groups = 0;
+    for (int b = 0; b < nblk; ++b)
+      for (int a = 0; a < natm; ++a) groups += (slots(a, b) + width - 1) / width;
+    const int run = (int)std::max<long long>(4, std::min<long long>(64, groups * p->nk / want));
+    return (run + 1) / 2 * 2;
+  };
+  const int con_run = run_length(chi::kPad, 152 * 64);
+  const int tc_run = t->tile > 0 ? run_length(t->tile, 152 * 9) : 0;
+  std::vector<int> first(natm);   // the chunk's blocks by falling number of the atom's slots
+  auto make_items = [&](const ChiChunk& c, ChiItems* it, int width, int run, size_t values,
+                        long long* pairs) {
+    it->item0 = (int)items.size();
+    it->row_of0 = (int)rows_of.size();
+    const int nb = c.b1 - c.b0;
     for (int a = 0; a < natm; ++a) {
-      const int o0 = (int)border.size(), row0 = (int)rows.size();
-      auto slots = [&](int b) {
-        return aoff[(size_t)b * (natm + 1) + a + 1] - aoff[(size_t)b * (natm + 1) + a];
-      };
-      std::vector<int> bl(c.b1 - c.b0);
-      std::iota(bl.begin(), bl.end(), c.b0);
-      std::stable_sort(bl.begin(), bl.end(), [&](int x, int y) { return slots(x) > slots(y); });
-      border.insert(border.end(), bl.begin(), bl.end());
-      for (int r0 = 0; r0 < (int)bl.size() && slots(bl[r0]) > 0; r0 += run) {
-        rows.push_back(make_int2((int)items.size() - c.item0, (slots(bl[r0]) + width - 1) / width));
-        for (int s = 0; s < slots(bl[r0]); s += width) {
+      const int row0 = (int)rows.size(), o0 = first[a];
+      for (int r0 = 0; r0 < nb && slots(a, border[o0 + r0]) > 0; r0 += run) {
+        const int ns = slots(a, border[o0 + r0]);
+        rows.push_back(make_int2((int)items.size() - it->item0, (ns + width - 1) / width));
+        for (int s = 0; s < ns; s += width) {
           int n = 0;
-          while (n < run && r0 + n < (int)bl.size() && slots(bl[r0 + n]) > s) ++n;
+          while (n < run && r0 + n < nb && slots(a, border[o0 + r0 + n]) > s) ++n;
           items.push_back(make_int4(a, s, o0 + r0, n));
-          t->item_pairs += (n + 1) / 2;
+          if (pairs) *pairs += (n + 1) / 2;
         }
       }
       rows_of.push_back(make_int2(row0, (int)rows.size() - row0));
     }
-    c.nitems = (int)items.size() - c.item0;
-    const size_t values = t->tile > 0
-                              ? tc_item_values(p->nocc)
-                              : 2 * (size_t)chi::kPad * chi::con_width(p->nocc, fp64);
-    t->part_bytes = std::max(t->part_bytes, sizeof(double) * values * (size_t)c.nitems * p->nk);
+    it->nitems = (int)items.size() - it->item0;
+    t->part_bytes =
+        std::max(t->part_bytes, sizeof(double) * values * (size_t)it->nitems * p->nk);
+  };
+  for (ChiChunk& c : t->chunks) {
+    for (int a = 0; a < natm; ++a) {
+      std::vector<int> bl(c.b1 - c.b0);
+      std::iota(bl.begin(), bl.end(), c.b0);
+      std::stable_sort(bl.begin(), bl.end(),
+                       [&](int x, int y) { return slots(a, x) > slots(a, y); });
+      first[a] = (int)border.size();
+      border.insert(border.end(), bl.begin(), bl.end());
+    }
+    make_items(c, &c.con, chi::kPad, con_run,
+               2 * (size_t)chi::kPad * chi::con_width(p->nocc, fp64), nullptr);
+    if (t->tile > 0)
+      make_items(c, &c.tc, t->tile, tc_run, tc_item_values(p->nocc), &t->item_pairs);
   }
   const int row_bytes = 32 * (fp64 ? 8 : 4);
   t->col_rows = 2 * (p->D[0] / 2 + 1) * p->D[1] * p->D[2];

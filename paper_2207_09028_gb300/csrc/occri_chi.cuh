@@ -15,10 +15,16 @@ struct ChiShell {
   int l, slot, orig, exact;   // first slot within the atom; index in the basis; FP32 exponents
 };
 
-// Blocks [b0, b1): one filling of the chi buffer, with the contraction's work items and the
-// first of its rows_of entries.
+// A contraction's work items for the blocks of one chunk and the first of its rows_of entries.
+struct ChiItems {
+  int item0 = 0, nitems = 0, row_of0 = 0;
+};
+
+// Blocks [b0, b1): one filling of the chi buffer. Items of the tensor cores' contraction (plans
+// that run it) and of the CUDA cores', which the adjoint takes in every plan.
 struct ChiChunk {
-  int b0, b1, item0, nitems, row_of0;
+  int b0 = 0, b1 = 0;
+  ChiItems tc, con;
 };
 
 struct ChiTables {
@@ -31,7 +37,7 @@ struct ChiTables {
   int signs = 0;                  // every phase of the mesh is a sign (axes of one or two points)
   int parts = 1;                  // CTAs per (block, atom) of chi_kernel
   int tile = 0;                   // slots per item of the tensor-core contraction, 0 without it
-  long long item_pairs = 0;       // pairs of blocks over all items
+  long long item_pairs = 0;       // pairs of blocks over the tensor-core items
   size_t chi_bytes = 0;
   // device
   ChiShell* shells = nullptr;     // [nshell] per atom, falling screening radius

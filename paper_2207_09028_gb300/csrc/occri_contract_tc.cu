@@ -356,18 +356,18 @@ cudaError_t run(const Plan& p, const chi::Params& q, const ChiChunk& c, double2*
                          (int)smem);
     return 1;
   });
-  const dim3 grid(c.nitems, p.nk);
+  const dim3 grid(c.tc.nitems, p.nk);
   if (hook) hook->before();
-  if (c.nitems > 0 && q.signs)
+  if (c.tc.nitems > 0 && q.signs)
     con_tc_kernel<N, true><<<grid, kThreads, smem, s>>>(q, p.chi->chi, (const float2*)p.Y, p.colmax,
-                                                        c.item0, c.nitems, p.status, p.wait_ns);
-  else if (c.nitems > 0)
+                                                        c.tc.item0, c.tc.nitems, p.status, p.wait_ns);
+  else if (c.tc.nitems > 0)
     con_tc_kernel<N, false><<<grid, kThreads, smem, s>>>(q, p.chi->chi, (const float2*)p.Y,
-                                                         p.colmax, c.item0, c.nitems, p.status,
+                                                         p.colmax, c.tc.item0, c.tc.nitems, p.status,
                                                          p.wait_ns);
   if (hook) hook->after();
-  sum_tc_kernel<N><<<dim3(q.nslots, p.nk), 256, 0, s>>>(q, p.colmax, p.kc, copy, c.row_of0,
-                                                                  c.nitems, scale,
+  sum_tc_kernel<N><<<dim3(q.nslots, p.nk), 256, 0, s>>>(q, p.colmax, p.kc, copy, c.tc.row_of0,
+                                                                  c.tc.nitems, scale,
                                                                   c.b0 > 0 ? 1 : 0);
   return cudaGetLastError();
 }

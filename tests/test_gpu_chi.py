@@ -103,3 +103,20 @@ def test_orbitals_two_blocks_per_warp(ragged, nocc):
     got = plan.orbitals(torch.from_numpy(w.C).cuda()).cpu().numpy().reshape(psi.shape)
     # the bar above: sqrt(n) u for n of about 100 images and AOs, with a margin of about 3
     assert np.abs(got - psi).max() <= 2e-6 * np.abs(psi).max()
+
+
+def test_adjoint_of_a_tensor_core_plan():
+    """The adjoint contracts on the CUDA cores in every plan: over items of their own."""
+    import torch
+    import paper_2207_09028_gb300 as occri
+    w = small_workload(mesh=(1, 1, 2), grid=(12, 12, 12), counts=(2, 1), nocc=3, seed=45)
+    G = torch.from_numpy(np.random.default_rng(6).standard_normal((w.nk, w.nao, w.nao)) + 0j).cuda()
+    C = torch.from_numpy(w.C).cuda()
+    out = {}
+    for prec in ("fp64", "mixed_tc"):
+        plan = occri.Plan.from_workload(w, precision=prec)
+        plan.build(C)
+        out[prec] = plan.vjp_full(C, 0.3, None, G).cpu().numpy()
+    # the bar of the mixed adjoint: FP32 sums of about 2,000 points, 2000 u = 1.2e-4 at most,
+    # sqrt(2000) u = 2.7e-6 as a random walk, with a margin of about 4
+    assert np.abs(out["mixed_tc"] - out["fp64"]).max() <= 1e-5 * np.abs(out["fp64"]).max()
