@@ -1,14 +1,15 @@
-// occri_ao.cu -- Bloch-summed AOs evaluated on the fly (integral-direct, Algorithm 4):
+// occri_ao.cu -- the orbitals without allocation, the fields' phases and output order.
 //   (a)+(b) psi_{ik}(r) = sum_mu C^k_{mu i} chi_{mu k}(r)                  (Eq. occmo)
-//   (e)     K_{mu i}(k) = -(Omega/(N_k N_g)) sum_r conj(chi_{mu k}(r)) Y_{ik}(r)  (Eq. occrik)
-// with chi_{mu k}(r) = sum_T e^{i k.T} phi_mu(r - A - T) (Sec. II.A).
+// with chi_{mu k}(r) = sum_T e^{i k.T} phi_mu(r - A - T) (Sec. II.A). orbitals_kernel evaluates
+// chi where it is used and stores none of it, for occri_orbitals_noalloc alone, which has no
+// memory for AO tiles; every other call takes the tiles of occri_chi.cu.
 //
 // The image sum is split as T = T0(r, A) + T': T0 brings r - A into the
 // Wigner-Seitz cell (precomputed per grid point and atom), T' runs over one
 // master list of lattice vectors sorted by length. Every thread of a warp walks
 // the same prefix of that list (a shell's prefix covers its screening radius
 // plus the largest |r - A - T0|), so the image offsets and the phase table
-// e^{i k.T'} are warp-uniform loads. chi itself is never stored.
+// e^{i k.T'} are warp-uniform loads.
 //
 // In FP32 the displacement r - A - T is formed from hi/lo float pairs so that
 // it is accurate to an ulp of its own size, not of |T|.
@@ -302,7 +303,7 @@ template cudaError_t launch_widen<double>(const Plan&, void*, cudaStream_t);
 
 // ------------------------------------------------------------------ orbitals without allocation
 //
-// occri_orbitals_noalloc runs the same kernels as occri_orbitals but keeps its
+// occri_orbitals_noalloc evaluates the AOs where it uses them and keeps its
 // scratch -- the normalised coefficients N_mu C^k_{mu i} and the orbitals in the
 // plan's working precision before widening -- in this file-scope device array
 // instead of the plan's workspaces. Every GPU that loads the library reserves
