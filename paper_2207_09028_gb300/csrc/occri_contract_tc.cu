@@ -10,10 +10,11 @@
 // memory in the tensor cores' layout, and one thread issues the stage's three FP16 products
 // (hi.hi + hi.lo + lo.hi) into tensor memory, 16 points to an accumulator, which leave it after
 // the stage for FP32 sums in registers: sums in tensor memory round toward zero (64 points to
-// an accumulator biased E_x by 1.1e-7 relative, long sums by 1e-6). The items' sums are added in a fixed order in FP64.
+// an accumulator biased E_x by 1.1e-7 relative, long sums by 1e-6). The items' sums are added in
+// a fixed order in FP64.
 //
-// What bounds it: chi is read once, 8 bytes per (k, slot, point), and everything else follows
-// that stream; with N = 16 the MMAs of a stage take a few hundred cycles. The earlier form
+// What bounds it: issue (74 % at 27 k, 94 AOs, 60^3: 1.18 ms), which is the split of chi, read
+// once, into its FP16 halves; with N = 16 the tensor pipe is 5 % busy. The earlier form
 // generated the AOs of the k-mesh's supercell in FP16 blocks instead (D_1 D_2 D_3 / 2 times the
 // products of this one, 36 % of them in reach): 2.09 of 3.43 ms of a build at 8 k, 104 AOs,
 // 36^3, 5.5 of 7.9 ms at 6 k, 50^3, and 50 of 426 ms at 64 k, 350 AOs, 60^3.
