@@ -408,9 +408,10 @@ int occri_batch_destroy(occri_batch *batch);
 /* ---- Fault injection, for tests of the error paths (no counterpart in the paper) ----
  * occri_plan_inject_fault(plan, OCCRI_FAULT_WAIT, ms): in the plan's following builds the
  *   producer warp of every bulk-copy accumulation pass (FP64 waves, and FP32 waves of
- *   nocc > 8, where shared memory allows) issues no copy, so each consumer's bounded
- *   wait runs out after ms milliseconds; the build then completes with a meaningless Y,
- *   and occri_plan_sync returns OCCRI_ETIMEOUT. No copy is in flight when a CTA leaves.
+ *   nocc > 8, where shared memory allows) issues no copy, and the tensor-core contraction
+ *   (OCCRI_MIXED_TC) issues no product, so each consumer's bounded wait runs out after ms
+ *   milliseconds; the build then completes with a meaningless Y or K_{mu i}, and
+ *   occri_plan_sync returns OCCRI_ETIMEOUT. Nothing is in flight when a CTA leaves.
  *   occri_plan_inject_fault(plan, OCCRI_FAULT_NONE, ms) restores normal builds with
  *   wait limit ms (the default limit is 2000 ms). ms must lie in (0, 60000].
  * occri_debug_fail_allocation(n): the n-th device allocation made by the library from

@@ -19,7 +19,7 @@
 // products of this one, 36 % of them in reach): 2.09 of 3.43 ms of a build at 8 k, 104 AOs,
 // 36^3, 5.5 of 7.9 ms at 6 k, 50^3, and 50 of 426 ms at 64 k, 350 AOs, 60^3.
 // Every mbarrier wait is bounded by the plan's wait limit; on timeout the kernel records
-// OCCRI_ETIMEOUT and stops issuing.
+// OCCRI_ETIMEOUT, stops issuing and waits once more (bounded too) for the products in flight.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -53,6 +53,18 @@ __device__ __forceinline__ int op_off(int rows, int row, int k) {
 __device__ __forceinline__ void fail(int* status) {
   if (status && atomicCAS(status, 0, (int)OCCRI_ETIMEOUT) == 0) status[1] = -1;
 }
+
+// A warp's bounded wait: lane 0 waits and the warp follows its verdict (what comes next is
+// warp-wide: tensor-memory loads need all 32 lanes), then every lane sees the phase itself.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, unsigned parity, long long limit_ns,
+                                          int lane) {
+  int ok = 1;
+  if (lane == 0) ok = tc::mbar_wait(bar, parity, limit_ns) ? 1 : 0;
+  ok = __shfl_sync(0xffffffffu, ok, 0);
+  if (ok && lane != 0) tc::mbar_try_wait(bar, parity);
+  return ok != 0;
+}
+constexpr long long kDrainNs = 2000000000LL;   // after a timeout: for the products in flight
 
 // FP16 hi/lo split of two values, packed as two 32-bit words (x0 in the low half)
 __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
@@ -94,7 +106,7 @@ template <int N, bool REAL>
 __global__ void __launch_bounds__(kThreads, N == 64 ? 2 : 3)
 con_tc_kernel(chi::Params p, const void* __restrict__ chi, const float2* __restrict__ Y,
               const unsigned* __restrict__ colmax, int item0, int nitems, int* status,
-              long long wait_ns) {
+              long long wait_ns, int fault) {
   constexpr int NI = N / 2;                       // orbitals, padded
   constexpr int AB = op_bytes(kM), BB = op_bytes(N);
   constexpr uint32_t kIdesc = tc::idesc_f16_f32(kM, N);
@@ -257,13 +269,16 @@ con_tc_kernel(chi::Params p, const void* __restrict__ chi, const float2* __restr
 #pragma unroll 1
   for (; st < nst; ++st) {
     if (st > 0) {
-      ok = tc::mbar_wait(tc::smem_u32(&bar.done), (unsigned)((st - 1) & 1), wait_ns);
+      ok = warp_wait(tc::smem_u32(&bar.done), (unsigned)((st - 1) & 1), wait_ns, lane);
       if (ok) take();
     }
     if (ok) store();
     tc::fence_proxy_async_smem();
-    if (!__syncthreads_and(ok ? 1 : 0)) break;
-    if (tid == 0) {
+    if (!__syncthreads_and(ok ? 1 : 0)) {   // one warp's timeout ends the CTA's work
+      ok = false;
+      break;
+    }
+    if (tid == 0 && fault != OCCRI_FAULT_WAIT) {   // (test-only fault: nothing is issued)
       tc::tc_fence_after();
       const uint32_t ah = tc::smem_u32(a_hi), al = tc::smem_u32(a_lo), bh = tc::smem_u32(b_hi),
                      bl = tc::smem_u32(b_lo);
@@ -281,10 +296,19 @@ con_tc_kernel(chi::Params p, const void* __restrict__ chi, const float2* __restr
     }
     if (st + 1 < nst) fetch(st + 1);
   }
-  // the last stage issued (after a timeout too: nothing is in flight when the CTA leaves)
-  const bool last = tc::mbar_wait(tc::smem_u32(&bar.done), (unsigned)((st - 1) & 1), wait_ns);
-  if (ok && last) take();
-  if (!ok || !last) fail(status);
+  // the last stage issued
+  const unsigned parity = (unsigned)((st - 1) & 1);
+  if (ok) {
+    ok = warp_wait(tc::smem_u32(&bar.done), parity, wait_ns, lane);
+    if (ok) take();
+  }
+  if (!ok) {
+    // the sums are void; the products in flight still read shared memory and write tensor
+    // memory, so the CTA keeps both until they are done (or this longer limit has passed too)
+    if (fault != OCCRI_FAULT_WAIT)
+      warp_wait(tc::smem_u32(&bar.done), parity, wait_ns > kDrainNs ? wait_ns : kDrainNs, lane);
+    if (lane == 0) fail(status);
+  }
   // part[k][item][row][column]
   double* o = p.part + ((size_t)k * nitems + w) * kM * N +
               (size_t)(32 * (warp & 3) + lane) * N + NI * (warp >> 2);
@@ -361,11 +385,12 @@ cudaError_t run(const Plan& p, const chi::Params& q, const ChiChunk& c, double2*
   if (hook) hook->before();
   if (c.tc.nitems > 0 && q.signs)
     con_tc_kernel<N, true><<<grid, kThreads, smem, s>>>(q, p.chi->chi, (const float2*)p.Y, p.colmax,
-                                                        c.tc.item0, c.tc.nitems, p.status, p.wait_ns);
+                                                        c.tc.item0, c.tc.nitems, p.status, p.wait_ns,
+                                                        p.fault);
   else if (c.tc.nitems > 0)
     con_tc_kernel<N, false><<<grid, kThreads, smem, s>>>(q, p.chi->chi, (const float2*)p.Y,
                                                          p.colmax, c.tc.item0, c.tc.nitems, p.status,
-                                                         p.wait_ns);
+                                                         p.wait_ns, p.fault);
   if (hook) hook->after();
   sum_tc_kernel<N><<<dim3(q.nslots, p.nk), 256, 0, s>>>(q, p.colmax, p.kc, copy, c.tc.row_of0,
                                                                   c.tc.nitems, scale,

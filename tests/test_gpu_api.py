@@ -150,6 +150,25 @@ def test_device_wait_timeout_is_reported_and_plan_recovers(torch_cuda):
         assert torch.allclose(Ex1, Ex0, rtol=1e-12)
 
 
+@pytest.mark.parametrize("mesh,nocc", [((1, 1, 2), 2), ((1, 1, 3), 12)])
+def test_contraction_timeout_is_reported_and_plan_recovers(torch_cuda, mesh, nocc):
+    """OCCRI_FAULT_WAIT in the tensor-core contraction: no product is issued, each warp's wait
+    gives up as one, and the next builds are the first one again."""
+    import paper_2207_09028_gb300 as occri
+    torch = torch_cuda
+    w = small_workload(mesh=mesh, grid=(12, 12, 12), counts=(6, 4), nocc=nocc, seed=85)
+    plan = occri.Plan.from_workload(w, precision="mixed_tc")
+    C = torch.from_numpy(w.C).cuda()
+    first = plan.build(C)
+    plan.inject_fault(occri.OCCRI_FAULT_WAIT, 50.0)
+    with pytest.raises(occri.OccriError) as e:
+        plan.build(C)
+    assert e.value.status == occri.OCCRI_ETIMEOUT
+    plan.inject_fault(occri.OCCRI_FAULT_NONE, 2000.0)
+    for _ in range(2):
+        assert all(torch.equal(x, y) for x, y in zip(plan.build(C), first))
+
+
 def test_inject_fault_rejects_bad_arguments(torch_cuda):
     import paper_2207_09028_gb300 as occri
     w = small_workload(mesh=(1, 1, 1), grid=(8, 8, 8), counts=(2, 1), nocc=2, seed=82)
