@@ -194,8 +194,9 @@ int occri_plan_set_stream(occri_plan *plan, void *cuda_stream);
 int occri_plan_sync(occri_plan *plan, int *bad_k);
 
 /* One exchange build, steps (a)-(f) (Algorithm 3 + ACE assembly).
- * C_dev : device, c128 [nk][nao][nocc] row-major, read only.
+ * C_dev : device, c128 [nk][nao][nocc] row-major, read only (but see KC_dev).
  * KC_dev: device, c128 [nk][nao][nocc] = K_{mu i}(k) (Eq. occrik), or NULL.
+ *         It may be the buffer of C, which is then overwritten after its last use.
  * K_dev : device, c128 [nk][nao][nao] ACE-form exchange matrix, or NULL.
  * Ex_dev: device, 1 double, E_x in Ha per cell, or NULL.
  * Asynchronous; call occri_plan_sync to observe OCCRI_ENOTPD. */

@@ -822,6 +822,12 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
   const bool timed = p->timing_every != 0;   // > 0: sampled waves too; -1: stage spans only
   long long launches = 0;
   const size_t orb = (size_t)p->nk * p->nocc * p->fs;
+  // The contraction writes the caller's K_{mu i} beside the plan's. The assembly still reads C
+  // after it: where the caller's two buffers overlap, a copy follows the assembly instead.
+  const size_t kc_bytes = sizeof(double2) * (size_t)p->nk * p->nao * p->nocc;
+  const uintptr_t kc_at = (uintptr_t)KC, c_at = (uintptr_t)C;
+  const bool kc_late = KC && kc_at < c_at + kc_bytes && c_at < kc_at + kc_bytes;
+  double2* const kc_out = kc_late ? nullptr : (double2*)KC;
   // streams that get a wave (a Gamma build has one wave)
   long long nwaves = 0;
   for (int k = 0; k < p->nk; ++k)
@@ -926,13 +932,14 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
           t = nullptr;
         }
       } spans(p, s, timed);
-      if (launch_contract_tc(*p, (double2*)KC, s, &spans) != cudaSuccess) return OCCRI_ECUDA;
+      if (launch_contract_tc(*p, kc_out, s, &spans) != cudaSuccess) return OCCRI_ECUDA;
       launches += tc_plan_launches(*p);
     } else {
       // Y carries N_g/(4 pi) (see PairParams), hence -Omega 4 pi / (N_k N_g^2)
       const double scale = -p->omega_cell * 4.0 * kPiD /
                            ((double)p->nk * (double)p->ng * (double)p->ng);
-      if (launch_contract_field<T>(*p, p->Y, p->kc, (double2*)KC, scale, s) != cudaSuccess) return OCCRI_ECUDA;
+      if (launch_contract_field<T>(*p, p->Y, p->kc, kc_out, scale, s) != cudaSuccess)
+        return OCCRI_ECUDA;
       launches += chi_launches(*p, true);
     }
     t.done(OCCRI_STAGE_CONTRACT, p->nk);
@@ -962,6 +969,9 @@ int build_impl(Plan* p, const double2* C, void* KC, void* K, double* Ex) {
     }
     t.done(OCCRI_STAGE_ASSEMBLE, p->nk);
   }
+  if (kc_late &&
+      cudaMemcpyAsync(KC, p->kc, kc_bytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+    return OCCRI_ECUDA;
   if (cudaGetLastError() != cudaSuccess) return OCCRI_ECUDA;
   p->have_kc = true;
   p->launches_per_build = launches;

@@ -125,6 +125,26 @@ def test_exchange_build_backward_after_another_build(torch_cuda):
     assert torch.allclose(g_ref, 4.0 / w.nk * KC, rtol=1e-11, atol=1e-14)
 
 
+@pytest.mark.parametrize("prec,mesh", [("fp64", (1, 1, 2)), ("mixed", (1, 1, 1)),
+                                       ("mixed_tc", (1, 1, 3))])
+@pytest.mark.parametrize("shift", [0, 3])
+def test_kc_written_over_c(torch_cuda, prec, mesh, shift):
+    """KC in the buffer of C, in its place and three values on: K, E_x and K_{mu i} are those of
+    separate buffers."""
+    import paper_2207_09028_gb300 as occri
+    torch = torch_cuda
+    w = small_workload(mesh=mesh, grid=(12, 12, 12), counts=(3, 2), nocc=3, seed=86)
+    plan = occri.Plan.from_workload(w, precision=prec)
+    C = torch.from_numpy(w.C).cuda()
+    kc, k, ex = plan.build(C)
+    buf = torch.zeros(C.numel() + shift, dtype=C.dtype, device="cuda")
+    over = buf[:C.numel()].view(C.shape).copy_(C)
+    KC = buf[shift:].view(C.shape)
+    K, Ex = torch.empty_like(k), torch.empty_like(ex)
+    plan.k_build(over, KC, K, Ex)
+    assert torch.equal(KC, kc) and torch.equal(K, k) and torch.equal(Ex, ex)
+
+
 # ------------------------------------------------------------------ error paths
 
 def test_device_wait_timeout_is_reported_and_plan_recovers(torch_cuda):
