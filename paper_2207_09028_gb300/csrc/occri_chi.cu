@@ -136,16 +136,16 @@ __device__ __forceinline__ void phase_sums(const cplx_t<T>* ph, int nkp, const T
 }
 
 // A narrow shell, one warp: every image its own entry (a lane reads back only what it wrote),
-// then chi of every k. Where the entries run out, the sums so far go to chi and the rest is
+// then chi of the k-points [ka, kb). Where the entries run out, the sums so far go to chi and the rest is
 // added.
 template <typename T, int L, int KT, typename GetRec>
 __device__ __forceinline__ void narrow_shell(const Params& p, const ChiShell& sh,
                                              const Disp<T>& d, int np, const GetRec& rec, T* ent,
-                                             int* ecls, cplx_t<T>* out, int kstride, int lane) {
+                                             int* ecls, cplx_t<T>* out, int kstride, int lane,
+                                             int ka, int kb) {
   constexpr int NM = 2 * L + 1;
   constexpr int CAP = kRows / NM;
   const cplx_t<T>* ph = reinterpret_cast<const cplx_t<T>*>(p.phase);
-  const int nk = p.a.nk;
   for (int j0 = 0; j0 < np; j0 += CAP) {
     const int ne = min(CAP, np - j0);
     for (int e = 0; e < ne; ++e) {
@@ -157,7 +157,7 @@ __device__ __forceinline__ void narrow_shell(const Params& p, const ChiShell& sh
       if (lane == 0) ecls[e] = r.cls;
     }
     __syncwarp();
-    for (int k0 = 0; k0 < nk; k0 += KT) {
+    for (int k0 = ka; k0 < kb; k0 += KT) {
       T xr[KT][NM], xi[KT][NM];
 #pragma unroll
       for (int b = 0; b < KT; ++b)
@@ -166,7 +166,7 @@ __device__ __forceinline__ void narrow_shell(const Params& p, const ChiShell& sh
       phase_sums<T, KT, NM>(ph, p.nkp, ent, ecls, ne, k0, lane, xr, xi);
 #pragma unroll
       for (int b = 0; b < KT; ++b) {
-        if (k0 + b >= nk) break;
+        if (k0 + b >= kb) break;
         cplx_t<T>* o = out + (size_t)(k0 + b) * kstride + lane;
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
@@ -597,10 +597,11 @@ chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
     }
     __syncthreads();
   }
-  int s = wide;
   T* ent = buf + warp * kRows * 32;
   int* ecls = eclss + warp * kRows;
-  for (s += warp + nw * blockIdx.z; s < nact; s += nw * gridDim.z) {
+  const int kz = FOLD ? 1 : p.kslices, per = (p.a.nk + 8 * kz - 1) / (8 * kz) * 8;
+  for (int it = warp + nw * blockIdx.z; it < (nact - wide) * kz; it += nw * gridDim.z) {
+    const int s = wide + it / kz, ka = per * (it % kz), kb = min(p.a.nk, ka + per);
     const ChiShell sh = p.shells[s0 + s];
     const int np = pre[sh.orig - s0];
     cplx_t<T>* out = p.signs ? reinterpret_cast<cplx_t<T>*>(reinterpret_cast<T*>(base) + 32 * sh.slot)
@@ -614,10 +615,10 @@ chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
       }
     } else {
       switch (sh.l) {
-        case 0: narrow_shell<T, 0, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
-        case 1: narrow_shell<T, 1, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
-        case 2: narrow_shell<T, 2, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
-        default: narrow_shell<T, 3, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane); break;
+        case 0: narrow_shell<T, 0, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane, ka, kb); break;
+        case 1: narrow_shell<T, 1, KS>(p, sh, d, np, rec, ent, ecls, out, kstride, lane, ka, kb); break;
+        case 2: narrow_shell<T, 2, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane, ka, kb); break;
+        default: narrow_shell<T, 3, KL>(p, sh, d, np, rec, ent, ecls, out, kstride, lane, ka, kb); break;
       }
     }
   }
@@ -630,6 +631,139 @@ chi_kernel(Params p, cplx_t<T>* __restrict__ chi, int blk0) {
         else base[o] = cplx_t<T>{T(0), T(0)};
       }
   }
+}
+
+// chi on meshes of many k-points that the transform does not take (shifted meshes, other axis
+// lengths), FP32: neighbouring shells of an atom, up to kDense AOs, at once. The warps evaluate a
+// batch of images into shared memory, then share the k-points, each with the sums of KD of them
+// and all kDense AOs in registers, so that a phase serves kDense products and chi is written
+// once per batch (every batch but the first adds). A group's shells have nearly the same reach;
+// the images that one lacks are zeros, and what its unused columns hold is not stored.
+// What bounds it: the phases (four wavefronts of the load path per 16 bytes that all lanes read) and
+// the products, about equally by count. One shell and warp at a time, a phase per product and chi read
+// and written again every 8 to 56 images: orbitals of 104 AOs at 9^3 k, 24^3, 23.0 ms against 8.1
+// (15.1 when they were summed without tiles).
+constexpr int kDense = 8;      // AOs of a group
+constexpr int KD = 4;          // k-points per warp
+// Least k-points of a mesh that takes it. Orbitals at 36^3, 104 and 350 AOs, narrow_shell against
+// this kernel: 12 k 642 / 719 and 1992 / 2355 us, 16 k 784 / 783 and 2498 / 2623, 20 k 964 / 953 and
+// 3178 / 3276, 27 k 1538 / 1151 and 5190 / 4043; at 12^3 it is ahead from 9 k on.
+constexpr int kDenseK = 16;
+constexpr int kDenseImages = 96;   // most images of a batch (1 KB each; two CTAs per SM)
+__global__ void __launch_bounds__(32 * kWarps, 2)
+chi_dense_kernel(Params p, float2* __restrict__ chi, int blk0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* val = reinterpret_cast<float*>(smem_raw);   // [image][column][lane]
+  int* ecls = reinterpret_cast<int*>(val + (size_t)p.batch * kDense * 32);
+  int* lnp = ecls + p.batch;                         // images << 2 | l of the atom's shells
+  const int blk = blk0 + blockIdx.x, a = blockIdx.y;
+  const size_t ab = (size_t)a * p.a.nblk + blk;
+  const int nact = p.nsh[ab];
+  if (nact == 0) return;
+  const int s0 = p.a.atom_shell0[a];
+  const unsigned short* pre = p.a.bpre + ab * p.a.nsa;
+  const size_t list0 = ab * p.a.lmax;
+  const int* cls = p.cls + (size_t)p.t0i[ab] * p.a.nimg;
+  for (int x = threadIdx.x; x < nact; x += blockDim.x) {
+    const ChiShell& sh = p.shells[s0 + x];
+    lnp[x] = pre[sh.orig - s0] << 2 | sh.l;
+  }
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  bool valid;
+  long long q;
+  const long long n = ao::block_point(p.a, blk, lane, &valid, &q);
+  Disp<float> d;
+  ao::load_disp(p.a, a, n, &d);
+  const int* aoff = p.aoff + (size_t)blk * (p.a.natm + 1);
+  const int kstride = 32 * aoff[p.a.natm];
+  float2* base = chi + (size_t)(p.boff[blk] * p.a.nk + aoff[a]) * 32 + lane;
+  // the CTA's k-points
+  const int nk = p.a.nk, per = (nk + KD * (int)gridDim.z - 1) / (KD * (int)gridDim.z) * KD;
+  const int ka = min(nk, per * (int)blockIdx.z), kb = min(nk, ka + per);
+  const float2* ph = reinterpret_cast<const float2*>(p.phase);
+  int last = 0;   // slots of the atom so far
+  for (int s = 0; s < nact;) {
+    int e = s, cols = 0;   // the group's shells [s, e)
+    while (e < nact && cols + 2 * (lnp[e] & 3) + 1 <= kDense) cols += 2 * (lnp[e++] & 3) + 1;
+    const int slot = p.shells[s0 + s].slot, images = lnp[s] >> 2;
+    for (int j0 = 0; j0 < images; j0 += p.batch) {
+      const int ne = min(p.batch, images - j0);
+      for (int j = warp; j < ne; j += kWarps) {
+        const Rec<float> r = load_rec<float>(p, list0, cls, j0 + j);
+        float* o = val + (size_t)j * kDense * 32 + lane;
+        for (int x = s; x < e; ++x) {
+          const ChiShell& sh = p.shells[s0 + x];
+          const bool in = j0 + j < lnp[x] >> 2;   // (past the shell's radius eval gives 0)
+          auto put = [&](auto L) {
+            constexpr int l = decltype(L)::value;
+            float v[2 * l + 1];
+            if (in) eval<l>(sh, d, r, v);
+#pragma unroll
+            for (int m = 0; m < 2 * l + 1; ++m) o[32 * m] = in ? v[m] : 0.f;
+            o += 32 * (2 * l + 1);
+          };
+          switch (lnp[x] & 3) {
+            case 0: put(std::integral_constant<int, 0>{}); break;
+            case 1: put(std::integral_constant<int, 1>{}); break;
+            case 2: put(std::integral_constant<int, 2>{}); break;
+            default: put(std::integral_constant<int, 3>{}); break;
+          }
+        }
+        if (lane == 0) ecls[j] = r.cls;
+      }
+      __syncthreads();
+      for (int k0 = ka + KD * warp; k0 < kb; k0 += KD * kWarps) {
+        float xr[KD][kDense], xi[KD][kDense];
+#pragma unroll
+        for (int b = 0; b < KD; ++b)
+#pragma unroll
+          for (int c = 0; c < kDense; ++c) xr[b][c] = xi[b][c] = 0.f;
+        // whole groups of KD: the table's rows are zero past the last k-point
+#pragma unroll 2
+        for (int j = 0; j < ne; ++j) {
+          const float4* row = reinterpret_cast<const float4*>(ph + (size_t)ecls[j] * p.nkp + k0);
+          const float* v = val + (size_t)j * kDense * 32 + lane;
+          float4 w[KD / 2];
+#pragma unroll
+          for (int b = 0; b < KD / 2; ++b) w[b] = __ldg(row + b);
+#pragma unroll
+          for (int c = 0; c < kDense; ++c) {
+            const float x = v[32 * c];
+#pragma unroll
+            for (int b = 0; b < KD / 2; ++b) {
+              xr[2 * b][c] += w[b].x * x;
+              xi[2 * b][c] += w[b].y * x;
+              xr[2 * b + 1][c] += w[b].z * x;
+              xi[2 * b + 1][c] += w[b].w * x;
+            }
+          }
+        }
+#pragma unroll
+        for (int b = 0; b < KD; ++b) {
+          if (k0 + b >= kb) break;
+          float2* o = base + (size_t)(k0 + b) * kstride + 32 * (size_t)slot;
+#pragma unroll
+          for (int c = 0; c < kDense; ++c) {
+            if (c >= cols) break;
+            float2 y = make_float2(xr[b][c], xi[b][c]);
+            if (j0 > 0) {
+              const float2 u = o[32 * c];
+              y.x += u.x;
+              y.y += u.y;
+            }
+            o[32 * c] = y;
+          }
+        }
+      }
+      __syncthreads();   // the batch's values are free
+    }
+    last = slot + cols;
+    s = e;
+  }
+  for (int x = last; x < aoff[a + 1] - aoff[a]; ++x)   // padding slots of the atom's last group
+    for (int k = ka + warp; k < kb; k += kWarps)
+      base[(size_t)k * kstride + 32 * (size_t)x] = make_float2(0.f, 0.f);
 }
 
 // List positions of every (atom, block) in order of class, once at plan creation: a warp per
@@ -1001,6 +1135,8 @@ Params params(const Plan& p) {
   q.buf_rows = t.buf_rows;
   q.warps = t.warps;
   q.signs = t.signs;
+  q.batch = t.batch;
+  q.kslices = t.kslices;
   return q;
 }
 
@@ -1009,27 +1145,49 @@ template <typename T> size_t chi_smem(int buf_rows, int lsm, int nsa) {
          (size_t)lsm * (sizeof(Rec<T>) + sizeof(unsigned short));
 }
 
+size_t dense_smem(int batch, int nsa) {
+  return (size_t)batch * (kDense * 32 * sizeof(float) + sizeof(int)) + (size_t)nsa * sizeof(int);
+}
+
+// A kernel's dynamic shared memory limit on each device, raised where a launch needs more.
+struct SmemLimit {
+  std::mutex mu;
+  size_t have[kMaxDevices] = {};
+  template <typename K>
+  cudaError_t raise(K kernel, int device, size_t bytes) {
+    std::lock_guard<std::mutex> lock(mu);
+    size_t& h = have[(device >= 0 && device < kMaxDevices) ? device : 0];
+    if (bytes <= h) return cudaSuccess;
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) h = bytes;
+    return e;
+  }
+};
+
 template <typename T, int KS, int KL, bool FOLD>
 cudaError_t run_chi_as(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t s) {
   const size_t sm = chi_smem<T>(q.buf_rows, q.lsm, q.a.nsa);
-  static std::mutex mu;
-  static size_t have[kMaxDevices] = {};
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    size_t& h = have[(p.device >= 0 && p.device < kMaxDevices) ? p.device : 0];
-    if (sm > h) {
-      const cudaError_t e = cudaFuncSetAttribute(
-          chi_kernel<T, KS, KL, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e != cudaSuccess) return e;
-      h = sm;
-    }
-  }
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(chi_kernel<T, KS, KL, FOLD>, p.device, sm);
+  if (e != cudaSuccess) return e;
   chi_kernel<T, KS, KL, FOLD><<<dim3(c.b1 - c.b0, p.natm, q.parts), 32 * q.warps, sm, s>>>(
       q, (cplx_t<T>*)p.chi->chi, c.b0);
   return cudaGetLastError();
 }
+cudaError_t run_dense(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t s) {
+  const size_t sm = dense_smem(q.batch, q.a.nsa);
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(chi_dense_kernel, p.device, sm);
+  if (e != cudaSuccess) return e;
+  chi_dense_kernel<<<dim3(c.b1 - c.b0, p.natm, q.parts), 32 * kWarps, sm, s>>>(
+      q, (float2*)p.chi->chi, c.b0);
+  return cudaGetLastError();
+}
 template <typename T, int KS, int KL>
 cudaError_t run_chi(const Plan& p, const Params& q, const ChiChunk& c, cudaStream_t s) {
+  if constexpr (sizeof(T) == 4)
+    if (q.batch > 0) return run_dense(p, q, c, s);
   return q.ncls <= kFold ? run_chi_as<T, KS, KL, true>(p, q, c, s)
                          : run_chi_as<T, KS, KL, false>(p, q, c, s);
 }
@@ -1264,11 +1422,22 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
       slots = (slots + chi::kPad - 1) / chi::kPad * chi::kPad;
       aoff[(size_t)b * (natm + 1) + a + 1] = aoff[(size_t)b * (natm + 1) + a] + slots;
     }
-  // residue classes of T0 + T' modulo the k-mesh's supercell, a table row per distinct T0
+  // Wide shells go through the transform over classes where the mesh is (nearly) full, its
+  // k-points are distinct and its lengths are compiled; columns as the shared memory allows.
   const int Dc = p->D[0] * p->D[1] * p->D[2], nimg = p->nimg;
-  const bool identity = Dc <= 4096;   // class = residue; beyond, the residues in use
+  bool dft = Dc <= 4096 && Dc <= 4 * p->nk;
+  for (int d = 0; d < 3; ++d) dft = dft && (p->D[d] <= 6 || p->D[d] == 8);
+  std::vector<int> kidx(dft ? Dc : 1, -1);
+  for (int k = 0; k < p->nk && dft; ++k) {
+    const int r = (p->kint_h[3 * k] * p->D[1] + p->kint_h[3 * k + 1]) * p->D[2] + p->kint_h[3 * k + 2];
+    if (kidx[r] >= 0) dft = false;
+    kidx[r] = k;
+  }
+  t->signs = dft && Dc <= chi::kFold && p->D[0] <= 2 && p->D[1] <= 2 && p->D[2] <= 2;
+  // residue classes of T0 + T' modulo the k-mesh's supercell, a table row per distinct T0; the
+  // transform takes class = residue, other meshes number the residues in use
   std::vector<int> id(Dc, -1), residue, cls, seen;
-  if (identity) {
+  if (dft) {
     residue.resize(Dc);
     std::iota(residue.begin(), residue.end(), 0);
     id = residue;
@@ -1298,6 +1467,12 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   t->ncls = std::max(1, (int)residue.size());
   t->nkp = (p->nk + 7) / 8 * 8;
   std::vector<double2> phase((size_t)t->ncls * t->nkp, make_double2(0.0, 0.0));
+  std::vector<double2> unit(residue.size() * p->nk > (size_t)Dc ? Dc : 0);   // e^{2 pi i n / Dc}
+  auto root = [&](long long num) {
+    const double ang = 2.0 * 3.14159265358979323846 * (double)num / (double)Dc;
+    return make_double2(std::cos(ang), std::sin(ang));
+  };
+  for (size_t n = 0; n < unit.size(); ++n) unit[n] = root((long long)n);
   for (size_t c = 0; c < residue.size(); ++c) {
     const int n[3] = {residue[c] / (p->D[1] * p->D[2]), residue[c] / p->D[2] % p->D[1],
                       residue[c] % p->D[2]};
@@ -1305,22 +1480,14 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
       long long num = 0;
       for (int d = 0; d < 3; ++d) num += (long long)p->kint_h[k * 3 + d] * n[d] * (Dc / p->D[d]);
       num %= Dc;
-      const double ang = 2.0 * 3.14159265358979323846 * (double)num / (double)Dc;
-      phase[c * t->nkp + k] = make_double2(std::cos(ang), std::sin(ang));
+      phase[c * t->nkp + k] = unit.empty() ? root(num) : unit[num];
     }
   }
-  // Wide shells go through the transform over classes where the mesh is (nearly) full, its
-  // k-points are distinct and its lengths are compiled; columns as the shared memory allows.
-  std::vector<int> kidx(identity ? Dc : 1, -1);
-  bool dft = identity && Dc <= 4 * p->nk;
-  for (int d = 0; d < 3; ++d) dft = dft && (p->D[d] <= 6 || p->D[d] == 8);
-  for (int k = 0; k < p->nk && dft; ++k) {
-    const int r = (p->kint_h[3 * k] * p->D[1] + p->kint_h[3 * k + 1]) * p->D[2] + p->kint_h[3 * k + 2];
-    if (kidx[r] >= 0) dft = false;
-    kidx[r] = k;
-  }
-  t->signs = dft && Dc <= chi::kFold && p->D[0] <= 2 && p->D[1] <= 2 && p->D[2] <= 2;
-  dft = dft && Dc > chi::kFold;   // up to kFold classes every shell takes one warp (fold_shell)
+  // Up to kFold classes every shell takes one warp (fold_shell). With few shells in all, a CTA
+  // per atom and block would transform its columns on a nearly idle GPU: on many k-points
+  // chi_dense_kernel spreads those instead (6x6x8 k, 10 AOs, 8^3: orbitals 100 -> 68 us).
+  const long long shells_all = (long long)nblk * natm * nsa;
+  dft = dft && Dc > chi::kFold && (fp64 || p->nk < 128 || shells_all >= 152 * 8);
   // chunks of blocks, offsets, and the contraction's items
   const size_t csz = (fp64 ? sizeof(double) : sizeof(float)) * (t->signs ? 1 : 2);
   const size_t slot_bytes = csz * 32 * (size_t)p->nk;
@@ -1423,7 +1590,18 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
                            : chi::chi_smem<float>(t->buf_rows, lmax, nsa);
   t->lsm = need <= 200 * 1024 ? lmax : 0;
   // several CTAs per (block, atom) where there are few of them (a Gamma cell)
-  t->parts = std::max(1, std::min(4, (int)(152LL * 4 / ((long long)nblk * natm))));
+  long long parts = 152LL * 4 / ((long long)nblk * natm);
+  if (!fp64 && !dft && p->nk >= chi::kDenseK) {
+    // batches of about equal size; the CTAs of a (block, atom) share the k-points
+    const int nb = (lmax + chi::kDenseImages - 1) / chi::kDenseImages;
+    t->batch = (lmax + nb - 1) / nb;
+    parts = std::min<long long>(parts, p->nk / (chi::KD * chi::kWarps));
+  } else {
+    // many k-points on a small grid: slices of them for narrow shells, a warp each
+    t->kslices = (int)std::max(1LL, std::min(p->nk / 32LL, 152LL * 16 / shells_all));
+    parts = std::min<long long>(std::max(4, (nsa * t->kslices + t->warps - 1) / t->warps), parts);
+  }
+  t->parts = (int)std::max(1LL, parts);
 
   std::vector<float2> phase_f;
   if (!fp64)

@@ -36,6 +36,8 @@ struct ChiTables {
   int buf_rows = 0, warps = 0;    // rows of chi_kernel's buffer, warps of its CTAs
   int signs = 0;                  // every phase of the mesh is a sign (axes of one or two points)
   int parts = 1;                  // CTAs per (block, atom) of chi_kernel
+  int kslices = 1;                // slices of the k-points that warps take of a narrow shell
+  int batch = 0;                  // images per batch of chi_dense_kernel (0: not this mesh)
   int tile = 0;                   // slots per item of the tensor-core contraction, 0 without it
   long long item_pairs = 0;       // pairs of blocks over the tensor-core items
   size_t chi_bytes = 0;
@@ -87,7 +89,7 @@ struct Params {
   const float* row_scale;
   const double* ao_norm;
   const int* kidx;
-  int nslots, ncls, nkp, lsm, parts, ncol, col_rows, buf_rows, warps, signs;
+  int nslots, ncls, nkp, lsm, parts, ncol, col_rows, buf_rows, warps, signs, batch, kslices;
 };
 
 Params params(const Plan& p);

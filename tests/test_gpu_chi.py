@@ -105,6 +105,48 @@ def test_orbitals_two_blocks_per_warp(ragged, nocc):
     assert np.abs(got - psi).max() <= 2e-6 * np.abs(psi).max()
 
 
+def _half_shifted(n):
+    ax = (np.arange(n) + 0.5) / n
+    return np.stack(np.meshgrid(ax, ax, ax, indexing="ij"), -1).reshape(-1, 3)
+
+
+MANY_K = {
+    # a length that the transform does not take, k-points past a group of four; about 340 images,
+    # four batches; groups of one to eight AOs (s and p together, d with s, f alone)
+    "axis17": dict(kfrac=[[0, 0, j / 17] for j in range(17)], counts=(3, 2, 1, 1), lo=0.12),
+    # several CTAs share the k-points
+    "shifted": dict(kfrac=_half_shifted(4), counts=(2, 1, 1), lo=0.15),
+    # one batch of a few images, blocks that some shells do not reach
+    "tight": dict(kfrac=[[0, j / 16, 0.5] for j in range(16)], counts=(2, 2, 1), a_ang=6.0,
+                  lo=0.4, hi=20.0),
+}
+
+
+@pytest.mark.parametrize("name", list(MANY_K))
+def test_many_k_points_without_the_transform(name):
+    """chi_dense_kernel (FP32) and a narrow shell's slices of the k-points (FP64) against the oracle,
+    and the tiles in the contraction against FP64."""
+    import torch
+    import paper_2207_09028_gb300 as occri
+    case = dict(MANY_K[name])
+    kfrac = case.pop("kfrac")
+    w = small_workload(mesh=(1, 1, 1), grid=(9, 9, 9), nocc=2, seed=33, complex_c=True, **case)
+    w = _with_kfrac(w, kfrac)
+    chi = O.bloch_aos(w.lattice, w.xyz, w.shell_atom, w.shell_l, w.shell_alpha, w.kfrac,
+                      grid=w.grid)
+    psi = O.orbitals_on_grid(chi, w.C)
+    C = torch.from_numpy(w.C).cuda()
+    # as above: sqrt(n) u with a margin of about 3, for n of about 350
+    for precision, bar in (("fp64", 1e-12), ("mixed", 4e-6)):
+        plan = occri.Plan.from_workload(w, precision=precision)
+        got = plan.orbitals(C).cpu().numpy().reshape(psi.shape)
+        assert np.abs(got - psi).max() <= bar * np.abs(psi).max(), precision
+    ref = occri.Plan.from_workload(w, precision="fp64").build(C)[0]
+    for precision in ("mixed", "mixed_tc"):
+        kc = occri.Plan.from_workload(w, precision=precision).build(C)[0]
+        assert (kc - ref).abs().max() <= 1e-5 * ref.abs().max()
+
+
 def test_adjoint_of_a_tensor_core_plan():
     """The adjoint contracts on the CUDA cores in every plan: over items of their own."""
     import torch
