@@ -932,54 +932,31 @@ orb_kernel(Params p, const chi_t<T, REAL>* __restrict__ chi, const typename CsT<
   }
 }
 
-// Sum over the lanes of a warp of NV values per lane, by halving: after the exchange over lane
-// bit b each lane keeps half of its values. Lane l ends with the sums of the values j with
-// j mod (NV / 32) free and the rest its bit-reversed position (index returned through idx).
-// FP32 values travel as hi + lo pairs (error-free sums), so nothing is lost across lanes.
-__device__ __forceinline__ void pair_add(float& ah, float& al, float bh, float bl) {
-  float s, e;
-  ao::two_sum(ah, bh, s, e);
-  ah = s;
-  al = al + bl + e;
-}
+// Sum in FP64 over the lanes of a warp of NV values per lane, by halving: after the exchange over
+// lane bit b each lane keeps half of its values. Lane l ends with the sums of the values
+// l (NV / 32) + j.
 template <typename T, int NV>
-__device__ __forceinline__ void halve_lanes(T (&v)[NV], double (&out)[NV / 32], int lane) {
+__device__ __forceinline__ void halve_lanes(const T (&v)[NV], double (&out)[NV / 32], int lane) {
   static_assert(NV % 32 == 0, "a whole number of values per lane");
-  if constexpr (sizeof(T) == 8) {
+  double w[NV / 2];   // the first exchange is of the working precision's values
 #pragma unroll
-    for (int step = 0; step < 5; ++step) {
-      const int half = NV >> (step + 1);
-      const bool up = (lane >> (4 - step)) & 1;
-#pragma unroll
-      for (int j = 0; j < half; ++j) {
-        const T mine = up ? v[j + half] : v[j], other = up ? v[j] : v[j + half];
-        v[j] = mine + __shfl_xor_sync(0xffffffffu, other, 16 >> step);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < NV / 32; ++j) out[j] = v[j];
-  } else {
-    T lo[NV];
-#pragma unroll
-    for (int j = 0; j < NV; ++j) lo[j] = T(0);
-#pragma unroll
-    for (int step = 0; step < 5; ++step) {
-      const int half = NV >> (step + 1);
-      const bool up = (lane >> (4 - step)) & 1;
-#pragma unroll
-      for (int j = 0; j < half; ++j) {
-        T mh = up ? v[j + half] : v[j], ml = up ? lo[j + half] : lo[j];
-        const T oh = up ? v[j] : v[j + half], ol = up ? lo[j] : lo[j + half];
-        const T rh = __shfl_xor_sync(0xffffffffu, oh, 16 >> step);
-        const T rl = step ? __shfl_xor_sync(0xffffffffu, ol, 16 >> step) : T(0);
-        pair_add(mh, ml, rh, rl);
-        v[j] = mh;
-        lo[j] = ml;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < NV / 32; ++j) out[j] = (double)v[j] + (double)lo[j];
+  for (int j = 0; j < NV / 2; ++j) {
+    const bool up = (lane >> 4) & 1;
+    const T mine = up ? v[j + NV / 2] : v[j], other = up ? v[j] : v[j + NV / 2];
+    w[j] = (double)mine + (double)__shfl_xor_sync(0xffffffffu, other, 16);
   }
+#pragma unroll
+  for (int step = 1; step < 5; ++step) {
+    const int half = NV >> (step + 1);
+    const bool up = (lane >> (4 - step)) & 1;
+#pragma unroll
+    for (int j = 0; j < half; ++j) {
+      const double mine = up ? w[j + half] : w[j], other = up ? w[j] : w[j + half];
+      w[j] = mine + __shfl_xor_sync(0xffffffffu, other, 16 >> step);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < NV / 32; ++j) out[j] = w[j];
 }
 
 // Partial sums over r of conj(chi) F: a warp takes kPad AOs of an atom over a run of the blocks
