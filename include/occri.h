@@ -89,7 +89,7 @@ typedef enum {
  *   real GEMM over the grid points: rows Re and Im of the Bloch AOs, columns Re and Im of Y,
  *   both split into FP16 hi + lo parts with power-of-two scalings, three FP16 products with
  *   FP32 accumulation per term; each 16-point product leaves tensor memory after its stage
- *   into FP32 running sums over at most 64 blocks of 32 points, and FP64 sums beyond. */
+ *   into FP32 running sums over at most 16 blocks of 32 points, and FP64 sums beyond. */
 typedef enum { OCCRI_FP64 = 0, OCCRI_MIXED = 1, OCCRI_MIXED_TC = 2 } occri_precision;
 
 typedef struct {

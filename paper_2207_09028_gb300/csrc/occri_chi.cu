@@ -1507,15 +1507,15 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   auto slots = [&](int a, int b) {
     return aoff[(size_t)b * (natm + 1) + a + 1] - aoff[(size_t)b * (natm + 1) + a];
   };
-  auto run_length = [&](int width, long long want) {
+  auto run_length = [&](int width, long long want, long long most) {
     long long groups = 0;
     for (int b = 0; b < nblk; ++b)
       for (int a = 0; a < natm; ++a) groups += (slots(a, b) + width - 1) / width;
-    const int run = (int)std::max<long long>(4, std::min<long long>(64, groups * p->nk / want));
+    const int run = (int)std::max<long long>(4, std::min(most, groups * p->nk / want));
     return (run + 1) / 2 * 2;
   };
-  const int con_run = run_length(chi::kPad, 152 * 64);
-  const int tc_run = t->tile > 0 ? run_length(t->tile, 152 * 9) : 0;
+  const int con_run = run_length(chi::kPad, 152 * 64, 64);
+  const int tc_run = t->tile > 0 ? run_length(t->tile, 152 * 9, kTcBlocks) : 0;
   std::vector<int> first(natm);   // the chunk's blocks by falling number of the atom's slots
   auto make_items = [&](const ChiChunk& c, ChiItems* it, int width, int run, size_t values,
                         long long* pairs) {

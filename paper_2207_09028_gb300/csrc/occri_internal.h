@@ -326,6 +326,7 @@ cudaError_t launch_widen(const Plan& p, void* out, cudaStream_t s);
 // The tensor-core contraction (OCCRI_MIXED_TC, occri_contract_tc.cu): K_{mu i} of the
 // accumulated Y into p.kc, from the chi buffer.
 constexpr int kTcTile = 64;                 // AO slots per tile (128 rows: Re and Im)
+constexpr int kTcBlocks = 16;               // point blocks (of 32) summed in FP32 before FP64
 // At Gamma the CUDA cores take it: with one k its few items leave the tensor cores' kernel waiting
 // for its stages (24^3, 26 AOs: builds of 115 against 100 us), and the products of the CUDA cores
 // are a little more exact (K there 1.4e-7 against 1.0e-7 from FP64).
