@@ -178,8 +178,10 @@ OCCRI_HDI void dft4(T (&re)[TOT], T (&im)[TOT]) {
   re[d] = d0r - jr; im[d] = d0i - ji;
 }
 
-// Five points: the sines enter as s_1 (t3 + (s_2/s_1) t4) and s_1 ((s_2/s_1) t3 - t4), the
-// outer factor in the last multiply-adds: 32 operations.
+// Five points: the sines enter as s_1 (t3 + (s_2/s_1) t4) and s_2 (t3 - (s_1/s_2) t4), the outer
+// factor in the last multiply-adds: 32 operations. Each row has its own outer factor because of
+// the rounding in FP32: like this the transform's gain is 0.8e-8 too large, as with four rounded
+// constants (0.9e-8); with s_1 outside in both it is 1.6e-8, which no sum averages out.
 template <int SIGN, int A, int S, typename T, int TOT>
 OCCRI_HDI void dft5(T (&re)[TOT], T (&im)[TOT]) {
   constexpr CS w1 = cs2pi(1, 5), w2 = cs2pi(2, 5);
@@ -190,16 +192,17 @@ OCCRI_HDI void dft5(T (&re)[TOT], T (&im)[TOT]) {
   const T t2r = re[e2] + re[e3], t2i = im[e2] + im[e3];
   const T t3r = re[e1] - re[e4], t3i = im[e1] - im[e4];
   const T t4r = re[e2] - re[e3], t4i = im[e2] - im[e3];
-  constexpr T c1 = T(w1.c), c2 = T(w2.c), s1 = T(SIGN * w1.s), r = T(w2.s / w1.s);
+  constexpr T c1 = T(w1.c), c2 = T(w2.c), s1 = T(SIGN * w1.s), s2 = T(SIGN * w2.s),
+              r1 = T(w2.s / w1.s), r2 = T(w1.s / w2.s);
   const T p1r = fma(c2, t2r, fma(c1, t1r, ar)), p1i = fma(c2, t2i, fma(c1, t1i, ai));
   const T p2r = fma(c1, t2r, fma(c2, t1r, ar)), p2i = fma(c1, t2i, fma(c2, t1i, ai));
-  const T q1r = fma(r, t4r, t3r), q1i = fma(r, t4i, t3i);    // times i s_1 below
-  const T q2r = fma(r, t3r, -t4r), q2i = fma(r, t3i, -t4i);
+  const T q1r = fma(r1, t4r, t3r), q1i = fma(r1, t4i, t3i);    // times i s_1 below
+  const T q2r = fma(-r2, t4r, t3r), q2i = fma(-r2, t4i, t3i);  // times i s_2
   re[e0] = ar + (t1r + t2r); im[e0] = ai + (t1i + t2i);
   re[e1] = fma(-s1, q1i, p1r); im[e1] = fma(s1, q1r, p1i);
   re[e4] = fma(s1, q1i, p1r); im[e4] = fma(-s1, q1r, p1i);
-  re[e2] = fma(-s1, q2i, p2r); im[e2] = fma(s1, q2r, p2i);
-  re[e3] = fma(s1, q2i, p2r); im[e3] = fma(-s1, q2r, p2i);
+  re[e2] = fma(-s2, q2i, p2r); im[e2] = fma(s2, q2r, p2i);
+  re[e3] = fma(s2, q2i, p2r); im[e3] = fma(-s2, q2r, p2i);
 }
 
 template <int R, int SIGN, int A, int S, typename T, int TOT>
@@ -374,17 +377,17 @@ __device__ __forceinline__ void pdft5(pk::u64 (&x)[TOT]) {
   const pk::u64 t3 = pk::sub_swap(x[e1], x[e4]);
   const pk::u64 t4 = pk::sub_swap(x[e2], x[e3]);
   const pk::u64 c1 = pk::splat(float(w1.c)), c2 = pk::splat(float(w2.c));
-  constexpr float s1 = float(SIGN * w1.s), r = float(w2.s / w1.s);
+  constexpr float s1 = float(SIGN * w1.s), s2 = float(SIGN * w2.s);
+  constexpr float r1 = float(w2.s / w1.s), r2 = float(w1.s / w2.s);
   const pk::u64 p1 = pk::fma(t2, c2, pk::fma(t1, c1, a));
   const pk::u64 p2 = pk::fma(t2, c1, pk::fma(t1, c2, a));
-  const pk::u64 q1 = pk::fma(t4, pk::splat(r), t3);              // t3 + r t4
-  const pk::u64 q2 = pk::fma(t3, pk::splat(-r), t4);             // -(r t3 - t4)
-  const pk::u64 up = pk::pack(-s1, s1), dn = pk::pack(s1, -s1);  // times i s_1, -i s_1
+  const pk::u64 q1 = pk::fma(t4, pk::splat(r1), t3);
+  const pk::u64 q2 = pk::fma(t4, pk::splat(-r2), t3);
   x[e0] = pk::add(pk::add(t1, t2), a);
-  x[e1] = pk::fma(q1, up, p1);
-  x[e4] = pk::fma(q1, dn, p1);
-  x[e2] = pk::fma(q2, dn, p2);
-  x[e3] = pk::fma(q2, up, p2);
+  x[e1] = pk::fma(q1, pk::pack(-s1, s1), p1);   // p1 + i s_1 q1
+  x[e4] = pk::fma(q1, pk::pack(s1, -s1), p1);
+  x[e2] = pk::fma(q2, pk::pack(-s2, s2), p2);
+  x[e3] = pk::fma(q2, pk::pack(s2, -s2), p2);
 }
 
 template <int R, int SIGN, int A, int S, int TOT>
