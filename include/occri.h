@@ -175,9 +175,11 @@ typedef struct occri_plan occri_plan;
  * this call: every later call on it makes that device current for its duration and then
  * restores the caller's. Among its workspaces are the kernel tables v/(4 pi) of every integer
  * k - k' on the mesh, formed here where they take at most 4 GiB (occri_tune_t.wave_tables),
- * and a buffer for the Bloch AOs of the grid (all of them where they take at most 8 GiB and a
- * quarter of the free memory, else 1 GiB or an eighth of it), filled by every call that needs
- * them.
+ * and a buffer for the Bloch AOs of the grid, filled by every call that needs them. It is
+ * allocated last: all of them where they take at most 8 GiB and a quarter of the memory then
+ * free (less what later calls of the plan allocate), else pieces of 1 GiB or an eighth of it,
+ * and where that cannot be had pieces of half the size, down to one block of 32 points. The
+ * pieces change the order of the sums of K_{mu i} over the grid, i.e. the rounding.
  * On success *out owns a plan to be destroyed with occri_plan_destroy; on failure *out is
  * NULL. */
 int occri_plan_create(occri_plan **out, const occri_cell *cell, const occri_kmesh *kmesh,
@@ -417,8 +419,9 @@ int occri_batch_destroy(occri_batch *batch);
  *   wait limit ms (the default limit is 2000 ms). ms must lie in (0, 60000].
  * occri_debug_fail_allocation(n): the n-th device allocation made by the library from
  *   now on (n >= 1, any plan, any thread) fails as if the device were out of memory, so
- *   that the entry point making it returns OCCRI_ENOMEM after freeing what it took;
- *   n <= 0 disarms. */
+ *   that the entry point making it returns OCCRI_ENOMEM after freeing what it took (the
+ *   buffer of the Bloch AOs, a plan's last allocation, takes smaller pieces instead where
+ *   it can); n <= 0 disarms. */
 enum { OCCRI_FAULT_NONE = 0, OCCRI_FAULT_WAIT = 1 };
 int occri_plan_inject_fault(occri_plan *plan, int fault, double wait_limit_ms);
 int occri_debug_fail_allocation(int nth);

@@ -1774,6 +1774,13 @@ int occri_plan_create(occri_plan** out, const occri_cell* cell, const occri_kmes
     e = cudaHostGetDevicePointer((void**)&p->status, p->status_h, 0);
   }
   if (e == cudaSuccess) e = cudaMemset(p->ace_ok, 0, sizeof(int) * (2 * (size_t)p->nk + 1));
+  if (e == cudaSuccess) {
+    // the adjoint's fields and coefficients, the bands' and the host calls' buffers
+    const size_t nkc = sizeof(double2) * (size_t)p->nk * nao * nocc;
+    const size_t later = 2 * orb * csz + 16 * (size_t)p->nk * chi_slots(*p) * nocc + 8 * nkc +
+                         sizeof(double2) * (size_t)p->nk * nao * nao;
+    e = chi_reserve(p, later, &tot);
+  }
   if (e == cudaSuccess && p->vq)
     e = precision == OCCRI_FP64 ? launch_qtables<double>(*p, p->stream)
                                 : launch_qtables<float>(*p, p->stream);

@@ -1303,6 +1303,7 @@ int chi_slots(const Plan& p) { return p.chi->nslots; }
 void chi_free(ChiTables* t) {
   if (!t) return;
   if (t->arena) cudaFree(t->arena);
+  if (t->chunk_arena) cudaFree(t->chunk_arena);
   delete t;
 }
 
@@ -1311,9 +1312,10 @@ namespace {
 // Tables laid out one after another (256-byte steps) for one allocation and one copy.
 struct Arena {
   std::vector<unsigned char> bytes;
+  static size_t align(size_t x) { return (x + 255) / 256 * 256; }
   template <typename X>
   size_t put(const std::vector<X>& v) {
-    const size_t at = (bytes.size() + 255) / 256 * 256;
+    const size_t at = align(bytes.size());
     bytes.resize(at + v.size() * sizeof(X));
     if (!v.empty()) std::memcpy(bytes.data() + at, v.data(), v.size() * sizeof(X));
     return at;
@@ -1465,20 +1467,81 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
   // chi_dense_kernel spreads those instead (6x6x8 k, 10 AOs, 8^3: orbitals 100 -> 68 us).
   const long long shells_all = (long long)nblk * natm * nsa;
   dft = dft && Dc > chi::kFold && (fp64 || p->nk < 128 || shells_all >= 152 * 8);
-  // chunks of blocks, offsets, and the contraction's items
-  const size_t csz = (fp64 ? sizeof(double) : sizeof(float)) * (t->signs ? 1 : 2);
-  const size_t slot_bytes = csz * 32 * (size_t)p->nk;
-  size_t all = 0, widest = 0;
-  for (int b = 0; b < nblk; ++b) {
-    const size_t n = slot_bytes * aoff[(size_t)b * (natm + 1) + natm];
-    all += n;
-    widest = std::max(widest, n);
+  t->aoff_h = aoff;
+  const int row_bytes = 32 * (fp64 ? 8 : 4);
+  t->col_rows = 2 * (p->D[0] / 2 + 1) * p->D[1] * p->D[2];
+  // 88 KB of columns leave room for two CTAs per SM; where that is under four AOs, one CTA
+  const long long col_bytes = (long long)t->col_rows * row_bytes;
+  const long long cols = (88 * 1024 / col_bytes >= 4 ? 88 : 176) * 1024 / col_bytes;
+  t->ncol = dft ? (int)std::min<long long>(chi::kCols, cols) : 0;
+  // without the transform nothing crosses warps: smaller CTAs
+  t->warps = t->ncol > 0 ? chi::kWarps : chi::kFoldWarps;
+  t->buf_rows = std::max(t->ncol * t->col_rows, t->warps * chi::kRows);
+  const size_t need = fp64 ? chi::chi_smem<double>(t->buf_rows, lmax, nsa)
+                           : chi::chi_smem<float>(t->buf_rows, lmax, nsa);
+  t->lsm = need <= 200 * 1024 ? lmax : 0;
+  // several CTAs per (block, atom) where there are few of them (a Gamma cell)
+  long long parts = 152LL * 4 / ((long long)nblk * natm);
+  if (!fp64 && !dft && p->nk >= chi::kDenseK) {
+    // batches of about equal size; the CTAs of a (block, atom) share the k-points
+    const int nb = (lmax + chi::kDenseImages - 1) / chi::kDenseImages;
+    t->batch = (lmax + nb - 1) / nb;
+    parts = std::min<long long>(parts, p->nk / (chi::KD * chi::kWarps));
+  } else {
+    // many k-points on a small grid: slices of them for narrow shells, a warp each
+    t->kslices = (int)std::max(1LL, std::min(p->nk / 32LL, 152LL * 16 / shells_all));
+    parts = std::min<long long>(std::max(4, (nsa * t->kslices + t->warps - 1) / t->warps), parts);
   }
-  size_t free_b = 0, dev_b = 0;
-  if (cudaMemGetInfo(&free_b, &dev_b) != cudaSuccess) return cudaGetLastError();
-  const size_t budget = all <= std::min(kChiKeepBytes, free_b / 4)
-                            ? std::max<size_t>(all, 1)
-                            : std::max(widest, std::min(kChiChunkBytes, free_b / 8));
+  t->parts = (int)std::max(1LL, parts);
+
+  std::vector<float2> phase_f;
+  if (!fp64)
+    for (const double2& z : phase) phase_f.push_back(make_float2((float)z.x, (float)z.y));
+  Arena tab;
+  const size_t o_sh = tab.put(shells), o_s0 = tab.put(slot0), o_ao = tab.put(slot_ao),
+               o_nsh = tab.put(nsh), o_aoff = tab.put(aoff), o_t0i = tab.put(t0i),
+               o_cls = tab.put(cls), o_ph = fp64 ? tab.put(phase) : tab.put(phase_f),
+               o_rs = tab.put(row_scale), o_ki = tab.put(kidx);
+  // then the lists in order of class (for the wide shells)
+  const bool sorted = t->ncol > 0;
+  const size_t o_ord = Arena::align(tab.bytes.size());
+  const size_t bytes = o_ord + (sorted ? sizeof(short) * (size_t)natm * nblk * lmax : 0);
+  *total += bytes;
+  cudaError_t e = device_malloc(&t->arena, bytes);
+  if (e != cudaSuccess) return e;
+  e = cudaMemcpy(t->arena, tab.bytes.data(), tab.bytes.size(), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return e;
+  unsigned char* d = (unsigned char*)t->arena;
+  t->shells = (ChiShell*)(d + o_sh);
+  t->slot0 = (int*)(d + o_s0);
+  t->slot_ao = (int*)(d + o_ao);
+  t->nsh = (unsigned short*)(d + o_nsh);
+  t->aoff = (int*)(d + o_aoff);
+  t->t0i = (unsigned short*)(d + o_t0i);
+  t->cls = (int*)(d + o_cls);
+  t->phase = d + o_ph;
+  t->row_scale = (float*)(d + o_rs);
+  t->kidx = (int*)(d + o_ki);
+  if (sorted) {
+    t->order = (unsigned short*)(d + o_ord);   // after the copies, on their stream
+    chi::order_kernel<<<(natm * nblk + 7) / 8, 256>>>(chi::params(*p), t->order);
+    e = cudaGetLastError();
+  }
+  return e;
+}
+
+namespace {
+
+// Chunks of blocks of at most `budget` bytes of chi (one block at least), the contractions' work
+// items in them, and their memory, whose device addresses go to t.
+cudaError_t chi_layout(Plan* p, size_t budget, size_t slot_bytes, size_t* total) {
+  ChiTables* t = p->chi;
+  const int natm = p->natm, nblk = p->nblk;
+  const bool fp64 = p->precision == OCCRI_FP64;
+  const std::vector<int>& aoff = t->aoff_h;
+  t->chunks.clear();
+  t->chi_bytes = t->part_bytes = 0;
+  t->item_pairs = 0;
   std::vector<long long> boff(nblk, 0);
   {
     ChiChunk c;
@@ -1554,79 +1617,53 @@ cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vect
     if (t->tile > 0)
       make_items(c, &c.tc, t->tile, tc_run, tc_item_values(p->nocc), &t->item_pairs);
   }
-  const int row_bytes = 32 * (fp64 ? 8 : 4);
-  t->col_rows = 2 * (p->D[0] / 2 + 1) * p->D[1] * p->D[2];
-  // 88 KB of columns leave room for two CTAs per SM; where that is under four AOs, one CTA
-  const long long col_bytes = (long long)t->col_rows * row_bytes;
-  const long long cols = (88 * 1024 / col_bytes >= 4 ? 88 : 176) * 1024 / col_bytes;
-  t->ncol = dft ? (int)std::min<long long>(chi::kCols, cols) : 0;
-  // without the transform nothing crosses warps: smaller CTAs
-  t->warps = t->ncol > 0 ? chi::kWarps : chi::kFoldWarps;
-  t->buf_rows = std::max(t->ncol * t->col_rows, t->warps * chi::kRows);
-  const size_t need = fp64 ? chi::chi_smem<double>(t->buf_rows, lmax, nsa)
-                           : chi::chi_smem<float>(t->buf_rows, lmax, nsa);
-  t->lsm = need <= 200 * 1024 ? lmax : 0;
-  // several CTAs per (block, atom) where there are few of them (a Gamma cell)
-  long long parts = 152LL * 4 / ((long long)nblk * natm);
-  if (!fp64 && !dft && p->nk >= chi::kDenseK) {
-    // batches of about equal size; the CTAs of a (block, atom) share the k-points
-    const int nb = (lmax + chi::kDenseImages - 1) / chi::kDenseImages;
-    t->batch = (lmax + nb - 1) / nb;
-    parts = std::min<long long>(parts, p->nk / (chi::KD * chi::kWarps));
-  } else {
-    // many k-points on a small grid: slices of them for narrow shells, a warp each
-    t->kslices = (int)std::max(1LL, std::min(p->nk / 32LL, 152LL * 16 / shells_all));
-    parts = std::min<long long>(std::max(4, (nsa * t->kslices + t->warps - 1) / t->warps), parts);
-  }
-  t->parts = (int)std::max(1LL, parts);
-
-  std::vector<float2> phase_f;
-  if (!fp64)
-    for (const double2& z : phase) phase_f.push_back(make_float2((float)z.x, (float)z.y));
   Arena tab;
-  const size_t o_sh = tab.put(shells), o_s0 = tab.put(slot0), o_ao = tab.put(slot_ao),
-               o_nsh = tab.put(nsh), o_aoff = tab.put(aoff), o_boff = tab.put(boff),
-               o_t0i = tab.put(t0i), o_cls = tab.put(cls),
-               o_ph = fp64 ? tab.put(phase) : tab.put(phase_f), o_it = tab.put(items),
-               o_bd = tab.put(border), o_rows = tab.put(rows), o_ro = tab.put(rows_of),
-               o_rs = tab.put(row_scale), o_ki = tab.put(kidx);
-  // then the lists in order of class (for the wide shells), the items' sums
-  // and chi
-  const bool sorted = t->ncol > 0;
-  auto align = [](size_t x) { return (x + 255) / 256 * 256; };
-  const size_t o_ord = align(tab.bytes.size());
-  const size_t o_part = align(o_ord + (sorted ? sizeof(short) * (size_t)natm * nblk * lmax : 0));
-  const size_t o_chi = align(o_part + t->part_bytes);
+  const size_t o_boff = tab.put(boff), o_it = tab.put(items), o_bd = tab.put(border),
+               o_rows = tab.put(rows), o_ro = tab.put(rows_of);
+  const size_t o_part = Arena::align(tab.bytes.size());   // the items' sums, then chi
+  const size_t o_chi = Arena::align(o_part + t->part_bytes);
   const size_t bytes = o_chi + std::max<size_t>(t->chi_bytes, 16);
+  cudaError_t e = device_malloc(&t->chunk_arena, bytes);
+  if (e != cudaSuccess) return e;
+  e = cudaMemcpy(t->chunk_arena, tab.bytes.data(), tab.bytes.size(), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return e;
   *total += bytes;
-  cudaError_t e = device_malloc(&t->arena, bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpy(t->arena, tab.bytes.data(), tab.bytes.size(), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return e;
-  unsigned char* d = (unsigned char*)t->arena;
-  t->shells = (ChiShell*)(d + o_sh);
-  t->slot0 = (int*)(d + o_s0);
-  t->slot_ao = (int*)(d + o_ao);
-  t->nsh = (unsigned short*)(d + o_nsh);
-  t->aoff = (int*)(d + o_aoff);
+  unsigned char* d = (unsigned char*)t->chunk_arena;
   t->boff = (long long*)(d + o_boff);
-  t->t0i = (unsigned short*)(d + o_t0i);
-  t->cls = (int*)(d + o_cls);
-  t->phase = d + o_ph;
   t->items = (int4*)(d + o_it);
   t->border = (int*)(d + o_bd);
   t->rows = (int2*)(d + o_rows);
   t->rows_of = (int2*)(d + o_ro);
-  t->row_scale = (float*)(d + o_rs);
-  t->kidx = (int*)(d + o_ki);
   t->part = (double*)(d + o_part);
   t->chi = d + o_chi;
-  if (sorted) {
-    t->order = (unsigned short*)(d + o_ord);   // after the copies, on their stream
-    chi::order_kernel<<<(natm * nblk + 7) / 8, 256>>>(chi::params(*p), t->order);
-    e = cudaGetLastError();
+  return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t chi_reserve(Plan* p, size_t later, size_t* total) {
+  const ChiTables& t = *p->chi;
+  const size_t csz = (p->precision == OCCRI_FP64 ? sizeof(double) : sizeof(float)) * (t.signs ? 1 : 2);
+  const size_t slot_bytes = csz * 32 * (size_t)p->nk;
+  size_t all = 0, widest = 0;
+  for (int b = 0; b < p->nblk; ++b) {
+    const size_t n = slot_bytes * t.aoff_h[(size_t)b * (p->natm + 1) + p->natm];
+    all += n;
+    widest = std::max(widest, n);
   }
-  return e;
+  size_t free_b = 0, dev_b = 0;
+  if (cudaMemGetInfo(&free_b, &dev_b) != cudaSuccess) return cudaGetLastError();
+  const size_t room = free_b > later ? free_b - later : 0;
+  size_t budget = all <= std::min(kChiKeepBytes, room / 4)
+                      ? std::max<size_t>(all, 1)
+                      : std::max(widest, std::min(kChiChunkBytes, room / 8));
+  while (true) {
+    const cudaError_t e = chi_layout(p, budget, slot_bytes, total);
+    // no memory: smaller chunks, down to one block
+    if (e != cudaErrorMemoryAllocation || t.chi_bytes <= widest) return e;
+    cudaGetLastError();
+    budget = std::max(widest, t.chi_bytes / 2);
+  }
 }
 
 template cudaError_t launch_slot_c<float>(const Plan&, const double2*, void*, double, cudaStream_t);

@@ -61,7 +61,9 @@ struct ChiTables {
   float* row_scale = nullptr;     // [nslots] tensor-core contraction: FP16 scale of a slot
   size_t part_bytes = 0;
   void* chi = nullptr;            // [block][k][slot][32 points], complex, or real with signs
-  void* arena = nullptr;          // the one allocation behind all of these
+  void* arena = nullptr;          // the allocation behind the tables
+  void* chunk_arena = nullptr;    // that of what depends on the chunks: boff to rows_of, part, chi
+  std::vector<int> aoff_h;        // aoff on the host
 };
 
 namespace chi {

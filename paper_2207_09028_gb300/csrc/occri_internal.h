@@ -248,14 +248,18 @@ constexpr int kPhasePadK = 4;
 // costs about what forming chi does, so more memory than this buys little.)
 constexpr size_t kChiKeepBytes = (size_t)8 << 30;
 constexpr size_t kChiChunkBytes = (size_t)1 << 30;
-// Tables and buffer of the plan's AOs (occri_chi.cu), from the shells, their screening radii,
-// the image lists of every (atom, block) with their prefixes, the lattice coordinates of the
-// images and the blocks' T0. What it allocated is freed by chi_free, also after a failure.
+// Tables of the plan's AOs (occri_chi.cu), from the shells, their screening radii, the image
+// lists of every (atom, block) with their prefixes, the lattice coordinates of the images and the
+// blocks' T0. What it allocated is freed by chi_free, also after a failure.
 cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vector<double>& rcut,
                        const std::vector<std::vector<unsigned short>>& lists,
                        const std::vector<unsigned short>& bpre, const std::vector<int>& img_n,
                        const std::vector<int>& t0, const std::vector<int>& atom_shell0,
                        size_t* total);
+// The chi buffer and the work items of its chunks, after everything else that the plan needs: they
+// take what leaves `later` bytes (of calls that allocate when first made) and three quarters of
+// the rest free, and where even that cannot be had, chunks of half the size, down to one block.
+cudaError_t chi_reserve(Plan* p, size_t later, size_t* total);
 void chi_free(ChiTables* t);
 int chi_slots(const Plan& p);      // rows of a coefficient table (AOs in slot order, padded)
 int chi_launches(const Plan& p, bool contract);   // kernels of the orbitals or the contraction

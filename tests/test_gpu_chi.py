@@ -147,6 +147,61 @@ def test_many_k_points_without_the_transform(name):
         assert (kc - ref).abs().max() <= 1e-5 * ref.abs().max()
 
 
+@pytest.mark.parametrize("mesh", [(1, 1, 2), (1, 1, 3)])   # real and complex tiles
+@pytest.mark.parametrize("precision", ["fp64", "mixed", "mixed_tc"])
+def test_aos_in_chunks(precision, mesh):
+    """Without the memory for all tiles a plan takes them in chunks: the same orbitals, and the same
+    sums but for their order."""
+    import torch
+    import paper_2207_09028_gb300 as occri
+    w = small_workload(mesh=mesh, grid=(15, 15, 15), counts=(3, 2, 1), nocc=3, seed=47)
+    C = torch.from_numpy(w.C).cuda()
+    rng = np.random.default_rng(8)
+    G = torch.from_numpy(rng.standard_normal((w.nk, w.nao, w.nao)) + 0j).cuda()
+
+    def results(plan):
+        psi = plan.orbitals(C).clone()
+        kc = plan.build(C)[0]
+        return psi, kc, plan.vjp_full(C, 0.3, None, G), plan.info()["launches_per_build"]
+
+    whole = results(occri.Plan.from_workload(w, precision=precision))
+    for nth in range(1, 60):   # the first failure that a plan survives is that of its tiles
+        occri.fail_allocation(nth)
+        try:
+            plan = occri.Plan.from_workload(w, precision=precision)
+            break
+        except occri.OccriError as e:
+            assert e.status == occri.OCCRI_ENOMEM
+        finally:
+            occri.fail_allocation(0)
+    parts = results(plan)
+    assert parts[3] > whole[3]
+    assert torch.equal(parts[0], whole[0])
+    # FP32: sums of about 3,000 points in another order, sqrt(3000) u = 3.3e-6 at most
+    tol = 1e-12 if precision == "fp64" else 3e-6
+    for x, y in zip(parts[1:3], whole[1:3]):
+        assert (x - y).abs().max() <= tol * y.abs().max()
+
+
+@pytest.mark.parametrize("mesh,nocc", [((1, 1, 3), 12), ((1, 1, 3), 20), ((1, 1, 17), 9)])
+def test_tensor_core_widths_on_complex_tiles(mesh, nocc):
+    """The tensor-core contraction of 32 and 64 columns where the tiles are complex."""
+    import torch
+    import paper_2207_09028_gb300 as occri
+    w = small_workload(mesh=mesh, grid=(9, 9, 9), counts=(6, 4, 1), nocc=nocc, seed=51)
+    chi = O.bloch_aos(w.lattice, w.xyz, w.shell_atom, w.shell_l, w.shell_alpha, w.kfrac,
+                      grid=w.grid)
+    psi = O.orbitals_on_grid(chi, w.C)
+    g0 = O.g0_value(w.kernel, w.omega, w.g0_mode, w.lattice, w.kfrac)
+    kc = O.occri_kc(w.lattice, w.grid, w.kfrac, psi, chi, w.kernel, w.omega, g0)
+    plan = occri.Plan.from_workload(w, precision="mixed_tc")
+    assert plan.info()["contraction_tc"] == 1
+    got = plan.build(torch.from_numpy(w.C).cuda())[0].cpu().numpy()
+    # the bar of the other builds above: a few FP32 roundings of each of the four orbitals of a
+    # term, at the size of the largest
+    assert np.abs(got - kc).max() <= 1e-5 * np.abs(kc).max()
+
+
 def test_adjoint_of_a_tensor_core_plan():
     """The adjoint contracts on the CUDA cores in every plan: over items of their own."""
     import torch
