@@ -154,20 +154,18 @@ __device__ __forceinline__ void orbital_shell(const AOParams& p, const ShellDev&
 
 // Scaled coefficients N_mu C^k_{mu i}, formed in FP64 (and split hi/lo for FP32).
 __global__ void scale_c_kernel_d(const double2* __restrict__ C, const double* __restrict__ nrm,
-                                 double2* __restrict__ out, int nao, int nocc, long long n,
-                                 double factor = 1.0) {
+                                 double2* __restrict__ out, int nao, int nocc, long long n) {
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x) {
-    const double s = factor * nrm[(e / nocc) % nao];
+    const double s = nrm[(e / nocc) % nao];
     out[e] = make_double2(s * C[e].x, s * C[e].y);
   }
 }
 __global__ void scale_c_kernel_f(const double2* __restrict__ C, const double* __restrict__ nrm,
-                                 float4* __restrict__ out, int nao, int nocc, long long n,
-                                 double factor = 1.0) {
+                                 float4* __restrict__ out, int nao, int nocc, long long n) {
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x) {
-    const double s = factor * nrm[(e / nocc) % nao];
+    const double s = nrm[(e / nocc) % nao];
     const double x = s * C[e].x, y = s * C[e].y;
     const float xh = (float)x, yh = (float)y;
     out[e] = make_float4(xh, yh, (float)(x - (double)xh), (float)(y - (double)yh));
@@ -178,13 +176,13 @@ __global__ void scale_c_kernel_f(const double2* __restrict__ C, const double* __
 // (168 registers, a 104-byte spill in FP32) were 7 % faster than two (255 registers).
 template <typename T, int NI, int KB>
 __global__ void __launch_bounds__(128, 3)
-orbitals_kernel(AOParams p, cplx_t<T>* __restrict__ psi, int i0, int kbase = 0) {
+orbitals_kernel(AOParams p, cplx_t<T>* __restrict__ psi, int i0) {
   const int blk = blockIdx.x * 4 + (threadIdx.x >> 5);
   if (blk >= p.nblk) return;
   bool valid;
   long long q;
   const long long n = block_point(p, blk, threadIdx.x & 31, &valid, &q);
-  const int k0 = kbase + blockIdx.y * KB;
+  const int k0 = blockIdx.y * KB;
   T ar[KB][NI], ai[KB][NI];
 #pragma unroll
   for (int b = 0; b < KB; ++b)

@@ -1708,7 +1708,7 @@ int occri_plan_create(occri_plan** out, const occri_cell* cell, const occri_kmes
   if (e == cudaSuccess) {
     std::vector<int> img_n;
     for (const Img& m : imgs) img_n.insert(img_n.end(), m.n, m.n + 3);
-    chk(chi_create(p, sh, rcut, lists, bpre, img_n, t0, atom_shell0, &tot));
+    chk(chi_create(p, sh, rcut, bpre, img_n, t0, atom_shell0, &tot));
   }
   if (e == cudaSuccess) {
     unsigned char* b = nullptr;

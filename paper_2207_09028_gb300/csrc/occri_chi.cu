@@ -1332,7 +1332,6 @@ static double shell_peak(int l, double alpha) {
 }
 
 cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vector<double>& rcut,
-                       const std::vector<std::vector<unsigned short>>& lists,
                        const std::vector<unsigned short>& bpre, const std::vector<int>& img_n,
                        const std::vector<int>& t0, const std::vector<int>& atom_shell0,
                        size_t* total) {

@@ -248,11 +248,10 @@ constexpr int kPhasePadK = 4;
 // costs about what forming chi does, so more memory than this buys little.)
 constexpr size_t kChiKeepBytes = (size_t)8 << 30;
 constexpr size_t kChiChunkBytes = (size_t)1 << 30;
-// Tables of the plan's AOs (occri_chi.cu), from the shells, their screening radii, the image
-// lists of every (atom, block) with their prefixes, the lattice coordinates of the images and the
-// blocks' T0. What it allocated is freed by chi_free, also after a failure.
+// Tables of the plan's AOs (occri_chi.cu), from the shells, their screening radii, the prefixes of
+// the image lists of every (atom, block), the lattice coordinates of the images and the blocks'
+// T0. What it allocated is freed by chi_free, also after a failure.
 cudaError_t chi_create(Plan* p, const std::vector<ShellDev>& sh, const std::vector<double>& rcut,
-                       const std::vector<std::vector<unsigned short>>& lists,
                        const std::vector<unsigned short>& bpre, const std::vector<int>& img_n,
                        const std::vector<int>& t0, const std::vector<int>& atom_shell0,
                        size_t* total);
