@@ -178,10 +178,14 @@ OCCRI_HDI void dft4(T (&re)[TOT], T (&im)[TOT]) {
   re[d] = d0r - jr; im[d] = d0i - ji;
 }
 
-// Five points: the sines enter as s_1 (t3 + (s_2/s_1) t4) and s_2 (t3 - (s_1/s_2) t4), the outer
-// factor in the last multiply-adds: 32 operations. Each row has its own outer factor because of
-// the rounding in FP32: like this the transform's gain is 0.8e-8 too large, as with four rounded
-// constants (0.9e-8); with s_1 outside in both it is 1.6e-8, which no sum averages out.
+// Five points: the sines enter as s_1 (t3 + (s_2/s_1) t4) and s_1 ((s_2/s_1) t3 - t4), the outer
+// factor in the last multiply-adds: 32 operations. In FP32 fl(s_1) fl(s_2/s_1) makes the
+// transform's gain 1.6e-8 too large, which no sum averages out. Where two stages of five follow
+// each other (25 points) that is more than rounding each constant by itself costs (3.3e-8 against
+// 1.9e-8): there the second row is s_2 (t3 - (s_1/s_2) t4) (0.8e-8 a stage, 1.7e-8). With one
+// stage the gains of whole lines stay within 0.3e-8 of those of rounded constants, and a 45-point
+// line in one thread's registers would be 2 % slower with the two constants more.
+template <int TOT> constexpr bool two_sines() { return TOT % 25 == 0; }
 template <int SIGN, int A, int S, typename T, int TOT>
 OCCRI_HDI void dft5(T (&re)[TOT], T (&im)[TOT]) {
   constexpr CS w1 = cs2pi(1, 5), w2 = cs2pi(2, 5);
@@ -197,12 +201,14 @@ OCCRI_HDI void dft5(T (&re)[TOT], T (&im)[TOT]) {
   const T p1r = fma(c2, t2r, fma(c1, t1r, ar)), p1i = fma(c2, t2i, fma(c1, t1i, ai));
   const T p2r = fma(c1, t2r, fma(c2, t1r, ar)), p2i = fma(c1, t2i, fma(c2, t1i, ai));
   const T q1r = fma(r1, t4r, t3r), q1i = fma(r1, t4i, t3i);    // times i s_1 below
-  const T q2r = fma(-r2, t4r, t3r), q2i = fma(-r2, t4i, t3i);  // times i s_2
+  constexpr T so = two_sines<TOT>() ? s2 : s1;                 // times i s_o
+  const T q2r = two_sines<TOT>() ? fma(-r2, t4r, t3r) : fma(r1, t3r, -t4r);
+  const T q2i = two_sines<TOT>() ? fma(-r2, t4i, t3i) : fma(r1, t3i, -t4i);
   re[e0] = ar + (t1r + t2r); im[e0] = ai + (t1i + t2i);
   re[e1] = fma(-s1, q1i, p1r); im[e1] = fma(s1, q1r, p1i);
   re[e4] = fma(s1, q1i, p1r); im[e4] = fma(-s1, q1r, p1i);
-  re[e2] = fma(-s2, q2i, p2r); im[e2] = fma(s2, q2r, p2i);
-  re[e3] = fma(s2, q2i, p2r); im[e3] = fma(-s2, q2r, p2i);
+  re[e2] = fma(-so, q2i, p2r); im[e2] = fma(so, q2r, p2i);
+  re[e3] = fma(so, q2i, p2r); im[e3] = fma(-so, q2r, p2i);
 }
 
 template <int R, int SIGN, int A, int S, typename T, int TOT>
@@ -382,12 +388,15 @@ __device__ __forceinline__ void pdft5(pk::u64 (&x)[TOT]) {
   const pk::u64 p1 = pk::fma(t2, c2, pk::fma(t1, c1, a));
   const pk::u64 p2 = pk::fma(t2, c1, pk::fma(t1, c2, a));
   const pk::u64 q1 = pk::fma(t4, pk::splat(r1), t3);
-  const pk::u64 q2 = pk::fma(t4, pk::splat(-r2), t3);
+  // -q2 where s_o = s_1: one multiply-add either way
+  const pk::u64 q2 = two_sines<TOT>() ? pk::fma(t4, pk::splat(-r2), t3)
+                                      : pk::fma(t3, pk::splat(-r1), t4);
+  constexpr float so = two_sines<TOT>() ? s2 : -s1;
   x[e0] = pk::add(pk::add(t1, t2), a);
   x[e1] = pk::fma(q1, pk::pack(-s1, s1), p1);   // p1 + i s_1 q1
   x[e4] = pk::fma(q1, pk::pack(s1, -s1), p1);
-  x[e2] = pk::fma(q2, pk::pack(-s2, s2), p2);
-  x[e3] = pk::fma(q2, pk::pack(s2, -s2), p2);
+  x[e2] = pk::fma(q2, pk::pack(-so, so), p2);
+  x[e3] = pk::fma(q2, pk::pack(so, -so), p2);
 }
 
 template <int R, int SIGN, int A, int S, int TOT>
