@@ -82,8 +82,9 @@ typedef enum {
 
 /* OCCRI_FP64: every step in double precision.
  * OCCRI_MIXED: AO evaluation, orbitals, pair densities, FFTs, the kernel multiply
- *   and the Y accumulation in FP32; the contraction (e) accumulates per thread in
- *   FP32 and across threads in FP64; assembly (f) and E_x in FP64.
+ *   and the Y accumulation in FP32; the contraction (e) accumulates per thread in FP32
+ *   (over at most 16 points), over the threads of a warp in 64-bit fixed point (no less
+ *   exact than FP64) and beyond in FP64; assembly (f) and E_x in FP64.
  * OCCRI_MIXED_TC: as OCCRI_MIXED, but at two and more k-points the contraction (e) runs on the
  *   tensor cores, per k as a
  *   real GEMM over the grid points: rows Re and Im of the Bloch AOs, columns Re and Im of Y,

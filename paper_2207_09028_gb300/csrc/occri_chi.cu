@@ -932,21 +932,29 @@ orb_kernel(Params p, const chi_t<T, REAL>* __restrict__ chi, const typename CsT<
   }
 }
 
-// Sum in FP64 over the lanes of a warp of NV values per lane, by halving: after the exchange over
-// lane bit b each lane keeps half of its values. Lane l ends with the sums of the values
-// l (NV / 32) + j.
-template <typename T, int NV>
-__device__ __forceinline__ void halve_lanes(const T (&v)[NV], double (&out)[NV / 32], int lane) {
-  static_assert(NV % 32 == 0, "a whole number of values per lane");
-  double w[NV / 2];   // the first exchange is of the working precision's values
+// Sums over the lanes of a warp of NV values per lane, by halving: after the exchange over lane
+// bit b each lane keeps half of its values. Lane l ends with the sums of the values
+// l (NV / 32) + j. NV words of shared memory per warp.
+//
+// FP64 values are added as they are. FP32 values are added as 64-bit integers in units of
+// 2^-57 of the largest lane's power of two, value by value: of a lane's 24 bits only those below
+// that unit are lost, so the sums are those of FP64 or better, and integer additions run at full
+// rate, where an SM adds two FP64 values per cycle (45^3, 8 k, nocc 8, items of 16 blocks: a build
+// 3.42 ms with FP64 sums of the lanes, 3.31 with these).
+__device__ __forceinline__ long long lane_fixed(unsigned bits, int e) {   // e: largest lane's exponent
+  const int x = bits >> 23 & 255;
+  const unsigned m = (bits & 0x7fffffu) | (x ? 0x800000u : 0u);
+  const unsigned long long q = ((unsigned long long)m << 40) >> min(7 + e - max(x, 1), 63);
+  return (int)bits < 0 ? -(long long)q : (long long)q;
+}
+template <int NV>
+__device__ __forceinline__ void halve_lanes(const double (&v)[NV], double (&out)[NV / 32], int lane,
+                                            unsigned*) {
+  double w[NV];
 #pragma unroll
-  for (int j = 0; j < NV / 2; ++j) {
-    const bool up = (lane >> 4) & 1;
-    const T mine = up ? v[j + NV / 2] : v[j], other = up ? v[j] : v[j + NV / 2];
-    w[j] = (double)mine + (double)__shfl_xor_sync(0xffffffffu, other, 16);
-  }
+  for (int j = 0; j < NV; ++j) w[j] = v[j];
 #pragma unroll
-  for (int step = 1; step < 5; ++step) {
+  for (int step = 0; step < 5; ++step) {
     const int half = NV >> (step + 1);
     const bool up = (lane >> (4 - step)) & 1;
 #pragma unroll
@@ -958,10 +966,53 @@ __device__ __forceinline__ void halve_lanes(const T (&v)[NV], double (&out)[NV /
 #pragma unroll
   for (int j = 0; j < NV / 32; ++j) out[j] = w[j];
 }
+template <int NV>
+__device__ __forceinline__ void halve_lanes(const float (&v)[NV], double (&out)[NV / 32], int lane,
+                                            unsigned* top) {
+  constexpr unsigned kAll = 0xffffffffu, kInf = 0x7f800000u;
+  // the largest lane's bits of value j go to top; where a lane holds an infinity or NaN, the sum's
+  auto largest = [&](int j) {
+    unsigned t = __reduce_max_sync(kAll, __float_as_uint(v[j]) & 0x7fffffffu);
+    if (t >= kInf) {   // (uniform)
+      double s = v[j];
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kAll, s, o);
+      t = __float_as_uint((float)s);
+    }
+    if (lane == 0) top[j] = t;
+    return (int)max(t >> 23 & 255u, 1u);
+  };
+  long long w[NV / 2];
+  const bool up0 = (lane >> 4) & 1;
+#pragma unroll
+  for (int j = 0; j < NV / 2; ++j) {
+    const int e0 = largest(j), e1 = largest(j + NV / 2), e = up0 ? e1 : e0;
+    const float mine = up0 ? v[j + NV / 2] : v[j], other = up0 ? v[j] : v[j + NV / 2];
+    w[j] = lane_fixed(__float_as_uint(mine), e) +
+           lane_fixed(__float_as_uint(__shfl_xor_sync(kAll, other, 16)), e);
+  }
+#pragma unroll
+  for (int step = 1; step < 5; ++step) {
+    const int half = NV >> (step + 1);
+    const bool up = (lane >> (4 - step)) & 1;
+#pragma unroll
+    for (int j = 0; j < half; ++j) {
+      const long long mine = up ? w[j + half] : w[j], other = up ? w[j] : w[j + half];
+      w[j] = mine + __shfl_xor_sync(kAll, other, 16 >> step);
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < NV / 32; ++j) {
+    const unsigned t = top[lane * (NV / 32) + j];
+    const int e = (int)max(t >> 23 & 255u, 1u);   // the unit is 2^(e - 183)
+    out[j] = (t & 0x7fffffffu) >= kInf ? (double)__uint_as_float(t)
+                                       : (double)w[j] * __hiloint2double((e + 840) << 20, 0);
+  }
+}
 
 // Partial sums over r of conj(chi) F: a warp takes kPad AOs of an atom over a run of the blocks
 // they reach (work items, made with the plan), sums per lane in the working precision, then
-// over the lanes in 64 bits. sum_kernel adds the items in a fixed order, so that the result
+// over the lanes exactly or in FP64. sum_kernel adds the items in a fixed order, so that the result
 // does not depend on the order in which they ran. What bounds it: issue and the load path, both
 // about half busy (60^3, 8 k, 94 AOs, real tiles: 0.38 ms); evaluating the AOs at each k-point
 // instead made the contraction over half of a build at 8 k, 104 AOs, 36^3.
@@ -1010,7 +1061,8 @@ con_kernel(Params p, const chi_t<T, REAL>* __restrict__ chi, const cplx_t<T>* __
     }
   }
   double sum[NV / 32];
-  halve_lanes<T, NV>(acc, sum, lane);
+  __shared__ unsigned top[8][NV];
+  halve_lanes<NV>(acc, sum, lane, top[threadIdx.x >> 5]);
   // lane l holds the values l (NV / 32) + j
   double* o = p.part + ((size_t)k * nitems + w) * NV + lane * (NV / 32);
 #pragma unroll
@@ -1562,7 +1614,9 @@ cudaError_t chi_layout(Plan* p, size_t budget, size_t slot_bytes, size_t* total)
   }
   // The contraction's items: a group of slots of an atom (kPad of them, or a tensor-core tile)
   // over up to `run` of the blocks that reach the group. `run` gives enough items to fill the
-  // GPU (about 16 warps per scheduler, or three rounds of CTAs) while the FP32 sums stay short.
+  // GPU (about 16 warps per scheduler, or three rounds of CTAs); FP32 sums, a point of a block per
+  // lane or 16 points per accumulator, go over 16 blocks at most (with 64 blocks to a lane the
+  // bands' columns at 40^3, 8 k were 1.7e-7 from FP64, with 16 1.5e-7).
   std::vector<int4> items;
   std::vector<int> border;
   std::vector<int2> rows, rows_of;
@@ -1576,7 +1630,7 @@ cudaError_t chi_layout(Plan* p, size_t budget, size_t slot_bytes, size_t* total)
     const int run = (int)std::max<long long>(4, std::min(most, groups * p->nk / want));
     return (run + 1) / 2 * 2;
   };
-  const int con_run = run_length(chi::kPad, 152 * 64, 64);
+  const int con_run = run_length(chi::kPad, 152 * 64, fp64 ? 64 : 16);
   const int tc_run = t->tile > 0 ? run_length(t->tile, 152 * 9, kTcBlocks) : 0;
   std::vector<int> first(natm);   // the chunk's blocks by falling number of the atom's slots
   auto make_items = [&](const ChiChunk& c, ChiItems* it, int width, int run, size_t values,

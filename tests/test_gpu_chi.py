@@ -202,6 +202,35 @@ def test_tensor_core_widths_on_complex_tiles(mesh, nocc):
     assert np.abs(got - kc).max() <= 1e-5 * np.abs(kc).max()
 
 
+@pytest.mark.parametrize("mesh,nocc", [((1, 1, 2), 3), ((1, 1, 3), 8)])
+def test_lane_sums_scale_and_pass_nan_on(mesh, nocc):
+    """The contraction's sums over a warp's lanes (FP32: integers scaled by the largest lane):
+    powers of two of C pass through every step exactly, zeros stay zeros and NaN stays NaN."""
+    import torch
+    import paper_2207_09028_gb300 as occri
+    w = small_workload(mesh=mesh, grid=(12, 12, 12), counts=(5, 3), nocc=nocc, seed=53)
+    plan = occri.Plan.from_workload(w, precision="mixed")
+    C = torch.from_numpy(w.C).cuda()
+
+    def kc(c):
+        return plan.k_build(c, KC=torch.empty_like(c), sync=False)[0]
+
+    ref = kc(C)
+    for e in (-20, 9):
+        assert torch.equal(kc(C * 2.0 ** e), ref * 2.0 ** (3 * e))
+    zero = C.clone()
+    zero[:, :, 1] = 0
+    got = kc(zero)
+    assert not got[:, :, 1].any() and torch.isfinite(torch.view_as_real(got)).all()
+    for bad in (float("nan"), float("inf")):
+        broken = C.clone()
+        broken[0, 0, 0] = bad
+        assert torch.isnan(torch.view_as_real(kc(broken))).all()
+    with pytest.raises(occri.OccriError):   # (the zero and NaN builds are not positive definite)
+        plan.sync()
+    assert torch.equal(kc(C), ref)
+
+
 def test_adjoint_of_a_tensor_core_plan():
     """The adjoint contracts on the CUDA cores in every plan: over items of their own."""
     import torch
