@@ -1014,7 +1014,7 @@ __device__ __forceinline__ void halve_lanes(const float (&v)[NV], double (&out)[
 // they reach (work items, made with the plan), sums per lane in the working precision, then
 // over the lanes exactly or in FP64. sum_kernel adds the items in a fixed order, so that the result
 // does not depend on the order in which they ran. What bounds it: issue and the load path, both
-// about half busy (60^3, 8 k, 94 AOs, real tiles: 0.38 ms); evaluating the AOs at each k-point
+// about half busy (60^3, 8 k, 94 AOs, real tiles: 0.51 ms); evaluating the AOs at each k-point
 // instead made the contraction over half of a build at 8 k, 104 AOs, 36^3.
 template <typename T, int NI, bool REAL>
 __global__ void __launch_bounds__(256, 2)
@@ -1614,9 +1614,9 @@ cudaError_t chi_layout(Plan* p, size_t budget, size_t slot_bytes, size_t* total)
   }
   // The contraction's items: a group of slots of an atom (kPad of them, or a tensor-core tile)
   // over up to `run` of the blocks that reach the group. `run` gives enough items to fill the
-  // GPU (about 16 warps per scheduler, or three rounds of CTAs); FP32 sums, a point of a block per
-  // lane or 16 points per accumulator, go over 16 blocks at most (with 64 blocks to a lane the
-  // bands' columns at 40^3, 8 k were 1.7e-7 from FP64, with 16 1.5e-7).
+  // GPU (about 16 warps per scheduler, or three rounds of CTAs); a lane's FP32 sums go over
+  // 16 blocks at most (with 64 the bands' columns at 40^3, 8 k were 1.7e-7 from FP64, with 16
+  // 1.5e-7).
   std::vector<int4> items;
   std::vector<int> border;
   std::vector<int2> rows, rows_of;
@@ -1631,7 +1631,7 @@ cudaError_t chi_layout(Plan* p, size_t budget, size_t slot_bytes, size_t* total)
     return (run + 1) / 2 * 2;
   };
   const int con_run = run_length(chi::kPad, 152 * 64, fp64 ? 64 : 16);
-  const int tc_run = t->tile > 0 ? run_length(t->tile, 152 * 9, kTcBlocks) : 0;
+  const int tc_run = t->tile > 0 ? run_length(t->tile, 152 * 9, tc_item_blocks(p->nocc)) : 0;
   std::vector<int> first(natm);   // the chunk's blocks by falling number of the atom's slots
   auto make_items = [&](const ChiChunk& c, ChiItems* it, int width, int run, size_t values,
                         long long* pairs) {

@@ -10,11 +10,11 @@
 // memory in the tensor cores' layout, and one thread issues the stage's three FP16 products
 // (hi.hi + hi.lo + lo.hi) into tensor memory, 16 points to an accumulator, which leave it after
 // the stage for FP32 sums in registers: sums in tensor memory round toward zero (64 points to
-// an accumulator biased E_x by 1.1e-7 relative, long sums by 1e-6). The items' sums are added in
-// a fixed order in FP64.
+// an accumulator biased E_x by 1.1e-7 relative, long sums by 1e-6). After 16 blocks these go on
+// in FP64; the items' sums are added in a fixed order.
 //
-// What bounds it: issue (74 % at 27 k, 94 AOs, 60^3: 1.18 ms), which is the split of chi, read
-// once, into its FP16 halves; with N = 16 the tensor pipe is 5 % busy. The earlier form
+// What bounds it: issue (66 % at 27 k, 94 AOs, 60^3: 1.39 ms), which is the split of chi, read
+// once, into its FP16 halves; with N = 16 the tensor pipe is 4 % busy. The earlier form
 // generated the AOs of the k-mesh's supercell in FP16 blocks instead (D_1 D_2 D_3 / 2 times the
 // products of this one, 36 % of them in reach): 2.09 of 3.43 ms of a build at 8 k, 104 AOs,
 // 36^3, 5.5 of 7.9 ms at 6 k, 50^3, and 50 of 426 ms at 64 k, 350 AOs, 60^3.
@@ -100,6 +100,12 @@ struct Smem {
   unsigned long long done;
   uint32_t tmem;
 };
+
+// FP32 sums end after kTcBlocks blocks. With 16 columns an item goes on over up to 64, its FP64 sums
+// added to in place (27 k, 94 AOs, 60^3: 1.39 ms against 1.52 with items of kTcBlocks; 48^3, 64 k
+// builds 44.2 -> 43.7 ms); wider kernels have no registers for that (nocc 20, 27 k, 30^3: 0.54
+// against 0.44 ms) and take items of kTcBlocks.
+template <int N> constexpr bool kFlush = N == 16;
 
 // One work item per CTA: kTcTile slots of an atom over a run of blocks, at one k.
 template <int N, bool REAL>
@@ -259,6 +265,25 @@ con_tc_kernel(chi::Params p, const void* __restrict__ chi, const float2* __restr
     }
     tc::tc_fence_before();
   };
+  // the item's FP64 sums, part[k][item][row][column]; this thread adds to its own
+  double* o = p.part + ((size_t)k * nitems + w) * kM * N +
+              (size_t)(32 * (warp & 3) + lane) * N + NI * (warp >> 2);
+  bool stored = false;
+  auto flush = [&]() {
+#pragma unroll
+    for (int j = 0; j < NI; j += 2) {
+      double2 t = make_double2((double)sum[j], (double)sum[j + 1]);
+      double2* d = reinterpret_cast<double2*>(o + j);
+      if (stored) {
+        const double2 u = *d;
+        t.x += u.x;
+        t.y += u.y;
+      }
+      *d = t;
+      sum[j] = sum[j + 1] = 0.f;
+    }
+    stored = true;
+  };
   bool ok = true;
   auto fetch = [&](int st) {
     load(st);
@@ -271,6 +296,8 @@ con_tc_kernel(chi::Params p, const void* __restrict__ chi, const float2* __restr
     if (st > 0) {
       ok = warp_wait(tc::smem_u32(&bar.done), (unsigned)((st - 1) & 1), wait_ns, lane);
       if (ok) take();
+      if constexpr (kFlush<N>)
+        if (st % (kTcBlocks / 2) == 0) flush();
     }
     if (ok) store();
     tc::fence_proxy_async_smem();
@@ -309,11 +336,7 @@ con_tc_kernel(chi::Params p, const void* __restrict__ chi, const float2* __restr
       warp_wait(tc::smem_u32(&bar.done), parity, wait_ns > kDrainNs ? wait_ns : kDrainNs, lane);
     if (lane == 0) fail(status);
   }
-  // part[k][item][row][column]
-  double* o = p.part + ((size_t)k * nitems + w) * kM * N +
-              (size_t)(32 * (warp & 3) + lane) * N + NI * (warp >> 2);
-#pragma unroll
-  for (int j = 0; j < NI; ++j) o[j] = (double)sum[j];
+  flush();
   tc::tc_fence_before();
   __syncthreads();   // every warp has read the accumulator
   if (warp == 0) tc::tmem_dealloc(tmem, COLS);
@@ -400,6 +423,7 @@ cudaError_t run(const Plan& p, const chi::Params& q, const ChiChunk& c, double2*
 
 }  // namespace tcc
 
+int tc_item_blocks(int nocc) { return tcc::width(nocc) == 16 ? 64 : kTcBlocks; }
 size_t tc_item_values(int nocc) { return (size_t)tcc::kM * tcc::width(nocc); }
 double tc_flops_per_stage(int nocc) { return 3.0 * 2.0 * tcc::kM * tcc::width(nocc) * tcc::kK; }
 long long tc_plan_stages(const Plan& p) { return p.chi->item_pairs * p.nk; }

@@ -334,6 +334,7 @@ constexpr int kTcBlocks = 16;               // point blocks (of 32) summed in FP
 // for its stages (24^3, 26 AOs: builds of 115 against 100 us), and the products of the CUDA cores
 // are a little more exact (K there 1.4e-7 against 1.0e-7 from FP64).
 inline bool tc_contraction(const Plan& p) { return p.precision == OCCRI_MIXED_TC && p.nk > 1; }
+int tc_item_blocks(int nocc);               // most blocks of a work item
 size_t tc_item_values(int nocc);            // sums one work item leaves
 long long tc_plan_stages(const Plan& p);    // stages (pairs of point blocks) per contraction
 int tc_plan_launches(const Plan& p);        // kernels one tensor-core contraction launches
