@@ -349,7 +349,8 @@ def tensor_roofline(info: dict, contract_ms: float, peak_tflops: float, peak_kin
     """Roofline of the tensor-core contraction: the MMA flops of its stages over the time of
     its GEMM kernels (CUDA events around each launch), against the measured dense bf16 rate
     (FP16 runs at the same rate on these tensor cores). `stage_ms`, the whole contraction
-    stage (with the Y conversion and the A-block generation), is reported beside it."""
+    stage (with the Y scales, the items' sums and any second pass over the AO tiles), is
+    reported beside it."""
     st = int(info.get("tc_stages", 0))
     fps = float(info.get("tc_flops_per_stage", 0.0))
     if not info.get("contraction_tc") or st <= 0 or contract_ms <= 0 or fps <= 0:

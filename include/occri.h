@@ -361,7 +361,7 @@ int occri_plan_stage_times(occri_plan *plan, double *ms, long long *launches, do
 /* occri_orbitals for callers that cannot allocate device memory at call time -- for
  * example hosts whose device memory is owned by another allocator. No counterpart in the
  * paper.
- * Same inputs, output and result as occri_orbitals, but the call's scratch (the
+ * Same inputs, output and (to rounding) result as occri_orbitals, but the call's scratch (the
  * normalised coefficients and the orbitals before widening) lives in one static
  * device array of OCCRI_STATIC_SCRATCH_BYTES instead of the plan's workspaces; the
  * call makes no cudaMalloc, cudaFree or other allocating call.
